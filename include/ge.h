@@ -58,7 +58,21 @@ typedef enum {
 } ge_precision;
 
 typedef enum {
-    GE_KERNEL_AUTO = 0,      /* GE_KERNEL_TEMPORAL with the built-in depth    */
+    GE_KERNEL_AUTO = 0,      /* composed steps where a call takes enough of
+                                them, else GE_KERNEL_TEMPORAL with the
+                                built-in depth.  The step is linear with
+                                constant coefficients, so k steps are one
+                                banded operator: built once per k and start
+                                parity and kept by the context, applied in one
+                                pass on the tensor cores (values and taps cut
+                                into digits whose products sum exactly; FP64:
+                                values to 2^-54 and taps to 2^-62 of the
+                                largest of 8192 neighbours, one rounding a
+                                pass) and as FP64 dot products near the walls
+                                and wherever a block of 64 points lies below
+                                2^-16 (FP32: 2^-10) of the values that reach
+                                it, down to 2^-100 of those.  The same scheme,
+                                reassociated; width k = 1; r in [1e-6, 1e6] */
     GE_KERNEL_CANONICAL = 1, /* one launch per step; Eqs. (cc)/(dd), (aa)/(bb)
                                 evaluated literally with fused multiply-adds
                                 in the order the equations print their terms

@@ -17,6 +17,7 @@
 #include <new>
 
 #include "ge_internal.h"
+#include "ge_prop.h"
 
 namespace {
 
@@ -92,6 +93,7 @@ struct ge_ctx {
     int tb_df_blocks_per_sm = 0;  // double-float kernel (GE_F64 contexts)
     ge::CanonCoef canon{};
     ge::TbParams tb{};   // launch-independent fields filled at creation
+    ge::PropState prop{}; // composed steps (GE_KERNEL_AUTO)
 };
 
 namespace {
@@ -241,6 +243,27 @@ ge_status run_tiled(ge_ctx *c, int64_t steps, int depth, bool df = false)
     return GE_OK;
 }
 
+// Composed steps (ge_prop.h); *taken = 0 when this call keeps the tiled kernel.
+ge_status run_composed(ge_ctx *c, int64_t steps, int *taken)
+{
+    *taken = 0;
+    // a requested stall times out tile loads: the tiled kernel's
+    if (c->tb.stall > 0 || !ge::prop_takes(c->n, c->r, steps, c->prec == GE_F64 ? 0 : (c->prec == GE_F32 ? 1 : 2)))
+        return GE_OK;
+    ge::PropTarget t{};
+    t.buf[0] = c->buf[0];
+    t.buf[1] = c->buf[1];
+    t.n = c->n;
+    t.r = c->r;
+    t.beta_l = c->beta_l;
+    t.beta_r = c->beta_r;
+    t.f64 = c->prec == GE_F64;
+    t.num_sms = c->num_sms;
+    t.err = c->err_dev;
+    const cudaError_t e = ge::prop_run(&c->prop, t, &c->cur, c->step, steps, taken, c->stream);
+    return e == cudaSuccess ? GE_OK : cuda_fail(e, "composed-step kernel launch");
+}
+
 // General sub-domain width k (ge_sweep.cu): up to `depth` steps per launch on
 // a tile in shared memory (multi), else, or where the width leaves too few
 // units per tile, one launch per step.
@@ -308,11 +331,8 @@ void release(ge_ctx *c)
 {
     if (!c)
         return;
-    for (int b = 0; b < 2; ++b)
-        if (c->buf[b])
-            cudaFree(c->buf[b]);
-    if (c->err_dev)
-        cudaFree(c->err_dev);
+    if (c->buf[0])
+        cudaFree(c->buf[0]);  // holds everything
     delete c;
 }
 
@@ -371,19 +391,20 @@ ge_status ge_create(ge_ctx **out, int64_t n, double r, double beta_l, double bet
         release(c);
         return cuda_fail(e, "ge_create: device query");
     }
-    const size_t bytes = (size_t)n_rows * ge::kRowBytes;
-    for (int b = 0; b < 2 && e == cudaSuccess; ++b)
-        e = cudaMalloc(&c->buf[b], bytes);
-    if (e == cudaSuccess)
-        e = cudaMalloc(reinterpret_cast<void **>(&c->err_dev), 256);
+    // one allocation for the two buffers, the error words and the composed
+    // steps' arrays (allocations and frees are most of a one-shot solve's
+    // set-up); the arrays need no initial values
+    const size_t bytes = ((size_t)n_rows * ge::kRowBytes + 255) & ~(size_t)255;
+    char *mem = nullptr;
+    e = cudaMalloc(reinterpret_cast<void **>(&mem), 2 * bytes + 256 + ge::prop_bytes(n, prec == GE_F64));
     if (e != cudaSuccess) {
         release(c);
         return cuda_fail(e, "ge_create: device allocation");
     }
-    for (int b = 0; b < 2 && e == cudaSuccess; ++b)
-        e = cudaMemsetAsync(c->buf[b], 0, bytes, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(c->err_dev, 0, 256, c->stream);
+    c->buf[0] = mem;
+    c->buf[1] = mem + bytes;
+    c->err_dev = reinterpret_cast<int *>(mem + 2 * bytes);
+    e = cudaMemsetAsync(mem, 0, 2 * bytes + 256, c->stream);
     if (e == cudaSuccess && u0_dev)
         e = cudaMemcpyAsync(c->buf[0], u0_dev, (size_t)n * elem_size(prec), cudaMemcpyDeviceToDevice,
                             c->stream);
@@ -393,6 +414,7 @@ ge_status ge_create(ge_ctx **out, int64_t n, double r, double beta_l, double bet
         release(c);
         return cuda_fail(e, "ge_create: initialising buffers");
     }
+    ge::prop_carve(&c->prop, reinterpret_cast<char *>(c->err_dev) + 256, n, prec == GE_F64);
     fill_coefficients(c);
     c->depth = table_depth(prec, n);
     ge_status st = make_tensor_maps(c);
@@ -402,6 +424,8 @@ ge_status ge_create(ge_ctx **out, int64_t n, double r, double beta_l, double bet
     }
     const int prec_idx = prec == GE_F64 ? 0 : (prec == GE_F32 ? 1 : 2);
     e = ge::tb_occupancy(prec_idx, &c->tb_blocks_per_sm);
+    if (e == cudaSuccess)
+        e = ge::prop_prepare();
     if (e == cudaSuccess && prec == GE_F64) {
         e = ge::tb_df_occupancy(&c->tb_df_blocks_per_sm);
         if (e == cudaSuccess && c->tb_df_blocks_per_sm < 1)
@@ -565,8 +589,12 @@ ge_status ge_step_n(ge_ctx *c, int64_t steps)
     case GE_KERNEL_TEMPORAL_DF:
         st = run_tiled(c, steps, effective_depth(c), true);
         break;
-    default:
-        st = run_tiled(c, steps, effective_depth(c));
+    default: {
+        int taken = 0;
+        st = c->kernel == GE_KERNEL_AUTO ? run_composed(c, steps, &taken) : GE_OK;
+        if (st == GE_OK && !taken)
+            st = run_tiled(c, steps, effective_depth(c));
+    }
     }
     if (st == GE_OK)
         c->step += steps;

@@ -1,0 +1,1366 @@
+// ge_prop.cu -- the kernels of composed steps (ge_prop.h): building an
+// operator's taps by binary powering, cutting the taps into digits, applying
+// an operator on the tensor cores away from the walls (tiles) and as FP64 dot
+// products near them (dots).
+//
+// Tiles.  A value and a tap are fixed-point numbers: integers of base-256
+// digits, the value relative to the largest magnitude of its tile, the tap
+// relative to the largest tap.  Digits are small integers, exact in FP16;
+// their products sum in the FP32 accumulators of tcgen05.mma without rounding
+// while a sum stays below 2^24, and the accumulators of equal weight i + j
+// (value digit j, tap digit i) join as 64-bit integers.  So a tile's result
+// is the exact fixed-point sum, rounded once.
+//   FP64: values to 2^-54 of the tile's largest, 7 digits; taps to about
+//     2^-62, 7 digits; the 34 products with i + j <= 7 (the rest is below
+//     2^-64 of the largest value).
+//   FP32: values to 2^-30, taps to about 2^-39, 4 digits each, 10 products.
+// Step by step the same k steps cost k multiply-adds a point on the FP64 (or
+// FP32) pipes; composed they cost the taps' width times the products on the
+// tensor cores, and the width grows with sqrt(k) only.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <cstdint>
+#include <mutex>
+
+#include "ge_internal.h"
+#include "ge_prop.h"
+#include "ge_tc.cuh"
+
+namespace ge {
+namespace {
+
+// ---- building an operator ------------------------------------------------
+
+// A tap of a row of parity `phase` of the chain starting at parity q: the
+// even rows' taps of the chain starting at parity 0, reversed when exactly
+// one of the two differs.
+__device__ __forceinline__ double tap(const double *e, int R, int q_phase, int d)
+{
+    d = (q_phase & 1) ? -d : d;
+    return (d >= -R && d <= R) ? e[d] : 0.0;
+}
+// The direction of those taps.
+__device__ __forceinline__ int dir(int q_phase) { return (q_phase & 1) ? -1 : 1; }
+
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// An unevaluated sum of two doubles.
+struct Dd {
+    double hi, lo;
+};
+__device__ __forceinline__ Dd two_sum(double a, double b)
+{
+    const double s = a + b, t = s - a;
+    return {s, (a - (s - t)) + (b - t)};
+}
+__device__ __forceinline__ Dd dd_add(Dd a, Dd b)
+{
+    const Dd s = two_sum(a.hi, b.hi);
+    return two_sum(s.hi, s.lo + (a.lo + b.lo));
+}
+__device__ __forceinline__ Dd dd_mul(Dd a, Dd b)
+{
+    const double p = a.hi * b.hi;
+    return two_sum(p, fma(a.hi, b.hi, -p) + fma(a.hi, b.lo, a.lo * b.hi));
+}
+
+// ---- the short chain: 128-bit fixed point
+
+// Signed fixed-point number of 126 fraction bits.
+struct Fix {
+    unsigned long long lo;
+    long long hi;
+};
+__device__ __forceinline__ Fix fix_sub(Fix a, Fix b)
+{
+    return {a.lo - b.lo, (long long)((unsigned long long)a.hi - (unsigned long long)b.hi - (a.lo < b.lo))};
+}
+__device__ __forceinline__ Fix fix_add(Fix a, Fix b)
+{
+    const unsigned long long lo = a.lo + b.lo;
+    return {lo, (long long)((unsigned long long)a.hi + (unsigned long long)b.hi + (lo < a.lo))};
+}
+// x times a fraction f 2^-64, rounded down in magnitude.
+__device__ __forceinline__ Fix fix_mul(Fix x, unsigned long long f)
+{
+    const bool neg = x.hi < 0;
+    if (neg)
+        x = fix_sub(Fix{0, 0}, x);
+    const unsigned long long xh = (unsigned long long)x.hi, l = xh * f, m = __umul64hi(x.lo, f);
+    const Fix r{l + m, (long long)(__umul64hi(xh, f) + (l + m < l))};
+    return neg ? fix_sub(Fix{0, 0}, r) : r;
+}
+// As a double-double.
+__device__ __forceinline__ Dd fix_dd(Fix x)
+{
+    const bool neg = x.hi < 0;
+    if (neg)
+        x = fix_sub(Fix{0, 0}, x);
+    const unsigned long long h = (unsigned long long)x.hi;
+    const double a = (double)(unsigned)(h >> 32) * 0x1p-30, b = (double)(unsigned)h * 0x1p-62;
+    const double c = (double)(unsigned)(x.lo >> 32) * 0x1p-94, d = (double)(unsigned)x.lo * 0x1p-126;
+    const Dd ab = two_sum(a, b), cd = two_sum(c, d);
+    const Dd r = two_sum(ab.hi, ab.lo + cd.hi);
+    const double e = ((ab.lo + cd.hi) - ab.lo);
+    const Dd v = two_sum(r.hi, r.lo + ((cd.hi - e) + cd.lo));
+    return neg ? Dd{-v.hi, -v.lo} : v;
+}
+
+// The chain of k <= kPropShort steps, step by step: rows of the operator as
+// vectors, the steps applied from the last back (a step is symmetric): the
+// even row of the infinite grid from parity 0, and rows 0 and 1 of the half
+// grid from both parities.  An element per thread, in 128-bit fixed point:
+// FP64 pairs would take ten operations an update on the SM's one FP64 unit
+// (19 cycles each a warp) where the integer pipes take a few cycles.
+constexpr int kShortThreads = (2 * kPropShort + 3 + 4 * (kPropShort + 3) + 31) / 32 * 32;
+
+__global__ void __launch_bounds__(kShortThreads) prop_short_kernel(double *e, double *el, double *h, double *hl, int hs, int k,
+                                                         PropCoef c)
+{
+    constexpr int kE = 2 * kPropShort + 3, kW = kPropShort + 3;  // elements of the infinite row, of a wall row
+    __shared__ Fix s_x[2][kE + 4 * kW + 2];
+    const int t = threadIdx.x;
+    const bool inf = t < kE, used = t < kE + 4 * kW;
+    const int w = (t - kE) / kW, pos = inf ? t - (kPropShort + 1) : (t - kE) % kW;  // lattice position
+    const int p = inf ? 0 : w >> 1, b = inf ? 0 : w & 1;
+    const int first = inf ? -(kPropShort + 1) : 0, last = kPropShort + (inf ? 1 : 2);
+    Fix x{0, used && pos == b ? (1ll << 62) : 0};
+    for (int s = k - 1; s >= 0; --s) {
+        const int par = (p + s) & 1, q = s & 1;
+        if (used)
+            s_x[q][t] = x;
+        __syncthreads();
+        if (used) {
+            const int m = ((pos + par) & 1) ? -1 : 1;  // the pair of parity par
+            if (pos + m >= first && pos + m <= last) {
+                x = fix_add(x, fix_mul(fix_sub(s_x[q][t + m], x), c.be_frac));
+            } else if (!inf && pos + m < 0) {
+                x = fix_mul(x, c.ka_frac);
+                if (c.ka[0] < 0.0)
+                    x = fix_sub(Fix{0, 0}, x);
+            }
+        }
+    }
+    __syncthreads();
+    if (used)
+        s_x[0][t] = x;
+    __syncthreads();
+    const int R = k + 1;
+    if (inf && pos >= -R && pos <= R) {
+        const Dd v = fix_dd(x);
+        e[pos] = v.hi;
+        el[pos] = v.lo;
+    } else if (used && !inf && pos <= R) {
+        // less the infinite grid's tap at distance pos - b
+        const int d = dir(p ^ b) * (pos - b);
+        const Dd v = fix_dd(fix_sub(x, s_x[0][d + kPropShort + 1]));
+        h[w * hs + pos] = v.hi;
+        hl[w * hs + pos] = v.lo;
+    }
+}
+
+// ---- doubling the chain
+
+// Chain of 2 k1 + delta steps from the chain of k1: Q_{2k+1} = Q_k Q_k C, the
+// extra first step mixing the columns of a pair.  A block takes 32 columns
+// (30 with delta: the outer two only lend their sums) of one row, a column
+// per thread, and its four warps a quarter of the terms each: a term costs
+// one multiply-add on the FP64 unit, which bounds the kernel, a broadcast and
+// a conflict-free read.  (A warp per entry, its lanes sharing the terms: 70 us
+// for the last level of k = 1999, r = 0.7; columns per thread: 38 us.)
+// Rounding leaves the whole operator a common factor near 1, which the finish
+// takes out.  `par`: the start parities whose wall arrays are needed (bit p).
+constexpr int kLevelPad = 36;  // zeros around the staged arrays: a block's columns overreach by at most 33
+
+__global__ void __launch_bounds__(128) prop_level_kernel(const PropLevel P)
+{
+    extern __shared__ double st[];
+    __shared__ double s_part[4][32], s_edge[2][4];
+    const int t = threadIdx.x, lane = t & 31, seg = t >> 5, R = P.R1, dl = P.delta;
+    const int ne = 2 * R + 1 + 2 * kLevelPad, nh = R + 1 + 2 * kLevelPad;
+    double *e = st + R + kLevelPad, *h = st + ne + kLevelPad;  // h: row class x at h + x nh
+    for (int i = t; i < ne; i += 128) {
+        const int d = i - R - kLevelPad;
+        st[i] = d >= -R && d <= R ? P.e0[d] : 0.0;
+    }
+#pragma unroll 1
+    for (int x = 0; x < 4; ++x)
+        for (int i = t; i < nh; i += 128) {
+            const int d = i - kLevelPad;
+            st[ne + x * nh + i] = d >= 0 && d <= R ? P.h0[x * P.hs + d] : 0.0;
+        }
+    __syncthreads();
+    const int per = dl ? 30 : 32;
+    const int b_int = (2 * P.R2 + 1 + per - 1) / per, b_wall = (P.R2 + 1 + per - 1) / per;
+    const int rows = P.par == 3 ? 4 : 2;
+    const bool wall = (int)blockIdx.x >= b_int;
+    const int wb = wall ? ((int)blockIdx.x - b_int) / b_wall : 0;
+    if (wb >= rows)
+        return;
+    const int pb = wb + (P.par == 2 ? 2 : 0), p = wall ? pb >> 1 : 0, b = wall ? pb & 1 : 0;
+    const int first = wall ? 0 : -P.R2;                        // first column of the row
+    const int blk = wall ? ((int)blockIdx.x - b_int) % b_wall : (int)blockIdx.x;
+    const int j0 = first + blk * per - dl, j = j0 + lane;      // this block's columns j0 .. j0 + 31
+    const int qs = (p + P.k1 + dl) & 1, qf = (p + dl) & 1;
+    const int s2 = dir(qs ^ b), s1e = dir(qf), s1o = -s1e;     // directions: the later chain's row, the earlier one's columns
+    double *g2 = st + ne + 4 * nh;  // the later chain's row b in full, a2 + h2
+    if (wall) {
+        const double *h2 = h + (qs * 2 + b) * nh;
+        for (int l = t; l < R + kLevelPad; l += 128)
+            g2[l] = (l - b <= R ? e[s2 * (l - b)] : 0.0) + h2[l];
+        __syncthreads();
+    }
+    // terms c[l] a1[j - l], l in [lo, hi] by this warp, a pair of columns l at a time
+    auto conv = [&](const double *c, int sc, int lo, int hi) {
+        if (hi < lo)
+            return 0.0;
+        const int n = hi - lo + 1, q = (n + 3) / 4;
+        int l = lo + seg * q;
+        const int end = l + q - 1 < hi ? l + q - 1 : hi;
+        // eight sums: rounding grows with the length of each
+        double x0[4] = {}, x1[4] = {};
+        if (l <= end && (l & 1)) {
+            x1[0] = c[sc * l] * e[s1o * (j - l)];
+            ++l;
+        }
+        for (; l + 7 <= end; l += 8) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                x0[u] = fma(c[sc * (l + 2 * u)], e[s1e * (j - l - 2 * u)], x0[u]);
+                x1[u] = fma(c[sc * (l + 2 * u + 1)], e[s1o * (j - l - 2 * u - 1)], x1[u]);
+            }
+        }
+        for (; l + 1 <= end; l += 2) {
+            x0[0] = fma(c[sc * l], e[s1e * (j - l)], x0[0]);
+            x1[0] = fma(c[sc * (l + 1)], e[s1o * (j - l - 1)], x1[0]);
+        }
+        if (l <= end)
+            x0[0] = fma(c[sc * l], e[s1e * (j - l)], x0[0]);
+        return ((x0[0] + x0[1]) + (x0[2] + x0[3])) + ((x1[0] + x1[1]) + (x1[2] + x1[3]));
+    };
+    // the columns' overreach: |j - l| <= R + 33 stays inside the padding
+    const int cl = j0 - R > b - R ? j0 - R : b - R, ch = j0 + 31 + R < b + R ? j0 + 31 + R : b + R;
+    double v;
+    if (!wall) {
+        v = conv(e - s2 * b, s2, cl, ch);
+    } else {
+        // sum over l >= 0 of h2 a1 + (a2 + h2) h1, less the infinite product's part from l < 0
+        const double *h2 = h + (qs * 2 + b) * nh;
+        v = conv(h2, 1, j0 - R > 0 ? j0 - R : 0, R) - conv(e - s2 * b, s2, cl, ch < -1 ? ch : -1);
+        const double *h1e = h + qf * 2 * nh, *h1o = h1e + nh;
+        const int hi = R - j0 + 1 < R + 1 ? R - j0 + 1 : R + 1;
+        if (hi >= 0) {
+            const int q = ((hi + 1 + 3) / 4 + 1) & ~1;
+            const int l0 = seg * q, end = l0 + q - 1 < hi ? l0 + q - 1 : hi;
+            const int jj = j > 0 ? j : 0;  // column -1 takes no part
+            double x0[4] = {}, x1[4] = {};
+            int l = l0;
+            for (; l + 6 <= end; l += 8) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    x0[u] = fma(g2[l + 2 * u], h1e[jj + l + 2 * u], x0[u]);
+                    x1[u] = fma(g2[l + 2 * u + 1], h1o[jj + l + 2 * u], x1[u]);
+                }
+            }
+            for (; l <= end; l += 2) {
+                x0[0] = fma(g2[l], h1e[jj + l], x0[0]);
+                x1[0] = fma(g2[l + 1], h1o[jj + l], x1[0]);
+            }
+            v += ((x0[0] + x0[1]) + (x0[2] + x0[3])) + ((x1[0] + x1[1]) + (x1[2] + x1[3]));
+        }
+    }
+    s_part[seg][lane] = v;
+    if (wall && dl && p == 1 && j0 < 0) {
+        // a singleton's column has no partner: the infinite product's own
+        // entries at columns 0 and -1, terms spread over the block
+        double a0 = 0.0, am = 0.0;
+        for (int d = -R + t; d <= R; d += 128) {
+            const double a2 = e[s2 * d];
+            const int l = b + d, s1 = dir(qf ^ l);
+            if (l <= R && l >= -R)
+                a0 = fma(a2, e[s1 * -l], a0);
+            if (-1 - l <= R && -1 - l >= -R)
+                am = fma(a2, e[s1 * (-1 - l)], am);
+        }
+        a0 = warp_sum(a0);
+        am = warp_sum(am);
+        if (lane == 0) {
+            s_edge[0][seg] = a0;
+            s_edge[1][seg] = am;
+        }
+    }
+    __syncthreads();
+    if (seg != 0)
+        return;
+    v = (s_part[0][lane] + s_part[1][lane]) + (s_part[2][lane] + s_part[3][lane]);
+    if (dl) {
+        const double up = __shfl_down_sync(0xffffffffu, v, 1), dn = __shfl_up_sync(0xffffffffu, v, 1);
+        double x = fma(P.c.al[0], v, P.c.be[0] * (((j + p) & 1) ? dn : up));
+        if (wall && p == 1 && j == 0) {
+            const double a0 = (s_edge[0][0] + s_edge[0][1]) + (s_edge[0][2] + s_edge[0][3]);
+            const double am = (s_edge[1][0] + s_edge[1][1]) + (s_edge[1][2] + s_edge[1][3]);
+            x = P.c.ka[0] * (a0 + v) - P.c.al[0] * a0 - P.c.be[0] * am;
+        }
+        v = x;
+    }
+    if (j < first || j > P.R2 || (dl && (lane == 0 || lane == 31)))
+        return;
+    if (wall) {
+        P.h1[pb * P.hs + j] = v;
+        P.hl1[pb * P.hs + j] = 0.0;
+    } else {
+        P.e1[j] = v;
+        P.el1[j] = 0.0;
+    }
+}
+
+// ---- the finished operator
+
+// The finished operator from the last level's arrays (small blocks, to spread
+// the double-doubles over the SMs' FP64 units):
+// taps and wall arrays divided by the taps' sum, the wall values' part, and
+// the rows of the tensor cores' operator as double-doubles, with their largest
+// magnitude: the exit folded into the last operator of a call (u = x1 w + x2
+// w_partner, pairs of the last step's parity) and the entry into the first
+// one (w = u + r (u_partner - u): a combination of columns), so that tiles
+// read and write the state as it is.
+//   F: with both walls 1 the constant state is steady, so F_i is what row i
+// misses of it: 1 - sum_j Q(i, j), plus the first point's own wall term,
+// which its right-hand side holds at parity 1.
+constexpr int kFinishThreads = 64;
+
+__global__ void __launch_bounds__(kFinishThreads) prop_finish_kernel(const PropLevel P, const PropFinish Q)
+{
+    __shared__ double part[kFinishThreads / 32];
+    __shared__ double s_miss;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, R = P.R1;
+    {
+        double s = 0.0;
+        for (int i = -R + t; i <= R; i += kFinishThreads)
+            s += P.e0[i];
+        s = warp_sum(s);
+        if (lane == 0)
+            part[warp] = s;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        Dd m{-1.0, 0.0};
+        for (int i = 0; i < kFinishThreads / 32; ++i) {
+            const Dd x = two_sum(m.hi, part[i]);
+            m.hi = x.hi;
+            m.lo += x.lo;
+        }
+        if (t == 0)
+            s_miss = -(m.hi + m.lo);
+    }
+    __syncthreads();
+    const double miss = s_miss;
+    const int gid = blockIdx.x * kFinishThreads + t, n_int = 2 * R + 1, n_h = 4 * (R + 1), RX = R + 4, n_x = 2 * (2 * RX + 1);
+    if (gid < n_int) {
+        P.e1[gid - R] = P.e0[gid - R] + fma(miss, P.e0[gid - R], P.el0[gid - R]);
+    } else if (gid < n_int + n_h) {
+        const int w = gid - n_int, i = w / (R + 1) * P.hs + w % (R + 1);
+        P.h1[i] = P.h0[i] + fma(miss, P.h0[i], P.hl0[i]);
+    } else if (Q.x && gid < n_int + n_h + n_x) {
+        const int i = gid - n_int - n_h, phase = i & 1, d = (i >> 1) - RX;
+        const int s = ((phase ^ Q.p0 ^ Q.k) & 1) ? -1 : 1, a = Q.p0 ^ phase;
+        // the row with the exit, at column phase + d
+        auto row = [&](int d) {
+            Dd v{tap(P.e0, R, a, d), tap(P.el0, R, a, d)};
+            if (Q.exit)
+                v = dd_add(dd_mul(Dd{Q.x1, 0.0}, v),
+                           dd_mul(Dd{Q.x2, 0.0}, Dd{tap(P.e0, R, a ^ 1, d - s), tap(P.el0, R, a ^ 1, d - s)}));
+            return v;
+        };
+        Dd v = row(d);
+        if (Q.entry) {
+            // v_j + r (v_partner - v_j), the pairs of parity 1 - p0
+            const Dd w = row(((phase + d + 1 - Q.p0) & 1) ? d - 1 : d + 1);
+            v = dd_add(v, dd_mul(Dd{Q.r, 0.0}, dd_add(w, Dd{-v.hi, -v.lo})));
+        }
+        Q.x[2 * i] = v.hi;
+        Q.x[2 * i + 1] = v.lo;
+        atomicMax(Q.x_max, (unsigned long long)__double_as_longlong(fabs(v.hi)));
+    }
+    const int o = blockIdx.x * (kFinishThreads / 32) + warp;
+    if (!Q.F || o >= 2 * (R + 2))
+        return;
+    const int p = o / (R + 2), i = o % (R + 2), b = i & 1;
+    if (!((P.par >> p) & 1))
+        return;
+    double s = 0.0;
+#pragma unroll 4
+    for (int d = -R + lane; d < -i; d += 32)
+        s += tap(P.e0, R, p ^ b, d);
+#pragma unroll 4
+    for (int x = i - b + lane; x <= R; x += 32)
+        s -= P.h0[(p * 2 + b) * P.hs + x];
+    s = warp_sum(s);
+    if (lane == 0) {
+        if (p == 1)
+            s -= Q.r * (tap(P.e0, R, p ^ b, -i) + (i - b <= R ? P.h0[(p * 2 + b) * P.hs + i - b] : 0.0));
+        s = fma(miss, s, s);
+        if (i == 0 && ((p + Q.k) & 1))
+            s += Q.r;
+        Q.F[p * P.hs + i] = s;
+    }
+}
+
+// Digit tables for the tensor cores.  The operand of a block of 64 outputs n
+// and window position k (64 + 2 W of them, from -W on) is the tap k - n - W;
+// eight consecutive k of a row are one 16-byte piece, and a piece depends on
+// n - k only (and on the parity of n): row rho of digit i's table holds
+// d = 56 + W_i - rho + t, t = 0..7, and the operand's piece (n, k = 8c) is
+// row n - 8c + 56 + 2 W_i.
+constexpr int kPropQ = 2 * kPropRMax + 13;
+
+// round(x 2^E), below 2^62 in magnitude.
+__device__ __forceinline__ long long fixed_of(double x, int E)
+{
+    const long long u = __double_as_longlong(x);
+    const int e = (int)(u >> 52) & 0x7ff;
+    unsigned long long m = (unsigned long long)u & 0x000fffffffffffffull;
+    if (e)
+        m |= 0x0010000000000000ull;
+    const int sh = (e ? e : 1) - 1075 + E;
+    if (sh >= 0) {
+        m <<= sh;
+    } else {
+        const int n = -sh < 60 ? -sh : 60;
+        m = (m + (1ull << (n - 1))) >> n;
+    }
+    return u < 0 ? -(long long)m : (long long)m;
+}
+
+__global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, const unsigned long long *x_max, int R,
+                                                           int nd, int hb_max, int tab_cap, unsigned char *tab,
+                                                           PropHeader *hdr)
+{
+    extern __shared__ long long q[];  // [2][kPropQ]
+    constexpr int kQ = kPropQ, kMid = kPropRMax + 6;
+    __shared__ long long s_sum[2];
+    __shared__ float s_abs[32];
+    __shared__ int s_W[8], s_row0[8];
+    __shared__ int s_ok;
+    const int t = threadIdx.x, RX = R + 4;
+    if (t < 8)
+        s_W[t] = 0;
+    if (t < 2)
+        s_sum[t] = 0;
+    // largest scale that keeps the top digit below 127 and a row's sum of
+    // magnitudes (1, more where the entry is folded in) below 2^62
+    const int count = 2 * (2 * RX + 1);
+    {
+        // (FP32 and integers throughout: one SM's FP64 unit would take longer)
+        float m = 0.0f;
+        for (int i = t; i < count; i += 1024)
+            m += fabsf((float)x[2 * i]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            m += __shfl_xor_sync(0xffffffffu, m, o);
+        if ((t & 31) == 0)
+            s_abs[t >> 5] = m;
+    }
+    __syncthreads();
+    float abs_sum = s_abs[t & 31];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        abs_sum += __shfl_xor_sync(0xffffffffu, abs_sum, o);  // of both phases: twice a row's
+    // 126 / max in [2^(ex - 1), 2^ex): the quotient's exponent, one less to be safe of its rounding
+    int ex, es;
+    frexpf(125.99f / (float)__longlong_as_double((long long)*x_max), &ex);
+    frexpf(0.499f * abs_sum, &es);
+    const int e0 = ex - 1 + 8 * (nd - 1), e1 = 62 - es, E = e0 < e1 ? e0 : e1;
+    auto add_sum = [&](int phase, long long v) {
+        // two phases alternate over the lanes: sum the even and the odd lanes
+        long long s = v;
+        for (int o = 16; o > 1; o >>= 1)
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((t & 31) < 2)
+            atomicAdd(reinterpret_cast<unsigned long long *>(&s_sum[phase]), (unsigned long long)s);
+    };
+    for (int i0 = 0; i0 < count; i0 += 1024) {
+        const int i = i0 + t, phase = i & 1, d = (i >> 1) - RX;
+        long long v = 0;
+        if (i < count) {
+            v = fixed_of(x[2 * i], E) + fixed_of(x[2 * i + 1], E);
+            q[phase * kQ + kMid + d] = v;
+        }
+        add_sum(phase, v);
+    }
+    __syncthreads();
+    // the rows' sum is exactly 1, so a constant stays what it is: the taps
+    // share what rounding left in proportion (put on one tap it would be
+    // white noise next to the smoothed field), the middle one takes the rest
+    const float unit = __int_as_float((127 - E) << 23);
+    const float miss[2] = {(float)((1LL << E) - s_sum[0]) * unit, (float)((1LL << E) - s_sum[1]) * unit};
+    __syncthreads();
+    if (t < 2)
+        s_sum[t] = 0;
+    __syncthreads();
+    for (int i0 = 0; i0 < count; i0 += 1024) {
+        const int i = i0 + t, phase = i & 1, d = (i >> 1) - RX;
+        long long v = 0;
+        if (i < count) {
+            v = q[phase * kQ + kMid + d];
+            v += __float2ll_rn((float)v * miss[phase]);
+            q[phase * kQ + kMid + d] = v;
+        }
+        add_sum(phase, v);
+    }
+    __syncthreads();
+    if (t < 2)
+        q[t * kQ + kMid] += (1LL << E) - s_sum[t];
+    __syncthreads();
+    const unsigned long long bias = nd == kPropNd64 ? 0x0080808080808080ull : 0x80808080ull;
+    int w[kPropNd64] = {};
+    for (int i = t; i < count; i += 1024) {
+        const int phase = i & 1, d = (i >> 1) - RX;
+        const unsigned long long y = (unsigned long long)q[phase * kQ + kMid + d] + bias;
+#pragma unroll
+        for (int j = 0; j < kPropNd64; ++j)
+            if (j < nd && ((y >> (8 * (nd - 1 - j))) & 255) != 128)
+                w[j] = max(w[j], d < 0 ? -d : d);
+    }
+#pragma unroll
+    for (int j = 0; j < kPropNd64; ++j) {
+        const int m = __reduce_max_sync(0xffffffffu, w[j]);
+        if ((t & 31) == 0)
+            atomicMax(&s_W[j], m);
+    }
+    __syncthreads();
+    if (t == 0) {
+        int rows = 0, ok = 1;
+        for (int j = 0; j < nd; ++j) {
+            int W = (s_W[j] + 15) / 16 * 16;
+            if (W > hb_max * kPropBlk) {
+                W = hb_max * kPropBlk;
+                ok = 0;
+            }
+            s_W[j] = W;
+            s_row0[j] = rows;
+            rows += 120 + 2 * W;
+        }
+        if (rows * 16 > tab_cap) {
+            ok = 0;
+            rows = 0;
+        }
+        s_ok = ok;
+        hdr->E = E;
+        hdr->room = 62 - es - E;
+        hdr->ok = ok;
+        hdr->rows = rows;
+        for (int j = 0; j < nd; ++j) {
+            hdr->W[j] = s_W[j];
+            hdr->row0[j] = s_row0[j];
+        }
+    }
+    __syncthreads();
+    if (!s_ok)
+        return;
+    for (int j = 0; j < nd; ++j) {
+        const int W = s_W[j], sh = 8 * (nd - 1 - j);
+        for (int rho = t; rho < 120 + 2 * W; rho += 1024) {
+            __align__(16) __half v[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const int d = 56 + W - rho + c;
+                unsigned long long y = bias;
+                if (d >= -RX && d <= RX)
+                    y += (unsigned long long)q[(rho & 1) * kQ + kMid + d];
+                v[c] = __int2half_rn((int)((y >> sh) & 255) - 128);
+            }
+            *reinterpret_cast<uint4 *>(tab + (size_t)(s_row0[j] + rho) * 16) = *reinterpret_cast<const uint4 *>(v);
+        }
+    }
+}
+
+// ---- reading the state ---------------------------------------------------
+
+// Point j's right-hand side w = (1 - r) u + r u_partner (+ the wall terms),
+// the groups those of parity 1 - p0 -- or the value itself after the first
+// operator, when the buffer holds w.
+template <typename T>
+__device__ __forceinline__ double load_w(const PropRun &P, long long j)
+{
+    const T *in = static_cast<const T *>(P.in);
+    const double u = (double)in[j];
+    if (!P.entry)
+        return u;
+    const long long m = ((j + 1 - P.p0) & 1) ? j - 1 : j + 1;
+    double w = P.omr * u;
+    if (m >= 0 && m < P.n)
+        w = fma(P.r, (double)in[m], w);
+    if (j == 0)
+        w += P.fl;
+    if (j == P.n - 1)
+        w += P.fr;
+    return w;
+}
+
+// ---- dot products --------------------------------------------------------
+
+// A few rows of a CTA: the rows near the walls (or all rows of a small grid),
+// and the blocks a tile left out.  The window of right-hand sides is staged
+// in shared memory as doubles; one warp takes one row's sum.  Bound by the
+// FP64 unit (two taps' widths of multiply-adds a row).
+constexpr int kDotRows = 8, kEdgeRows = 16;
+
+// How far right row i's sum reaches in k steps: k where the last step pairs
+// the row with its right neighbour, else k - 1 (and the other way to the left).
+__device__ __forceinline__ int reach_right(const PropRun &P, long long i)
+{
+    return ((i + P.p0 + P.k - 1) & 1) ? P.k - 1 : P.k;
+}
+constexpr int kDotWin = 2 * kPropRMax + 16;
+
+template <int ROWS>
+struct DotShared {
+    double row[ROWS + 2];
+    int bad[ROWS + 2];
+};
+
+// Rows [r0, rend) by NT threads (all of named barrier 1), up to ROWS of them;
+// s_w holds kDotWin doubles.
+template <typename T, int NT, int ROWS>
+__device__ __forceinline__ void dot_rows(const PropRun &P, DotShared<ROWS> &sh, double *s_w, long long r0, long long rend)
+{
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int pe = (P.p0 + P.k) & 1, R = P.R;
+    auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };
+    // with the exit at parity 1 the outer rows' partners lie outside the item
+    const int ext = P.exit && pe;
+    const long long lo = r0 - ext > 0 ? r0 - ext : 0;
+    const long long hi = rend + ext < P.n ? rend + ext : P.n;
+    const long long wlo = lo - R > 0 ? lo - R : 0;
+    const long long whi = hi + R < P.n ? hi + R : P.n;
+    if (t < ROWS + 2)
+        sh.bad[t] = 0;
+#pragma unroll 4
+    for (long long j = wlo + t; j < whi; j += NT)
+        s_w[j - wlo] = load_w<T>(P, j);
+    sync();
+    // a value that is not finite spoils every row it reaches in k steps, also
+    // beyond the taps that are kept
+    if (R < P.k) {
+        const long long clo = lo - P.k > 0 ? lo - P.k : 0, chi = hi + P.k < P.n ? hi + P.k : P.n;
+#pragma unroll 4
+        for (long long j = clo + t; j < chi; j += NT) {
+            if (!isfinite(j >= wlo && j < whi ? s_w[j - wlo] : load_w<T>(P, j))) {
+                for (int q = 0; q < (int)(hi - lo); ++q) {
+                    const long long d = j - (lo + q);
+                    const int right = reach_right(P, lo + q);
+                    if (d <= right && -d <= 2 * P.k - 1 - right)
+                        sh.bad[q] = 1;
+                }
+            }
+        }
+        sync();
+    }
+    for (int q = warp; q < (int)(hi - lo); q += NT / 32) {
+        const long long i = lo + q;
+        const int ph = (int)(i & 1), rev = (P.p0 ^ ph) & 1;
+        const int right = reach_right(P, i), left = 2 * P.k - 1 - right;
+        const long long jl = i - (left < R ? left : R) > 0 ? i - (left < R ? left : R) : 0;
+        const long long jh = i + (right < R ? right : R) < P.n - 1 ? i + (right < R ? right : R) : P.n - 1;
+        double s = 0.0;
+        {
+            const double *w = s_w + (jl - wlo);
+            const int m = (int)(jh - jl) + 1;
+            const double *e = rev ? P.e + (i - jl) : P.e - (i - jl);
+            const int se = rev ? -1 : 1;
+#pragma unroll 8
+            for (int x = lane; x < m; x += 32)
+                s = fma(__ldg(e + se * x), w[x], s);
+        }
+        // the left wall: h_{i&1}(j + i - (i & 1)) for j >= 0
+        const long long il = i - ph;
+        if (il <= R) {
+            const double *h = P.h + (P.p0 * 2 + ph) * P.hs + il;
+            const long long m = R - il < jh ? R - il : jh;
+#pragma unroll 8
+            for (int x = (int)jl + lane; x <= (int)m; x += 32)
+                s = fma(__ldg(h + x), s_w[x - wlo], s);
+            if (lane == 0 && P.bl != 0.0)
+                s = fma(P.bl, P.F[P.p0 * P.hs + i], s);
+        }
+        // the right wall, from the mirrored index
+        const long long im = P.n - 1 - i;
+        const int pm = (int)(im & 1);
+        const long long ir = im - pm;
+        if (ir <= R) {
+            const double *h = P.h + (P.pr * 2 + pm) * P.hs + ir;
+            const long long m = R - ir < P.n - 1 - jl ? R - ir : P.n - 1 - jl;
+            const double *w = s_w + (P.n - 1 - wlo);
+#pragma unroll 8
+            for (int x = (int)(P.n - 1 - jh) + lane; x <= (int)m; x += 32)
+                s = fma(__ldg(h + x), w[-x], s);
+            if (lane == 0 && P.br != 0.0)
+                s = fma(P.br, P.F[P.pr * P.hs + im], s);
+        }
+        s = warp_sum(s);
+        if (lane == 0)
+            sh.row[q] = sh.bad[q] ? s + __longlong_as_double(0x7ff8000000000000ll) : s;
+    }
+    sync();
+    if (t < (int)(rend - r0)) {
+        const long long i = r0 + t;
+        double v = sh.row[i - lo];
+        if (P.exit) {
+            const long long m = ((i + pe) & 1) ? i - 1 : i + 1;
+            v = (m >= 0 && m < P.n) ? fma(P.x2, sh.row[m - lo], P.x1 * v) : P.xs * v;
+        }
+        static_cast<T *>(P.out)[i] = (T)v;
+    }
+    sync();
+}
+
+// All rows of a grid too small for tiles, or the blocks the tiles listed.
+template <typename T>
+__global__ void __launch_bounds__(256) prop_dot_kernel(const __grid_constant__ PropRun P)
+{
+    __shared__ double s_w[kDotWin];
+    __shared__ DotShared<kDotRows> sh;
+    long long items = (P.n + kDotRows - 1) / kDotRows;
+    if (P.tiles > 0) {
+        items = (long long)*reinterpret_cast<volatile int *>(P.count) * (kPropBlk / kDotRows);
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            *P.count_next = 0;
+    }
+    for (long long it = blockIdx.x; it < items; it += gridDim.x) {
+        const long long r0 = P.tiles > 0 ? (long long)P.list[it / (kPropBlk / kDotRows)] * kPropBlk +
+                                               it % (kPropBlk / kDotRows) * kDotRows
+                                         : it * kDotRows;
+        dot_rows<T, 256, kDotRows>(P, sh, s_w, r0, r0 + kDotRows < P.n ? r0 + kDotRows : P.n);
+    }
+}
+
+// ---- tiles on the tensor cores -------------------------------------------
+
+// Blocks whose values all lie below 2^-kRange of the largest value they
+// depend on go to the dot products: the fixed-point sum would leave them too
+// few digits of their own.
+template <typename T>
+struct TileShape;
+template <>
+struct TileShape<double> {
+    static constexpr int ND = kPropNd64, kHb = kPropHb64, kTab = kPropTab64, kRange = 16;
+    static constexpr int kGroups = 9, kCols = 512;
+};
+template <>
+struct TileShape<float> {
+    static constexpr int ND = kPropNd32, kHb = kPropHb32, kTab = kPropTab32, kRange = 10;
+    static constexpr int kGroups = 4, kCols = 256;
+};
+
+// A value digit's plane: a 128-byte row of 64 FP16 digits per block of the
+// tile and its halo, the row's eight 16-byte pieces in descending order and
+// swizzled (piece position ^ row mod 8) as the tensor cores' 128-byte swizzle
+// reads them: a window that starts blocks further on is the same plane rows
+// further on, and every eight rows of a piece cover all banks.  (The same
+// plane unswizzled, rows of 16 bytes, took 85 to 90 cycles an MMA.)
+template <typename T>
+constexpr int kPlaneRows = kPropTileBlks + 2 * TileShape<T>::kHb;
+template <typename T>
+constexpr int kTileSmem = TileShape<T>::kTab + TileShape<T>::ND * kPlaneRows<T> * 128 + 1024;
+// The finished rows leave through the planes' space, padded so that the lanes
+// (a row each) write different banks.
+template <typename T>
+constexpr int kStageRow = kPropBlk * (int)sizeof(T) + 16;
+
+static_assert(kTileSmem<double> <= 232448 - 2048 && kTileSmem<float> <= 232448 - 2048, "tile exceeds shared memory");
+
+// Digit products of each accumulator, in issue order: sum g holds the products
+// of weight(g) whose tap digit lies in [lo(g), hi(g)].  FP64's weight 4 takes
+// two sums so that each stays exact; its first and last sum share one
+// accumulator (512 columns hold eight).
+struct Groups64 {
+    __host__ __device__ static constexpr int weight(int g) { return g <= 3 ? 7 - g : 8 - g; }
+    __host__ __device__ static constexpr int lo(int g) { return g == 0 ? 1 : g == 4 ? 3 : 0; }
+    __host__ __device__ static constexpr int hi(int g) { return g == 0 ? 6 : g == 3 ? 2 : weight(g); }
+};
+struct Groups32 {
+    __host__ __device__ static constexpr int weight(int g) { return 3 - g; }
+    __host__ __device__ static constexpr int lo(int) { return 0; }
+    __host__ __device__ static constexpr int hi(int g) { return weight(g); }
+};
+template <typename T>
+struct GroupsOf;
+template <>
+struct GroupsOf<double> {
+    using G = Groups64;
+};
+template <>
+struct GroupsOf<float> {
+    using G = Groups32;
+};
+
+// Exponent code of a value: 0 for zero, else its biased exponent (1 for
+// subnormals; all ones for infinities and NaN).
+__device__ __forceinline__ int code_of(double x)
+{
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    const int e = (int)(hi >> 20);
+    return e ? e : ((hi | (unsigned)__double2loint(x)) ? 1 : 0);
+}
+__device__ __forceinline__ int code_of(float x)
+{
+    const unsigned u = __float_as_uint(x) & 0x7fffffffu;
+    const int e = (int)(u >> 23);
+    return e ? e : (u ? 1 : 0);
+}
+template <typename T>
+constexpr int kCodeInf = sizeof(T) == 8 ? 2047 : 255;
+
+// round(x 2^(kVal - e)) for |x| < 2^e, e = code - bias + 1 of the tile's
+// largest value; `ref` is that largest code.
+__device__ __forceinline__ long long to_fixed(double x, int ref)
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)(u >> 52) & 0x7ff;
+    unsigned long long m = u & 0x000fffffffffffffull;
+    if (e)
+        m |= 0x0010000000000000ull;
+    // x = m 2^(ec - 1075), 2^e_tile = 2^(ref - 1022): shift by ec - ref + 1
+    const int sh = (e ? e : 1) - ref + 1;
+    if (sh >= 0) {
+        m <<= sh;
+    } else {
+        const int n = -sh < 60 ? -sh : 60;
+        m = (m + (1ull << (n - 1))) >> n;
+    }
+    return (long long)u < 0 ? -(long long)m : (long long)m;
+}
+__device__ __forceinline__ int to_fixed(float x, int ref)
+{
+    const unsigned u = __float_as_uint(x);
+    const int e = (int)(u >> 23) & 0xff;
+    unsigned m = u & 0x007fffffu;
+    if (e)
+        m |= 0x00800000u;
+    // x = m 2^(ec - 150), 2^e_tile = 2^(ref - 126): shift by ec - ref + 6
+    const int sh = (e ? e : 1) - ref + 6;
+    if (sh >= 0) {
+        m <<= sh;
+    } else {
+        const int n = -sh < 30 ? -sh : 30;
+        m = (m + (1u << (n - 1))) >> n;
+    }
+    return (int)u < 0 ? -(int)m : (int)m;
+}
+
+// x 2^e for a normal x whose product is normal too; and 2^e.
+__device__ __forceinline__ float add_exponent(float x, int e) { return __int_as_float(__float_as_int(x) + (e << 23)); }
+template <typename T>
+__device__ __forceinline__ T pow2(int e);
+template <>
+__device__ __forceinline__ double pow2<double>(int e)
+{
+    return __hiloint2double((e + 1023) << 20, 0);
+}
+template <>
+__device__ __forceinline__ float pow2<float>(int e)
+{
+    return __int_as_float((e + 127) << 23);
+}
+
+// z 2^e rounded to nearest even, for a normal result.  FP64 on the integer
+// pipes: the conversion instruction runs on the FP64 unit.
+template <typename T>
+__device__ __forceinline__ T from_fixed(long long z, int e);
+template <>
+__device__ __forceinline__ double from_fixed<double>(long long z, int e)
+{
+    const unsigned long long m = (unsigned long long)(z < 0 ? -z : z);
+    const int lead = __clzll((long long)m);                 // 2 .. 63 (64 for zero)
+    const unsigned long long w = m << (lead & 63);          // leading one at bit 63
+    unsigned long long f = w >> 11;
+    const unsigned low = (unsigned)w & 0x7ff;
+    f += (low > 0x400 || (low == 0x400 && (f & 1))) ? 1 : 0;
+    // exponent field of 2^(63 - lead + e), less the leading one's own unit
+    f += (unsigned long long)(unsigned)(1023 + 62 - lead + e) << 52;
+    if (m == 0)
+        f = 0;
+    return __longlong_as_double((long long)(f | ((unsigned long long)z & 0x8000000000000000ull)));
+}
+template <>
+__device__ __forceinline__ float from_fixed<float>(long long z, int e)
+{
+    return z ? add_exponent((float)z, e) : 0.0f;
+}
+
+// Two digits as FP16: bytes b of two biased values to (b - 128).
+__device__ __forceinline__ uint32_t half_pair(uint32_t a, uint32_t b, uint32_t sel)
+{
+    const uint32_t v = (__byte_perm(a, b, sel) & 0x00ff00ffu) | 0x64006400u;  // 1024 + byte
+    const __half2 h = __hsub2(*reinterpret_cast<const __half2 *>(&v), __float2half2_rn(1152.0f));
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// K-major operand with 128-byte rows and the 128-byte swizzle: groups of eight
+// rows 1024 bytes apart (the leading offset is unused).
+__device__ __forceinline__ uint64_t swizzled_desc(uint32_t addr)
+{
+    return ((addr & 0x3FFFF) >> 4) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+
+// K-major operand without swizzle: core matrices of 8 rows x 16 bytes
+// (contiguous, 128 bytes), `lead` bytes apart along K and 128 along the rows.
+__device__ __forceinline__ uint64_t plain_desc(uint32_t addr, uint32_t lead)
+{
+    return ((addr & 0x3FFFF) >> 4) | ((uint64_t)(lead >> 4) << 16) | ((uint64_t)(128 >> 4) << 32) | (1ull << 46);
+}
+
+// kind::f16 with FP16 operands and FP32 accumulators, M = 128, N = 64.
+constexpr uint32_t kIdescF16 = (1u << 4) | ((uint32_t)(kPropBlk >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+
+// 16 warps that convert and drain, 1 that issues the MMAs: the conversion and
+// the drain are chains of integer instructions with little else to hide their
+// latency.
+constexpr int kTileWarps = 16, kTileConv = 32 * kTileWarps, kTileThreads = kTileConv + 32;
+constexpr int kTileCols = kPropBlk / (kTileWarps / 4);  // points of a block a thread drains
+
+template <typename T>
+__global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid_constant__ PropRun P)
+{
+    using S = TileShape<T>;
+    using G = typename GroupsOf<T>::G;
+    constexpr int ND = S::ND, C = kPlaneRows<T>;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                          ~static_cast<uintptr_t>(1023));
+    unsigned char *xp = sm + S::kTab;  // value digits: [digit][C rows][128 bytes], then the finished rows
+    __shared__ __align__(8) uint64_t tab_full, done[S::kGroups], reuse;
+    __shared__ uint32_t tmem_sh;
+    __shared__ volatile int s_abort;
+    __shared__ int s_code[kPropTileBlks + 2 * S::kHb + 8];
+    __shared__ int s_max[2];  // largest code: the window, the whole cone
+    __shared__ int s_keep;    // blocks the tile itself answers
+    __shared__ PropHeader s_hdr;
+    __shared__ DotShared<kEdgeRows> s_dot;
+
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    if (t < (int)(sizeof(PropHeader) / 4))
+        reinterpret_cast<int *>(&s_hdr)[t] = reinterpret_cast<const int *>(P.hdr)[t];
+    if (t == 0) {
+        bar_init(&tab_full, 1);
+        for (int g = 0; g < S::kGroups; ++g)
+            bar_init(&done[g], 1);
+        bar_init(&reuse, kTileWarps);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_abort = 0;
+    }
+    if (warp == kTileWarps) {
+        tmem_alloc(&tmem_sh, S::kCols);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = tmem_sh;
+    const int hb = P.hb, ok_tab = s_hdr.ok && s_hdr.rows * 16 <= S::kTab;
+    if (t == 0 && ok_tab) {
+        bar_expect_tx(&tab_full, (uint32_t)s_hdr.rows * 16);
+        bulk_load(sm, P.tab, (uint32_t)s_hdr.rows * 16, &tab_full);
+    }
+    bool tab_waited = false;
+    uint32_t phase = 0;
+    const T *in = static_cast<const T *>(P.in);
+    T *out = static_cast<T *>(P.out);
+
+    const long long edge_l = P.rows_l / kEdgeRows;  // whole blocks
+    const long long edges = edge_l + (P.n - P.row_r + kEdgeRows - 1) / kEdgeRows;
+    for (long long tile = blockIdx.x; tile < P.tiles + edges; tile += gridDim.x) {
+        if (tile >= P.tiles) {
+            // rows near a wall, after the tiles: they fill the last wave
+            if (warp < kTileWarps) {
+                bulk_wait_read0();
+                asm volatile("bar.sync 1, %0;" ::"n"(kTileConv) : "memory");
+                const long long x = tile - P.tiles;
+                const long long r0 = x < edge_l ? x * kEdgeRows : P.row_r + (x - edge_l) * kEdgeRows;
+                dot_rows<T, kTileConv, kEdgeRows>(P, s_dot, reinterpret_cast<double *>(xp), r0,
+                                                  r0 + kEdgeRows < P.n ? r0 + kEdgeRows : P.n);
+            }
+            continue;
+        }
+        const long long b0 = P.blk0 + tile * kPropTileBlks;       // first output block
+        const int nb = (int)(P.blk1 - b0 < kPropTileBlks ? P.blk1 - b0 : kPropTileBlks);
+        const long long base = (b0 - hb) * kPropBlk;              // first point of the window
+        const int chunks = (kPropTileBlks + 2 * hb) * 8;          // 8 points each
+        constexpr int kIter = ((kPropTileBlks + 2 * S::kHb) * 8 + kTileConv - 1) / kTileConv;
+        if (t < 2)
+            s_max[t] = 0;
+        if (t == 2)
+            s_keep = 0;
+        __syncthreads();
+        // the window in registers, a chunk of 8 points per turn; the largest
+        // exponent of every block and of the window
+        T x[kIter][8];
+        if (warp < kTileWarps) {
+            int wmax = 0;
+            constexpr int kV = 16 / sizeof(T);
+#pragma unroll
+            for (int c = 0; c < kIter; ++c) {
+                const int u = c * kTileConv + t;
+                const long long j = base + (long long)u * 8;
+                // whole chunks only: the few points past the last one lie
+                // beyond every window that is used
+                const bool in_range = u < chunks && j + 8 <= P.n;
+#pragma unroll
+                for (int v = 0; v < 8 / kV; ++v) {
+                    uint4 q = make_uint4(0, 0, 0, 0);
+                    if (in_range)
+                        q = *reinterpret_cast<const uint4 *>(in + j + v * kV);
+                    *reinterpret_cast<uint4 *>(&x[c][v * kV]) = q;
+                }
+            }
+            // the next tile's window on its way to L2
+            if (tile + gridDim.x < P.tiles) {
+                const long long nx = base + (long long)gridDim.x * kPropTileBlks * kPropBlk + (long long)t * 128 / sizeof(T);
+                for (long long z = nx; z < nx - (long long)t * 128 / sizeof(T) + (long long)chunks * 8 && z < P.n;
+                     z += (long long)kTileConv * 128 / sizeof(T))
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(in + z));
+            }
+#pragma unroll
+            for (int c = 0; c < kIter; ++c) {
+                const int u = c * kTileConv + t;
+                int m = 0;
+#pragma unroll
+                for (int v = 0; v < 8; ++v) {
+                    const int q = code_of(x[c][v]);
+                    m = q > m ? q : m;
+                }
+                wmax = m > wmax ? m : wmax;
+                // eight lanes hold a block
+                for (int z = 1; z < 8; z <<= 1) {
+                    const int y = __shfl_xor_sync(0xffffffffu, m, z);
+                    m = y > m ? y : m;
+                }
+                if ((t & 7) == 0 && u < chunks)
+                    s_code[u >> 3] = m;
+            }
+            // the rest of the cone: everything that reaches the tile's blocks in k steps
+            int cmax = wmax;
+            const long long clo = b0 * kPropBlk - P.k - 2, chi = (b0 + nb) * kPropBlk + P.k + 2;
+            for (long long j = (clo > 0 ? clo : 0) + t; j < base; j += kTileConv)
+                cmax = max(cmax, code_of(in[j]));
+            for (long long j = base + (long long)chunks * 8 + t; j < (chi < P.n ? chi : P.n); j += kTileConv)
+                cmax = max(cmax, code_of(in[j]));
+            for (long long j = (P.n & ~7LL) + t; j < P.n && j < chi; j += kTileConv)  // the ragged end
+                cmax = max(cmax, code_of(in[j]));
+            bulk_wait_read0();  // the last tile's rows have left the planes
+            wmax = __reduce_max_sync(0xffffffffu, wmax);
+            cmax = __reduce_max_sync(0xffffffffu, cmax);
+            if (lane == 0) {
+                atomicMax(&s_max[0], wmax);
+                atomicMax(&s_max[1], cmax);
+            }
+        }
+        __syncthreads();
+        const int ref = s_max[0], cone = s_max[1];
+        if (t < nb) {
+            const int q = s_code[hb + t];
+            const bool listed = cone > 0 && (!ok_tab || cone == kCodeInf<T> || q < cone - S::kRange || q == 0);
+            if (listed)
+                P.list[atomicAdd(P.count, 1)] = (int)(b0 + t);
+            else if (cone > 0)
+                s_keep = 1;
+        }
+        if (warp < kTileWarps && cone != kCodeInf<T>) {
+#pragma unroll
+            for (int c = 0; c < kIter; ++c) {
+                const int u = c * kTileConv + t;
+                if (u < chunks) {
+                    // biased fixed-point values: every byte is a digit + 128
+                    unsigned char *dst = xp + (u >> 3) * 128 + ((7 - (u & 7)) ^ ((u >> 3) & 7)) * 16;
+                    uint32_t lo[8], hi[8];
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) {
+                        if (ND == kPropNd64) {
+                            const unsigned long long y =
+                                (unsigned long long)to_fixed((double)x[c][v], ref) + 0x0080808080808080ull;
+                            lo[v] = (uint32_t)y;
+                            hi[v] = (uint32_t)(y >> 32);
+                        } else {
+                            lo[v] = (uint32_t)to_fixed((float)x[c][v], ref) + 0x80808080u;
+                        }
+                    }
+#pragma unroll
+                    for (int d = 0; d < ND; ++d) {
+                        const int byte = ND - 1 - d;
+                        const uint32_t sel = byte < 4 ? (uint32_t)(byte | (byte << 4) | ((byte + 4) << 8) | ((byte + 4) << 12))
+                                                      : (uint32_t)((byte - 4) | ((byte - 4) << 4) | (byte << 8) | (byte << 12));
+                        uint4 q;
+                        q.x = byte < 4 ? half_pair(lo[0], lo[1], sel) : half_pair(hi[0], hi[1], sel);
+                        q.y = byte < 4 ? half_pair(lo[2], lo[3], sel) : half_pair(hi[2], hi[3], sel);
+                        q.z = byte < 4 ? half_pair(lo[4], lo[5], sel) : half_pair(hi[4], hi[5], sel);
+                        q.w = byte < 4 ? half_pair(lo[6], lo[7], sel) : half_pair(hi[6], hi[7], sel);
+                        *reinterpret_cast<uint4 *>(dst + (size_t)d * C * 128) = q;
+                    }
+                }
+            }
+        }
+        fence_async_smem();
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        const bool keep = s_keep != 0;
+        if (warp == kTileWarps) {
+            if (keep) {
+                // the whole warp runs the loop, so descriptors stay in uniform
+                // registers; one lane issues
+                const bool leader = elect_one();
+                bool ok = true;
+                if (!tab_waited) {
+                    ok = bar_wait(&tab_full, 0, kWaitLimitCycles, &s_abort);
+                    tab_waited = true;
+                }
+                const uint32_t tab0 = saddr(sm), x0 = saddr(xp);
+#pragma unroll 1
+                for (int g = 0; ok && g < S::kGroups; ++g) {
+                    const int w = G::weight(g), lo = G::lo(g), hi = G::hi(g);
+                    uint32_t acc = 0;
+                    if (g * kPropBlk >= S::kCols) {
+                        // sum 0's accumulator again, once the warps have read it
+                        ok = bar_wait(&reuse, phase, kWaitLimitCycles, &s_abort);
+                        tc_fence_after();
+                        if (!ok)
+                            break;
+                    }
+                    const uint32_t dcol = tbase + (uint32_t)(g * kPropBlk % S::kCols);
+#pragma unroll 1
+                    for (int i = lo; i <= hi; ++i) {
+                        const int W = __shfl_sync(0xffffffffu, s_hdr.W[i], 0);
+                        const int row0 = __shfl_sync(0xffffffffu, s_hdr.row0[i], 0);
+                        // window position -W: block -W >> 6, piece q of its row (descending, as the
+                        // table's rows run); four steps go 64 points on, to the next row
+                        const int q = (-W & 63) >> 3;
+                        uint64_t ad = swizzled_desc(x0 + (uint32_t)(((w - i) * C + hb + (-W >> 6)) * 128));
+                        uint64_t bd = plain_desc(tab0 + (uint32_t)(row0 + 48 + 2 * W) * 16, 128);
+                        const int steps = (kPropBlk + 2 * W) / 16;
+                        const uint64_t a0 = (uint64_t)(6 - q), a1 = (uint64_t)(6 - ((q + 2) & 7) + ((q + 2) & 8)),
+                                       a2 = (uint64_t)(6 - ((q + 4) & 7) + ((q + 4) & 8)),
+                                       a3 = (uint64_t)(6 - ((q + 6) & 7) + ((q + 6) & 8));
+                        int s = 0;
+#pragma unroll 1
+                        for (; s + 4 <= steps; s += 4) {
+                            tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, acc);
+                            tc_mma_if(leader, dcol, ad + a1, bd - 16, kIdescF16, 1);
+                            tc_mma_if(leader, dcol, ad + a2, bd - 32, kIdescF16, 1);
+                            tc_mma_if(leader, dcol, ad + a3, bd - 48, kIdescF16, 1);
+                            acc = 1;
+                            ad += 8;
+                            bd -= 64;
+                        }
+                        if (s < steps) {
+                            tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, 1);
+                            if (s + 1 < steps)
+                                tc_mma_if(leader, dcol, ad + a1, bd - 16, kIdescF16, 1);
+                            if (s + 2 < steps)
+                                tc_mma_if(leader, dcol, ad + a2, bd - 32, kIdescF16, 1);
+                        }
+                    }
+                    if (lane == 0)
+                        tc_commit(&done[g]);
+                    __syncwarp();
+                }
+                if (!ok && lane == 0) {
+                    atomicExch(P.err, kDevTimeout);
+                    s_abort = 1;
+                }
+            }
+            __syncwarp();
+        } else if (keep) {
+            // drain: kTileCols columns (points of a block) of the lane's block
+            const int row = (warp & 3) * 32 + lane, col = (warp >> 2) * kTileCols;
+            // units of the sums: weight 5 (FP32: 3), and up to 8 bits below
+            // where the taps' scale leaves the 64-bit sum that room
+            const int room = s_hdr.room, xs = sizeof(T) == 4 ? 0 : room < 8 ? room : 8;
+            long long acc[kTileCols];
+#pragma unroll
+            for (int v = 0; v < kTileCols; ++v)
+                acc[v] = 0;
+            bool ok = true;
+#pragma unroll
+            for (int g = 0; g < S::kGroups; ++g) {
+                ok = ok && bar_wait(&done[g], phase, kWaitLimitCycles, &s_abort);
+                if (!__any_sync(0xffffffffu, !ok)) {
+                    tc_fence_after();
+                    uint32_t v[kTileCols];
+                    tmem_ld16(tbase + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(g * kPropBlk % S::kCols + col), v);
+                    tmem_wait_ld();
+                    if (g == 0 && S::kGroups * kPropBlk > S::kCols) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0)
+                            bar_arrive(&reuse);
+                    }
+                    const int w = G::weight(g);
+#pragma unroll
+                    for (int q = 0; q < kTileCols; ++q) {
+                        const int z = __float2int_rn(__uint_as_float(v[q]));
+                        if (ND == kPropNd64)
+                            acc[q] = w == 7   ? (long long)z
+                                     : w == 6 ? ((acc[q] + ((long long)z << 8) + (0x8000 >> xs)) >> (16 - xs))
+                                              : acc[q] + ((long long)z << (8 * (5 - (w < 6 ? w : 5)) + xs));
+                        else
+                            acc[q] += (long long)z << (8 * (3 - (w < 4 ? w : 3)));
+                    }
+                }
+            }
+            if (__any_sync(0xffffffffu, !ok)) {
+                if (lane == 0) {
+                    atomicExch(P.err, kDevTimeout);
+                    s_abort = 1;
+                }
+            } else if (row < nb) {
+                // out = acc 2^x: FP64 x = e + 2 - E - xs, FP32 x = e - 6 - E, 2^e above the tile's largest value
+                const int ex = sizeof(T) == 8 ? ref - 1022 + 2 - s_hdr.E - xs : ref - 126 - 6 - s_hdr.E;
+                unsigned char *o = xp + row * kStageRow<T> + col * (int)sizeof(T);
+                const bool plain = sizeof(T) == 8 ? ex >= -1021 && ex <= 959 : ex >= -125 && ex <= 63;
+                const T s1 = pow2<T>(ex / 2), s2 = pow2<T>(ex - ex / 2);
+                if (plain) {
+#pragma unroll
+                    for (int v = 0; v < kTileCols; v += 16 / sizeof(T)) {
+                        T y[16 / sizeof(T)];
+#pragma unroll
+                        for (int z = 0; z < (int)(16 / sizeof(T)); ++z)
+                            y[z] = from_fixed<T>(acc[v + z], ex);
+                        *reinterpret_cast<uint4 *>(o + v * sizeof(T)) = *reinterpret_cast<const uint4 *>(y);
+                    }
+                } else {  // near the ends of the exponent range
+#pragma unroll
+                    for (int v = 0; v < kTileCols; ++v)
+                        reinterpret_cast<volatile T *>(o)[v] = (T)acc[v] * s1 * s2;
+                }
+            }
+            // every row by one bulk copy (a row per thread storing 16-byte
+            // pieces: 15000 cycles a tile)
+            fence_async_smem();
+            asm volatile("bar.sync 1, %0;" ::"n"(kTileConv) : "memory");
+            if (t < nb && !s_abort) {
+                bulk_store(out + (b0 + t) * kPropBlk, xp + t * kStageRow<T>, kPropBlk * (uint32_t)sizeof(T));
+                bulk_commit();
+            }
+        } else if (cone == 0) {
+            const int row = (warp & 3) * 32 + lane, col = (warp >> 2) * kTileCols;
+            if (row < nb) {
+                T *o = out + (b0 + row) * kPropBlk + col;
+                for (int v = 0; v < kTileCols; ++v)
+                    o[v] = (T)0;
+            }
+        }
+        if (keep)
+            phase ^= 1;
+        tc_fence_before();
+        __syncthreads();
+        tc_fence_after();
+        if (s_abort)
+            break;
+    }
+    bulk_wait0();
+    // the table's copy and MMAs in flight end before the CTA does
+    if (t == 0 && ok_tab)
+        bar_drain(&tab_full, 0, kWaitLimitCycles);
+    if (s_abort && t == 0)
+        bar_drain(&done[S::kGroups - 1], phase ^ 1, kWaitLimitCycles);
+    __syncthreads();
+    if (warp == kTileWarps)
+        tmem_dealloc(tbase, S::kCols);
+}
+
+}  // namespace
+
+cudaError_t prop_prepare()
+{
+    // once per device: the attributes, and every kernel loaded before a stream
+    // capture may need it
+    static std::mutex lock;
+    static unsigned long long ready[4];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess)
+        return e;
+    std::lock_guard<std::mutex> hold(lock);
+    if (dev < 256 && (ready[dev >> 6] >> (dev & 63)) & 1)
+        return cudaSuccess;
+    cudaFuncAttributes fa;
+    e = cudaFuncSetAttribute(prop_tile_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kTileSmem<double>);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(prop_tile_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kTileSmem<float>);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(prop_digits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 2 * kPropQ * 8);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(prop_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (7 * kPropRMax + 11 * kLevelPad + 8) * 8);
+    const void *rest[] = {(const void *)prop_short_kernel, (const void *)prop_finish_kernel,
+                          (const void *)prop_dot_kernel<double>, (const void *)prop_dot_kernel<float>};
+    for (const void *f : rest)
+        if (e == cudaSuccess)
+            e = cudaFuncGetAttributes(&fa, f);
+    if (e == cudaSuccess && dev < 256)
+        ready[dev >> 6] |= 1ull << (dev & 63);
+    return e;
+}
+
+cudaError_t prop_launch_short(double *e, double *el, double *h, double *hl, int hs, int k, const PropCoef &c,
+                              cudaStream_t s)
+{
+    prop_short_kernel<<<1, kShortThreads, 0, s>>>(e, el, h, hl, hs, k, c);
+    return cudaGetLastError();
+}
+
+cudaError_t prop_launch_level(const PropLevel &a, cudaStream_t s)
+{
+    const int per = a.delta ? 30 : 32;
+    const int grid = (2 * a.R2 + 1 + per - 1) / per + (a.par == 3 ? 4 : 2) * ((a.R2 + 1 + per - 1) / per);
+    const size_t bytes = (size_t)(2 * a.R1 + 1 + 2 * kLevelPad + 4 * (a.R1 + 1 + 2 * kLevelPad) + a.R1 + kLevelPad) * 8;
+    prop_level_kernel<<<grid, 128, bytes, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t prop_launch_finish(const PropLevel &a, const PropFinish &f, cudaStream_t s)
+{
+    const int R = a.R1, threads = 2 * R + 1 + 4 * (R + 1) + (f.x ? 2 * (2 * R + 9) : 0);
+    const int warps = f.F ? 2 * (R + 2) : 0;
+    const int bw = (warps * 32 + kFinishThreads - 1) / kFinishThreads, bt = (threads + kFinishThreads - 1) / kFinishThreads;
+    prop_finish_kernel<<<bw > bt ? bw : bt, kFinishThreads, 0, s>>>(a, f);
+    return cudaGetLastError();
+}
+
+cudaError_t prop_launch_digits(const PropSet &set, const PropFinish &f, int R, int f64, int hb_max, cudaStream_t s)
+{
+    prop_digits_kernel<<<1, 1024, 2 * kPropQ * 8, s>>>(f.x, f.x_max, R, f64 ? kPropNd64 : kPropNd32, hb_max,
+                                                                    f64 ? kPropTab64 : kPropTab32, set.tab, set.hdr);
+    return cudaGetLastError();
+}
+
+cudaError_t prop_launch_tiles(const PropRun &a, int f64, int grid, cudaStream_t s)
+{
+    if (f64)
+        prop_tile_kernel<double><<<grid, kTileThreads, kTileSmem<double>, s>>>(a);
+    else
+        prop_tile_kernel<float><<<grid, kTileThreads, kTileSmem<float>, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t prop_launch_dots(const PropRun &a, int f64, int grid, cudaStream_t s)
+{
+    if (f64)
+        prop_dot_kernel<double><<<grid, 256, 0, s>>>(a);
+    else
+        prop_dot_kernel<float><<<grid, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace ge

@@ -1,0 +1,126 @@
+"""Composed steps (GE_KERNEL_AUTO): k steps as one banded operator, on the
+tensor cores away from the walls and as FP64 dot products near them, against
+the oracle and the tiled kernel.
+
+Tolerances: FP64 1e-12 relative max-norm (tests/tolerances.py), FP32 1e-5, as
+for every other path.  Where the data's magnitude changes from block to block
+(64 points) each block is held to its own largest value: the operator takes
+dot products for blocks below 2^-16 of what reaches them, and the others keep
+at least 54 - 16 - 1 bits, so 2^-37 a pass and at most a few passes: 1e-10.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from tolerances import tol64
+from paper_1310_3422_gb300 import binding as B
+from paper_1310_3422_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+def auto_run(u0, r, bl, br, steps, prec=B.GE_F64, step0=0):
+    x = torch.as_tensor(np.asarray(u0), dtype=B.dtype_of(prec), device=DEV).contiguous()
+    ctx = B.ge_create(len(u0), r, bl, br, prec, x)
+    B.ge_write_state(ctx, x, step0)
+    B.ge_step_n(ctx, steps)
+    out = torch.empty_like(x)
+    B.ge_read_state(ctx, out)
+    B.ge_sync(ctx)
+    assert B.ge_get_step(ctx) == step0 + steps
+    B.ge_destroy(ctx)
+    return out.double().cpu().numpy()
+
+
+def rel_max(got, want):
+    return float(np.max(np.abs(got - want)) / np.max(np.abs(want)))
+
+
+# all dot products below 8192 points; above, tiles of 128 blocks of 64 points
+# between the two wall ranges: one block, one tile more or less, odd ends
+@pytest.mark.parametrize("n", [16, 17, 65, 1000, 8191, 8192, 9281, 17407, 17473, 40001])
+@pytest.mark.parametrize("steps", [20, 21, 200, 777])
+@pytest.mark.parametrize("r", [0.01, 0.7, 2.0, 6.0])
+def test_matches_the_oracle(n, steps, r):
+    step0 = steps & 1
+    u0 = inputs.random_state(n, seed=n + steps)
+    want = oracle.run(u0, r, 0.3, -0.8, steps, step0)
+    assert rel_max(auto_run(u0, r, 0.3, -0.8, steps, step0=step0), want) <= tol64(r)
+    f0 = u0.astype(np.float32).astype(np.float64)
+    want = oracle.run(f0, r, 0.3, -0.8, steps, step0)
+    for prec in (B.GE_F32, B.GE_F32_COMP):
+        assert rel_max(auto_run(f0, r, 0.3, -0.8, steps, prec, step0), want) <= 1e-5
+
+
+@pytest.mark.parametrize("prec,tol", [(B.GE_F64, 1e-10), (B.GE_F32, 1e-3)])
+def test_each_block_keeps_its_own_digits(prec, tol):
+    """A pulse on a zero ground, steps between magnitudes, and a ramp over 30 decades."""
+    n, r, steps = 50000, 1.5, 140
+    u0 = np.zeros(n)
+    u0[9000:9400] = 1.0
+    u0[20000:30000] = 1e-20 * inputs.random_state(10000, seed=3)
+    u0[25000:25064] += 1.0
+    u0[35000:45000] = 10.0 ** np.linspace(-20, 0, 10000)
+    u0 = u0.astype(np.float32).astype(np.float64)
+    want = oracle.run(u0, r, 0.0, 0.0, steps)
+    got = auto_run(u0, r, 0.0, 0.0, steps, prec)
+    floor = 1e-30 if prec == B.GE_F64 else 1e-25
+    for a in range(0, n, 64):
+        big = np.max(np.abs(want[a:a + 64]))
+        if big > floor:
+            assert np.max(np.abs(got[a:a + 64] - want[a:a + 64])) <= tol * big, a
+    assert not got[np.flatnonzero(want == 0.0)].any()
+
+
+@pytest.mark.parametrize("r,steps", [(0.05, 300), (2.0, 100)])
+def test_values_that_are_not_finite_reach_as_far_as_step_by_step(r, steps):
+    n = 30000
+    u0 = inputs.random_state(n, seed=9)
+    u0[12000], u0[25001] = np.nan, np.nan
+    want = oracle.run(u0, r, 0.1, 0.2, steps)
+    got = auto_run(u0, r, 0.1, 0.2, steps)
+    assert np.array_equal(np.isfinite(got), np.isfinite(want))
+    ok = np.isfinite(want)
+    assert rel_max(got[ok], want[ok]) <= tol64(r)
+
+
+def test_magnitudes_near_the_ends_of_the_exponent_range():
+    n, r, steps = 20000, 2.0, 200
+    u0 = inputs.random_state(n, seed=4)
+    want = oracle.run(u0, r, 0.0, 0.0, steps)
+    for e in (-1000, 1000):
+        got = auto_run(np.ldexp(u0, e), r, 0.0, 0.0, steps)
+        assert rel_max(np.ldexp(got, -e), want) <= tol64(r)
+
+
+def test_captured_graph_and_later_direct_calls():
+    """A call captured from a fresh context builds its operator in the graph;
+    replays and direct calls (the same steps, others, and more kinds than the
+    context keeps) give the same results."""
+    n, r = 20001, 1.2
+    u0 = inputs.random_state(n, seed=12)
+    x = torch.tensor(u0, device=DEV)
+    out = torch.empty_like(x)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ctx = B.ge_create(n, r, 0.2, -0.1, B.GE_F64, x, stream)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            B.ge_write_state(ctx, x, 0)
+            B.ge_step_n(ctx, 300)
+            B.ge_read_state(ctx, out)
+        for steps in ("replay", 300, 40, 41, 60, "replay", 80, 100, 300, "replay"):
+            out.zero_()
+            if steps == "replay":
+                graph.replay()
+            else:
+                B.ge_write_state(ctx, x, 0)
+                B.ge_step_n(ctx, steps)
+                B.ge_read_state(ctx, out)
+            B.ge_sync(ctx)
+            want = oracle.run(u0, r, 0.2, -0.1, 300 if steps == "replay" else steps)
+            assert rel_max(out.cpu().numpy(), want) <= tol64(r), steps
+        del graph
+    torch.cuda.synchronize()
