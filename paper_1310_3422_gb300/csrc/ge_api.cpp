@@ -90,6 +90,7 @@ struct ge_ctx {
     int *err_dev = nullptr;
     int num_sms = 0;
     int tb_blocks_per_sm = 0;
+    int tb_rounds_per_sm = 0;     // its cooperative form
     int tb_df_blocks_per_sm = 0;  // double-float kernel (GE_F64 contexts)
     ge::CanonCoef canon{};
     ge::TbParams tb{};   // launch-independent fields filled at creation
@@ -210,6 +211,21 @@ int effective_depth(const ge_ctx *c)
     return (c->prec == GE_F64) ? kDefaultDepthF64 : kDefaultDepthF32;
 }
 
+// Where the tiled kernel runs (grid_cap aside).
+ge::TbTarget tiled_target(const ge_ctx *c)
+{
+    ge::TbTarget t{};
+    t.tmap[0] = &c->tmap[0];
+    t.tmap[1] = &c->tmap[1];
+    t.buf[0] = c->buf[0];
+    t.buf[1] = c->buf[1];
+    t.n = c->n;
+    t.n_rows = c->n_rows;
+    t.err = c->err_dev;
+    t.tile_ctr = c->err_dev + 48;  // two tile-queue words (48, 49)
+    return t;
+}
+
 // Advance `steps` steps with the tiled kernel, `depth` steps per launch
 // (df: the double-float kernel, after its per-call prescale); the launches
 // and the scale mirror are planned by ge::tb_run.
@@ -225,15 +241,7 @@ ge_status run_tiled(ge_ctx *c, int64_t steps, int depth, bool df = false)
         if (e != cudaSuccess)
             return cuda_fail(e, "double-float prescale launch");
     }
-    ge::TbTarget t{};
-    t.tmap[0] = &c->tmap[0];
-    t.tmap[1] = &c->tmap[1];
-    t.buf[0] = c->buf[0];
-    t.buf[1] = c->buf[1];
-    t.n = c->n;
-    t.n_rows = c->n_rows;
-    t.err = c->err_dev;
-    t.tile_ctr = c->err_dev + 48;  // two tile-queue words (48, 49)
+    ge::TbTarget t = tiled_target(c);
     t.grid_cap = (long long)c->num_sms * (df ? c->tb_df_blocks_per_sm : c->tb_blocks_per_sm);
     const cudaError_t e = ge::tb_run(t, base, growth_lo, df, prec, &c->cur, c->step, steps, depth, c->stream);
     if (e == cudaErrorInvalidValue)
@@ -260,6 +268,12 @@ ge_status run_composed(ge_ctx *c, int64_t steps, int *taken)
     t.f64 = c->prec == GE_F64;
     t.num_sms = c->num_sms;
     t.err = c->err_dev;
+    t.tiled = tiled_target(c);
+    t.base = &c->tb;
+    t.growth_lo = c->onepg_lo;
+    t.prec = c->prec == GE_F64 ? 0 : (c->prec == GE_F32 ? 1 : 2);
+    t.depth = effective_depth(c);
+    t.rounds_grid = c->num_sms * c->tb_rounds_per_sm;
     const cudaError_t e = ge::prop_run(&c->prop, t, &c->cur, c->step, steps, taken, c->stream);
     return e == cudaSuccess ? GE_OK : cuda_fail(e, "composed-step kernel launch");
 }
@@ -424,6 +438,8 @@ ge_status ge_create(ge_ctx **out, int64_t n, double r, double beta_l, double bet
     }
     const int prec_idx = prec == GE_F64 ? 0 : (prec == GE_F32 ? 1 : 2);
     e = ge::tb_occupancy(prec_idx, &c->tb_blocks_per_sm);
+    if (e == cudaSuccess)
+        e = ge::tb_rounds_occupancy(prec_idx, &c->tb_rounds_per_sm);
     if (e == cudaSuccess)
         e = ge::prop_prepare();
     if (e == cudaSuccess && prec == GE_F64) {

@@ -108,6 +108,15 @@ struct TbParams {
                           // the launches of a stream alternate between two words, so no
                           // memset runs between them
     float dfc[7][2];      // (hi, lo) of g, kappa, r, 1 - r, x1, x2, xs
+    double out_scale;     // != 0 without an exit: the factor that takes the scale out again
+};
+
+// A solve's launches as the rounds of one (tb_rounds_kernel).
+constexpr int kMaxRounds = 64;
+struct TbRounds {
+    int rounds;
+    int *barrier;         // grid barrier's count, zero at the start
+    TbParams r[kMaxRounds];
 };
 
 // Prescale exponent word of the double-float kernel: for the smallest e with
@@ -257,6 +266,12 @@ cudaError_t launch_sweep_tb_f32(const float *in, float *out, long long n, int pa
 // prec: 0 = FP64, 1 = FP32, 2 = FP32 compensated.  tmap: 128-byte-aligned
 // CUtensorMap (opaque here) describing the source buffer.
 cudaError_t launch_tb(int prec, const void *tmap, const TbParams &p, int grid, cudaStream_t s);
+// The rounds of one cooperative launch (t0, t1: maps of the source buffers of
+// the even and the odd rounds), and their co-resident CTAs per SM.
+struct PropRun;
+cudaError_t launch_tb_rounds(int prec, const void *t0, const void *t1, const TbRounds &q, const PropRun &d, int grid,
+                             cudaStream_t s);
+cudaError_t tb_rounds_occupancy(int prec, int *blocks_per_sm);
 // A launch of exactly one block step and nothing else (no entry, exit;
 // plain FP32): the streaming kernel, from buffer `in` to `out`.
 cudaError_t launch_tb_stream(int prec, const void *in, void *out, const TbParams &p, cudaStream_t s);
@@ -314,6 +329,13 @@ struct TbTarget {
 // launch error.
 cudaError_t tb_run(const TbTarget &t, const TbParams &base, double growth_lo, bool df, int prec, int *cur,
                    long long step0, long long steps, int depth, cudaStream_t s);
+
+// Fill the rounds of `n_mid` block steps from parity p_first (entry before,
+// exit after as asked, the scale taken out otherwise), an odd number of them,
+// so that the result lands in the buffer opposite `cur`.  False when they do
+// not fit.
+bool tb_plan_rounds(const TbTarget &t, const TbParams &base, double growth_lo, int prec, int cur, int p_first,
+                    long long n_mid, bool entry, bool exit, int depth, TbRounds *out);
 
 // Record the calling thread's last-failure text (read by ge_last_error()).
 void set_last_error(const char *msg);

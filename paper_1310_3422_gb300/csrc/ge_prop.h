@@ -18,6 +18,8 @@
 #include <cstdint>
 #include <cuda_runtime_api.h>
 
+#include "ge_internal.h"
+
 namespace ge {
 
 // Most taps kept per side (FP32; an FP64 context keeps up to kPropR64Max).
@@ -68,6 +70,7 @@ struct PropState {
     int *list = nullptr;          // blocks that need dot products
     int *count = nullptr;         // two words: the current launch's and the next one's
     long long clock = 0;
+    TbRounds rounds;              // scratch of the launch being planned
     int rcap = 0, hs = 0;         // taps the arrays hold per side, stride of the wall arrays
 };
 
@@ -78,6 +81,12 @@ struct PropTarget {
     int f64;             // element type of the state
     int num_sms;
     int *err;
+    // the step-by-step form of an operator (tb_rounds_kernel), for data that
+    // would need dot products nearly everywhere
+    TbTarget tiled;
+    const TbParams *base;
+    double growth_lo;
+    int prec, depth, rounds_grid;
 };
 
 // Arguments of the kernels that advance the state.
@@ -102,6 +111,8 @@ struct PropRun {
     // dot products: rows [0, rows_l) and [row_r, n), and the listed blocks
     long long rows_l, row_r;
     int *list, *count, *count_next;
+    int gate_min;      // more listed blocks than this: left to the step-by-step form
+    int *zero[3];      // words the tiles clear for it: barrier, two tile queues
 };
 
 // Pair and singleton coefficients of one step, (high, low) parts.

@@ -386,8 +386,33 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
             a.row_r = a.blk1 * kPropBlk;
             const long long edges = a.rows_l / 16 + (t.n - a.row_r + 15) / 16;
             const int grid = (int)std::min<long long>(a.tiles + edges, t.num_sms);
+            // listed blocks past which the whole grid step by step is sooner
+            // done than their dot products: a block's 64 rows of 2 R taps at
+            // 2e11 multiply-adds a second, against the tiled kernel's rate
+            // and its wall tiles' time a step
+            const double rate = t.prec == 0 ? 8e11 : t.prec == 1 ? 1.8e13 : 5.8e12, wall = t.prec == 0 ? 4.4e-6 : 0.85e-6;
+            const double tiled_s = std::max((double)t.n * s.k / rate, wall * s.k) + 20e-6;
+            a.gate_min = (int)std::min(tiled_s / (128.0 * a.R / 2e11), 2e9);
+            const bool gated = a.gate_min < a.blk1 - a.blk0 &&
+                               tb_plan_rounds(t.tiled, *t.base, t.growth_lo, t.prec, *cur, p0, s.k, s.entry, s.exit,
+                                              t.depth, &st->rounds);
+            if (gated) {
+                st->rounds.barrier = st->count + 2;
+                a.zero[0] = st->count + 2;
+                a.zero[1] = t.tiled.tile_ctr;
+                a.zero[2] = t.tiled.tile_ctr + 1;
+            } else {
+                a.gate_min = 2000000000;
+            }
             if ((e = prop_launch_tiles(a, t.f64, grid, stream)) != cudaSuccess)
                 return e;
+            if (gated) {
+                if ((e = launch_tb_rounds(t.prec, t.tiled.tmap[*cur], t.tiled.tmap[*cur ^ 1], st->rounds, a,
+                                          t.rounds_grid, stream)) != cudaSuccess)
+                    return e;
+                *cur ^= 1;
+                continue;
+            }
             items = 2LL * t.num_sms;
         } else {
             a.rows_l = t.n;

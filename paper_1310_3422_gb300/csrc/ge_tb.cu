@@ -39,6 +39,7 @@
 // form x <- x + d (x_partner - x), d = 2r/(1+2r), and each point's updates
 // are Kahan-summed into (hi, lo); lo lives in registers for the launch.
 #include "ge.h"
+#include "ge_prop_dev.cuh"
 #include "ge_tb_dev.cuh"
 
 namespace ge {
@@ -182,6 +183,11 @@ __device__ __forceinline__ void run_scaled(Real (&v)[K], const TbParams &P, Exch
         } else {
             stage<0, kExit, EDGE>(v, L, R, sp, c);
         }
+    } else if (P.out_scale != 0.0) {
+        const Real sc = (Real)P.out_scale;
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+            v[j] *= sc;
     }
 }
 
@@ -281,9 +287,20 @@ struct Layout {
         sizeof(Real) == 8 ? GE_TB_MINBLOCKS_F64 : (COMP ? GE_TB_MINBLOCKS_COMP : GE_TB_MINBLOCKS_F32);
 };
 
+// Shared memory of a CTA beside its two tile buffers.
+template <typename Real, int NW>
+struct TbShared {
+    uint64_t mbar[3];  // two tile buffers, and one nothing arrives on
+    Real slot[2][NW][2];
+    long long next;
+};
+
+// The CTA's tiles of one launch, or of one round of tb_rounds_kernel; `it`
+// counts the tiles this CTA has loaded (the buffers and their barriers'
+// phases alternate with it).  False when a tile load did not complete.
 template <typename Real, bool COMP>
-__global__ void __launch_bounds__(Layout<Real, COMP>::NT, Layout<Real, COMP>::MINB)
-    tb_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ TbParams P)
+__device__ __forceinline__ bool tb_tiles(const CUtensorMap *tmap, const TbParams &P, unsigned char *tiles,
+                                         TbShared<Real, Layout<Real, COMP>::NT / 32> &sh, long long &it)
 {
     using LY = Layout<Real, COMP>;
     constexpr bool WT = LY::WT;
@@ -291,12 +308,7 @@ __global__ void __launch_bounds__(Layout<Real, COMP>::NT, Layout<Real, COMP>::MI
     constexpr int NW = NT / 32;
     constexpr int CH = kRowBytes / 16;
     constexpr uint32_t kTileBytes = kTileRows * kRowBytes;
-
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char *tiles = reinterpret_cast<unsigned char *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    __shared__ __align__(8) uint64_t mbar[3];  // two tile buffers, and one nothing arrives on
-    __shared__ Real slot[2][NW][2];
+    uint64_t *mbar = sh.mbar;
 
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int hr = P.H / KR;  // halo rows of the tile
@@ -306,40 +318,28 @@ __global__ void __launch_bounds__(Layout<Real, COMP>::NT, Layout<Real, COMP>::MI
     const int ht = P.H / K;                                   // halo threads per warp side
     const int my_row = WT ? (warp * (32 - 2 * ht) + lane) * RPT : t;
     const bool writes = WT ? (lane >= ht && lane < 32 - ht) : true;
-    Exch<Real, NW, WT> x{slot, 0, lane, warp};
-
-    if (t == 0) {
-        mbar_init(&mbar[0], 1);
-        mbar_init(&mbar[1], 1);
-        mbar_init(&mbar[2], 1);
-        fence_mbar_init();
-        // the next launch's tile queue starts empty (it runs after this one)
-        if (blockIdx.x == 0 && P.tile_ctr_next)
-            *P.tile_ctr_next = 0;
-    }
-    __syncthreads();
+    Exch<Real, NW, WT> x{sh.slot, 0, lane, warp};
 
     // tiles come from the launch's dynamic queue (queue_tile): thread 0
     // takes the next position while the current tile is computed
-    __shared__ long long s_next;
     long long k = blockIdx.x;
     if (t == 0 && k < P.n_tiles) {
-        mbar_arrive_expect_tx(&mbar[0], kTileBytes);
-        tma_load_rows(tiles, &tmap, &mbar[0], (int)(queue_tile(k, P.n_tiles) * ur - hr));
+        mbar_arrive_expect_tx(&mbar[it & 1], kTileBytes);
+        tma_load_rows(tiles + (it & 1) * kTileBytes, tmap, &mbar[it & 1], (int)(queue_tile(k, P.n_tiles) * ur - hr));
     }
-    for (long long it = 0; k < P.n_tiles; ++it) {
+    for (; k < P.n_tiles; ++it) {
         const int b = (int)(it & 1);
         unsigned char *cur = tiles + b * kTileBytes;
         const long long tile = queue_tile(k, P.n_tiles);
         bool prefetch = false;
         if (t == 0) {
             const long long nk = (long long)gridDim.x + atomicAdd(P.tile_ctr, 1);
-            s_next = nk;
+            sh.next = nk;
             prefetch = nk < P.n_tiles;
             if (prefetch) {
                 fence_proxy_async_smem();
                 mbar_arrive_expect_tx(&mbar[b ^ 1], kTileBytes);
-                tma_load_rows(tiles + (b ^ 1) * kTileBytes, &tmap, &mbar[b ^ 1],
+                tma_load_rows(tiles + (b ^ 1) * kTileBytes, tmap, &mbar[b ^ 1],
                               (int)(queue_tile(nk, P.n_tiles) * ur - hr));
             }
         }
@@ -347,9 +347,9 @@ __global__ void __launch_bounds__(Layout<Real, COMP>::NT, Layout<Real, COMP>::MI
         if (__syncthreads_or(!ok)) {
             if (t == 0)
                 tile_wait_failed(P.err, mbar, b, it, prefetch);
-            return;
+            return false;
         }
-        const long long next = s_next;  // written by thread 0 before the barrier
+        const long long next = sh.next;  // written by thread 0 before the barrier
 
         Real v[K];
 #pragma unroll
@@ -408,6 +408,100 @@ __global__ void __launch_bounds__(Layout<Real, COMP>::NT, Layout<Real, COMP>::MI
         }
         __syncthreads();
         k = next;
+    }
+    return true;
+}
+
+template <typename Real, bool COMP>
+__device__ __forceinline__ unsigned char *tb_start(unsigned char *smem_raw,
+                                                   TbShared<Real, Layout<Real, COMP>::NT / 32> &sh)
+{
+    if (threadIdx.x == 0) {
+        mbar_init(&sh.mbar[0], 1);
+        mbar_init(&sh.mbar[1], 1);
+        mbar_init(&sh.mbar[2], 1);
+        fence_mbar_init();
+    }
+    return reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+}
+
+template <typename Real, bool COMP>
+__global__ void __launch_bounds__(Layout<Real, COMP>::NT, Layout<Real, COMP>::MINB)
+    tb_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ TbParams P)
+{
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ __align__(8) TbShared<Real, Layout<Real, COMP>::NT / 32> sh;
+    unsigned char *tiles = tb_start<Real, COMP>(smem_raw, sh);
+    // the next launch's tile queue starts empty (it runs after this one)
+    if (threadIdx.x == 0 && blockIdx.x == 0 && P.tile_ctr_next)
+        *P.tile_ctr_next = 0;
+    __syncthreads();
+    long long it = 0;
+    tb_tiles<Real, COMP>(&tmap, P, tiles, sh, it);
+}
+
+// After a composed operator's tiles (ge_prop.h): the blocks they listed as dot
+// products, or, when more than gate_min are listed, the whole grid step by
+// step, the launches of the solve as rounds of this one cooperative launch
+// that meet at a grid barrier (bounded; a CTA that recorded a failure
+// releases the others' waits).  Which is known on the device only: as
+// launches that look at the count, the steps would cost 3 us each when they
+// are not needed.  (2^22 points of spikes on zeros, FP64, r = 1, 1000 steps:
+// 25.5 ms of dot products, 8.1 ms this way, 8.5 ms as the tiled kernel's own
+// launches.)
+template <typename Real, bool COMP>
+__global__ void __launch_bounds__(Layout<Real, COMP>::NT, Layout<Real, COMP>::MINB)
+    tb_rounds_kernel(const __grid_constant__ CUtensorMap t0, const __grid_constant__ CUtensorMap t1,
+                     const __grid_constant__ TbRounds Q, const __grid_constant__ PropRun D)
+{
+    extern __shared__ unsigned char smem_raw[];
+    const int listed = *reinterpret_cast<const volatile int *>(D.count);
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *D.count_next = 0;
+    if (listed <= D.gate_min) {
+        __shared__ DotShared<kDotRows> dots;
+        static_assert(kDotWin * 8 <= 2 * kTileRows * kRowBytes, "the window fits the tile buffers");
+        for (long long it = blockIdx.x; it < (long long)listed * (kPropBlk / kDotRows); it += gridDim.x)
+            dot_listed<Real, Layout<Real, COMP>::NT>(D, dots, reinterpret_cast<double *>(smem_raw), it);
+        return;
+    }
+    __shared__ __align__(8) TbShared<Real, Layout<Real, COMP>::NT / 32> sh;
+    __shared__ int s_ok;
+    unsigned char *tiles = tb_start<Real, COMP>(smem_raw, sh);
+    __syncthreads();
+    long long it = 0;
+    for (int rd = 0; rd < Q.rounds; ++rd) {
+        const TbParams &P = Q.r[rd];
+        // the word the next round takes its tiles from: last used a round ago
+        if (threadIdx.x == 0 && blockIdx.x == 0)
+            *P.tile_ctr_next = 0;
+        if (!tb_tiles<Real, COMP>((rd & 1) ? &t1 : &t0, P, tiles, sh, it))
+            return;
+        if (rd + 1 == Q.rounds)
+            return;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            atomicAdd(Q.barrier, 1);
+            const int want = (rd + 1) * (int)gridDim.x;
+            const long long start = clock64();
+            int ok = 1;
+            while (*reinterpret_cast<volatile int *>(Q.barrier) < want) {
+                if (*reinterpret_cast<volatile int *>(P.err) != kDevOk || clock64() - start > kWaitLimitCycles) {
+                    ok = 0;
+                    atomicExch(P.err, kDevTimeout);
+                    break;
+                }
+            }
+            __threadfence();
+            // other CTAs' stores, read next by TMA
+            asm volatile("fence.proxy.async.global;" ::: "memory");
+            s_ok = ok;
+        }
+        __syncthreads();
+        if (!s_ok)
+            return;
     }
 }
 
@@ -558,6 +652,27 @@ cudaError_t launch_one(const void *tmap, const TbParams &p, int grid, cudaStream
 }
 
 template <typename Real, bool COMP>
+cudaError_t launch_rounds_one(const void *t0, const void *t1, const TbRounds &q, const PropRun &d, int grid,
+                              cudaStream_t s)
+{
+    CUtensorMap a = *static_cast<const CUtensorMap *>(t0), b = *static_cast<const CUtensorMap *>(t1);
+    void *args[] = {&a, &b, const_cast<TbRounds *>(&q), const_cast<PropRun *>(&d)};
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(tb_rounds_kernel<Real, COMP>), dim3(grid),
+                                       dim3(Layout<Real, COMP>::NT), args, tb_smem_bytes(), s);
+}
+
+template <typename Real, bool COMP>
+cudaError_t rounds_occupancy(int *blocks)
+{
+    cudaError_t e = cudaFuncSetAttribute(tb_rounds_kernel<Real, COMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         tb_smem_bytes());
+    if (e != cudaSuccess)
+        return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, tb_rounds_kernel<Real, COMP>, Layout<Real, COMP>::NT,
+                                                         tb_smem_bytes());
+}
+
+template <typename Real, bool COMP>
 cudaError_t set_attr_and_occupancy(int *blocks)
 {
     cudaError_t e = cudaFuncSetAttribute(tb_kernel<Real, COMP>,
@@ -623,6 +738,25 @@ cudaError_t launch_tb(int prec, const void *tmap, const TbParams &p, int grid, c
     if (prec == 1)
         return launch_one<float, false>(tmap, p, grid, s);
     return launch_one<float, true>(tmap, p, grid, s);
+}
+
+cudaError_t tb_rounds_occupancy(int prec, int *blocks)
+{
+    if (prec == 0)
+        return rounds_occupancy<double, false>(blocks);
+    if (prec == 1)
+        return rounds_occupancy<float, false>(blocks);
+    return rounds_occupancy<float, true>(blocks);
+}
+
+cudaError_t launch_tb_rounds(int prec, const void *t0, const void *t1, const TbRounds &q, const PropRun &d, int grid,
+                             cudaStream_t s)
+{
+    if (prec == 0)
+        return launch_rounds_one<double, false>(t0, t1, q, d, grid, s);
+    if (prec == 1)
+        return launch_rounds_one<float, false>(t0, t1, q, d, grid, s);
+    return launch_rounds_one<float, true>(t0, t1, q, d, grid, s);
 }
 
 }  // namespace ge

@@ -141,4 +141,69 @@ cudaError_t tb_run(const TbTarget &t, const TbParams &base, double growth_lo, bo
     return cudaSuccess;
 }
 
+bool tb_plan_rounds(const TbTarget &t, const TbParams &base, double growth_lo, int prec, int cur, int p_first,
+                    long long n_mid, bool entry, bool exit, int depth, TbRounds *out)
+{
+    depth = tb_clamp_depth(base, depth);
+    if (depth < 1)
+        return false;
+    long long rounds = (n_mid + depth - 1) / depth;
+    rounds |= 1;
+    if (rounds > kMaxRounds - 1) {
+        rounds = kMaxRounds - 1;
+        depth = tb_clamp_depth(base, (int)((n_mid + rounds - 1) / rounds));
+        if ((long long)depth * rounds < n_mid)
+            return false;
+    }
+    const int every = base.rescale_every;
+    double sigma = 1.0, sigma_lo = 0.0;
+    int until = every;
+    long long done = 0;
+    for (int i = 0; i < (int)rounds; ++i) {
+        TbParams p = base;
+        const bool last = i + 1 == (int)rounds;
+        const long long to = n_mid * (i + 1) / rounds;
+        p.do_entry = entry && i == 0;
+        p.n_mid = (int)(to - done);
+        p.do_exit = exit && last;
+        p.p_first = (int)((p_first + done) & 1);
+        p.sigma_in = sigma;
+        p.rescale_phase = until;
+        if (every > 0) {
+            int ev = 0;
+            for (int m = 0; m < p.n_mid; ++m) {
+                dd_mul(sigma, sigma_lo, p.onepg, growth_lo);
+                if (--until == 0) {
+                    until = every;
+                    int e2 = 0;
+                    std::frexp(sigma, &e2);
+                    p.rs_exp[ev++] = (short)(e2 - 1);
+                    sigma = std::ldexp(sigma, 1 - e2);
+                    sigma_lo = std::ldexp(sigma_lo, 1 - e2);
+                }
+            }
+        }
+        if (p.do_exit) {
+            p.x1 = dd_div(base.x1, sigma, sigma_lo);
+            p.x2 = dd_div(base.x2, sigma, sigma_lo);
+            p.xs = dd_div(base.xs, sigma, sigma_lo);
+        } else if (last && every > 0) {
+            p.out_scale = dd_div(1.0, sigma, sigma_lo);
+        }
+        if (!tb_geometry(prec, p.do_entry + p.n_mid + p.do_exit, &p.H, &p.U))
+            return false;
+        p.n = t.n;
+        p.n_rows = t.n_rows;
+        p.n_tiles = (t.n + p.U - 1) / p.U;
+        p.out = t.buf[(cur + i + 1) & 1];
+        p.err = t.err;
+        p.tile_ctr = t.tile_ctr + (i & 1);
+        p.tile_ctr_next = t.tile_ctr + ((i + 1) & 1);
+        out->r[i] = p;
+        done = to;
+    }
+    out->rounds = (int)rounds;
+    return true;
+}
+
 }  // namespace ge

@@ -86,6 +86,24 @@ def test_values_that_are_not_finite_reach_as_far_as_step_by_step(r, steps):
     assert rel_max(got[ok], want[ok]) <= tol64(r)
 
 
+@pytest.mark.parametrize("prec,n,r,steps", [
+    (B.GE_F64, 1 << 20, 1.0, 60), (B.GE_F64, (1 << 19) + 7, 4.0, 801), (B.GE_F32, (1 << 18) + 1, 4.0, 2001),
+    (B.GE_F32_COMP, 1 << 18, 4.0, 2000)])
+def test_grids_of_spikes_go_step_by_step(prec, n, r, steps):
+    """Most blocks far below their neighbours: the whole grid takes the steps
+    themselves, as rounds of one launch (the longer runs: several operators,
+    the middle ones between right-hand sides, the scale taken out)."""
+    u0 = np.zeros(n)
+    u0[::4999] = 1.0
+    want = oracle.run(u0, r, 0.2, -0.1, steps)
+    got = auto_run(u0, r, 0.2, -0.1, steps, prec)
+    assert rel_max(got, want) <= (tol64(r) if prec == B.GE_F64 else 1e-5)
+    if prec == B.GE_F64:  # blocks between the spikes keep their own digits
+        for a in range(64 * 20, n - 64 * 20, 64 * 37):
+            big = np.max(np.abs(want[a:a + 64]))
+            assert np.max(np.abs(got[a:a + 64] - want[a:a + 64])) <= 1e-10 * big, a
+
+
 def test_magnitudes_near_the_ends_of_the_exponent_range():
     n, r, steps = 20000, 2.0, 200
     u0 = inputs.random_state(n, seed=4)
