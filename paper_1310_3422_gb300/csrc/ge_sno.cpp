@@ -82,6 +82,8 @@ struct ge_sno {
     float *out = nullptr, *dout = nullptr, *loss = nullptr;  // [B n], [B n], [B]
     float *dA = nullptr, *dB = nullptr;   // [B n][max(C, H)] gradient scratch
     float *dvh = nullptr;                 // [B][2M][C]
+    float *sums = nullptr;                // column sums' scratch, and their blocks' counts (zero between launches)
+    int *sum_tickets = nullptr;
     // tensor-core inference path (ge_sno_tc.cu; plain mode, C = 64, 2M = 32,
     // H = 128, n a multiple of 128): transposed B operands and tensor maps
     bool tc = true;                       // use it where the shape allows
@@ -161,18 +163,46 @@ ge::GemmArgs &act_fmt(ge::GemmArgs &g, bool bf)
 
 // Weight gradient of a pointwise layer: dW[in][out] = X^T dY over R rows
 // (X rows ldx apart; split-K with atomics, FP32), db = column sums of dY.
+// The lift's 4 features and the last projection's single column are weighted
+// column sums instead of GEMMs.
 ge_status weight_grad(ge_sno *s, const void *X, int in, int ldx, const void *dY, int out, long long R, float *dW,
                       float *db)
 {
     const bool bf = bf16_mode(s);
+    ge::SnoSums a{};
+    a.rows = R;
+    a.part = s->sums;
+    a.ticket = s->sum_tickets;
+    if (out == 1 && ldx == in) {
+        a.x = X;
+        a.cols = in;
+        a.w = dY;
+        a.ldw = 1;
+        a.nw = 1;
+        a.wsum = dW;
+        a.wtot = db;
+        SNO_TRY(ge::sno_colsum(a, bf ? 1 : 0, s->stream));
+        return GE_OK;
+    }
+    a.x = dY;
+    a.cols = out;
+    a.sum = db;
+    if (in == 4) {
+        a.w = X;
+        a.ldw = ldx;
+        a.nw = 4;
+        a.wsum = dW;
+        SNO_TRY(ge::sno_colsum(a, bf ? 1 : 0, s->stream));
+        return GE_OK;
+    }
     SNO_TRY(cudaMemsetAsync(dW, 0, sizeof(float) * in * out, s->stream));
     ge::GemmArgs g = gemm(X, 1, ldx, dY, out, 1, dW, out, in, out, (int)R);
     act_fmt(g, bf).out_bf16 = 0;
-    long long ks = R / 1024;
+    long long ks = R / 512;
     g.ksplit = (int)(ks < 1 ? 1 : (ks > 512 ? 512 : ks));
     SNO_TRY(ge::sno_gemm(g, 1, s->split, s->stream));
     if (db)
-        SNO_TRY(ge::sno_colsum(dY, db, R, out, bf ? 1 : 0, s->stream));
+        SNO_TRY(ge::sno_colsum(a, bf ? 1 : 0, s->stream));
     return GE_OK;
 }
 
@@ -299,12 +329,7 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
     g.bias = P + s->off_qb1;
     g.act = s->h;
     SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
-    g = gemm(s->h, H, 1, weight(s, s->off_q2), 1, 1, out, 1, (int)R, 1, H);
-    g.bias = P + s->off_qb2;
-    g.C0 = u0;
-    g.beta = 1.0f;
-    act_fmt(g, bf).out_bf16 = 0;
-    SNO_TRY(ge::sno_gemm(g, 1, s->split, st));
+    SNO_TRY(ge::sno_row_dot(s->h, weight(s, s->off_q2), P + s->off_qb2, u0, out, R, H, bf ? 1 : 0, st));
     return GE_OK;
 }
 
@@ -378,12 +403,10 @@ ge_status backward(ge_sno *s, int B)
     if ((rc = weight_grad(s, s->h, H, H, s->dout, 1, R, Gd + s->off_q2, Gd + s->off_qb2)) != GE_OK)
         return rc;
     // dhpre = (dout Q2^T) * GELU'(hpre)
-    ge::GemmArgs g = gemm(s->dout, 1, 1, weight(s, s->off_q2), 1, 1, s->dA, H, (int)R, H, 1);
-    g.dgelu_pre = s->hpre;
-    SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
+    SNO_TRY(ge::sno_outer_dgelu(s->dout, weight(s, s->off_q2), s->hpre, s->dA, R, H, bf ? 1 : 0, st));
     if ((rc = weight_grad(s, s->v[s->L], C, C, s->dA, H, R, Gd + s->off_q1, Gd + s->off_qb1)) != GE_OK)
         return rc;
-    g = gemm(s->dA, H, 1, weight(s, s->off_q1), 1, H, s->dB, C, (int)R, C, H);  // dv_L = dhpre Q1^T
+    ge::GemmArgs g = gemm(s->dA, H, 1, weight(s, s->off_q1), 1, H, s->dB, C, (int)R, C, H);  // dv_L = dhpre Q1^T
     SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
     // dv holds the gradient of the current layer's pre-activation: the last
     // layer has no activation, and every lower one's GELU' is applied in the
@@ -571,6 +594,10 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
     e = e ? e : alloc(&s->loss, max_batch);
     e = e ? e : alloc(&s->dA, R * (C > H ? C : H));
     e = e ? e : alloc(&s->dB, R * (C > H ? C : H));
+    e = e ? e : alloc(&s->sums, ge::sno_sum_floats(C > H ? C : H));
+    e = e ? e : alloc_bytes(reinterpret_cast<void **>(&s->sum_tickets), 4LL * ge::sno_sum_tickets(C > H ? C : H));
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(s->sum_tickets, 0, 4LL * ge::sno_sum_tickets(C > H ? C : H), s->stream);
     e = e ? e : alloc_bytes(&s->wt, 2LL * layers * C * C);
     e = e ? e : alloc_bytes(&s->q1t, 2LL * H * C);
     e = e ? e : alloc_bytes(&s->wst, 2LL * layers * M * 4 * C * C);

@@ -113,7 +113,29 @@ cudaError_t sno_features(const float *u0, const float *r, const float *bl, const
 cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int modes, int c, int bf16, cudaStream_t s,
                               bool k_major = false);
 cudaError_t sno_spec_reduce(const float *dw, float *drr, float *dri, int modes, int c, cudaStream_t s);
-cudaError_t sno_colsum(const void *x, float *out, long long rows, int cols, int bf16, cudaStream_t s);
+// Column sums of x [rows][cols], plain and weighted by w [rows][ldw]'s first
+// nw (0, 1 or 4) columns; sum, wsum [nw][cols] and wtot (of w's first column)
+// may be NULL.  part: sno_sum_floats(cols) floats of scratch, ticket:
+// sno_sum_tickets(cols) ints, zero before the first call.
+struct SnoSums {
+    const void *x;
+    long long rows;
+    int cols;
+    const void *w;
+    int ldw, nw;
+    float *part;
+    int *ticket;
+    float *sum, *wsum, *wtot;
+};
+long long sno_sum_floats(int cols);
+int sno_sum_tickets(int cols);
+cudaError_t sno_colsum(const SnoSums &a, int bf16, cudaStream_t s);
+// out[i, j] = d[i] q[j] GELU'(pre[i, j]).
+cudaError_t sno_outer_dgelu(const void *d, const void *q, const void *pre, void *out, long long rows, int cols, int bf16,
+                            cudaStream_t s);
+// out[i] = u0[i] + q2[0] + sum_j h[i, j] q[j].
+cudaError_t sno_row_dot(const void *h, const void *q, const float *q2, const float *u0, float *out, long long rows, int cols,
+                        int bf16, cudaStream_t s);
 cudaError_t sno_rel_l2(const float *pred, const float *target, void *dpred, float *loss, int n, int batch, int bf16,
                        cudaStream_t s);
 cudaError_t sno_adam(float *p, const float *g, float *m, float *v, long long n, float lr, float b1, float b2,

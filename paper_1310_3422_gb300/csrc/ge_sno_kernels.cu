@@ -391,9 +391,13 @@ __device__ __forceinline__ void mainloop_f32(const GemmArgs &g, int bz, int ksli
     }
 }
 
-// Main loop, BF16 operands: the slices of both products run through two
-// shared-memory stages; the copies of slice i+1 are in flight while slice i
-// is multiplied.
+// Main loop, BF16 operands: the slices of both products run through kStages
+// shared-memory stages; the copies of the next slices are in flight while
+// slice i is multiplied.  (Most of the network's GEMMs are a few dozen CTAs
+// with a long K: with two stages each slice waited for its copies, 0.75 us a
+// slice; TBD.)
+constexpr int kStages = 4;
+
 __device__ __forceinline__ void mainloop_bf16(const GemmArgs &g, int bz, int kslice, int ks_n, int i0, int j0,
                                               float (&acc)[2][4][4], __nv_bfloat16 (*As)[TILE],
                                               __nv_bfloat16 (*Bs)[TILE], int t, int wm, int wn, int lane)
@@ -405,24 +409,28 @@ __device__ __forceinline__ void mainloop_bf16(const GemmArgs &g, int bz, int ksl
     auto issue = [&](int i) {
         const Seg &sg = i < n0 ? s0 : s1;
         const int k0 = sg.kbeg + (i < n0 ? i : i - n0) * BK;
-        __nv_bfloat16 *as = As[i & 1], *bs = Bs[i & 1];
+        __nv_bfloat16 *as = As[i % kStages], *bs = Bs[i % kStages];
         stage_bf16(as, static_cast<const __nv_bfloat16 *>(sg.A), sg.la_i, sg.la_k, i0, g.M, k0, sg.kend, sg.va, t);
         stage_bf16(bs, static_cast<const __nv_bfloat16 *>(sg.B), sg.lb_j, sg.lb_k, j0, g.N, k0, sg.kend, sg.vb, t);
         cp_async_commit();
     };
-    if (nt > 0)
-        issue(0);
+    // a group per slice, empty past the end, so that the count in flight is fixed
+#pragma unroll
+    for (int i = 0; i < kStages - 1; ++i) {
+        if (i < nt)
+            issue(i);
+        else
+            cp_async_commit();
+    }
     for (int i = 0; i < nt; ++i) {
-        if (i + 1 < nt) {
-            issue(i + 1);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
+        cp_async_wait<kStages - 2>();
+        __syncthreads();  // slice i has landed, and every warp is done with slice i - 1
+        if (i + kStages - 1 < nt)
+            issue(i + kStages - 1);
+        else
+            cp_async_commit();
         const Seg &sg = i < n0 ? s0 : s1;
-        mma_tile<false>(As + (i & 1), Bs + (i & 1), acc, wm, wn, lane, sg.la_k == 1, sg.lb_k == 1);
-        __syncthreads();
+        mma_tile<false>(As + i % kStages, Bs + i % kStages, acc, wm, wn, lane, sg.la_k == 1, sg.lb_k == 1);
     }
 }
 
@@ -562,7 +570,7 @@ __device__ __forceinline__ void epilogue(const GemmArgs &g, int bz, int ks_n, in
 template <bool SPLIT, int MODE>
 __global__ void __launch_bounds__(NT, MODE == 0 ? 1 : 4) gemm_kernel(GemmArgs g)
 {
-    constexpr int NS = (SPLIT || MODE == 2) ? 2 : 1;  // split parts, or pipeline stages
+    constexpr int NS = MODE == 2 ? kStages : SPLIT ? 2 : 1;  // pipeline stages, or split parts
     __shared__ __align__(16) __nv_bfloat16 As[NS][TILE];
     __shared__ __align__(16) __nv_bfloat16 Bs[NS][TILE];
     const int ks_n = g.ksplit > 1 ? g.ksplit : 1;
@@ -661,25 +669,203 @@ __global__ void spec_reduce_kernel(const float *__restrict__ dw, float *__restri
     }
 }
 
-// Column sums (bias gradients): out[j] = sum_i x[i, j], x is rows x cols
-// (FP32 or BF16).
-__global__ void colsum_kernel(const void *__restrict__ x, float *__restrict__ out, long long rows, int cols, int bf16)
-{
-    const int j = blockIdx.x;
-    float s = 0.0f;
-    for (long long i = threadIdx.x; i < rows; i += blockDim.x)
-        s += bf16 ? __bfloat162float(static_cast<const __nv_bfloat16 *>(x)[i * cols + j])
-                  : static_cast<const float *>(x)[i * cols + j];
-    __shared__ float red[256];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w)
-            red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
+// 16 bytes of a matrix row as floats.
+template <typename T>
+struct Chunk;
+template <>
+struct Chunk<float> {
+    static constexpr int E = 4;
+    static __device__ __forceinline__ void load(const float *p, float (&v)[4])
+    {
+        const float4 q = *reinterpret_cast<const float4 *>(p);
+        v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
     }
-    if (threadIdx.x == 0)
-        out[j] = red[0];
+};
+template <>
+struct Chunk<__nv_bfloat16> {
+    static constexpr int E = 8;
+    static __device__ __forceinline__ void load(const __nv_bfloat16 *p, float (&v)[8])
+    {
+        const uint4 q = *reinterpret_cast<const uint4 *>(p);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w[i]));
+            v[2 * i] = f.x;
+            v[2 * i + 1] = f.y;
+        }
+    }
+};
+__device__ __forceinline__ float to_f(float x) { return x; }
+__device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
+
+// Column sums of x [rows][cols] (bias gradients), plain and weighted by the
+// columns of w [rows][ldw]:
+//   sum[j] = sum_i x[i, j],  wsum[f][j] = sum_i w[i, f] x[i, j] (f < NW),
+//   wtot = sum_i w[i, 0];  each may be NULL.
+// With NW = 4 and w the features it is the lift's weight gradient, with NW =
+// 1 and w the output's gradient that of the last projection: products with 4
+// or 1 rows, which a 64-row GEMM tile took 81 and 42 us for (65,536 rows).
+// Bound by reading x once: blocks of 256 threads take rows in turn, 16 bytes
+// a thread (V; else single values), and the last block to finish adds the
+// blocks' sums in their order, so the result does not depend on timing.  (A
+// block per column, striding through the rows: 47 us for 8 MB, now TBD us.)
+constexpr int kSumBlocks = 192;
+
+template <typename T, int NW, bool V>
+__global__ void __launch_bounds__(256) colsum_kernel(const T *__restrict__ x, long long rows, int cols,
+                                                     const T *__restrict__ w, int ldw, float *__restrict__ part,
+                                                     int *__restrict__ ticket, float *__restrict__ sum,
+                                                     float *__restrict__ wsum, float *__restrict__ wtot)
+{
+    constexpr int E = V ? Chunk<T>::E : 1, TPR = V ? 64 / E : 32, CW = E * TPR, G = 256 / TPR, S = 1 + NW;
+    __shared__ float red[G][CW];
+    __shared__ float tot[G];
+    __shared__ int last;
+    const int t = threadIdx.x, tc = t % TPR, g = t / TPR, c0 = blockIdx.y * CW, c = c0 + tc * E;
+    const bool in = c < cols;
+    float acc[S][E] = {}, at = 0.0f;
+#pragma unroll 4
+    for (long long i = (long long)blockIdx.x * G + g; i < rows; i += (long long)gridDim.x * G) {
+        float v[E], wv[NW > 0 ? NW : 1];
+        if constexpr (V) {
+            if (in)
+                Chunk<T>::load(x + i * cols + c, v);
+        } else {
+            v[0] = in ? to_f(x[i * cols + c]) : 0.0f;
+        }
+#pragma unroll
+        for (int f = 0; f < NW; ++f)
+            wv[f] = to_f(w[i * ldw + f]);
+        if (!in)
+            continue;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            acc[0][e] += v[e];
+#pragma unroll
+            for (int f = 0; f < NW; ++f)
+                acc[1 + f][e] = fmaf(wv[f], v[e], acc[1 + f][e]);
+        }
+        if (NW > 0 && tc == 0)
+            at += wv[0];
+    }
+    const long long stride = (long long)S * cols + 1;
+    float *mine = part + blockIdx.x * stride;
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            red[g][tc * E + e] = acc[q][e];
+        if (tc == 0)
+            tot[g] = at;
+        __syncthreads();
+        if (t < CW && c0 + t < cols) {
+            float v = 0.0f;
+            for (int i = 0; i < G; ++i)
+                v += red[i][t];
+            mine[(long long)q * cols + c0 + t] = v;
+        }
+        if (t == 0 && q == 0 && blockIdx.y == 0) {
+            float v = 0.0f;
+            for (int i = 0; i < G; ++i)
+                v += tot[i];
+            mine[(long long)S * cols] = v;
+        }
+    }
+    __threadfence();
+    __syncthreads();
+    if (t == 0)
+        last = atomicAdd(ticket + blockIdx.y, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!last)
+        return;
+    __threadfence();
+    if (t == 0)
+        ticket[blockIdx.y] = 0;  // the next launch's
+    for (int o = t; o < S * CW; o += 256) {
+        const int q = o / CW, j = c0 + o % CW;
+        float *out = q == 0 ? sum : wsum;
+        if (j >= cols || !out)
+            continue;
+        float v = 0.0f;
+#pragma unroll 8
+        for (int i = 0; i < (int)gridDim.x; ++i)
+            v += __ldcg(part + i * stride + (long long)q * cols + j);
+        out[(q == 0 ? 0 : (long long)(q - 1) * cols) + j] = v;
+    }
+    if (wtot && blockIdx.y == 0 && t == 255) {
+        float v = 0.0f;
+        for (int i = 0; i < (int)gridDim.x; ++i)
+            v += __ldcg(part + i * stride + (long long)S * cols);
+        *wtot = v;
+    }
+}
+
+// Gradient of the hidden layer's pre-activation: out[i, j] = d[i] q[j]
+// GELU'(pre[i, j]).  An elementwise pass over pre and out (as a GEMM with K =
+// 1: 52 us for 65,536 x 128 BF16, now TBD us).
+template <bool EXACT, typename T, bool V>
+__global__ void __launch_bounds__(256) outer_dgelu_kernel(const T *__restrict__ d, const T *__restrict__ q,
+                                                          const T *__restrict__ pre, T *__restrict__ out,
+                                                          long long rows, int cols)
+{
+    constexpr int E = V ? Chunk<T>::E : 1;
+    const long long total = rows * cols / E;
+    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < total; i += (long long)gridDim.x * 256) {
+        const long long r = i * E / cols;
+        const int j = (int)(i * E - r * cols);
+        const float dv = to_f(d[r]);
+        float p[E];
+        __align__(16) T o[E];
+        if constexpr (V)
+            Chunk<T>::load(pre + i * E, p);
+        else
+            p[0] = to_f(pre[i]);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            o[e] = static_cast<T>(dv * to_f(q[j + e]) * gelu_grad<EXACT>(p[e]));
+        if constexpr (V)
+            *reinterpret_cast<uint4 *>(out + i * E) = *reinterpret_cast<const uint4 *>(o);
+        else
+            out[i] = o[0];
+    }
+}
+
+// out[i] = u0[i] + q2[0] + sum_j h[i, j] q[j], a warp per row.  (As a GEMM
+// with one column: 23 us for 65,536 x 128 BF16, now TBD us.)
+template <typename T, bool V>
+__global__ void __launch_bounds__(256) row_dot_kernel(const T *__restrict__ h, const T *__restrict__ q,
+                                                      const float *__restrict__ q2, const float *__restrict__ u0,
+                                                      float *__restrict__ out, long long rows, int cols)
+{
+    constexpr int E = V ? Chunk<T>::E : 1;
+    const int lane = threadIdx.x & 31;
+    const long long step = (long long)gridDim.x * 8;
+    // the lane's first weights stay in registers (all of them up to 32 E columns)
+    float w[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        w[e] = lane * E + e < cols ? to_f(q[lane * E + e]) : 0.0f;
+#pragma unroll 4
+    for (long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); i < rows; i += step) {
+        float s = 0.0f;
+        for (int j = lane * E; j < cols; j += 32 * E) {
+            float a[E];
+            if constexpr (V)
+                Chunk<T>::load(h + i * cols + j, a);
+            else
+                a[0] = to_f(h[i * cols + j]);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                s = fmaf(a[e], j == lane * E ? w[e] : to_f(q[j + e]), s);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0)
+            out[i] = u0[i] + q2[0] + s;
+    }
 }
 
 // Relative L2 loss per sample and its gradient: loss_b = ||p - y|| / ||y||,
@@ -1093,10 +1279,83 @@ cudaError_t sno_spec_reduce(const float *dw, float *drr, float *dri, int modes, 
     return cudaGetLastError();
 }
 
-cudaError_t sno_colsum(const void *x, float *out, long long rows, int cols, int bf16, cudaStream_t s)
+namespace {
+
+template <typename T, int NW>
+void launch_colsum(const SnoSums &a, cudaStream_t s)
 {
-    colsum_kernel<<<cols, 256, 0, s>>>(x, out, rows, cols, bf16);
+    const T *x = static_cast<const T *>(a.x), *w = static_cast<const T *>(a.w);
+    const bool v = a.cols % Chunk<T>::E == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+    const int cw = v ? 64 : 32;
+    const dim3 grid(kSumBlocks, (a.cols + cw - 1) / cw);
+    if (v)
+        colsum_kernel<T, NW, true><<<grid, 256, 0, s>>>(x, a.rows, a.cols, w, a.ldw, a.part, a.ticket, a.sum, a.wsum, a.wtot);
+    else
+        colsum_kernel<T, NW, false><<<grid, 256, 0, s>>>(x, a.rows, a.cols, w, a.ldw, a.part, a.ticket, a.sum, a.wsum, a.wtot);
+}
+
+template <typename T>
+cudaError_t pick_colsum(const SnoSums &a, cudaStream_t s)
+{
+    switch (a.nw) {
+    case 0: launch_colsum<T, 0>(a, s); break;
+    case 1: launch_colsum<T, 1>(a, s); break;
+    case 4: launch_colsum<T, 4>(a, s); break;
+    default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
+}
+
+template <bool EXACT, typename T>
+cudaError_t launch_outer(const void *d, const void *q, const void *pre, void *out, long long rows, int cols, cudaStream_t s)
+{
+    const bool v = cols % Chunk<T>::E == 0 && ((reinterpret_cast<uintptr_t>(pre) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+    const long long total = rows * cols / (v ? Chunk<T>::E : 1);
+    const int grid = grid_for(total);
+    const T *dt = static_cast<const T *>(d), *qt = static_cast<const T *>(q), *pt = static_cast<const T *>(pre);
+    if (v)
+        outer_dgelu_kernel<EXACT, T, true><<<grid, 256, 0, s>>>(dt, qt, pt, static_cast<T *>(out), rows, cols);
+    else
+        outer_dgelu_kernel<EXACT, T, false><<<grid, 256, 0, s>>>(dt, qt, pt, static_cast<T *>(out), rows, cols);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_row_dot(const void *h, const void *q, const float *q2, const float *u0, float *out, long long rows,
+                           int cols, cudaStream_t s)
+{
+    const T *ht = static_cast<const T *>(h), *qt = static_cast<const T *>(q);
+    const bool v = cols % Chunk<T>::E == 0 && (reinterpret_cast<uintptr_t>(h) & 15) == 0;
+    const int grid = grid_for(rows * 8);
+    if (v)
+        row_dot_kernel<T, true><<<grid, 256, 0, s>>>(ht, qt, q2, u0, out, rows, cols);
+    else
+        row_dot_kernel<T, false><<<grid, 256, 0, s>>>(ht, qt, q2, u0, out, rows, cols);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+long long sno_sum_floats(int cols) { return (long long)kSumBlocks * (5LL * cols + 1); }
+int sno_sum_tickets(int cols) { return (cols + 31) / 32; }
+
+cudaError_t sno_colsum(const SnoSums &a, int bf16, cudaStream_t s)
+{
+    return bf16 ? pick_colsum<__nv_bfloat16>(a, s) : pick_colsum<float>(a, s);
+}
+
+cudaError_t sno_outer_dgelu(const void *d, const void *q, const void *pre, void *out, long long rows, int cols, int bf16,
+                            cudaStream_t s)
+{
+    return bf16 ? launch_outer<false, __nv_bfloat16>(d, q, pre, out, rows, cols, s)
+                : launch_outer<true, float>(d, q, pre, out, rows, cols, s);
+}
+
+cudaError_t sno_row_dot(const void *h, const void *q, const float *q2, const float *u0, float *out, long long rows, int cols,
+                        int bf16, cudaStream_t s)
+{
+    return bf16 ? launch_row_dot<__nv_bfloat16>(h, q, q2, u0, out, rows, cols, s)
+                : launch_row_dot<float>(h, q, q2, u0, out, rows, cols, s);
 }
 
 cudaError_t sno_rel_l2(const float *pred, const float *target, void *dpred, float *loss, int n, int batch, int bf16,
