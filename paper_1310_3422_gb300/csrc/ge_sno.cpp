@@ -95,7 +95,13 @@ struct ge_sno {
     // the weight-derived operands above (and the rounded weights pw, pw16)
     // no longer match the parameters: set when the parameters change
     bool tc_stale = true;
+    void *ws = nullptr;                   // [L][M][2C in][2C out] BF16 (the backward mixing's operand)
+    void *FT16 = nullptr, *GT16 = nullptr;  // F^T [n][2M], G^T [2M][n] BF16 (backward)
     int *err = nullptr;                   // device error word of the tensor-core kernels
+    // training: F^T, G^T, the spectral weights, the gradients' spectra (dy as
+    // mixing rows, dvh as a layer's operand) and buffers, W of each layer
+    CUtensorMap tm_ft, tm_gt, tm_ws, tm_dy, tm_dvh, tm_dA, tm_dB, tm_dAs, tm_dBs;
+    std::vector<CUtensorMap> tm_w;
     CUtensorMap tm_g, tm_y, tm_wt, tm_q1t, tm_f, tm_wst;
     std::vector<CUtensorMap> tm_v;        // one per activation buffer v[0..L]
     std::vector<CUtensorMap> tm_vs;       // store maps of v[1..L] (index l: v[l + 1])
@@ -247,8 +253,9 @@ bool tc_active(const ge_sno *s) { return s->tc && !s->split && tc_shape(s) && s-
 
 // Inference with the tensor-core kernels for the truncated DFT, the fused
 // layers and the projection (the mode mixing keeps the mma.sync GEMM).
-ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br,
-                     float *out);
+ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br, float *out,
+                     bool keep);
+ge_status project_keep(ge_sno *s, const float *u0, float *out, long long R);
 
 // Forward pass for B problems into out ([B n], FP32).  keep: also store the
 // pre-activations the backward pass needs (training).
@@ -262,8 +269,8 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
     const float *P = s->pw;  // FP32 rounded weights: biases and the spectral matrices' source
     const void *F = bf ? s->F16 : static_cast<const void *>(s->F);
     const void *G = bf ? s->G16 : static_cast<const void *>(s->G);
-    if (!keep && tc_active(s))
-        return forward_tc(s, B, u0, r, bl, br, out);
+    if (tc_active(s))
+        return forward_tc(s, B, u0, r, bl, br, out, keep);
     SNO_TRY(ge::sno_round_bf16(s->params, s->pw, bf ? s->pw16 : nullptr, s->n_params, st));
     // lift (K = 4: no GEMM); the features themselves only for the backward pass
     if (keep)
@@ -325,35 +332,60 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
         SNO_TRY(ge::sno_dot_finish(u0, P + s->off_qb2, s->dA, slots, out, R, st));
         return GE_OK;
     }
-    g = gemm(s->v[s->L], C, 1, weight(s, s->off_q1), H, 1, s->hpre, H, (int)R, H, C);
+    return project_keep(s, u0, out, R);
+}
+
+// The projection of a training pass: hpre, h and the output.
+ge_status project_keep(ge_sno *s, const float *u0, float *out, long long R)
+{
+    const int C = s->C, H = s->H;
+    const bool bf = bf16_mode(s);
+    const float *P = s->pw;
+    ge::GemmArgs g = gemm(s->v[s->L], C, 1, weight(s, s->off_q1), H, 1, s->hpre, H, (int)R, H, C);
     g.bias = P + s->off_qb1;
     g.act = s->h;
-    SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
-    SNO_TRY(ge::sno_row_dot(s->h, weight(s, s->off_q2), P + s->off_qb2, u0, out, R, H, bf ? 1 : 0, st));
+    SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, s->stream));
+    SNO_TRY(ge::sno_row_dot(s->h, weight(s, s->off_q2), P + s->off_qb2, u0, out, R, H, bf ? 1 : 0, s->stream));
     return GE_OK;
 }
 
-ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br,
-                     float *out)
+ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br, float *out,
+                     bool keep)
 {
     const int n = s->n, C = s->C, M = s->M, H = s->H;
     const long long R = (long long)B * n;
     cudaStream_t st = s->stream;
     const float *P = s->pw;
-    if (s->tc_stale) {
-        // operands derived from the weights, once per parameter change: the
-        // rounded weights, the K-major copies W^T (per layer) and Q1^T, and
-        // the K-major spectral weights Wspec_m^T
-        SNO_TRY(ge::sno_round_bf16(s->params, s->pw, s->pw16, s->n_params, st));
-        for (int l = 0; l < s->L; ++l)
-            SNO_TRY(ge::sno_transpose_rows(at(s->pw16, s->lay[l].w, true), at(s->wt, (long long)l * C * C, true), 1,
-                                           C, C, st));
-        SNO_TRY(ge::sno_transpose_rows(at(s->pw16, s->off_q1, true), s->q1t, 1, C, H, st));
-        for (int l = 0; l < s->L; ++l)
-            SNO_TRY(ge::sno_spec_assemble(P + s->lay[l].rr, P + s->lay[l].ri,
-                                          at(s->wst, (long long)l * M * 4 * C * C, true), M, C, 1, st, true));
-        s->tc_stale = false;
+    if (s->tc_stale || keep) {
+        // operands derived from the weights: the rounded weights, the K-major
+        // copies W^T (per layer) and Q1^T, and the spectral matrices both
+        // ways.  Inference rebuilds them once per parameter change; a
+        // training pass always does, so that one captured in a graph uses
+        // the parameters of its replay.
+        ge::SnoPrepare w{};
+        w.params = s->params;
+        w.count = s->n_params;
+        w.pw = s->pw;
+        w.pw16 = s->pw16;
+        w.wt = s->wt;
+        w.ws = s->ws;
+        w.wst = s->wst;
+        w.q1t = s->q1t;
+        w.c = C;
+        w.modes = M;
+        w.layers = s->L;
+        w.h = H;
+        w.lay0 = s->lay[0].rr;
+        w.lay_size = 2LL * M * C * C + (long long)C * C + C;
+        w.q1 = s->off_q1;
+        SNO_TRY(ge::sno_prepare(w, st));
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        SNO_TRY(cudaStreamIsCapturing(st, &cap));
+        if (!keep || cap == cudaStreamCaptureStatusNone)
+            s->tc_stale = false;
     }
+    if (keep)
+        SNO_TRY(ge::sno_features(u0, r, bl, br, s->feat, B, n, 1, st));
     SNO_TRY(ge::sno_lift(u0, r, bl, br, weight(s, s->off_w0), P + s->off_b0, s->v[0], B, n, C, 1, st));
     ge::SnoTcArgs a{};
     a.n_tiles = R / 128;
@@ -372,11 +404,15 @@ ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const fl
         a.gelu = l < s->L - 1 ? 1 : 0;
         a.bias = P + o.b;
         a.out = s->v[l + 1];
+        a.pre = keep && l < s->L - 1 ? s->pre[l] : nullptr;
         const ge::SnoTcMaps m{&s->tm_g, &s->tm_y, &s->tm_v[l], &s->tm_wt, &s->tm_vs[l]};
         SNO_TRY(ge::sno_tc_layer(m, a, s->num_sms, st));
     }
+    if (keep)
+        return project_keep(s, u0, out, R);
     a.b2_row = 0;
     a.gelu = 1;
+    a.pre = nullptr;
     a.bias = P + s->off_qb1;
     a.q2w = P + s->off_q2;
     a.q2b = P + s->off_qb2;
@@ -412,6 +448,12 @@ ge_status backward(ge_sno *s, int B)
     // layer has no activation, and every lower one's GELU' is applied in the
     // epilogue of the GEMM that makes its gradient.
     void *dv = s->dB, *dnext = s->dA;
+    const bool tc = tc_active(s);
+    ge::SnoTcArgs ta{};
+    ta.n_tiles = R / 128;
+    ta.tiles_per_problem = n / 128;
+    ta.err = s->err;
+    ta.limit = ge::kWaitLimitCycles;
     for (int l = s->L - 1; l >= 0; --l) {
         const LayerOff &o = s->lay[l];
         const void *ws = at(s->wspec, (long long)l * M * 4 * C * C, bf);
@@ -420,11 +462,16 @@ ge_status backward(ge_sno *s, int B)
         if ((rc = weight_grad(s, s->v[l], C, C, dpre, C, R, Gd + o.w, Gd + o.b)) != GE_OK)
             return rc;
         // spectral path: dy[b] = G^T dpre[b]
-        g = gemm(G, 1, 2 * M, dpre, C, 1, s->y, C, 2 * M, C, n);
-        g.sA = 0;
-        g.sB = (long long)n * C;
-        g.sC = 2LL * M * C;
-        SNO_TRY(ge::sno_gemm(act_fmt(g, bf), B, s->split, st));
+        if (tc) {
+            ta.out = s->y;
+            SNO_TRY(ge::sno_tc_dft(&s->tm_gt, dv == s->dB ? &s->tm_dB : &s->tm_dA, ta, s->num_sms, st));
+        } else {
+            g = gemm(G, 1, 2 * M, dpre, C, 1, s->y, C, 2 * M, C, n);
+            g.sA = 0;
+            g.sB = (long long)n * C;
+            g.sC = 2LL * M * C;
+            SNO_TRY(ge::sno_gemm(act_fmt(g, bf), B, s->split, st));
+        }
         // dWspec_m = vh[:, m]^T dy[:, m]  (FP32)
         g = gemm(s->vh[l], 1, 2LL * M * C, s->y, 2LL * M * C, 1, s->dwspec, 2 * C, 2 * C, 2 * C, B);
         g.sA = 2 * C;
@@ -433,6 +480,20 @@ ge_status backward(ge_sno *s, int B)
         act_fmt(g, bf).out_bf16 = 0;
         SNO_TRY(ge::sno_gemm(g, M, s->split, st));
         SNO_TRY(ge::sno_spec_reduce(s->dwspec, Gd + o.rr, Gd + o.ri, M, C, st));
+        if (tc) {
+            // dvh[:, m] = dy[:, m] Wspec_m^T, then both paths as one layer
+            const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->dvh, s->err, ge::kWaitLimitCycles};
+            SNO_TRY(ge::sno_tc_mix(&s->tm_dy, &s->tm_ws, x, M, st));
+            ta.b2_row = 0;
+            ta.out = dnext;
+            ta.dg = l > 0 ? s->pre[l - 1] : nullptr;
+            const bool from_b = dv == s->dB;
+            const ge::SnoTcMaps m{&s->tm_ft, &s->tm_dvh, from_b ? &s->tm_dB : &s->tm_dA, &s->tm_w[l],
+                                  from_b ? &s->tm_dAs : &s->tm_dBs};
+            SNO_TRY(ge::sno_tc_layer(m, ta, s->num_sms, st));
+            std::swap(dv, dnext);
+            continue;
+        }
         // dvh[:, m] = dy[:, m] Wspec_m^T
         g = gemm(s->y, 2LL * M * C, 1, ws, 1, 2 * C, s->dvh, 2LL * M * C, B, 2 * C, 2 * C);
         g.sA = 2 * C;
@@ -601,6 +662,9 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
     e = e ? e : alloc_bytes(&s->wt, 2LL * layers * C * C);
     e = e ? e : alloc_bytes(&s->q1t, 2LL * H * C);
     e = e ? e : alloc_bytes(&s->wst, 2LL * layers * M * 4 * C * C);
+    e = e ? e : alloc_bytes(&s->ws, 2LL * layers * M * 4 * C * C);
+    e = e ? e : alloc_bytes(&s->FT16, 2 * 2 * M * n);
+    e = e ? e : alloc_bytes(&s->GT16, 2 * 2 * M * n);
     e = e ? e : alloc_bytes(reinterpret_cast<void **>(&s->err), 256);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(s->err, 0, 256, s->stream);
@@ -630,6 +694,17 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
         s->tm_vh.resize(layers);
         for (int l = 0; l < layers && ok; ++l)
             ok = bf16_map(&s->tm_vh[l], s->vh[l], max_batch, 2 * modes * width, 64, 128);
+        // training: the same kernels on the transposed operands and the gradients
+        ok = ok && bf16_map(&s->tm_ft, s->FT16, n, 2 * modes, 2 * modes, 128) &&
+             bf16_map(&s->tm_gt, s->GT16, 2 * modes, n, 64, 2 * modes) &&
+             bf16_map(&s->tm_ws, s->ws, (long long)layers * modes * 2 * width, 2 * width, 64, 128) &&
+             bf16_map(&s->tm_dy, s->y, max_batch, 2 * modes * width, 64, 128) &&
+             bf16_map(&s->tm_dvh, s->dvh, (long long)max_batch * 2 * modes, width, width, 2 * modes) &&
+             bf16_map(&s->tm_dA, s->dA, R, width, width, 128) && bf16_map(&s->tm_dB, s->dB, R, width, width, 128) &&
+             bf16_map(&s->tm_dAs, s->dA, R, width, 32, 32) && bf16_map(&s->tm_dBs, s->dB, R, width, 32, 32);
+        s->tm_w.resize(layers);
+        for (int l = 0; l < layers && ok; ++l)
+            ok = bf16_map(&s->tm_w[l], static_cast<char *>(s->pw16) + 2 * s->lay[l].w, width, width, width, 64);
         s->tc_ready = ok;
     }
     // DFT bases: F[2m][j] = cos(2 pi m j / n), F[2m+1][j] = -sin(...);
@@ -663,10 +738,15 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
         p[s->off_q1 + i] = (float)rng.uniform(1.0 / std::sqrt((double)C));
     for (long long i = 0; i < H; ++i)
         p[s->off_q2 + i] = (float)rng.uniform(1.0 / std::sqrt((double)H));
-    std::vector<uint16_t> F16(F.size()), G16(Gm.size());
+    std::vector<uint16_t> F16(F.size()), G16(Gm.size()), FT16(F.size()), GT16(Gm.size());
     for (size_t i = 0; i < F.size(); ++i) {
         F16[i] = bf16_bits(F[i]);
         G16[i] = bf16_bits(Gm[i]);
+    }
+    for (int k = 0; k < 2 * modes; ++k)
+        for (int j = 0; j < n; ++j) {
+            FT16[(size_t)j * 2 * modes + k] = F16[(size_t)k * n + j];
+            GT16[(size_t)k * n + j] = G16[(size_t)j * 2 * modes + k];
     }
     e = cudaMemcpyAsync(s->F, F.data(), sizeof(float) * F.size(), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess)
@@ -675,6 +755,10 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
         e = cudaMemcpyAsync(s->F16, F16.data(), 2 * F16.size(), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->G16, G16.data(), 2 * G16.size(), cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(s->FT16, FT16.data(), 2 * FT16.size(), cudaMemcpyHostToDevice, s->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(s->GT16, GT16.data(), 2 * GT16.size(), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->params, p.data(), sizeof(float) * p.size(), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess)

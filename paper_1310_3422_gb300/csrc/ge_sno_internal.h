@@ -85,6 +85,8 @@ struct SnoTcArgs {
     void *out;              // layer: next activation, BF16 [rows][C]; projection: FP32 [rows]
     int *err;               // device error word (GE_ETIMEOUT on a wait that gave up)
     long long limit;        // wait limit in SM cycles
+    void *pre;              // layer: also the value before GELU, BF16 [rows][C], or NULL
+    const void *dg;         // layer: multiply by GELU' of these BF16 [rows][C], or NULL
 };
 cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s);
 cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s);
@@ -105,13 +107,9 @@ struct SnoTcMixArgs {
     long long limit;     // wait limit in SM cycles
 };
 cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s);
-// yt[b][c][k] = y[b][k][c] for BF16 [batch][k_rows][c_cols] blocks (the
-// K-major copies W^T and Q1^T).
-cudaError_t sno_transpose_rows(const void *y, void *yt, long long batch, int k_rows, int c_cols, cudaStream_t s);
 cudaError_t sno_features(const float *u0, const float *r, const float *bl, const float *br, void *f, int batch,
                          int n, int bf16, cudaStream_t s);
-cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int modes, int c, int bf16, cudaStream_t s,
-                              bool k_major = false);
+cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int modes, int c, int bf16, cudaStream_t s);
 cudaError_t sno_spec_reduce(const float *dw, float *drr, float *dri, int modes, int c, cudaStream_t s);
 // Column sums of x [rows][cols], plain and weighted by w [rows][ldw]'s first
 // nw (0, 1 or 4) columns; sum, wsum [nw][cols] and wtot (of w's first column)
@@ -140,6 +138,20 @@ cudaError_t sno_rel_l2(const float *pred, const float *target, void *dpred, floa
                        cudaStream_t s);
 cudaError_t sno_adam(float *p, const float *g, float *m, float *v, long long n, float lr, float b1, float b2,
                      float eps, float c1, float c2, cudaStream_t s);
+// The weights and everything the tensor-core kernels derive from them, in one
+// pass: pw and pw16 (rounded to BF16), and in BF16 per layer W^T [C out][C in]
+// (wt), the spectral matrices [2C in][2C out] (ws) and transposed (wst), and
+// Q1^T [H][C] (q1t).
+struct SnoPrepare {
+    const float *params;
+    long long count;
+    float *pw;
+    void *pw16, *wt, *ws, *wst, *q1t;
+    int c, modes, layers, h;
+    long long lay0, lay_size;  // first layer's Rr, parameters of a layer (Rr, Ri, W, b)
+    long long q1;              // first parameter of Q1
+};
+cudaError_t sno_prepare(const SnoPrepare &a, cudaStream_t s);
 cudaError_t sno_round_bf16(const float *x, float *y, void *y16, long long n, cudaStream_t s);
 // v0[b n + j][c] = b0[c] + sum_k feature_k(b, j) W0[k][c] (features as in
 // sno_features, rounded to BF16 when bf16); W0 BF16 or FP32 as v0.

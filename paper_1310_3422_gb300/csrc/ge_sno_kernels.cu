@@ -391,13 +391,9 @@ __device__ __forceinline__ void mainloop_f32(const GemmArgs &g, int bz, int ksli
     }
 }
 
-// Main loop, BF16 operands: the slices of both products run through kStages
-// shared-memory stages; the copies of the next slices are in flight while
-// slice i is multiplied.  (Most of the network's GEMMs are a few dozen CTAs
-// with a long K: with two stages each slice waited for its copies, 0.75 us a
-// slice; TBD.)
-constexpr int kStages = 4;
-
+// Main loop, BF16 operands: the slices of both products run through two
+// shared-memory stages; the copies of slice i+1 are in flight while slice i
+// is multiplied.
 __device__ __forceinline__ void mainloop_bf16(const GemmArgs &g, int bz, int kslice, int ks_n, int i0, int j0,
                                               float (&acc)[2][4][4], __nv_bfloat16 (*As)[TILE],
                                               __nv_bfloat16 (*Bs)[TILE], int t, int wm, int wn, int lane)
@@ -409,28 +405,24 @@ __device__ __forceinline__ void mainloop_bf16(const GemmArgs &g, int bz, int ksl
     auto issue = [&](int i) {
         const Seg &sg = i < n0 ? s0 : s1;
         const int k0 = sg.kbeg + (i < n0 ? i : i - n0) * BK;
-        __nv_bfloat16 *as = As[i % kStages], *bs = Bs[i % kStages];
+        __nv_bfloat16 *as = As[i & 1], *bs = Bs[i & 1];
         stage_bf16(as, static_cast<const __nv_bfloat16 *>(sg.A), sg.la_i, sg.la_k, i0, g.M, k0, sg.kend, sg.va, t);
         stage_bf16(bs, static_cast<const __nv_bfloat16 *>(sg.B), sg.lb_j, sg.lb_k, j0, g.N, k0, sg.kend, sg.vb, t);
         cp_async_commit();
     };
-    // a group per slice, empty past the end, so that the count in flight is fixed
-#pragma unroll
-    for (int i = 0; i < kStages - 1; ++i) {
-        if (i < nt)
-            issue(i);
-        else
-            cp_async_commit();
-    }
+    if (nt > 0)
+        issue(0);
     for (int i = 0; i < nt; ++i) {
-        cp_async_wait<kStages - 2>();
-        __syncthreads();  // slice i has landed, and every warp is done with slice i - 1
-        if (i + kStages - 1 < nt)
-            issue(i + kStages - 1);
-        else
-            cp_async_commit();
+        if (i + 1 < nt) {
+            issue(i + 1);
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
+        }
+        __syncthreads();
         const Seg &sg = i < n0 ? s0 : s1;
-        mma_tile<false>(As + i % kStages, Bs + i % kStages, acc, wm, wn, lane, sg.la_k == 1, sg.lb_k == 1);
+        mma_tile<false>(As + (i & 1), Bs + (i & 1), acc, wm, wn, lane, sg.la_k == 1, sg.lb_k == 1);
+        __syncthreads();
     }
 }
 
@@ -570,7 +562,7 @@ __device__ __forceinline__ void epilogue(const GemmArgs &g, int bz, int ks_n, in
 template <bool SPLIT, int MODE>
 __global__ void __launch_bounds__(NT, MODE == 0 ? 1 : 4) gemm_kernel(GemmArgs g)
 {
-    constexpr int NS = MODE == 2 ? kStages : SPLIT ? 2 : 1;  // pipeline stages, or split parts
+    constexpr int NS = (SPLIT || MODE == 2) ? 2 : 1;  // split parts, or pipeline stages
     __shared__ __align__(16) __nv_bfloat16 As[NS][TILE];
     __shared__ __align__(16) __nv_bfloat16 Bs[NS][TILE];
     const int ks_n = g.ksplit > 1 ? g.ksplit : 1;
@@ -624,10 +616,8 @@ __global__ void features_kernel(const float *__restrict__ u0, const float *__res
 // vector (re, im): [[Rr^T, Ri^T], [-Ri^T, Rr^T]] with R = Rr + i Ri (C x C,
 // out x in).  Layout of rr/ri: [m][out][in]; of w: [m][2C][2C].
 __global__ void spec_assemble_kernel(const float *__restrict__ rr, const float *__restrict__ ri,
-                                     void *__restrict__ w, int modes, int c, int bf16, int k_major)
+                                     void *__restrict__ w, int modes, int c, int bf16)
 {
-    // k_major: store each mode's matrix transposed, [2C out][2C in] (the
-    // K-major B operand of the tensor-core mixing)
     const long long total = (long long)modes * 2 * c * 2 * c;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
         const int m = (int)(e / (4LL * c * c));
@@ -645,11 +635,10 @@ __global__ void spec_assemble_kernel(const float *__restrict__ rr, const float *
             v = -ri[ro];
         else
             v = rr[ro];
-        const long long o = k_major ? (long long)m * 4 * c * c + (long long)col * 2 * c + row : e;
         if (bf16)
-            static_cast<__nv_bfloat16 *>(w)[o] = __float2bfloat16_rn(v);
+            static_cast<__nv_bfloat16 *>(w)[e] = __float2bfloat16_rn(v);
         else
-            static_cast<float *>(w)[o] = v;
+            static_cast<float *>(w)[e] = v;
     }
 }
 
@@ -937,6 +926,45 @@ __global__ void round_bf16_kernel(const float *__restrict__ x, float *__restrict
 }
 
 // Lift without a GEMM (K = 4): one thread per point and 8 channels.
+// (see SnoPrepare)
+__global__ void prepare_kernel(const SnoPrepare a)
+{
+    const int c = a.c;
+    const long long spec = (long long)a.modes * c * c;
+    __nv_bfloat16 *pw16 = static_cast<__nv_bfloat16 *>(a.pw16), *wt = static_cast<__nv_bfloat16 *>(a.wt);
+    __nv_bfloat16 *ws = static_cast<__nv_bfloat16 *>(a.ws), *wst = static_cast<__nv_bfloat16 *>(a.wst);
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.count; i += (long long)gridDim.x * blockDim.x) {
+        const __nv_bfloat16 v = __float2bfloat16_rn(a.params[i]);
+        a.pw[i] = __bfloat162float(v);
+        pw16[i] = v;
+        const long long rel = i - a.lay0;
+        if (rel >= 0 && rel < a.lay_size * a.layers) {
+            const int l = (int)(rel / a.lay_size);
+            const long long o = rel % a.lay_size;
+            if (o < 2 * spec) {
+                const bool im = o >= spec;
+                const long long q = im ? o - spec : o;
+                const int m = (int)(q / ((long long)c * c)), r = (int)(q % ((long long)c * c));
+                const int out = r / c, in = r % c, d = 2 * c;
+                const long long base = ((long long)l * a.modes + m) * 4 * c * c;
+                // [[Rr^T, Ri^T], [-Ri^T, Rr^T]]
+                const int r0 = in, c0 = im ? c + out : out, r1 = c + in, c1 = im ? out : c + out;
+                const __nv_bfloat16 v1 = im ? __hneg(v) : v;
+                ws[base + (long long)r0 * d + c0] = v;
+                ws[base + (long long)r1 * d + c1] = v1;
+                wst[base + (long long)c0 * d + r0] = v;
+                wst[base + (long long)c1 * d + r1] = v1;
+            } else if (o < 2 * spec + (long long)c * c) {
+                const int r = (int)(o - 2 * spec);
+                wt[(long long)l * c * c + (long long)(r % c) * c + r / c] = v;
+            }
+        } else if (i >= a.q1 && i < a.q1 + (long long)c * a.h) {
+            const int r = (int)(i - a.q1);
+            static_cast<__nv_bfloat16 *>(a.q1t)[(long long)(r % a.h) * c + r / a.h] = v;
+        }
+    }
+}
+
 constexpr int kLiftMaxC = 256;
 
 template <typename T, typename I>
@@ -1266,10 +1294,15 @@ cudaError_t sno_features(const float *u0, const float *r, const float *bl, const
     return cudaGetLastError();
 }
 
-cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int modes, int c, int bf16, cudaStream_t s,
-                              bool k_major)
+cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int modes, int c, int bf16, cudaStream_t s)
 {
-    spec_assemble_kernel<<<grid_for(4LL * modes * c * c), 256, 0, s>>>(rr, ri, w, modes, c, bf16, k_major ? 1 : 0);
+    spec_assemble_kernel<<<grid_for(4LL * modes * c * c), 256, 0, s>>>(rr, ri, w, modes, c, bf16);
+    return cudaGetLastError();
+}
+
+cudaError_t sno_prepare(const SnoPrepare &a, cudaStream_t s)
+{
+    prepare_kernel<<<grid_for(a.count), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -1,4 +1,4 @@
-// ge_sno_tc.cu -- the surrogate's inference GEMMs on the fifth-generation
+// ge_sno_tc.cu -- the surrogate's GEMMs on the fifth-generation
 // tensor cores: tcgen05.mma with the accumulator in tensor memory (TMEM),
 // operands staged in shared memory by 2D TMA copies, and the epilogue fused.
 // The paper has no counterpart (the surrogate is a deployment variant of the
@@ -11,7 +11,9 @@
 //       inverse truncated DFT, y [2M][C] the mode-mixed spectrum of the
 //       tile's problem, v the tile's activations, W [C][C] the pointwise
 //       weights.  Two products accumulate into one TMEM tile: K = 2M = 32
-//       (G y) and K = C = 64 (v W).
+//       (G y) and K = C = 64 (v W).  In training it also writes pre; the
+//       layer's backward pass is the same kernel on other operands,
+//       (F^T dvh + dpre W^T) * GELU'(pre of the layer below);
 //   projection (MODE 1): out = u0 + q2 + sum_h GELU(v Q1 + q1)_h Q2_h, one
 //       FP32 value per row; the hidden layer (N = H = 128) lives in TMEM
 //       only, and each thread sums its row in a fixed order;
@@ -23,8 +25,8 @@
 // read them.  B operands: the spectrum y [2M][C] and the activations v (in
 // the DFT) are read as stored, MN-major (N = 64 channels contiguous, one
 // 128-byte swizzle atom wide); W and Q1 go through transposed copies W^T
-// [C][C] and Q1^T [H][C] (K-major; a small kernel below writes them when
-// the parameters change).  One MMA instruction covers 128 rows x N columns
+// [C][C] and Q1^T [H][C] (K-major; sno_prepare writes them when the
+// parameters change).  One MMA instruction covers 128 rows x N columns
 // x 16 of K.
 //
 // Warp roles (160 threads): warp 4 lane 0 is the producer: it issues the TMA
@@ -102,6 +104,14 @@ __device__ __forceinline__ float gelu_hw(float x)
     return 0.5f * x * (1.0f + t);
 }
 
+// Its derivative.
+__device__ __forceinline__ float gelu_grad_hw(float x)
+{
+    float t;
+    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(x * (kGeluK0 + kGeluK0K1 * x * x)));
+    return 0.5f * (1.0f + t) + 0.5f * x * (1.0f - t * t) * (kGeluK0 + 3.0f * kGeluK0K1 * x * x);
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);  // .x = a (low half), .y = b
@@ -131,7 +141,9 @@ struct TcShape {
     static constexpr int kSmem = (int)(2 * kStage + kB2 + kOut + 1024);
 };
 
-template <int MODE>
+// TRAIN: the training epilogues (P.pre, P.dg, no bias); inference keeps its
+// own instance, 8% faster than one that decides at run time.
+template <int MODE, bool TRAIN>
 __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constant__ CUtensorMap tmA1,
                                                             const __grid_constant__ CUtensorMap tmB1,
                                                             const __grid_constant__ CUtensorMap tmA2,
@@ -167,7 +179,7 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
         tmem_relinquish();
     }
     for (int i = t; i < N; i += kTcThreads) {
-        s_bias[i] = P.bias[i];
+        s_bias[i] = !TRAIN || P.bias ? P.bias[i] : 0.0f;
         // the projection keeps Q2 / 2 (exact): GELU's factor 1/2 moves onto it
         s_q2[i] = MODE == 1 ? 0.5f * P.q2w[i] : 0.0f;
     }
@@ -283,16 +295,37 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t *r = h ? r1 : r0;
-                    uint32_t w[16];
+                    uint32_t w[16], keep[16];
+                    if (TRAIN && P.dg) {
+                        const uint4 *d = reinterpret_cast<const uint4 *>(P.dg) + row * (N / 8) + 4 * h;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const uint4 x = d[q];
+                            keep[4 * q] = x.x, keep[4 * q + 1] = x.y, keep[4 * q + 2] = x.z, keep[4 * q + 3] = x.w;
+                        }
+                    }
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         float a = __uint_as_float(r[2 * c]) + s_bias[32 * h + 2 * c];
                         float b = __uint_as_float(r[2 * c + 1]) + s_bias[32 * h + 2 * c + 1];
+                        if (TRAIN && P.dg) {
+                            const float2 d = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&keep[c]));
+                            a *= gelu_grad_hw(d.x);
+                            b *= gelu_grad_hw(d.y);
+                        } else if (TRAIN && P.pre) {
+                            keep[c] = pack_bf16(a, b);
+                        }
                         if (P.gelu) {
                             a = gelu_hw(a);
                             b = gelu_hw(b);
                         }
                         w[c] = pack_bf16(a, b);
+                    }
+                    if (TRAIN && P.pre) {
+                        uint4 *d = reinterpret_cast<uint4 *>(P.pre) + row * (N / 8) + 4 * h;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            d[q] = make_uint4(keep[4 * q], keep[4 * q + 1], keep[4 * q + 2], keep[4 * q + 3]);
                     }
                     // the buffer is free once the previous store has read it
                     if (lane == 0)
@@ -530,7 +563,7 @@ __global__ void __launch_bounds__(kDftThreads) sno_tc_dft_kernel(const __grid_co
 // the [2C][2C] real form of the complex mode weights.  A CTA takes 128
 // problems of one mode: A = those problems' vh[., m] rows (K-major, two
 // 64-wide 128-byte-swizzled boxes), B = Wspec_m^T [N][K] (K-major, written so
-// by the K-major variant of the spectral-weight assembly), one 128 x 128 FP32
+// by sno_prepare; Wspec_m itself in the backward pass), one 128 x 128 FP32
 // accumulator in TMEM after 8 MMAs of K = 16.  Thread 0 issues the four loads
 // and the MMAs; the four warps then read back their 32 rows each and write
 // y[b, m] as BF16 (rows past the batch are not written).
@@ -624,33 +657,18 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
         tmem_dealloc(tbase, 128);
 }
 
-// yT[b][c][k] = y[b][k][c]  (BF16, K = 2M rows, C columns per problem);
-// 32-bit indices (the caller checks that every index fits)
-__global__ void transpose_rows_kernel(const __nv_bfloat16 *__restrict__ y, __nv_bfloat16 *__restrict__ yt,
-                                      int batch, int k_rows, int c_cols)
-{
-    const int per = k_rows * c_cols;
-    const int total = batch * per;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
-        const int b = e / per;
-        const int rem = e - b * per;
-        const int c = rem / k_rows, k = rem - c * k_rows;
-        yt[e] = y[b * per + k * c_cols + c];
-    }
-}
-
-template <int MODE>
+template <int MODE, bool TRAIN>
 cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
     using S = TcShape<MODE>;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(sno_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(sno_tc_kernel<MODE, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              S::kSmem);
         // the largest shared-memory carve-out, so that as many CTAs fit as
         // TMEM allows (3 layer CTAs of 74 KB need about 225 KB)
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(sno_tc_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
+            e = cudaFuncSetAttribute(sno_tc_kernel<MODE, TRAIN>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess)
             return e;
@@ -663,7 +681,7 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
     if (per_sm == 0) {
         cudaFuncAttributes fa{};
         int dev = 0, sm_bytes = 0, reserve = 0;
-        cudaError_t e = cudaFuncGetAttributes(&fa, sno_tc_kernel<MODE>);
+        cudaError_t e = cudaFuncGetAttributes(&fa, sno_tc_kernel<MODE, TRAIN>);
         if (e == cudaSuccess)
             e = cudaGetDevice(&dev);
         if (e == cudaSuccess)
@@ -690,7 +708,7 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
     const CUtensorMap *a1 = static_cast<const CUtensorMap *>(MODE == 0 ? m.a1 : m.a2);
     const CUtensorMap *b1 = static_cast<const CUtensorMap *>(MODE == 0 ? m.b1 : m.a2);
     const CUtensorMap *o = static_cast<const CUtensorMap *>(MODE == 0 ? m.out : m.a2);
-    sno_tc_kernel<MODE><<<(int)grid, kTcThreads, S::kSmem, s>>>(*a1, *b1, *static_cast<const CUtensorMap *>(m.a2),
+    sno_tc_kernel<MODE, TRAIN><<<(int)grid, kTcThreads, S::kSmem, s>>>(*a1, *b1, *static_cast<const CUtensorMap *>(m.a2),
                                                               *static_cast<const CUtensorMap *>(m.b2), *o, a);
     return cudaGetLastError();
 }
@@ -699,12 +717,12 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
 
 cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
-    return launch_tc<0>(m, a, sms, s);
+    return a.pre || a.dg || !a.bias ? launch_tc<0, true>(m, a, sms, s) : launch_tc<0, false>(m, a, sms, s);
 }
 
 cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
-    return launch_tc<1>(m, a, sms, s);
+    return launch_tc<1, false>(m, a, sms, s);
 }
 
 cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a, int sms, cudaStream_t s)
@@ -761,21 +779,6 @@ cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixAr
     const dim3 grid((unsigned)((a.batch + 127) / 128), (unsigned)modes);
     sno_tc_mix_kernel<<<grid, kMixThreads, kMixSmem, s>>>(*static_cast<const CUtensorMap *>(map_vh),
                                                           *static_cast<const CUtensorMap *>(map_wst), a);
-    return cudaGetLastError();
-}
-
-cudaError_t sno_transpose_rows(const void *y, void *yt, long long batch, int k_rows, int c_cols, cudaStream_t s)
-{
-    const long long total = batch * k_rows * c_cols;
-    if (total >= (1LL << 31) - 256LL * 4096)
-        return cudaErrorInvalidValue;
-    long long blocks = (total + 255) / 256;
-    if (blocks > 4096)
-        blocks = 4096;
-    if (blocks < 1)
-        return cudaSuccess;
-    transpose_rows_kernel<<<(int)blocks, 256, 0, s>>>(static_cast<const __nv_bfloat16 *>(y),
-                                                       static_cast<__nv_bfloat16 *>(yt), (int)batch, k_rows, c_cols);
     return cudaGetLastError();
 }
 
