@@ -100,8 +100,8 @@ struct ge_sno {
     int *err = nullptr;                   // device error word of the tensor-core kernels
     // training: F^T, G^T, the spectral weights, the gradients' spectra (dy as
     // mixing rows, dvh as a layer's operand) and buffers, W of each layer
-    CUtensorMap tm_ft, tm_gt, tm_ws, tm_dy, tm_dvh, tm_dA, tm_dB, tm_dAs, tm_dBs;
-    std::vector<CUtensorMap> tm_w;
+    CUtensorMap tm_ft, tm_gt, tm_ws, tm_dy, tm_dvh, tm_dA, tm_dB, tm_dAs, tm_dBs, tm_dAh, tm_q1, tm_h, tm_hpre;
+    std::vector<CUtensorMap> tm_w, tm_pre;
     CUtensorMap tm_g, tm_y, tm_wt, tm_q1t, tm_f, tm_wst;
     std::vector<CUtensorMap> tm_v;        // one per activation buffer v[0..L]
     std::vector<CUtensorMap> tm_vs;       // store maps of v[1..L] (index l: v[l + 1])
@@ -145,11 +145,6 @@ ge::GemmArgs gemm(const void *A, long long lda_i, long long lda_k, const void *B
 bool bf16_mode(const ge_sno *s) { return !s->split; }
 
 // Element `off` of a buffer in the mode's storage type.
-const void *at(const void *base, long long off, bool bf)
-{
-    return static_cast<const char *>(base) + off * (bf ? 2 : 4);
-}
-
 void *at(void *base, long long off, bool bf) { return static_cast<char *>(base) + off * (bf ? 2 : 4); }
 
 // The weights as the GEMMs read them: BF16 copy or FP32 rounded values.
@@ -169,8 +164,7 @@ ge::GemmArgs &act_fmt(ge::GemmArgs &g, bool bf)
 
 // Weight gradient of a pointwise layer: dW[in][out] = X^T dY over R rows
 // (X rows ldx apart; split-K with atomics, FP32), db = column sums of dY.
-// The lift's 4 features and the last projection's single column are weighted
-// column sums instead of GEMMs.
+// The lift's 4 features are weighted column sums instead of a GEMM.
 ge_status weight_grad(ge_sno *s, const void *X, int in, int ldx, const void *dY, int out, long long R, float *dW,
                       float *db)
 {
@@ -179,17 +173,6 @@ ge_status weight_grad(ge_sno *s, const void *X, int in, int ldx, const void *dY,
     a.rows = R;
     a.part = s->sums;
     a.ticket = s->sum_tickets;
-    if (out == 1 && ldx == in) {
-        a.x = X;
-        a.cols = in;
-        a.w = dY;
-        a.ldw = 1;
-        a.nw = 1;
-        a.wsum = dW;
-        a.wtot = db;
-        SNO_TRY(ge::sno_colsum(a, bf ? 1 : 0, s->stream));
-        return GE_OK;
-    }
     a.x = dY;
     a.cols = out;
     a.sum = db;
@@ -255,7 +238,6 @@ bool tc_active(const ge_sno *s) { return s->tc && !s->split && tc_shape(s) && s-
 // layers and the projection (the mode mixing keeps the mma.sync GEMM).
 ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br, float *out,
                      bool keep);
-ge_status project_keep(ge_sno *s, const float *u0, float *out, long long R);
 
 // Forward pass for B problems into out ([B n], FP32).  keep: also store the
 // pre-activations the backward pass needs (training).
@@ -332,20 +314,11 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
         SNO_TRY(ge::sno_dot_finish(u0, P + s->off_qb2, s->dA, slots, out, R, st));
         return GE_OK;
     }
-    return project_keep(s, u0, out, R);
-}
-
-// The projection of a training pass: hpre, h and the output.
-ge_status project_keep(ge_sno *s, const float *u0, float *out, long long R)
-{
-    const int C = s->C, H = s->H;
-    const bool bf = bf16_mode(s);
-    const float *P = s->pw;
-    ge::GemmArgs g = gemm(s->v[s->L], C, 1, weight(s, s->off_q1), H, 1, s->hpre, H, (int)R, H, C);
+    g = gemm(s->v[s->L], C, 1, weight(s, s->off_q1), H, 1, s->hpre, H, (int)R, H, C);
     g.bias = P + s->off_qb1;
     g.act = s->h;
-    SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, s->stream));
-    SNO_TRY(ge::sno_row_dot(s->h, weight(s, s->off_q2), P + s->off_qb2, u0, out, R, H, bf ? 1 : 0, s->stream));
+    SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
+    SNO_TRY(ge::sno_row_dot(s->h, weight(s, s->off_q2), P + s->off_qb2, u0, out, R, H, bf ? 1 : 0, st));
     return GE_OK;
 }
 
@@ -404,21 +377,19 @@ ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const fl
         a.gelu = l < s->L - 1 ? 1 : 0;
         a.bias = P + o.b;
         a.out = s->v[l + 1];
-        a.pre = keep && l < s->L - 1 ? s->pre[l] : nullptr;
-        const ge::SnoTcMaps m{&s->tm_g, &s->tm_y, &s->tm_v[l], &s->tm_wt, &s->tm_vs[l]};
+        a.keep = keep && l < s->L - 1 ? 1 : 0;
+        const ge::SnoTcMaps m{&s->tm_g, &s->tm_y, &s->tm_v[l], &s->tm_wt, &s->tm_vs[l], &s->tm_pre[l]};
         SNO_TRY(ge::sno_tc_layer(m, a, s->num_sms, st));
     }
-    if (keep)
-        return project_keep(s, u0, out, R);
     a.b2_row = 0;
     a.gelu = 1;
-    a.pre = nullptr;
+    a.keep = keep ? 1 : 0;
     a.bias = P + s->off_qb1;
     a.q2w = P + s->off_q2;
     a.q2b = P + s->off_qb2;
     a.u0 = u0;
     a.out = out;
-    const ge::SnoTcMaps m{nullptr, nullptr, &s->tm_v[s->L], &s->tm_q1t, nullptr};
+    const ge::SnoTcMaps m{nullptr, nullptr, &s->tm_v[s->L], &s->tm_q1t, &s->tm_h, &s->tm_hpre};
     SNO_TRY(ge::sno_tc_projection(m, a, s->num_sms, st));
     return GE_OK;
 }
@@ -435,20 +406,47 @@ ge_status backward(ge_sno *s, int B)
     const int ldf = bf ? 8 : 4;
     float *Gd = s->grads;
     ge_status rc;
-    // projection: out = h Q2 + q2
-    if ((rc = weight_grad(s, s->h, H, H, s->dout, 1, R, Gd + s->off_q2, Gd + s->off_qb2)) != GE_OK)
-        return rc;
-    // dhpre = (dout Q2^T) * GELU'(hpre)
-    SNO_TRY(ge::sno_outer_dgelu(s->dout, weight(s, s->off_q2), s->hpre, s->dA, R, H, bf ? 1 : 0, st));
-    if ((rc = weight_grad(s, s->v[s->L], C, C, s->dA, H, R, Gd + s->off_q1, Gd + s->off_qb1)) != GE_OK)
-        return rc;
-    ge::GemmArgs g = gemm(s->dA, H, 1, weight(s, s->off_q1), 1, H, s->dB, C, (int)R, C, H);  // dv_L = dhpre Q1^T
-    SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
+    const bool tc = tc_active(s);
+    if (tc)  // sno_tc_grad adds to its results
+        SNO_TRY(cudaMemsetAsync(Gd, 0, sizeof(float) * s->n_params, st));
+    ge::SnoTcGradArgs tg{};
+    tg.rows = R;
+    tg.err = s->err;
+    tg.limit = ge::kWaitLimitCycles;
+    // projection: out = h Q2 + q2; and dhpre = (dout Q2^T) * GELU'(hpre)
+    ge::SnoSums q{};
+    q.x = s->h;
+    q.rows = R;
+    q.cols = H;
+    q.w = s->dout;
+    q.ldw = 1;
+    q.nw = 1;
+    q.part = s->sums;
+    q.ticket = s->sum_tickets;
+    q.wsum = Gd + s->off_q2;
+    q.wtot = Gd + s->off_qb2;
+    q.q = weight(s, s->off_q2);
+    q.pre = s->hpre;
+    q.out = s->dA;
+    SNO_TRY(ge::sno_colsum(q, bf ? 1 : 0, st));
+    // dQ1, dq1 and dv_L = dhpre Q1^T
+    ge::GemmArgs g{};
+    if (tc) {
+        tg.dw = Gd + s->off_q1;
+        tg.db = Gd + s->off_qb1;
+        SNO_TRY(ge::sno_tc_grad(&s->tm_v[s->L], &s->tm_dAh, tg, H, s->num_sms, st));
+        const ge::SnoTcMixArgs x{(int)R, 0, C, s->dB, s->err, ge::kWaitLimitCycles};
+        SNO_TRY(ge::sno_tc_rows(&s->tm_dAh, &s->tm_q1, x, st));
+    } else {
+        if ((rc = weight_grad(s, s->v[s->L], C, C, s->dA, H, R, Gd + s->off_q1, Gd + s->off_qb1)) != GE_OK)
+            return rc;
+        g = gemm(s->dA, H, 1, weight(s, s->off_q1), 1, H, s->dB, C, (int)R, C, H);
+        SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
+    }
     // dv holds the gradient of the current layer's pre-activation: the last
     // layer has no activation, and every lower one's GELU' is applied in the
     // epilogue of the GEMM that makes its gradient.
     void *dv = s->dB, *dnext = s->dA;
-    const bool tc = tc_active(s);
     ge::SnoTcArgs ta{};
     ta.n_tiles = R / 128;
     ta.tiles_per_problem = n / 128;
@@ -458,20 +456,43 @@ ge_status backward(ge_sno *s, int B)
         const LayerOff &o = s->lay[l];
         const void *ws = at(s->wspec, (long long)l * M * 4 * C * C, bf);
         const void *dpre = dv;
+        if (tc) {
+            const bool from_b = dv == s->dB;
+            const CUtensorMap *map = from_b ? &s->tm_dB : &s->tm_dA;
+            // pointwise path weights
+            tg.dw = Gd + o.w;
+            tg.db = Gd + o.b;
+            SNO_TRY(ge::sno_tc_grad(&s->tm_v[l], map, tg, C, s->num_sms, st));
+            // spectral path: dy[b] = G^T dpre[b], dWspec_m = vh[:, m]^T dy[:, m],
+            // dvh[:, m] = dy[:, m] Wspec_m^T
+            ta.out = s->y;
+            SNO_TRY(ge::sno_tc_dft(&s->tm_gt, map, ta, s->num_sms, st));
+            ge::SnoTcGradArgs ts = tg;
+            ts.rows = B;
+            ts.drr = Gd + o.rr;
+            ts.dri = Gd + o.ri;
+            SNO_TRY(ge::sno_tc_grad_spec(&s->tm_vh[l], &s->tm_dy, ts, M, st));
+            const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->dvh, s->err, ge::kWaitLimitCycles};
+            SNO_TRY(ge::sno_tc_mix(&s->tm_dy, &s->tm_ws, x, M, st));
+            // gradient of v_l, both paths as one layer, times GELU'(pre_{l-1})
+            // when v_l is an activation
+            ta.b2_row = 0;
+            ta.out = dnext;
+            ta.dg = l > 0 ? s->pre[l - 1] : nullptr;
+            const ge::SnoTcMaps m{&s->tm_ft, &s->tm_dvh, map, &s->tm_w[l], from_b ? &s->tm_dAs : &s->tm_dBs, nullptr};
+            SNO_TRY(ge::sno_tc_layer(m, ta, s->num_sms, st));
+            std::swap(dv, dnext);
+            continue;
+        }
         // pointwise path weights
         if ((rc = weight_grad(s, s->v[l], C, C, dpre, C, R, Gd + o.w, Gd + o.b)) != GE_OK)
             return rc;
         // spectral path: dy[b] = G^T dpre[b]
-        if (tc) {
-            ta.out = s->y;
-            SNO_TRY(ge::sno_tc_dft(&s->tm_gt, dv == s->dB ? &s->tm_dB : &s->tm_dA, ta, s->num_sms, st));
-        } else {
-            g = gemm(G, 1, 2 * M, dpre, C, 1, s->y, C, 2 * M, C, n);
-            g.sA = 0;
-            g.sB = (long long)n * C;
-            g.sC = 2LL * M * C;
-            SNO_TRY(ge::sno_gemm(act_fmt(g, bf), B, s->split, st));
-        }
+        g = gemm(G, 1, 2 * M, dpre, C, 1, s->y, C, 2 * M, C, n);
+        g.sA = 0;
+        g.sB = (long long)n * C;
+        g.sC = 2LL * M * C;
+        SNO_TRY(ge::sno_gemm(act_fmt(g, bf), B, s->split, st));
         // dWspec_m = vh[:, m]^T dy[:, m]  (FP32)
         g = gemm(s->vh[l], 1, 2LL * M * C, s->y, 2LL * M * C, 1, s->dwspec, 2 * C, 2 * C, 2 * C, B);
         g.sA = 2 * C;
@@ -480,20 +501,6 @@ ge_status backward(ge_sno *s, int B)
         act_fmt(g, bf).out_bf16 = 0;
         SNO_TRY(ge::sno_gemm(g, M, s->split, st));
         SNO_TRY(ge::sno_spec_reduce(s->dwspec, Gd + o.rr, Gd + o.ri, M, C, st));
-        if (tc) {
-            // dvh[:, m] = dy[:, m] Wspec_m^T, then both paths as one layer
-            const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->dvh, s->err, ge::kWaitLimitCycles};
-            SNO_TRY(ge::sno_tc_mix(&s->tm_dy, &s->tm_ws, x, M, st));
-            ta.b2_row = 0;
-            ta.out = dnext;
-            ta.dg = l > 0 ? s->pre[l - 1] : nullptr;
-            const bool from_b = dv == s->dB;
-            const ge::SnoTcMaps m{&s->tm_ft, &s->tm_dvh, from_b ? &s->tm_dB : &s->tm_dA, &s->tm_w[l],
-                                  from_b ? &s->tm_dAs : &s->tm_dBs};
-            SNO_TRY(ge::sno_tc_layer(m, ta, s->num_sms, st));
-            std::swap(dv, dnext);
-            continue;
-        }
         // dvh[:, m] = dy[:, m] Wspec_m^T
         g = gemm(s->y, 2LL * M * C, 1, ws, 1, 2 * C, s->dvh, 2LL * M * C, B, 2 * C, 2 * C);
         g.sA = 2 * C;
@@ -520,9 +527,7 @@ ge_status backward(ge_sno *s, int B)
             g.sDg = (long long)n * C;
         }
         SNO_TRY(ge::sno_gemm(act_fmt(g, bf), B, s->split, st));
-        void *t = dv;
-        dv = dnext;
-        dnext = t;
+        std::swap(dv, dnext);
     }
     // lift
     return weight_grad(s, s->feat, 4, ldf, dv, C, R, Gd + s->off_w0, Gd + s->off_b0);
@@ -702,6 +707,13 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
              bf16_map(&s->tm_dvh, s->dvh, (long long)max_batch * 2 * modes, width, width, 2 * modes) &&
              bf16_map(&s->tm_dA, s->dA, R, width, width, 128) && bf16_map(&s->tm_dB, s->dB, R, width, width, 128) &&
              bf16_map(&s->tm_dAs, s->dA, R, width, 32, 32) && bf16_map(&s->tm_dBs, s->dB, R, width, 32, 32);
+        // dhpre as rows of H, Q1 as stored, the stores of h and the pre-activations
+        ok = ok && bf16_map(&s->tm_dAh, s->dA, R, hidden, 64, 128) &&
+             bf16_map(&s->tm_q1, static_cast<char *>(s->pw16) + 2 * s->off_q1, width, hidden, 64, 64) &&
+             bf16_map(&s->tm_h, s->h, R, hidden, 32, 32) && bf16_map(&s->tm_hpre, s->hpre, R, hidden, 32, 32);
+        s->tm_pre.resize(layers);
+        for (int l = 0; l < layers && ok; ++l)
+            ok = bf16_map(&s->tm_pre[l], s->pre[l], R, width, 32, 32);
         s->tm_w.resize(layers);
         for (int l = 0; l < layers && ok; ++l)
             ok = bf16_map(&s->tm_w[l], static_cast<char *>(s->pw16) + 2 * s->lay[l].w, width, width, width, 64);

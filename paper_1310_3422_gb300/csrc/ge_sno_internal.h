@@ -68,10 +68,13 @@ cudaError_t sno_gemm(const GemmArgs &g, int batch, bool split, cudaStream_t s);
 //               MN-major), a2 = v [rows][C] (box 64 x 128, 128-byte swizzle),
 //               b2 = W^T of all layers [L * C][C] (box 64 x 64, 128-byte
 //               swizzle);
-//   projection: a2 = v as above, b2 = Q1^T [H][C] (box 64 x 128).
+//   projection: a2 = v as above, b2 = Q1^T [H][C] (box 64 x 128);
+//   in training also store maps (box 32 x 32, 64-byte swizzle) of the value
+//   before GELU (pre) and, for the projection, of the hidden layer (out).
 struct SnoTcMaps {
     const void *a1, *b1, *a2, *b2;
     const void *out;  // layer: store map of the next activation [rows][C] (box 32 x 32, 64-byte swizzle)
+    const void *pre;  // or NULL
 };
 struct SnoTcArgs {
     long long n_tiles;      // rows / 128
@@ -85,7 +88,7 @@ struct SnoTcArgs {
     void *out;              // layer: next activation, BF16 [rows][C]; projection: FP32 [rows]
     int *err;               // device error word (GE_ETIMEOUT on a wait that gave up)
     long long limit;        // wait limit in SM cycles
-    void *pre;              // layer: also the value before GELU, BF16 [rows][C], or NULL
+    int keep;               // training forward: also write pre (layer) or hidden layer and pre (projection)
     const void *dg;         // layer: multiply by GELU' of these BF16 [rows][C], or NULL
 };
 cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s);
@@ -98,6 +101,8 @@ cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a,
 // map_vh over vh [batch rows][2M * 2C] (box 64 x 128, 128-byte swizzle),
 // map_wst over the K-major spectral weights Wspec_m^T of all layers
 // [L * M * 2C][2C] (box 64 x 128); grid = (ceil(batch / 128), modes).
+// sno_tc_rows is the same product with one "mode" and 64 output columns:
+// y [rows][64] = x [rows][128] B^T, B [64][128] (box 64 x 64).
 struct SnoTcMixArgs {
     int batch;           // problems (rows of vh and y)
     int b_row0;          // first row of this layer's block of map_wst (l * M * 2C)
@@ -107,6 +112,25 @@ struct SnoTcMixArgs {
     long long limit;     // wait limit in SM cycles
 };
 cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s);
+cudaError_t sno_tc_rows(const void *map_x, const void *map_b, const SnoTcMixArgs &a, cudaStream_t s);
+// Weight gradients on the tensor cores, dW = X^T dY over the rows of both:
+//   sno_tc_grad:  X [rows][64] (map_x, box 64 x 128), dY [rows][cols] with
+//       cols = 64 or 128 (map_y, box 64 x 128); adds to dw [64][cols] and
+//       the column sums of dY to db [cols] (both 16-byte aligned).
+//   sno_tc_grad_spec:  per mode m, X and dY the columns 128 m .. 128 m + 127
+//       of vh and dy [rows][2M * C] (same boxes); writes dRr and dRi
+//       [modes][C out][C in], C = 64.
+struct SnoTcGradArgs {
+    long long rows;
+    float *dw, *db;      // sno_tc_grad
+    float *drr, *dri;    // sno_tc_grad_spec
+    int *err;            // device error word
+    long long limit;     // wait limit in SM cycles
+};
+cudaError_t sno_tc_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, int cols, int sms,
+                        cudaStream_t s);
+cudaError_t sno_tc_grad_spec(const void *map_vh, const void *map_dy, const SnoTcGradArgs &a, int modes,
+                             cudaStream_t s);
 cudaError_t sno_features(const float *u0, const float *r, const float *bl, const float *br, void *f, int batch,
                          int n, int bf16, cudaStream_t s);
 cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int modes, int c, int bf16, cudaStream_t s);
@@ -124,13 +148,13 @@ struct SnoSums {
     float *part;
     int *ticket;
     float *sum, *wsum, *wtot;
+    // nw = 1: also out[i, j] = w[i] q[j] GELU'(pre[i, j]), unless out is NULL
+    const void *q, *pre;
+    void *out;
 };
 long long sno_sum_floats(int cols);
 int sno_sum_tickets(int cols);
 cudaError_t sno_colsum(const SnoSums &a, int bf16, cudaStream_t s);
-// out[i, j] = d[i] q[j] GELU'(pre[i, j]).
-cudaError_t sno_outer_dgelu(const void *d, const void *q, const void *pre, void *out, long long rows, int cols, int bf16,
-                            cudaStream_t s);
 // out[i] = u0[i] + q2[0] + sum_j h[i, j] q[j].
 cudaError_t sno_row_dot(const void *h, const void *q, const float *q2, const float *u0, float *out, long long rows, int cols,
                         int bf16, cudaStream_t s);

@@ -695,25 +695,38 @@ __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float
 // With NW = 4 and w the features it is the lift's weight gradient, with NW =
 // 1 and w the output's gradient that of the last projection: products with 4
 // or 1 rows, which a 64-row GEMM tile took 81 and 42 us for (65,536 rows).
+// HEAD (with NW = 1) also writes the gradient of the hidden layer's
+// pre-activation in the same pass, out[i, j] = w[i] q[j] GELU'(pre[i, j]); as
+// a GEMM with K = 1 it took 52 us for 65,536 x 128 BF16.
 // Bound by reading x once: blocks of 256 threads take rows in turn, 16 bytes
 // a thread (V; else single values), and the last block to finish adds the
-// blocks' sums in their order, so the result does not depend on timing.  (A
-// block per column, striding through the rows: 47 us for 8 MB, now TBD us.)
+// blocks' sums in a fixed order, so the result does not depend on timing; it
+// is one block, so all its threads share the sums and keep several loads in
+// flight.  65,536 rows, BF16, cold caches: a block per column striding
+// through the rows took 47 us for plain sums of 64 columns; now the last
+// projection's gradients with dhpre (48 MB) take 24.5 us, the lift's 19.7 us
+// (21.6 + 12.4 and 32.7 us before the last block's sums were shared).
 constexpr int kSumBlocks = 192;
 
-template <typename T, int NW, bool V>
-__global__ void __launch_bounds__(256) colsum_kernel(const T *__restrict__ x, long long rows, int cols,
-                                                     const T *__restrict__ w, int ldw, float *__restrict__ part,
-                                                     int *__restrict__ ticket, float *__restrict__ sum,
-                                                     float *__restrict__ wsum, float *__restrict__ wtot)
+template <typename T, int NW, bool V, bool HEAD>
+__global__ void __launch_bounds__(256) colsum_kernel(const SnoSums a)
 {
     constexpr int E = V ? Chunk<T>::E : 1, TPR = V ? 64 / E : 32, CW = E * TPR, G = 256 / TPR, S = 1 + NW;
-    __shared__ float red[G][CW];
+    static_assert(!HEAD || NW == 1, "the weight is the output's gradient");
+    __shared__ float red[256 / CW > G ? 256 / CW : G][CW];
     __shared__ float tot[G];
     __shared__ int last;
+    const T *x = static_cast<const T *>(a.x), *w = static_cast<const T *>(a.w);
+    const long long rows = a.rows;
+    const int cols = a.cols, ldw = a.ldw;
     const int t = threadIdx.x, tc = t % TPR, g = t / TPR, c0 = blockIdx.y * CW, c = c0 + tc * E;
     const bool in = c < cols;
-    float acc[S][E] = {}, at = 0.0f;
+    float acc[S][E] = {}, at = 0.0f, qv[E];
+    if constexpr (HEAD) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            qv[e] = in ? to_f(static_cast<const T *>(a.q)[c + e]) : 0.0f;
+    }
 #pragma unroll 4
     for (long long i = (long long)blockIdx.x * G + g; i < rows; i += (long long)gridDim.x * G) {
         float v[E], wv[NW > 0 ? NW : 1];
@@ -723,11 +736,37 @@ __global__ void __launch_bounds__(256) colsum_kernel(const T *__restrict__ x, lo
         } else {
             v[0] = in ? to_f(x[i * cols + c]) : 0.0f;
         }
+        if constexpr (V && NW == 4) {
+            // a row of features is 16 bytes (BF16 rows are padded to 8)
+            float f[Chunk<T>::E];
+            Chunk<T>::load(w + i * Chunk<T>::E, f);
 #pragma unroll
-        for (int f = 0; f < NW; ++f)
-            wv[f] = to_f(w[i * ldw + f]);
+            for (int k = 0; k < 4; ++k)
+                wv[k] = f[k];
+        } else {
+#pragma unroll
+            for (int f = 0; f < NW; ++f)
+                wv[f] = to_f(w[i * ldw + f]);
+        }
         if (!in)
             continue;
+        if constexpr (HEAD) {
+            const T *pre = static_cast<const T *>(a.pre) + i * cols + c;
+            T *out = static_cast<T *>(a.out) + i * cols + c;
+            float p[E];
+            __align__(16) T o[E];
+            if constexpr (V)
+                Chunk<T>::load(pre, p);
+            else
+                p[0] = to_f(pre[0]);
+#pragma unroll
+            for (int e = 0; e < E; ++e)
+                o[e] = static_cast<T>(wv[0] * qv[e] * gelu_grad<sizeof(T) == 4>(p[e]));
+            if constexpr (V)
+                *reinterpret_cast<uint4 *>(out) = *reinterpret_cast<const uint4 *>(o);
+            else
+                out[0] = o[0];
+        }
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             acc[0][e] += v[e];
@@ -739,7 +778,7 @@ __global__ void __launch_bounds__(256) colsum_kernel(const T *__restrict__ x, lo
             at += wv[0];
     }
     const long long stride = (long long)S * cols + 1;
-    float *mine = part + blockIdx.x * stride;
+    float *mine = a.part + blockIdx.x * stride;
 #pragma unroll
     for (int q = 0; q < S; ++q) {
         __syncthreads();
@@ -765,64 +804,51 @@ __global__ void __launch_bounds__(256) colsum_kernel(const T *__restrict__ x, lo
     __threadfence();
     __syncthreads();
     if (t == 0)
-        last = atomicAdd(ticket + blockIdx.y, 1) == (int)gridDim.x - 1;
+        last = atomicAdd(a.ticket + blockIdx.y, 1) == (int)gridDim.x - 1;
     __syncthreads();
     if (!last)
         return;
     __threadfence();
     if (t == 0)
-        ticket[blockIdx.y] = 0;  // the next launch's
-    for (int o = t; o < S * CW; o += 256) {
-        const int q = o / CW, j = c0 + o % CW;
-        float *out = q == 0 ? sum : wsum;
-        if (j >= cols || !out)
-            continue;
-        float v = 0.0f;
-#pragma unroll 8
-        for (int i = 0; i < (int)gridDim.x; ++i)
-            v += __ldcg(part + i * stride + (long long)q * cols + j);
-        out[(q == 0 ? 0 : (long long)(q - 1) * cols) + j] = v;
-    }
-    if (wtot && blockIdx.y == 0 && t == 255) {
-        float v = 0.0f;
-        for (int i = 0; i < (int)gridDim.x; ++i)
-            v += __ldcg(part + i * stride + (long long)S * cols);
-        *wtot = v;
-    }
-}
-
-// Gradient of the hidden layer's pre-activation: out[i, j] = d[i] q[j]
-// GELU'(pre[i, j]).  An elementwise pass over pre and out (as a GEMM with K =
-// 1: 52 us for 65,536 x 128 BF16, now TBD us).
-template <bool EXACT, typename T, bool V>
-__global__ void __launch_bounds__(256) outer_dgelu_kernel(const T *__restrict__ d, const T *__restrict__ q,
-                                                          const T *__restrict__ pre, T *__restrict__ out,
-                                                          long long rows, int cols)
-{
-    constexpr int E = V ? Chunk<T>::E : 1;
-    const long long total = rows * cols / E;
-    for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < total; i += (long long)gridDim.x * 256) {
-        const long long r = i * E / cols;
-        const int j = (int)(i * E - r * cols);
-        const float dv = to_f(d[r]);
-        float p[E];
-        __align__(16) T o[E];
-        if constexpr (V)
-            Chunk<T>::load(pre + i * E, p);
-        else
-            p[0] = to_f(pre[i]);
+        a.ticket[blockIdx.y] = 0;  // the next launch's
+    // thread (k, j): blocks k, k + 256 / CW, ... of column c0 + j
+    const int k = t / CW, j = c0 + t % CW;
+    float s[S] = {};
+    if (j < cols) {
+#pragma unroll 4
+        for (int i = k; i < (int)gridDim.x; i += 256 / CW)
 #pragma unroll
-        for (int e = 0; e < E; ++e)
-            o[e] = static_cast<T>(dv * to_f(q[j + e]) * gelu_grad<EXACT>(p[e]));
-        if constexpr (V)
-            *reinterpret_cast<uint4 *>(out + i * E) = *reinterpret_cast<const uint4 *>(o);
-        else
-            out[i] = o[0];
+            for (int q = 0; q < S; ++q)
+                s[q] += __ldcg(a.part + i * stride + (long long)q * cols + j);
+    }
+#pragma unroll
+    for (int q = 0; q < S; ++q) {
+        float *out = q == 0 ? a.sum : a.wsum;
+        __syncthreads();
+        red[k][t % CW] = s[q];
+        __syncthreads();
+        if (k == 0 && j < cols && out) {
+            float v = 0.0f;
+            for (int i = 0; i < 256 / CW; ++i)
+                v += red[i][t];
+            out[(q == 0 ? 0 : (long long)(q - 1) * cols) + j] = v;
+        }
+    }
+    if (a.wtot && blockIdx.y == 0 && t < 32) {
+        float v = 0.0f;
+#pragma unroll 6
+        for (int i = t; i < (int)gridDim.x; i += 32)
+            v += __ldcg(a.part + i * stride + (long long)S * cols);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (t == 0)
+            *a.wtot = v;
     }
 }
 
 // out[i] = u0[i] + q2[0] + sum_j h[i, j] q[j], a warp per row.  (As a GEMM
-// with one column: 23 us for 65,536 x 128 BF16, now TBD us.)
+// with one column: 23 us for 65,536 x 128 BF16, now 16 us.)
 template <typename T, bool V>
 __global__ void __launch_bounds__(256) row_dot_kernel(const T *__restrict__ h, const T *__restrict__ q,
                                                       const float *__restrict__ q2, const float *__restrict__ u0,
@@ -929,38 +955,34 @@ __global__ void round_bf16_kernel(const float *__restrict__ x, float *__restrict
 // (see SnoPrepare)
 __global__ void prepare_kernel(const SnoPrepare a)
 {
-    const int c = a.c;
-    const long long spec = (long long)a.modes * c * c;
+    const unsigned c = a.c, cc = c * c, spec = a.modes * cc, lay0 = (unsigned)a.lay0, lay = (unsigned)a.lay_size;
+    const unsigned q1 = (unsigned)a.q1, d = 2 * c;
     __nv_bfloat16 *pw16 = static_cast<__nv_bfloat16 *>(a.pw16), *wt = static_cast<__nv_bfloat16 *>(a.wt);
     __nv_bfloat16 *ws = static_cast<__nv_bfloat16 *>(a.ws), *wst = static_cast<__nv_bfloat16 *>(a.wst);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.count; i += (long long)gridDim.x * blockDim.x) {
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (unsigned)a.count; i += gridDim.x * blockDim.x) {
         const __nv_bfloat16 v = __float2bfloat16_rn(a.params[i]);
         a.pw[i] = __bfloat162float(v);
         pw16[i] = v;
-        const long long rel = i - a.lay0;
-        if (rel >= 0 && rel < a.lay_size * a.layers) {
-            const int l = (int)(rel / a.lay_size);
-            const long long o = rel % a.lay_size;
+        if (i >= lay0 && i - lay0 < lay * a.layers) {
+            const unsigned rel = i - lay0, l = rel / lay, o = rel - l * lay;
             if (o < 2 * spec) {
                 const bool im = o >= spec;
-                const long long q = im ? o - spec : o;
-                const int m = (int)(q / ((long long)c * c)), r = (int)(q % ((long long)c * c));
-                const int out = r / c, in = r % c, d = 2 * c;
-                const long long base = ((long long)l * a.modes + m) * 4 * c * c;
+                const unsigned q = im ? o - spec : o, m = q / cc, r = q - m * cc, out = r / c, in = r - out * c;
+                const size_t base = (size_t)(l * a.modes + m) * 4 * cc;
                 // [[Rr^T, Ri^T], [-Ri^T, Rr^T]]
-                const int r0 = in, c0 = im ? c + out : out, r1 = c + in, c1 = im ? out : c + out;
+                const unsigned r0 = in, c0 = im ? c + out : out, r1 = c + in, c1 = im ? out : c + out;
                 const __nv_bfloat16 v1 = im ? __hneg(v) : v;
-                ws[base + (long long)r0 * d + c0] = v;
-                ws[base + (long long)r1 * d + c1] = v1;
-                wst[base + (long long)c0 * d + r0] = v;
-                wst[base + (long long)c1 * d + r1] = v1;
-            } else if (o < 2 * spec + (long long)c * c) {
-                const int r = (int)(o - 2 * spec);
-                wt[(long long)l * c * c + (long long)(r % c) * c + r / c] = v;
+                ws[base + r0 * d + c0] = v;
+                ws[base + r1 * d + c1] = v1;
+                wst[base + c0 * d + r0] = v;
+                wst[base + c1 * d + r1] = v1;
+            } else if (o < 2 * spec + cc) {
+                const unsigned r = o - 2 * spec;
+                wt[(size_t)l * cc + (r % c) * c + r / c] = v;
             }
-        } else if (i >= a.q1 && i < a.q1 + (long long)c * a.h) {
-            const int r = (int)(i - a.q1);
-            static_cast<__nv_bfloat16 *>(a.q1t)[(long long)(r % a.h) * c + r / a.h] = v;
+        } else if (i >= q1 && i - q1 < c * a.h) {
+            const unsigned r = i - q1;
+            static_cast<__nv_bfloat16 *>(a.q1t)[(r % a.h) * c + r / a.h] = v;
         }
     }
 }
@@ -1302,6 +1324,8 @@ cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int mod
 
 cudaError_t sno_prepare(const SnoPrepare &a, cudaStream_t s)
 {
+    if (a.count >= 1LL << 31)  // the kernel's 32-bit indices
+        return cudaErrorInvalidValue;
     prepare_kernel<<<grid_for(a.count), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
@@ -1314,42 +1338,34 @@ cudaError_t sno_spec_reduce(const float *dw, float *drr, float *dri, int modes, 
 
 namespace {
 
-template <typename T, int NW>
+template <typename T, int NW, bool HEAD>
 void launch_colsum(const SnoSums &a, cudaStream_t s)
 {
-    const T *x = static_cast<const T *>(a.x), *w = static_cast<const T *>(a.w);
-    const bool v = a.cols % Chunk<T>::E == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(a.x) |
+                         (HEAD ? reinterpret_cast<uintptr_t>(a.pre) | reinterpret_cast<uintptr_t>(a.out) : 0) |
+                         (NW == 4 ? reinterpret_cast<uintptr_t>(a.w) : 0);
+    const bool v = a.cols % Chunk<T>::E == 0 && (at & 15) == 0 && (NW != 4 || a.ldw == Chunk<T>::E);
     const int cw = v ? 64 : 32;
     const dim3 grid(kSumBlocks, (a.cols + cw - 1) / cw);
     if (v)
-        colsum_kernel<T, NW, true><<<grid, 256, 0, s>>>(x, a.rows, a.cols, w, a.ldw, a.part, a.ticket, a.sum, a.wsum, a.wtot);
+        colsum_kernel<T, NW, true, HEAD><<<grid, 256, 0, s>>>(a);
     else
-        colsum_kernel<T, NW, false><<<grid, 256, 0, s>>>(x, a.rows, a.cols, w, a.ldw, a.part, a.ticket, a.sum, a.wsum, a.wtot);
+        colsum_kernel<T, NW, false, HEAD><<<grid, 256, 0, s>>>(a);
 }
 
 template <typename T>
 cudaError_t pick_colsum(const SnoSums &a, cudaStream_t s)
 {
-    switch (a.nw) {
-    case 0: launch_colsum<T, 0>(a, s); break;
-    case 1: launch_colsum<T, 1>(a, s); break;
-    case 4: launch_colsum<T, 4>(a, s); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
-}
-
-template <bool EXACT, typename T>
-cudaError_t launch_outer(const void *d, const void *q, const void *pre, void *out, long long rows, int cols, cudaStream_t s)
-{
-    const bool v = cols % Chunk<T>::E == 0 && ((reinterpret_cast<uintptr_t>(pre) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
-    const long long total = rows * cols / (v ? Chunk<T>::E : 1);
-    const int grid = grid_for(total);
-    const T *dt = static_cast<const T *>(d), *qt = static_cast<const T *>(q), *pt = static_cast<const T *>(pre);
-    if (v)
-        outer_dgelu_kernel<EXACT, T, true><<<grid, 256, 0, s>>>(dt, qt, pt, static_cast<T *>(out), rows, cols);
+    if (a.nw == 0)
+        launch_colsum<T, 0, false>(a, s);
+    else if (a.nw == 1 && a.out)
+        launch_colsum<T, 1, true>(a, s);
+    else if (a.nw == 1)
+        launch_colsum<T, 1, false>(a, s);
+    else if (a.nw == 4)
+        launch_colsum<T, 4, false>(a, s);
     else
-        outer_dgelu_kernel<EXACT, T, false><<<grid, 256, 0, s>>>(dt, qt, pt, static_cast<T *>(out), rows, cols);
+        return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
 
@@ -1375,13 +1391,6 @@ int sno_sum_tickets(int cols) { return (cols + 31) / 32; }
 cudaError_t sno_colsum(const SnoSums &a, int bf16, cudaStream_t s)
 {
     return bf16 ? pick_colsum<__nv_bfloat16>(a, s) : pick_colsum<float>(a, s);
-}
-
-cudaError_t sno_outer_dgelu(const void *d, const void *q, const void *pre, void *out, long long rows, int cols, int bf16,
-                            cudaStream_t s)
-{
-    return bf16 ? launch_outer<false, __nv_bfloat16>(d, q, pre, out, rows, cols, s)
-                : launch_outer<true, float>(d, q, pre, out, rows, cols, s);
 }
 
 cudaError_t sno_row_dot(const void *h, const void *q, const float *q2, const float *u0, float *out, long long rows, int cols,

@@ -82,16 +82,18 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n)
 
 // B operand descriptor, MN-major with a 128-byte swizzle, for a tile of K
 // rows of 64 BF16 N values (one swizzle atom wide, as TMA stores a box 128
-// bytes wide): 8-row K groups 1024 bytes apart (the same stride in both
-// offset fields: with one atom across N, only the K direction has a stride).
-// The instruction descriptor marks B MN-major with bit 16.
+// bytes wide): 8-row K groups 1024 bytes apart.  The instruction descriptor
+// marks A MN-major with bit 15, B with bit 16.
 constexpr uint32_t kIdescBMn = 1u << 16;
-__device__ __forceinline__ uint64_t smem_desc_mn128(const void *tile)
+__device__ __forceinline__ uint64_t smem_desc_mn128(const void *tile, uint32_t atom_stride = 1024)
 {
+    // atom_stride: bytes from one 64-wide atom across M or N to the next
+    // (the leading byte offset), for operands of two atoms
     const uint64_t addr = saddr(tile);
-    return ((addr & 0x3FFFF) >> 4) | ((uint64_t)(1024 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
-           (2ull << 61);
+    return ((addr & 0x3FFFF) >> 4) | ((uint64_t)(atom_stride >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           (1ull << 46) | (2ull << 61);
 }
+constexpr uint32_t kIdescAMn = 1u << 15;
 
 // GELU, tanh form: GELU(x) = x (1 + tanh(k0 (x + k1 x^3))) / 2
 constexpr float kGeluK0 = 0.7978845608028654f, kGeluK0K1 = 0.7978845608028654f * 0.044715f;
@@ -118,10 +120,27 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
+__device__ __forceinline__ uint32_t half_bf16x2(uint32_t x)
+{
+    const __nv_bfloat162 h = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(&x), __floats2bfloat162_rn(0.5f, 0.5f));
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+// A lane's row of 32 BF16 into a warp's staging buffer of 32 such rows: the
+// 16-byte chunk q of row `lane` sits at chunk q ^ ((lane >> 1) & 3), the
+// 64-byte swizzle the store's tensor map reads.
+__device__ __forceinline__ void stage_rows(unsigned char *stg, int lane, const uint32_t (&w)[16])
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<uint4 *>(stg + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4)) =
+            make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+}
+
 constexpr int kTcThreads = 160;
 constexpr int kTileM = 128;
 
-template <int MODE>
+template <int MODE, bool TRAIN>
 struct TcShape {
     static constexpr int N = MODE == 0 ? 64 : 128;                  // output columns (TMEM columns per stage)
     static constexpr uint32_t kA2 = kTileM * 128;                    // v tile: 128 rows x 64 BF16
@@ -136,12 +155,13 @@ struct TcShape {
     static constexpr int kAccs = MODE == 0 ? 2 : 1;
     static constexpr uint32_t kTmemCols = kAccs * N;
     // layer: per epilogue warp a 2 KB staging buffer of its 32 output rows x
-    // 32 columns (64-byte swizzle), written to global memory by a TMA store
-    static constexpr uint32_t kOut = MODE == 0 ? 4 * 2048 : 0;
+    // 32 columns (64-byte swizzle), written to global memory by a TMA store;
+    // in training a second one, for the value before GELU, in both modes
+    static constexpr uint32_t kOut = TRAIN ? 8 * 2048 : MODE == 0 ? 4 * 2048 : 0;
     static constexpr int kSmem = (int)(2 * kStage + kB2 + kOut + 1024);
 };
 
-// TRAIN: the training epilogues (P.pre, P.dg, no bias); inference keeps its
+// TRAIN: the training epilogues (P.keep, P.dg, no bias); inference keeps its
 // own instance, 8% faster than one that decides at run time.
 template <int MODE, bool TRAIN>
 __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constant__ CUtensorMap tmA1,
@@ -149,9 +169,10 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                                                             const __grid_constant__ CUtensorMap tmA2,
                                                             const __grid_constant__ CUtensorMap tmB2,
                                                             const __grid_constant__ CUtensorMap tmOut,
+                                                            const __grid_constant__ CUtensorMap tmPre,
                                                             const __grid_constant__ SnoTcArgs P)
 {
-    using S = TcShape<MODE>;
+    using S = TcShape<MODE, TRAIN>;
     constexpr int N = S::N;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>(
@@ -264,6 +285,16 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
         // ---- epilogue warps 0-3: TMEM lanes 32 warp .. 32 warp + 31 ------
         for (long long i = 0; i < my_tiles; ++i) {
             const int s = (int)(i & 1);
+            const long long g = (long long)blockIdx.x + i * gridDim.x;
+            const long long row = g * kTileM + warp * 32 + lane;
+            uint4 dg[TRAIN && MODE == 0 ? 8 : 1];
+            if (TRAIN && MODE == 0 && P.dg) {
+                // under the tile's loads and MMAs
+                const uint4 *d = reinterpret_cast<const uint4 *>(P.dg) + row * (N / 8);
+#pragma unroll
+                for (int q = 0; q < (TRAIN && MODE == 0 ? 8 : 1); ++q)
+                    dg[q] = d[q];
+            }
             const bool ok = bar_wait(&mma_done[s], (uint32_t)((i >> 1) & 1), P.limit, &s_abort);
             if (__any_sync(0xffffffffu, !ok)) {
                 if (lane == 0 && !s_abort) {
@@ -273,8 +304,6 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                 break;
             }
             tc_fence_after();
-            const long long g = (long long)blockIdx.x + i * gridDim.x;
-            const long long row = g * kTileM + warp * 32 + lane;
             const int ac = (int)(i % S::kAccs);
             const uint32_t taddr = tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)(ac * N);
             if (MODE == 0) {
@@ -287,32 +316,24 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                 if (lane == 0)
                     bar_arrive(&acc_empty[ac]);
                 // the warp's 32 rows leave through its staging buffer, 32
-                // columns (64 bytes a row) at a time: the 16-byte chunk q of
-                // row `lane` sits at chunk q ^ ((lane >> 1) & 3), the 64-byte
-                // swizzle the store's tensor map reads
+                // columns (64 bytes a row) at a time
                 unsigned char *stg = sm + 2 * S::kStage + S::kB2 + warp * 2048;
                 const long long row0 = g * kTileM + warp * 32;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t *r = h ? r1 : r0;
                     uint32_t w[16], keep[16];
-                    if (TRAIN && P.dg) {
-                        const uint4 *d = reinterpret_cast<const uint4 *>(P.dg) + row * (N / 8) + 4 * h;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const uint4 x = d[q];
-                            keep[4 * q] = x.x, keep[4 * q + 1] = x.y, keep[4 * q + 2] = x.z, keep[4 * q + 3] = x.w;
-                        }
-                    }
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         float a = __uint_as_float(r[2 * c]) + s_bias[32 * h + 2 * c];
                         float b = __uint_as_float(r[2 * c + 1]) + s_bias[32 * h + 2 * c + 1];
                         if (TRAIN && P.dg) {
-                            const float2 d = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&keep[c]));
+                            const uint4 &x = dg[TRAIN ? 4 * h + (c >> 2) : 0];
+                            const uint32_t y = (c & 3) == 0 ? x.x : (c & 3) == 1 ? x.y : (c & 3) == 2 ? x.z : x.w;
+                            const float2 d = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&y));
                             a *= gelu_grad_hw(d.x);
                             b *= gelu_grad_hw(d.y);
-                        } else if (TRAIN && P.pre) {
+                        } else if (TRAIN && P.keep) {
                             keep[c] = pack_bf16(a, b);
                         }
                         if (P.gelu) {
@@ -321,24 +342,19 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                         }
                         w[c] = pack_bf16(a, b);
                     }
-                    if (TRAIN && P.pre) {
-                        uint4 *d = reinterpret_cast<uint4 *>(P.pre) + row * (N / 8) + 4 * h;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            d[q] = make_uint4(keep[4 * q], keep[4 * q + 1], keep[4 * q + 2], keep[4 * q + 3]);
-                    }
                     // the buffer is free once the previous store has read it
                     if (lane == 0)
                         bulk_wait_read0();
                     __syncwarp();
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        *reinterpret_cast<uint4 *>(stg + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4)) =
-                            make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+                    stage_rows(stg, lane, w);
+                    if (TRAIN && P.keep)
+                        stage_rows(stg + 4 * 2048, lane, keep);
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) {
                         tma_store_2d(&tmOut, stg, 32 * h, (int)row0);
+                        if (TRAIN && P.keep)
+                            tma_store_2d(&tmPre, stg + 4 * 2048, 32 * h, (int)row0);
                         bulk_commit();
                     }
                 }
@@ -360,6 +376,7 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                     tmem_ld32(taddr + 64 * h, r[0]);
                     tmem_ld32(taddr + 64 * h + 32, r[1]);
                     tmem_wait_ld();
+                    uint32_t wp[TRAIN ? 2 : 1][16], wh[TRAIN ? 2 : 1][16];
 #pragma unroll
                     for (int c = 0; c < 64; c += 2) {
                         const int col = 64 * h + c;
@@ -373,7 +390,35 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                         float t0, t1;
                         asm("tanh.approx.f32 %0, %1;" : "=f"(t0) : "f"(af.x));
                         asm("tanh.approx.f32 %0, %1;" : "=f"(t1) : "f"(af.y));
-                        part[(c >> 1) & 3] = f2_fma(f2_fma(x, f2(t0, t1), x), f2(wq.x, wq.y), part[(c >> 1) & 3]);
+                        uint64_t x2 = f2_fma(x, f2(t0, t1), x);  // 2 GELU(x)
+                        if (TRAIN) {
+                            // h is stored in BF16, and the output is the product
+                            // with what is stored (the backward pass uses it)
+                            const float2 xf = f2_split(x), hf = f2_split(x2);
+                            const uint32_t hb = pack_bf16(hf.x, hf.y);
+                            wp[TRAIN ? c >> 5 : 0][(c & 31) >> 1] = pack_bf16(xf.x, xf.y);
+                            wh[TRAIN ? c >> 5 : 0][(c & 31) >> 1] = half_bf16x2(hb);
+                            x2 = f2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xFFFF0000u));
+                        }
+                        part[(c >> 1) & 3] = f2_fma(x2, f2(wq.x, wq.y), part[(c >> 1) & 3]);
+                    }
+                    if (TRAIN) {
+                        unsigned char *stg = sm + 2 * S::kStage + S::kB2 + warp * 2048;
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            if (lane == 0)
+                                bulk_wait_read0();
+                            __syncwarp();
+                            stage_rows(stg, lane, wh[TRAIN ? q : 0]);
+                            stage_rows(stg + 4 * 2048, lane, wp[TRAIN ? q : 0]);
+                            fence_async_smem();
+                            __syncwarp();
+                            if (lane == 0) {
+                                tma_store_2d(&tmOut, stg, 64 * h + 32 * q, (int)(g * kTileM + warp * 32));
+                                tma_store_2d(&tmPre, stg + 4 * 2048, 64 * h + 32 * q, (int)(g * kTileM + warp * 32));
+                                bulk_commit();
+                            }
+                        }
                     }
                 }
                 const float2 accf = f2_split(f2_add(f2_add(part[0], part[1]), f2_add(part[2], part[3])));
@@ -387,8 +432,8 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
             }
         }
     }
-    // the layer's output stores have landed before the CTA exits
-    if (MODE == 0 && warp < 4 && lane == 0)
+    // the output stores have landed before the CTA exits
+    if ((MODE == 0 || TRAIN) && warp < 4 && lane == 0)
         bulk_wait0();
     tc_fence_before();
     __syncthreads();
@@ -409,15 +454,19 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
 // bytes apart and 16 points (one K step) 2048 bytes on.  A CTA takes whole
 // problems: the n / 128 chunks (8 MMAs each) accumulate into one TMEM tile,
 // then warp 0 (TMEM lanes 0 .. 31 = the 2M transform rows) writes vh[b] as
-// BF16 [2M][C].  Warp 1's lane 0 is the producer (two stages of TMA loads,
+// BF16 [2M][C].  Warp 1's lane 0 is the producer (ST stages of TMA loads,
 // the MMAs, commits); two accumulators, so the next problem's MMAs run
 // under the previous one's write-out.  Bounded waits as in sno_tc_kernel.
+// Two stages let four CTAs share an SM, the choice for many problems; with at
+// most one problem per SM (a training batch) a CTA is alone and the latency
+// of its loads counts, so all 8 chunks of 1024 points are in flight (64 problems: 10.9 -> 9.8 us).
 constexpr int kDftThreads = 64;
 constexpr uint32_t kDftAtom = 32 * 128;              // F rows of one 64-point half of a chunk
 constexpr uint32_t kDftV = 128 * 128;                // the activation tile
 constexpr uint32_t kDftStage = 2 * kDftAtom + kDftV;  // 24 KB: F halves first, so A's unused rows stay inside
-constexpr int kDftSmem = (int)(2 * kDftStage) + 1024;
+constexpr int dft_smem(int stages) { return stages * (int)kDftStage + 1024; }
 
+template <int ST>
 __global__ void __launch_bounds__(kDftThreads) sno_tc_dft_kernel(const __grid_constant__ CUtensorMap tmF,
                                                                  const __grid_constant__ CUtensorMap tmV,
                                                                  const __grid_constant__ SnoTcArgs P)
@@ -427,14 +476,16 @@ __global__ void __launch_bounds__(kDftThreads) sno_tc_dft_kernel(const __grid_co
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    __shared__ __align__(8) uint64_t full[2], freed[2], done[2], acc_empty[2];
+    __shared__ __align__(8) uint64_t full[ST], freed[ST], done[2], acc_empty[2];
     __shared__ uint32_t tmem_base_sh;
     __shared__ volatile int s_abort;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     if (t == 0) {
-        for (int s = 0; s < 2; ++s) {
+        for (int s = 0; s < ST; ++s) {
             bar_init(&full[s], 1);
             bar_init(&freed[s], 1);
+        }
+        for (int s = 0; s < 2; ++s) {
             bar_init(&done[s], 1);
             bar_init(&acc_empty[s], 1);
         }
@@ -457,7 +508,7 @@ __global__ void __launch_bounds__(kDftThreads) sno_tc_dft_kernel(const __grid_co
             // ---- producer: loads and MMAs, item = (problem, chunk) ----------
             const long long items = mine * kChunks;
             auto load = [&](long long it) {
-                const int s = (int)(it & 1);
+                const int s = (int)(it % ST);
                 const long long b = (long long)blockIdx.x + (it / kChunks) * gridDim.x;
                 const int ch = (int)(it % kChunks);
                 unsigned char *st = sm + s * kDftStage;
@@ -468,21 +519,21 @@ __global__ void __launch_bounds__(kDftThreads) sno_tc_dft_kernel(const __grid_co
             };
             long long issued = 0, committed = 0;
             bool ok = true;
-            load(0);
-            issued = 1;
+            for (; issued < ST - 1 && issued < items; ++issued)
+                load(issued);
             for (long long it = 0; ok && it < items; ++it) {
-                const int s = (int)(it & 1);
+                const int s = (int)(it % ST);
                 const long long prob = it / kChunks;
                 const int ch = (int)(it % kChunks);
-                if (it + 1 < items) {
-                    // stage (it + 1) & 1 is free once the MMAs of item it - 1 are done
-                    if (it >= 1 && !(ok = bar_wait(&freed[(it + 1) & 1], (uint32_t)(((it - 1) >> 1) & 1), P.limit,
-                                                    &s_abort)))
+                if (it + ST - 1 < items) {
+                    // its stage is free once the MMAs of item it - 1 are done
+                    if (it >= 1 && !(ok = bar_wait(&freed[(it - 1) % ST], (uint32_t)(((it - 1) / ST) & 1), P.limit,
+                                                   &s_abort)))
                         break;
-                    load(it + 1);
-                    issued = it + 2;
+                    load(it + ST - 1);
+                    issued = it + ST;
                 }
-                if (!(ok = bar_wait(&full[s], (uint32_t)((it >> 1) & 1), P.limit, &s_abort)))
+                if (!(ok = bar_wait(&full[s], (uint32_t)((it / ST) & 1), P.limit, &s_abort)))
                     break;
                 const int a = (int)(prob & 1);  // accumulator of this problem
                 if (ch == 0 && prob >= 2 &&
@@ -507,9 +558,9 @@ __global__ void __launch_bounds__(kDftThreads) sno_tc_dft_kernel(const __grid_co
                 atomicExch(P.err, kDevTimeout);
                 s_abort = 1;
                 for (long long j = committed; j < issued; ++j)
-                    bar_drain(&full[j & 1], (uint32_t)((j >> 1) & 1), kWaitLimitCycles);
+                    bar_drain(&full[j % ST], (uint32_t)((j / ST) & 1), kWaitLimitCycles);
                 if (committed > 0)
-                    bar_drain(&freed[(committed - 1) & 1], (uint32_t)(((committed - 1) >> 1) & 1), kWaitLimitCycles);
+                    bar_drain(&freed[(committed - 1) % ST], (uint32_t)(((committed - 1) / ST) & 1), kWaitLimitCycles);
             }
         }
         __syncwarp();
@@ -571,11 +622,12 @@ constexpr int kMixThreads = 128;
 constexpr uint32_t kMixHalf = 128 * 128;  // one 64-wide box of 128 rows
 constexpr int kMixSmem = (int)(4 * kMixHalf) + 1024;
 
+template <int N>
 __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                  const __grid_constant__ CUtensorMap tmB,
                                                                  const __grid_constant__ SnoTcMixArgs P)
 {
-    constexpr uint32_t idesc = idesc_bf16(128, 128);
+    constexpr uint32_t idesc = idesc_bf16(128, N);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -601,7 +653,7 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
     tc_fence_after();
     const uint32_t tbase = tmem_base_sh;
     if (t == 0) {
-        bar_expect_tx(&full, 4 * kMixHalf);
+        bar_expect_tx(&full, 2 * kMixHalf + 2 * N * 128);
         tma_2d(sa, &tmA, m * 128, row0, &full);
         tma_2d(sa + kMixHalf, &tmA, m * 128 + 64, row0, &full);
         tma_2d(sb, &tmB, 0, P.b_row0 + m * 128, &full);
@@ -634,9 +686,9 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
         tc_fence_after();
         const int b = row0 + warp * 32 + lane;
         uint4 *dst = reinterpret_cast<uint4 *>(static_cast<unsigned char *>(P.y) +
-                                               ((long long)b * P.row_elems + (long long)m * 128) * 2);
+                                               ((long long)b * P.row_elems + (long long)m * N) * 2);
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
+        for (int h = 0; h < N / 32; ++h) {
             uint32_t r[32];
             tmem_ld32(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)(32 * h), r);
             tmem_wait_ld();
@@ -657,10 +709,210 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
         tmem_dealloc(tbase, 128);
 }
 
+// ---- weight gradients on the tensor cores -----------------------------------
+//
+// dW = X^T dY, the sum over all grid points (rows) of products of two
+// activations [rows][64 or 128] as they lie in memory: the rows are the K
+// dimension, both operands are MN-major.  A CTA takes every gridDim.x-th
+// chunk of 128 rows: up to four stages of TMA loads in flight, 8 MMAs of K =
+// 16 a chunk into one FP32 accumulator in TMEM, then the result is added to
+// global memory.
+//   KIND 0 / 1: X [rows][64], dY [rows][64 / 128].  The instruction has 128
+//       rows of A and X gives 64: the others come from a constant tile whose
+//       first column is 1 (the second atom of A, at its own stride), so that
+//       accumulator row 64 is the column sum of dY, the bias gradient.
+//   KIND 2: one CTA per mode, X and dY [rows = problems][128]; D = X^T dY is
+//       folded to the complex weights' gradients before it is stored.
+// Bound by the latency of the loads and of the adds (16 MB in KIND 0: 2.4 us
+// at the copy rate).  65,536 rows, cold caches: KIND 0 takes 11.1 us, KIND 1
+// 12.9 us; as mma.sync tiles with split K, a column-sum pass and a memset
+// they took 38 and 40 us.  KIND 2, 64 problems: 7.5 us, before 19.4 us with
+// the folding as a pass of its own.
+template <int KIND>
+struct GradShape {
+    static constexpr int AT = KIND == 2 ? 2 : 1, NB = KIND == 0 ? 1 : 2;  // 64-wide atoms of X and dY
+    static constexpr uint32_t kAtom = 128 * 128;
+    static constexpr uint32_t kStage = (AT + NB) * kAtom;
+    static constexpr int ST = KIND == 2 ? 2 : 4;
+    static constexpr uint32_t kOnes = KIND == 2 ? 0 : 16 * 128;
+    static constexpr int kSmem = (int)(ST * kStage + kOnes) + 1024;
+};
+constexpr int kGradThreads = 160;
+
+__device__ __forceinline__ void red_add4(float *p, float a, float b, float c, float d)
+{
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(kGradThreads) sno_tc_grad_kernel(const __grid_constant__ CUtensorMap tmX,
+                                                                   const __grid_constant__ CUtensorMap tmY,
+                                                                   const __grid_constant__ SnoTcGradArgs P)
+{
+    using S = GradShape<KIND>;
+    constexpr int N = 64 * S::NB, ST = S::ST;
+    constexpr uint32_t idesc = idesc_bf16(128, N) | kIdescAMn | kIdescBMn;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *sm = reinterpret_cast<unsigned char *>(
+        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    unsigned char *ones = sm + ST * S::kStage;
+    __shared__ __align__(8) uint64_t full[ST], freed[ST], done;
+    __shared__ uint32_t tmem_base_sh;
+    __shared__ volatile int s_abort;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    if (t == 0) {
+        for (int s = 0; s < ST; ++s) {
+            bar_init(&full[s], 1);
+            bar_init(&freed[s], 1);
+        }
+        bar_init(&done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_abort = 0;
+    }
+    if (warp == 0) {
+        tmem_alloc(&tmem_base_sh, N);
+        tmem_relinquish();
+    }
+    // 16 K rows of 64 values, value 0 = 1: in row k the 16-byte chunk 0 lies
+    // at chunk k & 7 (128-byte swizzle)
+    for (int i = t; i < (int)S::kOnes / 16; i += kGradThreads)
+        reinterpret_cast<uint4 *>(ones)[i] = make_uint4((i & 7) == ((i >> 3) & 7) ? 0x3F80u : 0u, 0u, 0u, 0u);
+    fence_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = tmem_base_sh;
+    const long long chunks = (P.rows + 127) / 128;
+    const long long mine = chunks > (long long)blockIdx.x ? (chunks - 1 - (long long)blockIdx.x) / gridDim.x + 1 : 0;
+    const int x0 = KIND == 2 ? (int)blockIdx.y * 128 : 0;
+
+    if (warp == 4) {
+        auto load = [&](long long it) {
+            if (lane == 0) {
+                const int s = (int)(it % ST);
+                const int row = (int)(((long long)blockIdx.x + it * gridDim.x) * 128);
+                unsigned char *st = sm + s * S::kStage;
+                bar_expect_tx(&full[s], S::kStage);
+                for (int q = 0; q < S::AT; ++q)
+                    tma_2d(st + q * S::kAtom, &tmX, x0 + 64 * q, row, &full[s]);
+                for (int q = 0; q < S::NB; ++q)
+                    tma_2d(st + (S::AT + q) * S::kAtom, &tmY, x0 + 64 * q, row, &full[s]);
+            }
+        };
+        long long issued = 0, committed = 0;
+        bool ok = true;
+        for (; issued < ST && issued < mine; ++issued)
+            load(issued);
+        for (long long it = 0; it < mine; ++it) {
+            const int s = (int)(it % ST);
+            if (!(ok = __all_sync(0xffffffffu, bar_wait(&full[s], (uint32_t)((it / ST) & 1), P.limit, &s_abort))))
+                break;
+            unsigned char *st = sm + s * S::kStage;
+            const long long left = P.rows - ((long long)blockIdx.x + it * gridDim.x) * 128;
+            const int valid = left < 128 ? (int)left : 128, steps = (valid + 15) / 16;
+            if (valid < 16 * steps) {
+                // rows past the end (another batch's): zero in both operands
+                for (int i = lane; i < (16 * steps - valid) * 8; i += 32)
+                    for (int q = 0; q < S::AT + S::NB; ++q)
+                        *reinterpret_cast<uint4 *>(st + q * S::kAtom + valid * 128 + i * 16) = make_uint4(0, 0, 0, 0);
+                fence_async_smem();
+            }
+            __syncwarp();
+            if (lane == 0) {
+                tc_fence_after();
+                unsigned char *b = st + S::AT * S::kAtom;
+                for (int k = 0; k < steps; ++k) {
+                    unsigned char *a = st + k * 2048;
+                    const uint32_t second = KIND == 2 ? S::kAtom : (uint32_t)(ones - a);
+                    tc_mma(tbase, smem_desc_mn128(a, second), smem_desc_mn128(b + k * 2048, S::kAtom), idesc,
+                           (it > 0 || k > 0) ? 1u : 0u);
+                }
+                tc_commit(&freed[s]);
+                if (it == mine - 1)
+                    tc_commit(&done);
+            }
+            committed = it + 1;
+            // refill the stage of the item before
+            if (it >= 1 && it - 1 + ST < mine) {
+                const long long q = it - 1;
+                if (!(ok = __all_sync(0xffffffffu, bar_wait(&freed[q % ST], (uint32_t)((q / ST) & 1), P.limit,
+                                                            &s_abort))))
+                    break;
+                load(q + ST);
+                issued = q + ST + 1;
+            }
+        }
+        if (!ok && lane == 0) {
+            atomicExch(P.err, kDevTimeout);
+            s_abort = 1;
+            for (long long j = committed; j < issued; ++j)
+                bar_drain(&full[j % ST], (uint32_t)((j / ST) & 1), kWaitLimitCycles);
+            if (committed > 0)
+                bar_drain(&freed[(committed - 1) % ST], (uint32_t)(((committed - 1) / ST) & 1), kWaitLimitCycles);
+        }
+        __syncwarp();
+    } else if (mine > 0) {
+        const bool ok = __all_sync(0xffffffffu, bar_wait(&done, 0, P.limit, &s_abort));
+        if (!ok && lane == 0 && !s_abort) {
+            atomicExch(P.err, kDevTimeout);
+            s_abort = 1;
+        }
+        tc_fence_after();
+        const uint32_t taddr = tbase + ((uint32_t)(warp * 32) << 16);
+        const int row = warp * 32 + lane;
+        if (KIND == 2) {
+            // thread i holds row i of D; with R_im the rows 64 .. 127,
+            //   dRr[o][i] = D[i][o] + D[64 + i][64 + o]
+            //   dRi[o][i] = D[i][64 + o] - D[64 + i][o]
+            float *other = reinterpret_cast<float *>(sm);  // the stages are read: [128 columns][64 rows]
+            if (ok && warp >= 2)
+                for (int h = 0; h < 4; ++h) {
+                    uint32_t r[32];
+                    tmem_ld32(taddr + 32 * h, r);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < 32; ++c)
+                        other[(32 * h + c) * 64 + row - 64] = __uint_as_float(r[c]);
+                }
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (ok && warp < 2)
+                for (int h = 0; h < 4; ++h) {
+                    uint32_t r[32];
+                    tmem_ld32(taddr + 32 * h, r);
+                    tmem_wait_ld();
+                    float *dst = (h < 2 ? P.drr : P.dri) + (long long)blockIdx.y * 64 * 64;
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) {
+                        const int o = 32 * (h & 1) + c;
+                        const float v = __uint_as_float(r[c]), w = other[(h < 2 ? 64 + o : o) * 64 + row];
+                        dst[o * 64 + row] = h < 2 ? v + w : v - w;
+                    }
+                }
+        } else if (ok && warp < 3) {
+            float *dst = row < 64 ? P.dw + row * N : P.db;
+            for (int h = 0; h < N / 32; ++h) {
+                uint32_t r[32];
+                tmem_ld32(taddr + 32 * h, r);
+                tmem_wait_ld();
+                if (row <= 64)
+#pragma unroll
+                    for (int c = 0; c < 32; c += 4)
+                        red_add4(dst + 32 * h + c, __uint_as_float(r[c]), __uint_as_float(r[c + 1]),
+                                 __uint_as_float(r[c + 2]), __uint_as_float(r[c + 3]));
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0)
+        tmem_dealloc(tbase, N);
+}
+
 template <int MODE, bool TRAIN>
 cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
-    using S = TcShape<MODE>;
+    using S = TcShape<MODE, TRAIN>;
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(sno_tc_kernel<MODE, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -691,8 +943,9 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
         if (e != cudaSuccess)
             return e;
         int fit = sm_bytes / (S::kSmem + (int)fa.sharedSizeBytes + reserve);
-        const int tmem_cap = 512 / (int)S::kTmemCols;
+        const int tmem_cap = 512 / (int)S::kTmemCols, reg_cap = 65536 / ((fa.numRegs + 7) / 8 * 8 * kTcThreads);
         per_sm = fit < tmem_cap ? fit : tmem_cap;
+        per_sm = per_sm < reg_cap ? per_sm : reg_cap;
         if (per_sm < 1)
             return cudaErrorInvalidConfiguration;
     }
@@ -701,42 +954,32 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
         grid = a.n_tiles;
     if (grid < 1)
         return cudaSuccess;
-    if (!m.a2 || !m.b2 || (MODE == 0 && (!m.a1 || !m.b1 || !m.out)))
+    if (!m.a2 || !m.b2 || (MODE == 0 && (!m.a1 || !m.b1 || !m.out)) || (TRAIN && a.keep && (!m.out || !m.pre)))
         return cudaErrorInvalidValue;
     // the projection has no first product and no output map: those
     // parameters repeat a2
     const CUtensorMap *a1 = static_cast<const CUtensorMap *>(MODE == 0 ? m.a1 : m.a2);
     const CUtensorMap *b1 = static_cast<const CUtensorMap *>(MODE == 0 ? m.b1 : m.a2);
-    const CUtensorMap *o = static_cast<const CUtensorMap *>(MODE == 0 ? m.out : m.a2);
+    const CUtensorMap *o = static_cast<const CUtensorMap *>(MODE == 0 || TRAIN ? m.out : m.a2);
+    const CUtensorMap *pre = static_cast<const CUtensorMap *>(TRAIN && m.pre ? m.pre : m.a2);
     sno_tc_kernel<MODE, TRAIN><<<(int)grid, kTcThreads, S::kSmem, s>>>(*a1, *b1, *static_cast<const CUtensorMap *>(m.a2),
-                                                              *static_cast<const CUtensorMap *>(m.b2), *o, a);
+                                                              *static_cast<const CUtensorMap *>(m.b2), *o, *pre, a);
     return cudaGetLastError();
 }
 
-}  // namespace
-
-cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
-{
-    return a.pre || a.dg || !a.bias ? launch_tc<0, true>(m, a, sms, s) : launch_tc<0, false>(m, a, sms, s);
-}
-
-cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
-{
-    return launch_tc<1, false>(m, a, sms, s);
-}
-
-cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a, int sms, cudaStream_t s)
+template <int ST>
+cudaError_t launch_dft(const CUtensorMap &f, const CUtensorMap &v, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
     static int per_sm = 0;
     if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(sno_tc_dft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDftSmem);
+        cudaError_t e = cudaFuncSetAttribute(sno_tc_dft_kernel<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, dft_smem(ST));
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(sno_tc_dft_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+            e = cudaFuncSetAttribute(sno_tc_dft_kernel<ST>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      cudaSharedmemCarveoutMaxShared);
         cudaFuncAttributes fa{};
         int dev = 0, sm_bytes = 0, reserve = 0;
         if (e == cudaSuccess)
-            e = cudaFuncGetAttributes(&fa, sno_tc_dft_kernel);
+            e = cudaFuncGetAttributes(&fa, sno_tc_dft_kernel<ST>);
         if (e == cudaSuccess)
             e = cudaGetDevice(&dev);
         if (e == cudaSuccess)
@@ -745,29 +988,27 @@ cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a,
             e = cudaDeviceGetAttribute(&reserve, cudaDevAttrReservedSharedMemoryPerBlock, dev);
         if (e != cudaSuccess)
             return e;
-        const int fit = sm_bytes / (kDftSmem + (int)fa.sharedSizeBytes + reserve);
+        const int fit = sm_bytes / (dft_smem(ST) + (int)fa.sharedSizeBytes + reserve);
         per_sm = fit < 4 ? fit : 4;  // 128 TMEM columns each
         if (per_sm < 1)
             return cudaErrorInvalidConfiguration;
     }
-    if (!map_f || !map_v || a.tiles_per_problem < 1)
-        return cudaErrorInvalidValue;
     const long long problems = a.n_tiles / a.tiles_per_problem;
     long long grid = (long long)sms * per_sm;
     if (grid > problems)
         grid = problems;
     if (grid < 1)
         return cudaSuccess;
-    sno_tc_dft_kernel<<<(int)grid, kDftThreads, kDftSmem, s>>>(*static_cast<const CUtensorMap *>(map_f),
-                                                              *static_cast<const CUtensorMap *>(map_v), a);
+    sno_tc_dft_kernel<ST><<<(int)grid, kDftThreads, dft_smem(ST), s>>>(f, v, a);
     return cudaGetLastError();
 }
 
-cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s)
+template <int N>
+cudaError_t launch_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s)
 {
     static bool ready = false;
     if (!ready) {
-        cudaError_t e = cudaFuncSetAttribute(sno_tc_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMixSmem);
+        cudaError_t e = cudaFuncSetAttribute(sno_tc_mix_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMixSmem);
         if (e != cudaSuccess)
             return e;
         ready = true;
@@ -777,9 +1018,74 @@ cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixAr
     if (a.batch == 0)
         return cudaSuccess;
     const dim3 grid((unsigned)((a.batch + 127) / 128), (unsigned)modes);
-    sno_tc_mix_kernel<<<grid, kMixThreads, kMixSmem, s>>>(*static_cast<const CUtensorMap *>(map_vh),
+    sno_tc_mix_kernel<N><<<grid, kMixThreads, kMixSmem, s>>>(*static_cast<const CUtensorMap *>(map_vh),
                                                           *static_cast<const CUtensorMap *>(map_wst), a);
     return cudaGetLastError();
+}
+
+template <int KIND>
+cudaError_t launch_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, dim3 grid, cudaStream_t s)
+{
+    using S = GradShape<KIND>;
+    static bool ready = false;
+    if (!ready) {
+        cudaError_t e =
+            cudaFuncSetAttribute(sno_tc_grad_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
+        if (e != cudaSuccess)
+            return e;
+        ready = true;
+    }
+    if (!map_x || !map_y || a.rows < 0 || a.rows > 0x7FFFFF00LL)
+        return cudaErrorInvalidValue;
+    if (a.rows == 0 || grid.x == 0 || grid.y == 0)
+        return cudaSuccess;
+    sno_tc_grad_kernel<KIND><<<grid, kGradThreads, S::kSmem, s>>>(*static_cast<const CUtensorMap *>(map_x),
+                                                                  *static_cast<const CUtensorMap *>(map_y), a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
+{
+    return a.keep || a.dg || !a.bias ? launch_tc<0, true>(m, a, sms, s) : launch_tc<0, false>(m, a, sms, s);
+}
+
+cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
+{
+    return a.keep ? launch_tc<1, true>(m, a, sms, s) : launch_tc<1, false>(m, a, sms, s);
+}
+
+cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a, int sms, cudaStream_t s)
+{
+    if (!map_f || !map_v || a.tiles_per_problem < 1)
+        return cudaErrorInvalidValue;
+    const CUtensorMap &f = *static_cast<const CUtensorMap *>(map_f), &v = *static_cast<const CUtensorMap *>(map_v);
+    return a.n_tiles / a.tiles_per_problem <= sms ? launch_dft<8>(f, v, a, sms, s) : launch_dft<2>(f, v, a, sms, s);
+}
+
+cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s)
+{
+    return launch_mix<128>(map_vh, map_wst, a, modes, s);
+}
+
+cudaError_t sno_tc_rows(const void *map_x, const void *map_b, const SnoTcMixArgs &a, cudaStream_t s)
+{
+    return launch_mix<64>(map_x, map_b, a, 1, s);
+}
+
+cudaError_t sno_tc_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, int cols, int sms, cudaStream_t s)
+{
+    if (cols != 64 && cols != 128)
+        return cudaErrorInvalidValue;
+    const long long chunks = (a.rows + 127) / 128, per = (chunks + sms - 1) / sms;
+    const dim3 grid((unsigned)(per > 0 ? (chunks + per - 1) / per : 0), 1);
+    return cols == 64 ? launch_grad<0>(map_x, map_y, a, grid, s) : launch_grad<1>(map_x, map_y, a, grid, s);
+}
+
+cudaError_t sno_tc_grad_spec(const void *map_vh, const void *map_dy, const SnoTcGradArgs &a, int modes, cudaStream_t s)
+{
+    return launch_grad<2>(map_vh, map_dy, a, dim3(1, (unsigned)modes), s);
 }
 
 }  // namespace ge
