@@ -20,6 +20,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <mutex>
 
@@ -581,17 +583,24 @@ __global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, cons
 template <typename T>
 __global__ void __launch_bounds__(256) prop_dot_kernel(const __grid_constant__ PropRun P)
 {
-    __shared__ double s_w[kDotWin];
+    extern __shared__ double s_w[];
+    double *taps = s_w + kDotWin;
     __shared__ DotShared<kDotRows> sh;
     if (P.tiles > 0) {
         const long long items = (long long)*reinterpret_cast<const volatile int *>(P.count) * (kPropBlk / kDotRows);
         if (blockIdx.x == 0 && threadIdx.x == 0)
             *P.count_next = 0;
+        if (blockIdx.x < items)
+            dot_stage<256>(P, reinterpret_cast<typename PairOf<T>::E *>(taps));
         for (long long it = blockIdx.x; it < items; it += gridDim.x)
-            dot_listed<T, 256>(P, sh, s_w, it);
+            dot_listed<T, 256, true>(P, sh, s_w, taps, it);
     } else {
-        for (long long r0 = blockIdx.x * (long long)kDotRows; r0 < P.n; r0 += gridDim.x * (long long)kDotRows)
-            dot_rows<T, 256, kDotRows>(P, sh, s_w, r0, r0 + kDotRows < P.n ? r0 + kDotRows : P.n);
+        dot_stage<256>(P, reinterpret_cast<typename PairOf<T>::E *>(taps));
+        const int shift = item_shift(P);
+        for (long long r0 = blockIdx.x * (long long)kDotRows - shift; r0 < P.n; r0 += gridDim.x * (long long)kDotRows) {
+            const long long r1 = r0 + kDotRows;
+            dot_rows<T, 256, kDotRows, 1, true>(P, sh, s_w, taps, r0 > 0 ? r0 : 0, r1 < P.n ? r1 : P.n);
+        }
     }
 }
 
@@ -774,13 +783,61 @@ __device__ __forceinline__ uint64_t plain_desc(uint32_t addr, uint32_t lead)
 // kind::f16 with FP16 operands and FP32 accumulators, M = 128, N = 64.
 constexpr uint32_t kIdescF16 = (1u << 4) | ((uint32_t)(kPropBlk >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 
-// 16 warps that convert and drain, 1 that issues the MMAs: the conversion and
-// the drain are chains of integer instructions with little else to hide their
-// latency.
-constexpr int kTileWarps = 16, kTileConv = 32 * kTileWarps, kTileThreads = kTileConv + 32;
+// 16 warps that convert and drain: chains of integer instructions with little
+// else to hide their latency.  2 that issue the MMAs, every other sum each:
+// one warp issues one in 54 cycles, and spends 200 to 300 between two digit
+// products, where the tensor cores take 48.
+constexpr int kTileWarps = 16, kMmaWarps = 2;
+constexpr int kTileConv = 32 * kTileWarps, kTileThreads = kTileConv + 32 * kMmaWarps;
+constexpr int kEdgeParts = kTileWarps / kEdgeRows, kEdgeScratch = 32 * kEdgeParts * (kEdgeRows + 2);
 constexpr int kTileCols = kPropBlk / (kTileWarps / 4);  // points of a block a thread drains
+static_assert((kDotWin + kEdgeScratch + dot_taps(kPropR64Max)) * 8 <= kTileSmem<double> - 1024 &&
+                  (kDotWin + kEdgeScratch + dot_taps(kPropRMax)) * 8 <= kTileSmem<float> - 1024,
+              "the rows near a wall fit");
 
-template <typename T>
+// SPLIT: a cluster of 2, 4 or 8 CTAs per tile, for grids with fewer tiles than
+// SMs.  Each CTA issues its share of every digit product's MMAs, in units of
+// four; the sums are integers, so the shares add up to what one CTA's sum
+// would have been, bit for bit.  They meet in shared memory as 64-bit
+// integers, and each CTA finishes its share of the points of every block.
+// The conversion is not shared: a digit product's window is its own, and
+// their union is nearly the whole one.  The launcher weighs the tile's time
+// against that of the wall rows, which need the CTAs without a tile: n =
+// 100,003, k = 1999, FP64 takes 4 CTAs a tile, 68 -> 49 us a call (8: 57, 2:
+// 59); n = 500,000 takes 2, 82 -> 67 us; n = 300,001, FP32, two operators:
+// 100 -> 82 us.
+constexpr int kPartHigh = kPropTileBlks * kPropBlk * 8;  // bytes of a CTA's sums [64 points][128 blocks]; FP64: 16 last bits follow
+// One partial sum from each CTA of the cluster, and for FP64 its last bits.
+template <typename T, int C>
+__device__ __forceinline__ void add_parts(uint32_t addr, uint32_t addr_low, long long &hi, int &low)
+{
+    long long h[C];
+    unsigned short l[C];
+#pragma unroll
+    for (int p = 0; p < C; ++p) {
+        uint32_t a, b;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(p));
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(b) : "r"(addr_low), "r"(p));
+        asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(h[p]) : "r"(a) : "memory");
+        if (sizeof(T) == 8)
+            asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(l[p]) : "r"(b) : "memory");
+    }
+    hi = low = 0;
+#pragma unroll
+    for (int p = 0; p < C; ++p) {
+        hi += h[p];
+        if (sizeof(T) == 8)
+            low += l[p];
+    }
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <typename T, bool SPLIT>
 __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid_constant__ PropRun P)
 {
     using S = TileShape<T>;
@@ -799,6 +856,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
     __shared__ int s_left;
     __shared__ PropHeader s_hdr;
     __shared__ DotShared<kEdgeRows> s_dot;
+    __shared__ int4 s_prod[S::kGroups * ND];  // see below
+    __shared__ int s_used;                    // split: sums this CTA has products of
 
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     if (t < (int)(sizeof(PropHeader) / 4))
@@ -808,6 +867,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
         for (int g = 0; g < S::kGroups; ++g)
             bar_init(&done[g], 1);
         bar_init(&reuse, kTileWarps);
+        s_used = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_abort = 0;
     }
@@ -821,28 +881,77 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
     const uint32_t tbase = tmem_sh;
     if (blockIdx.x == 0 && t < 3 && P.zero[t])
         *P.zero[t] = 0;
+    const int ctas = SPLIT ? P.split : 1, lg = SPLIT ? 31 - __clz(ctas) : 0, rank = SPLIT ? (int)blockIdx.x & (ctas - 1) : 0;
+    // split: a tile per cluster; the CTAs without one start with the rows near
+    // a wall (edge_rounds items each), and what is left is everyone's
+    const int spare = SPLIT ? (int)gridDim.x - (int)P.tiles * ctas : 0, me = SPLIT ? (int)blockIdx.x - (int)P.tiles * ctas : 0;
+    const int shift = item_shift(P);
+    const long long edge_l = item_count(P.rows_l, kEdgeRows, shift);
+    const long long edges = edge_l + item_count(P.n - P.row_r, kEdgeRows, shift);
+    const long long early = SPLIT ? ((long long)spare * P.edge_rounds < edges ? (long long)spare * P.edge_rounds : edges) : 0;
+    const long long first = !SPLIT ? (long long)blockIdx.x
+                            : me < 0 ? (long long)blockIdx.x >> lg
+                            : me < early ? P.tiles + me
+                                         : P.tiles + early + blockIdx.x;
+    auto after = [&](long long x) {
+        if (!SPLIT || x >= P.tiles + early)
+            return x + (long long)gridDim.x;
+        if (x >= P.tiles && x + spare < P.tiles + early)
+            return x + spare;
+        return P.tiles + early + (long long)blockIdx.x;
+    };
     const int hb = P.hb, ok_tab = s_hdr.ok && s_hdr.rows * 16 <= S::kTab;
-    if (t == 0 && ok_tab) {
+    const bool has_tab = ok_tab && first < P.tiles;
+    if (t == 0 && has_tab) {
         bar_expect_tx(&tab_full, (uint32_t)s_hdr.rows * 16);
         bulk_load(sm, P.tab, (uint32_t)s_hdr.rows * 16, &tab_full);
     }
-    bool tab_waited = false;
+    // the digit products' first descriptors and steps, in issue order
+    for (int z = t; z < S::kGroups * ND; z += kTileThreads) {
+        const int g = z / ND, i = z % ND;
+        if (i < G::lo(g) || i > G::hi(g))
+            continue;
+        const int W = s_hdr.W[i], steps = (kPropBlk + 2 * W) / 16, units = (steps + 3) / 4;
+        int u0 = 0, u1 = units;
+        if (SPLIT) {
+            const int turn = (g + 3 * i) & (ctas - 1);
+            u0 = (units * rank + turn) >> lg;
+            u1 = (units * (rank + 1) + turn) >> lg;
+            if (u1 > u0)
+                atomicOr(&s_used, 1 << g);
+        }
+        // window position -W: block -W >> 6, piece q of its row (descending, as the
+        // table's rows run); four steps go 64 points on, to the next row
+        int4 p;
+        p.x = (int)((uint32_t)(((G::weight(g) - i) * C + hb + (-W >> 6)) * 128) >> 4) + 8 * u0;
+        p.y = s_hdr.row0[i] + 48 + 2 * W - 64 * u0;
+        p.z = (-W & 63) >> 3;
+        p.w = (4 * u1 < steps ? 4 * u1 : steps) - 4 * u0;
+        s_prod[z] = p;
+    }
+    bool tab_waited = false, staged = false;
     uint32_t phase = 0;
     const T *in = static_cast<const T *>(P.in);
     T *out = static_cast<T *>(P.out);
 
-    const long long edge_l = P.rows_l / kEdgeRows;  // whole blocks
-    const long long edges = edge_l + (P.n - P.row_r + kEdgeRows - 1) / kEdgeRows;
-    for (long long tile = blockIdx.x; tile < P.tiles + edges; tile += gridDim.x) {
+    for (long long tile = first; tile < P.tiles + edges; tile = after(tile)) {
         if (tile >= P.tiles) {
             // rows near a wall, after the tiles: they fill the last wave
+            double *s_w = reinterpret_cast<double *>(sm), *taps = s_w + kDotWin + kEdgeScratch;
             if (warp < kTileWarps) {
-                bulk_wait_read0();
-                asm volatile("bar.sync 1, %0;" ::"n"(kTileConv) : "memory");
+                if (!staged) {
+                    // the tables' and planes' space: nothing still writes or reads it
+                    bulk_wait_read0();
+                    if (has_tab)
+                        bar_drain(&tab_full, 0, kWaitLimitCycles);
+                    asm volatile("bar.sync 1, %0;" ::"n"(kTileConv) : "memory");
+                    dot_stage<kTileConv>(P, reinterpret_cast<typename PairOf<T>::E *>(taps));
+                    staged = true;
+                }
                 const long long x = tile - P.tiles;
-                const long long r0 = x < edge_l ? x * kEdgeRows : P.row_r + (x - edge_l) * kEdgeRows;
-                dot_rows<T, kTileConv, kEdgeRows>(P, s_dot, reinterpret_cast<double *>(xp), r0,
-                                                  r0 + kEdgeRows < P.n ? r0 + kEdgeRows : P.n);
+                const long long a = x < edge_l ? 0 : P.row_r, b = x < edge_l ? P.rows_l : P.n;
+                const long long r0 = a + (x < edge_l ? x : x - edge_l) * kEdgeRows - shift, r1 = r0 + kEdgeRows;
+                dot_rows<T, kTileConv, kEdgeRows, kEdgeParts, true>(P, s_dot, s_w, taps, r0 > a ? r0 : a, r1 < b ? r1 : b);
             }
             continue;
         }
@@ -880,7 +989,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                 }
             }
             // the next tile's window on its way to L2
-            if (tile + gridDim.x < P.tiles) {
+            if (!SPLIT && tile + gridDim.x < P.tiles) {
                 const long long nx = base + (long long)gridDim.x * kPropTileBlks * kPropBlk + (long long)t * 128 / sizeof(T);
                 for (long long z = nx; z < nx - (long long)t * 128 / sizeof(T) + (long long)chunks * 8 && z < P.n;
                      z += (long long)kTileConv * 128 / sizeof(T))
@@ -907,10 +1016,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
             // the rest of the cone: everything that reaches the tile's blocks in k steps
             int cmax = wmax;
             const long long clo = b0 * kPropBlk - P.k - 2, chi = (b0 + nb) * kPropBlk + P.k + 2;
-            for (long long j = (clo > 0 ? clo : 0) + t; j < base; j += kTileConv)
-                cmax = max(cmax, code_of(in[j]));
-            for (long long j = base + (long long)chunks * 8 + t; j < (chi < P.n ? chi : P.n); j += kTileConv)
-                cmax = max(cmax, code_of(in[j]));
+            auto scan = [&](long long a, long long b) {
+                for (long long j = a + t; j < b; j += 4 * kTileConv)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        cmax = max(cmax, code_of(j + u * kTileConv < b ? in[j + u * kTileConv] : (T)0));
+            };
+            scan(clo > 0 ? clo : 0, base);
+            scan(base + (long long)chunks * 8, chi < P.n ? chi : P.n);
             for (long long j = (P.n & ~7LL) + t; j < P.n && j < chi; j += kTileConv)  // the ragged end
                 cmax = max(cmax, code_of(in[j]));
             bulk_wait_read0();  // the last tile's rows have left the planes
@@ -922,15 +1035,16 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
             }
         }
         __syncthreads();
-        if (s_left)
+        // (a cluster's CTAs must agree, and have one tile only)
+        if (!SPLIT && s_left)
             break;
         const int ref = s_max[0], cone = s_max[1];
         if (t < nb) {
             const int q = s_code[hb + t];
             const bool listed = cone > 0 && (!ok_tab || cone == kCodeInf<T> || q < cone - S::kRange || q == 0);
-            if (listed)
+            if (listed && rank == 0)
                 P.list[atomicAdd(P.count, 1)] = (int)(b0 + t);
-            else if (cone > 0)
+            else if (!listed && cone > 0)
                 s_keep = 1;
         }
         if (warp < kTileWarps && cone != kCodeInf<T>) {
@@ -972,7 +1086,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
         __syncthreads();
         tc_fence_after();
         const bool keep = s_keep != 0;
-        if (warp == kTileWarps) {
+        if (warp >= kTileWarps) {
             if (keep) {
                 // the whole warp runs the loop, so descriptors stay in uniform
                 // registers; one lane issues
@@ -982,10 +1096,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                     ok = bar_wait(&tab_full, 0, kWaitLimitCycles, &s_abort);
                     tab_waited = true;
                 }
-                const uint32_t tab0 = saddr(sm), x0 = saddr(xp);
+                const uint64_t ad0 = swizzled_desc(saddr(xp)), bd0 = plain_desc(saddr(sm), 128);
 #pragma unroll 1
-                for (int g = 0; ok && g < S::kGroups; ++g) {
-                    const int w = G::weight(g), lo = G::lo(g), hi = G::hi(g);
+                for (int g = warp - kTileWarps; ok && g < S::kGroups; g += kMmaWarps) {
+                    const int lo = G::lo(g), hi = G::hi(g);
                     uint32_t acc = 0;
                     if (g * kPropBlk >= S::kCols) {
                         // sum 0's accumulator again, once the warps have read it
@@ -997,20 +1111,16 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                     const uint32_t dcol = tbase + (uint32_t)(g * kPropBlk % S::kCols);
 #pragma unroll 1
                     for (int i = lo; i <= hi; ++i) {
-                        const int W = __shfl_sync(0xffffffffu, s_hdr.W[i], 0);
-                        const int row0 = __shfl_sync(0xffffffffu, s_hdr.row0[i], 0);
-                        // window position -W: block -W >> 6, piece q of its row (descending, as the
-                        // table's rows run); four steps go 64 points on, to the next row
-                        const int q = (-W & 63) >> 3;
-                        uint64_t ad = swizzled_desc(x0 + (uint32_t)(((w - i) * C + hb + (-W >> 6)) * 128));
-                        uint64_t bd = plain_desc(tab0 + (uint32_t)(row0 + 48 + 2 * W) * 16, 128);
-                        const int steps = (kPropBlk + 2 * W) / 16;
+                        const int4 p = s_prod[g * ND + i];
+                        const int q = __shfl_sync(0xffffffffu, p.z, 0), end = __shfl_sync(0xffffffffu, p.w, 0);
+                        uint64_t ad = ad0 + (uint32_t)__shfl_sync(0xffffffffu, p.x, 0);
+                        uint64_t bd = bd0 + (uint32_t)__shfl_sync(0xffffffffu, p.y, 0);
                         const uint64_t a0 = (uint64_t)(6 - q), a1 = (uint64_t)(6 - ((q + 2) & 7) + ((q + 2) & 8)),
                                        a2 = (uint64_t)(6 - ((q + 4) & 7) + ((q + 4) & 8)),
                                        a3 = (uint64_t)(6 - ((q + 6) & 7) + ((q + 6) & 8));
                         int s = 0;
 #pragma unroll 1
-                        for (; s + 4 <= steps; s += 4) {
+                        for (; s + 4 <= end; s += 4) {
                             tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, acc);
                             tc_mma_if(leader, dcol, ad + a1, bd - 16, kIdescF16, 1);
                             tc_mma_if(leader, dcol, ad + a2, bd - 32, kIdescF16, 1);
@@ -1019,12 +1129,13 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                             ad += 8;
                             bd -= 64;
                         }
-                        if (s < steps) {
-                            tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, 1);
-                            if (s + 1 < steps)
+                        if (s < end) {
+                            tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, SPLIT ? acc : 1);
+                            if (s + 1 < end)
                                 tc_mma_if(leader, dcol, ad + a1, bd - 16, kIdescF16, 1);
-                            if (s + 2 < steps)
+                            if (s + 2 < end)
                                 tc_mma_if(leader, dcol, ad + a2, bd - 32, kIdescF16, 1);
+                            acc = 1;
                         }
                     }
                     if (lane == 0)
@@ -1043,7 +1154,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
             // units of the sums: weight 5 (FP32: 3), and up to 8 bits below
             // where the taps' scale leaves the 64-bit sum that room
             const int room = s_hdr.room, xs = sizeof(T) == 4 ? 0 : room < 8 ? room : 8;
-            long long acc[kTileCols];
+            long long acc[kTileCols], low[SPLIT && sizeof(T) == 8 ? kTileCols : 1];
 #pragma unroll
             for (int v = 0; v < kTileCols; ++v)
                 acc[v] = 0;
@@ -1063,10 +1174,18 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                             bar_arrive(&reuse);
                     }
                     const int w = G::weight(g);
+                    const bool mine = !SPLIT || ((s_used >> g) & 1);
 #pragma unroll
                     for (int q = 0; q < kTileCols; ++q) {
-                        const int z = __float2int_rn(__uint_as_float(v[q]));
-                        if (ND == kPropNd64)
+                        const int z = mine ? __float2int_rn(__uint_as_float(v[q])) : 0;
+                        if (SPLIT && ND == kPropNd64) {
+                            // weights 7 and 6 apart: their last bits are rounded off the whole sum
+                            if (w >= 6)
+                                low[SPLIT && sizeof(T) == 8 ? q : 0] =
+                                    w == 7 ? (long long)z : low[SPLIT && sizeof(T) == 8 ? q : 0] + ((long long)z << 8);
+                            else
+                                acc[q] += (long long)z << (8 * (5 - (w < 6 ? w : 5)) + xs);
+                        } else if (ND == kPropNd64)
                             acc[q] = w == 7   ? (long long)z
                                      : w == 6 ? ((acc[q] + ((long long)z << 8) + (0x8000 >> xs)) >> (16 - xs))
                                               : acc[q] + ((long long)z << (8 * (5 - (w < 6 ? w : 5)) + xs));
@@ -1079,6 +1198,17 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                 if (lane == 0) {
                     atomicExch(P.err, kDevTimeout);
                     s_abort = 1;
+                }
+            } else if (SPLIT) {
+#pragma unroll
+                for (int v = 0; v < kTileCols; ++v) {
+                    const int at = (col + v) * kPropTileBlks + row;
+                    if (sizeof(T) == 8) {
+                        const long long l = low[SPLIT && sizeof(T) == 8 ? v : 0];
+                        acc[v] += l >> (16 - xs);
+                        reinterpret_cast<unsigned short *>(sm + kPartHigh)[at] = (unsigned short)(l & ((1 << (16 - xs)) - 1));
+                    }
+                    reinterpret_cast<long long *>(sm)[at] = acc[v];
                 }
             } else if (row < nb) {
                 // out = acc 2^x: FP64 x = e + 2 - E - xs, FP32 x = e - 6 - E, 2^e above the tile's largest value
@@ -1101,21 +1231,60 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                         reinterpret_cast<volatile T *>(o)[v] = (T)acc[v] * s1 * s2;
                 }
             }
-            // every row by one bulk copy (a row per thread storing 16-byte
-            // pieces: 15000 cycles a tile)
-            fence_async_smem();
-            asm volatile("bar.sync 1, %0;" ::"n"(kTileConv) : "memory");
-            if (t < nb && !s_abort) {
-                bulk_store(out + (b0 + t) * kPropBlk, xp + t * kStageRow<T>, kPropBlk * (uint32_t)sizeof(T));
-                bulk_commit();
+            if (!SPLIT) {
+                // every row by one bulk copy (a row per thread storing 16-byte
+                // pieces: 15000 cycles a tile)
+                fence_async_smem();
+                asm volatile("bar.sync 1, %0;" ::"n"(kTileConv) : "memory");
+                if (t < nb && !s_abort) {
+                    bulk_store(out + (b0 + t) * kPropBlk, xp + t * kStageRow<T>, kPropBlk * (uint32_t)sizeof(T));
+                    bulk_commit();
+                }
             }
-        } else if (cone == 0) {
+        } else if (cone == 0 && rank == 0) {
             const int row = (warp & 3) * 32 + lane, col = (warp >> 2) * kTileCols;
             if (row < nb) {
                 T *o = out + (b0 + row) * kPropBlk + col;
                 for (int v = 0; v < kTileCols; ++v)
                     o[v] = (T)0;
             }
+        }
+        if (SPLIT) {
+            __syncwarp();
+            cluster_sync();
+            if (keep && warp < kTileWarps) {
+                const int share = kPropBlk / ctas, room = s_hdr.room, xs = sizeof(T) == 4 ? 0 : room < 8 ? room : 8;
+                const int ex = sizeof(T) == 8 ? ref - 1022 + 2 - s_hdr.E - xs : ref - 126 - 6 - s_hdr.E;
+                const bool plain = sizeof(T) == 8 ? ex >= -1021 && ex <= 959 : ex >= -125 && ex <= 63;
+                const T s1 = pow2<T>(ex / 2), s2 = pow2<T>(ex - ex / 2);
+                // a warp reads 32 blocks' sums of one point (contiguous: reads
+                // from another CTA's memory cost by the piece)
+#pragma unroll 2
+                for (int u = t; u < share * kPropTileBlks; u += kTileConv) {
+                    const int row = u % kPropTileBlks, col = rank * share + u / kPropTileBlks;
+                    if (row >= nb)
+                        continue;
+                    const uint32_t cell = (uint32_t)(col * kPropTileBlks + row), at = saddr(sm) + cell * 8,
+                                   at_low = saddr(sm) + kPartHigh + cell * 2;
+                    long long z;
+                    int low;
+                    if (ctas == 2)
+                        add_parts<T, 2>(at, at_low, z, low);
+                    else if (ctas == 4)
+                        add_parts<T, 4>(at, at_low, z, low);
+                    else
+                        add_parts<T, 8>(at, at_low, z, low);
+                    if (sizeof(T) == 8)
+                        z += (low + (0x8000 >> xs)) >> (16 - xs);
+                    T *o = out + (b0 + row) * kPropBlk + col;
+                    if (plain)
+                        *o = from_fixed<T>(z, ex);
+                    else
+                        *reinterpret_cast<volatile T *>(o) = (T)z * s1 * s2;
+                }
+            }
+            __syncwarp();
+            cluster_sync();
         }
         if (keep)
             phase ^= 1;
@@ -1127,10 +1296,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
     }
     bulk_wait0();
     // the table's copy and MMAs in flight end before the CTA does
-    if (t == 0 && ok_tab)
+    if (t == 0 && has_tab)
         bar_drain(&tab_full, 0, kWaitLimitCycles);
-    if (s_abort && t == 0)
-        bar_drain(&done[S::kGroups - 1], phase ^ 1, kWaitLimitCycles);
+    if (s_abort && t < kMmaWarps)
+        bar_drain(&done[S::kGroups - 1 - t], phase ^ 1, kWaitLimitCycles);
     __syncthreads();
     if (warp == kTileWarps)
         tmem_dealloc(tbase, S::kCols);
@@ -1152,19 +1321,23 @@ cudaError_t prop_prepare()
     if (dev < 256 && (ready[dev >> 6] >> (dev & 63)) & 1)
         return cudaSuccess;
     cudaFuncAttributes fa;
-    e = cudaFuncSetAttribute(prop_tile_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kTileSmem<double>);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(prop_tile_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kTileSmem<float>);
+    auto smem = [&](auto *f, int bytes) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    smem(prop_tile_kernel<double, false>, kTileSmem<double>);
+    smem(prop_tile_kernel<double, true>, kTileSmem<double>);
+    smem(prop_tile_kernel<float, false>, kTileSmem<float>);
+    smem(prop_tile_kernel<float, true>, kTileSmem<float>);
+    smem(prop_dot_kernel<double>, (kDotWin + dot_taps(kPropRMax)) * 8);
+    smem(prop_dot_kernel<float>, (kDotWin + dot_taps(kPropRMax)) * 8);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(prop_digits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  2 * kPropQ * 8);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(prop_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (7 * kPropRMax + 11 * kLevelPad + 8) * 8);
-    const void *rest[] = {(const void *)prop_short_kernel, (const void *)prop_finish_kernel,
-                          (const void *)prop_dot_kernel<double>, (const void *)prop_dot_kernel<float>};
+    const void *rest[] = {(const void *)prop_short_kernel, (const void *)prop_finish_kernel};
     for (const void *f : rest)
         if (e == cudaSuccess)
             e = cudaFuncGetAttributes(&fa, f);
@@ -1205,21 +1378,108 @@ cudaError_t prop_launch_digits(const PropSet &set, const PropFinish &f, int R, i
     return cudaGetLastError();
 }
 
-cudaError_t prop_launch_tiles(const PropRun &a, int f64, int grid, cudaStream_t s)
+// Clusters of 2, 4 and 8 CTAs the device holds at once (a cluster lies within
+// one group of SMs), asked once per device.
+static cudaError_t split_clusters(int f64, int ctas, int *clusters)
 {
+    static std::mutex lock;
+    static int known[64][2][9];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess)
+        return e;
+    std::lock_guard<std::mutex> hold(lock);
+    int *k = dev < 64 ? &known[dev][f64 ? 1 : 0][ctas] : nullptr;
+    if (k && *k) {
+        *clusters = *k - 1;
+        return cudaSuccess;
+    }
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)ctas);
+    c.blockDim = dim3(kTileThreads);
+    c.dynamicSmemBytes = (size_t)(f64 ? kTileSmem<double> : kTileSmem<float>);
+    c.attrs = &at;
+    c.numAttrs = 1;
+    e = f64 ? cudaOccupancyMaxActiveClusters(clusters, prop_tile_kernel<double, true>, &c)
+            : cudaOccupancyMaxActiveClusters(clusters, prop_tile_kernel<float, true>, &c);
+    if (e == cudaSuccess && k)
+        *k = *clusters + 1;
+    return e;
+}
+
+cudaError_t prop_launch_tiles(PropRun a, int f64, int num_sms, cudaStream_t s)
+{
+    const int shift = item_shift(a);
+    const long long edges = item_count(a.rows_l, kEdgeRows, shift) + item_count(a.n - a.row_r, kEdgeRows, shift);
+    // Fewer tiles than SMs: the cluster size, and the rounds of wall rows for
+    // the CTAs without a tile, that should be done first, in cycles (measured
+    // on this device: loading and converting a tile, an MMA, finishing it, an
+    // item of wall rows; a digit's reach is on average 0.62 of the halo).
+    int best = 1, split_grid = 0;
+    const double mmas = (f64 ? 34.0 : 10.0) * (4 + 5 * a.hb), start = f64 ? 15500 : 11000;
+    const double item = f64 ? 7000 + 16.0 * a.R : 6500 + 6.0 * a.R;
+    if (a.tiles < num_sms) {
+        const double rounds = std::ceil((double)edges / (double)(num_sms - a.tiles));
+        double least = std::max(start + 50 * mmas + 6000, 4000 + rounds * item);
+        for (int ctas = 2; ctas <= 8 && a.tiles * ctas <= num_sms; ctas *= 2) {
+            int clusters = 0;
+            cudaError_t e = split_clusters(f64, ctas, &clusters);
+            if (e != cudaSuccess)
+                return e;
+            if (a.tiles > clusters)
+                break;
+            const int grid = (int)std::min<long long>(clusters, a.tiles + (edges + ctas - 1) / ctas) * ctas;
+            const int spare = grid - (int)a.tiles * ctas;
+            const double tile = start + 60 * mmas / ctas + 11000;
+            const int all = spare > 0 ? (int)((edges + spare - 1) / spare) : 0;
+            const int under = spare > 0 ? std::min(all, (int)((tile - 4000) / item)) : 0;
+            for (int r : {under, all}) {
+                const long long left = std::max(0LL, edges - (long long)r * spare);
+                const double total = std::max(tile, 4000 + r * item) + (double)((left + grid - 1) / grid) * (item + 4000);
+                if (total < least) {
+                    least = total;
+                    best = ctas;
+                    a.edge_rounds = r;
+                    a.split = ctas;
+                    split_grid = grid;
+                }
+            }
+        }
+    }
+    if (best > 1) {
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)best;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cudaLaunchConfig_t c{};
+        c.gridDim = dim3((unsigned)split_grid);
+        c.blockDim = dim3(kTileThreads);
+        c.dynamicSmemBytes = (size_t)(f64 ? kTileSmem<double> : kTileSmem<float>);
+        c.stream = s;
+        c.attrs = &at;
+        c.numAttrs = 1;
+        return f64 ? cudaLaunchKernelEx(&c, prop_tile_kernel<double, true>, a)
+                   : cudaLaunchKernelEx(&c, prop_tile_kernel<float, true>, a);
+    }
+    const int grid = (int)(a.tiles + edges < num_sms ? a.tiles + edges : num_sms);
     if (f64)
-        prop_tile_kernel<double><<<grid, kTileThreads, kTileSmem<double>, s>>>(a);
+        prop_tile_kernel<double, false><<<grid, kTileThreads, kTileSmem<double>, s>>>(a);
     else
-        prop_tile_kernel<float><<<grid, kTileThreads, kTileSmem<float>, s>>>(a);
+        prop_tile_kernel<float, false><<<grid, kTileThreads, kTileSmem<float>, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t prop_launch_dots(const PropRun &a, int f64, int grid, cudaStream_t s)
 {
+    const size_t bytes = (size_t)(kDotWin + dot_taps(a.R)) * 8;
     if (f64)
-        prop_dot_kernel<double><<<grid, 256, 0, s>>>(a);
+        prop_dot_kernel<double><<<grid, 256, bytes, s>>>(a);
     else
-        prop_dot_kernel<float><<<grid, 256, 0, s>>>(a);
+        prop_dot_kernel<float><<<grid, 256, bytes, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -112,6 +112,8 @@ struct PropRun {
     long long rows_l, row_r;
     int *list, *count, *count_next;
     int gate_min;      // more listed blocks than this: left to the step-by-step form
+    int split;         // CTAs per tile, and items of wall rows for each CTA without one (set by the launcher)
+    int edge_rounds;
     int *zero[3];      // words the tiles clear for it: barrier, two tile queues
 };
 
@@ -146,7 +148,7 @@ cudaError_t prop_launch_short(double *e, double *el, double *h, double *hl, int 
 cudaError_t prop_launch_level(const PropLevel &a, cudaStream_t s);
 cudaError_t prop_launch_finish(const PropLevel &a, const PropFinish &f, cudaStream_t s);
 cudaError_t prop_launch_digits(const PropSet &set, const PropFinish &f, int R, int f64, int hb_max, cudaStream_t s);
-cudaError_t prop_launch_tiles(const PropRun &a, int f64, int grid, cudaStream_t s);
+cudaError_t prop_launch_tiles(PropRun a, int f64, int num_sms, cudaStream_t s);
 cudaError_t prop_launch_dots(const PropRun &a, int f64, int grid, cudaStream_t s);
 cudaError_t prop_prepare();  // per-device kernel attributes
 

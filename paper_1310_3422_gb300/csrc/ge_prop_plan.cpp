@@ -384,8 +384,6 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
             a.tiles = (a.blk1 - a.blk0 + kPropTileBlks - 1) / kPropTileBlks;
             a.rows_l = a.blk0 * kPropBlk;
             a.row_r = a.blk1 * kPropBlk;
-            const long long edges = a.rows_l / 16 + (t.n - a.row_r + 15) / 16;
-            const int grid = (int)std::min<long long>(a.tiles + edges, t.num_sms);
             // listed blocks past which the whole grid step by step is sooner
             // done than their dot products: a block's 64 rows of 2 R taps at
             // 2e11 multiply-adds a second, against the tiled kernel's rate
@@ -404,7 +402,7 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
             } else {
                 a.gate_min = 2000000000;
             }
-            if ((e = prop_launch_tiles(a, t.f64, grid, stream)) != cudaSuccess)
+            if ((e = prop_launch_tiles(a, t.f64, t.num_sms, stream)) != cudaSuccess)
                 return e;
             if (gated) {
                 if ((e = launch_tb_rounds(t.prec, t.tiled.tmap[*cur], t.tiled.tmap[*cur ^ 1], st->rounds, a,
@@ -417,7 +415,7 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
         } else {
             a.rows_l = t.n;
             a.row_r = t.n;
-            items = (t.n + 7) / 8;
+            items = t.n / 8 + 1;
         }
         const int grid = (int)std::min<long long>(items, 8LL * t.num_sms);
         if ((e = prop_launch_dots(a, t.f64, grid, stream)) != cudaSuccess)

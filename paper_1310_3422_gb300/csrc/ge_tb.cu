@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(Layout<Real, COMP>::NT, Layout<Real, COMP>::MI
         __shared__ DotShared<kDotRows> dots;
         static_assert(kDotWin * 8 <= 2 * kTileRows * kRowBytes, "the window fits the tile buffers");
         for (long long it = blockIdx.x; it < (long long)listed * (kPropBlk / kDotRows); it += gridDim.x)
-            dot_listed<Real, Layout<Real, COMP>::NT>(D, dots, reinterpret_cast<double *>(smem_raw), it);
+            dot_listed<Real, Layout<Real, COMP>::NT>(D, dots, reinterpret_cast<double *>(smem_raw), nullptr, it);
         return;
     }
     __shared__ __align__(8) TbShared<Real, Layout<Real, COMP>::NT / 32> sh;

@@ -142,3 +142,37 @@ def test_captured_graph_and_later_direct_calls():
             assert rel_max(out.cpu().numpy(), want) <= tol64(r), steps
         del graph
     torch.cuda.synchronize()
+
+
+# 2, 11, 30, 70 and 75 tiles: clusters of 8, 8, 4, 2 and 2 CTAs a tile, where
+# the device holds that many; 97 tiles in the larger grid: one CTA each
+@pytest.mark.parametrize("n", [20000, 93001, 249990, 580003, 619000])
+@pytest.mark.parametrize("r,steps", [(0.01, 21), (0.7, 300), (0.7, 2000)])
+@pytest.mark.parametrize("prec", [B.GE_F64, B.GE_F32, B.GE_F32_COMP])
+def test_split_tiles_give_the_same_bits(n, r, steps, prec):
+    """Integer sums split over a cluster are the unsplit ones: the start of a
+    larger grid, whose tiles are not split, gives the same bits away from the
+    smaller grid's right wall (a tile and its halo, at most 16 blocks)."""
+    if prec != B.GE_F64:
+        steps = max(steps, 150)  # fewer go step by step, from 128 + n 192 / 2^24
+    u0 = inputs.random_state(800000, seed=3)
+    want = auto_run(u0, r, 0.3, -0.8, steps, prec)
+    got = auto_run(u0[:n], r, 0.3, -0.8, steps, prec)
+    m = n - 8192 - 17 * 64
+    assert np.array_equal(got[:m], want[:m])
+    assert np.all(np.isfinite(got))
+
+
+# an FP32 row's sum runs in FP32 between 2^-70 and 2^90, else in FP64; above
+# 8192 points these are the rows near a wall
+@pytest.mark.parametrize("n", [1000, 9281])
+@pytest.mark.parametrize("exp", [-100, -71, -69, 88, 91, 100])
+def test_fp32_rows_at_any_magnitude(n, exp):
+    """The scheme is linear: data and walls times 2^exp give the result times
+    2^exp, within the FP32 tolerance."""
+    r, steps = 0.7, 300
+    u0 = inputs.random_state(n, seed=exp + 200).astype(np.float32).astype(np.float64)
+    want = oracle.run(u0, r, 0.25, -0.75, steps, 0)
+    s = 2.0 ** exp
+    got = auto_run(u0 * s, r, 0.25 * s, -0.75 * s, steps, B.GE_F32)
+    assert rel_max(got / s, want) <= 1e-5
