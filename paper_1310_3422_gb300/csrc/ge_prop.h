@@ -162,8 +162,9 @@ void prop_carve(PropState *st, void *mem, long long n, int f64);
 // (prec as in tb_run).
 bool prop_takes(long long n, double r, long long steps, int prec);
 // Advance `steps` steps; *cur as in tb_run.  *taken = 0: nothing done (every
-// operator slot belongs to a captured graph).
+// operator slot belongs to a captured graph).  build_only: put the operators
+// on the stream, and nothing else.
 cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long step0, long long steps, int *taken,
-                     cudaStream_t s);
+                     cudaStream_t s, bool build_only = false);
 
 }  // namespace ge

@@ -253,7 +253,7 @@ cudaError_t build_set(PropState *st, const PropTarget &t, PropSet &s, int pr, in
 }  // namespace
 
 cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long step0, long long steps, int *taken,
-                     cudaStream_t stream)
+                     cudaStream_t stream, bool build_only)
 {
     *taken = 0;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -342,6 +342,8 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
             w.set->valid = 1;
     }
     *taken = 1;
+    if (build_only)
+        return cudaSuccess;
     if ((e = cudaMemsetAsync(st->count, 0, 2 * sizeof(int), stream)) != cudaSuccess)
         return e;
     for (long long i = 0; i <= full; ++i) {
