@@ -783,6 +783,97 @@ __device__ __forceinline__ uint64_t plain_desc(uint32_t addr, uint32_t lead)
 // kind::f16 with FP16 operands and FP32 accumulators, M = 128, N = 64.
 constexpr uint32_t kIdescF16 = (1u << 4) | ((uint32_t)(kPropBlk >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 
+// Eight values as digits, one 16-byte piece of each plane.
+template <typename T>
+__device__ __forceinline__ void convert8(const T (&x)[8], int ref, unsigned char *dst, size_t plane)
+{
+    constexpr int ND = TileShape<T>::ND;
+    uint32_t lo[8], hi[8];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        if (ND == kPropNd64) {
+            const unsigned long long y = (unsigned long long)to_fixed((double)x[v], ref) + 0x0080808080808080ull;
+            lo[v] = (uint32_t)y;
+            hi[v] = (uint32_t)(y >> 32);
+        } else {
+            lo[v] = (uint32_t)to_fixed((float)x[v], ref) + 0x80808080u;
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        const int byte = ND - 1 - d;
+        const uint32_t sel = byte < 4 ? (uint32_t)(byte | (byte << 4) | ((byte + 4) << 8) | ((byte + 4) << 12))
+                                      : (uint32_t)((byte - 4) | ((byte - 4) << 4) | (byte << 8) | (byte << 12));
+        uint4 q;
+        q.x = byte < 4 ? half_pair(lo[0], lo[1], sel) : half_pair(hi[0], hi[1], sel);
+        q.y = byte < 4 ? half_pair(lo[2], lo[3], sel) : half_pair(hi[2], hi[3], sel);
+        q.z = byte < 4 ? half_pair(lo[4], lo[5], sel) : half_pair(hi[4], hi[5], sel);
+        q.w = byte < 4 ? half_pair(lo[6], lo[7], sel) : half_pair(hi[6], hi[7], sel);
+        *reinterpret_cast<uint4 *>(dst + (size_t)d * plane) = q;
+    }
+}
+
+// One sum's value into a point's 64-bit accumulator (weight w; units: see the drain).
+template <typename T>
+__device__ __forceinline__ long long fold(long long acc, int w, int z, int xs)
+{
+    if (sizeof(T) == 8)
+        return w == 7   ? (long long)z
+               : w == 6 ? ((acc + ((long long)z << 8) + (0x8000 >> xs)) >> (16 - xs))
+                        : acc + ((long long)z << (8 * (5 - (w < 6 ? w : 5)) + xs));
+    return acc + ((long long)z << (8 * (3 - (w < 4 ? w : 3))));
+}
+
+// N finished points of a row to the staging buffer: out = acc 2^ex.
+template <typename T, int N>
+__device__ __forceinline__ void finish_row(const long long (&acc)[N], int ex, unsigned char *o)
+{
+    const bool plain = sizeof(T) == 8 ? ex >= -1021 && ex <= 959 : ex >= -125 && ex <= 63;
+    if (plain) {
+#pragma unroll
+        for (int v = 0; v < N; v += 16 / sizeof(T)) {
+            T y[16 / sizeof(T)];
+#pragma unroll
+            for (int z = 0; z < (int)(16 / sizeof(T)); ++z)
+                y[z] = from_fixed<T>(acc[v + z], ex);
+            *reinterpret_cast<uint4 *>(o + v * sizeof(T)) = *reinterpret_cast<const uint4 *>(y);
+        }
+    } else {  // near the ends of the exponent range
+        const T s1 = pow2<T>(ex / 2), s2 = pow2<T>(ex - ex / 2);
+#pragma unroll
+        for (int v = 0; v < N; ++v)
+            reinterpret_cast<volatile T *>(o)[v] = (T)acc[v] * s1 * s2;
+    }
+}
+
+// The four MMAs of 64 points of a window, `end` steps of 16 in all: ad, bd at
+// the first step, q the window's first piece of its row.
+__device__ __forceinline__ void issue_product(bool leader, uint32_t dcol, uint64_t ad, uint64_t bd, int q, int end,
+                                              uint32_t &acc)
+{
+    const uint64_t a0 = (uint64_t)(6 - q), a1 = (uint64_t)(6 - ((q + 2) & 7) + ((q + 2) & 8)),
+                   a2 = (uint64_t)(6 - ((q + 4) & 7) + ((q + 4) & 8)), a3 = (uint64_t)(6 - ((q + 6) & 7) + ((q + 6) & 8));
+    int s = 0;
+#pragma unroll 1
+    for (; s + 4 <= end; s += 4) {
+        tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, acc);
+        tc_mma_if(leader, dcol, ad + a1, bd - 16, kIdescF16, 1);
+        tc_mma_if(leader, dcol, ad + a2, bd - 32, kIdescF16, 1);
+        tc_mma_if(leader, dcol, ad + a3, bd - 48, kIdescF16, 1);
+        acc = 1;
+        ad += 8;
+        bd -= 64;
+    }
+    if (s < end) {
+        tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, acc);
+        if (s + 1 < end)
+            tc_mma_if(leader, dcol, ad + a1, bd - 16, kIdescF16, 1);
+        if (s + 2 < end)
+            tc_mma_if(leader, dcol, ad + a2, bd - 32, kIdescF16, 1);
+        acc = 1;
+    }
+}
+
 // 16 warps that convert and drain: chains of integer instructions with little
 // else to hide their latency.  2 that issue the MMAs, every other sum each:
 // one warp issues one in 54 cycles, and spends 200 to 300 between two digit
@@ -882,23 +973,24 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
     if (blockIdx.x == 0 && t < 3 && P.zero[t])
         *P.zero[t] = 0;
     const int ctas = SPLIT ? P.split : 1, lg = SPLIT ? 31 - __clz(ctas) : 0, rank = SPLIT ? (int)blockIdx.x & (ctas - 1) : 0;
-    // split: a tile per cluster; the CTAs without one start with the rows near
-    // a wall (edge_rounds items each), and what is left is everyone's
-    const int spare = SPLIT ? (int)gridDim.x - (int)P.tiles * ctas : 0, me = SPLIT ? (int)blockIdx.x - (int)P.tiles * ctas : 0;
+    // Tiles (split: one per cluster), then the rows near a wall: the CTAs with
+    // a tile less (split: without one) take edge_rounds items each, and what
+    // is left is everyone's.
+    const int busy = SPLIT ? (int)P.tiles * ctas : (int)(P.tiles % gridDim.x);  // CTAs with a tile more
+    const int spare = busy ? (int)gridDim.x - busy : 0, me = (int)blockIdx.x - busy;
     const int shift = item_shift(P);
     const long long edge_l = item_count(P.rows_l, kEdgeRows, shift);
     const long long edges = edge_l + item_count(P.n - P.row_r, kEdgeRows, shift);
-    const long long early = SPLIT ? ((long long)spare * P.edge_rounds < edges ? (long long)spare * P.edge_rounds : edges) : 0;
-    const long long first = !SPLIT ? (long long)blockIdx.x
-                            : me < 0 ? (long long)blockIdx.x >> lg
-                            : me < early ? P.tiles + me
-                                         : P.tiles + early + blockIdx.x;
+    const long long early = (long long)spare * P.edge_rounds < edges ? (long long)spare * P.edge_rounds : edges;
+    const long long first_edge = spare > 0 && me >= 0 && me < early ? P.tiles + me : P.tiles + early + blockIdx.x;
+    const long long first = SPLIT ? (me < 0 ? (long long)blockIdx.x >> lg : first_edge)
+                                  : ((long long)blockIdx.x < P.tiles ? (long long)blockIdx.x : first_edge);
     auto after = [&](long long x) {
-        if (!SPLIT || x >= P.tiles + early)
-            return x + (long long)gridDim.x;
-        if (x >= P.tiles && x + spare < P.tiles + early)
-            return x + spare;
-        return P.tiles + early + (long long)blockIdx.x;
+        if (x < P.tiles)
+            return !SPLIT && x + gridDim.x < P.tiles ? x + (long long)gridDim.x : first_edge;
+        if (x < P.tiles + early)
+            return x + spare < P.tiles + early ? x + spare : P.tiles + early + (long long)blockIdx.x;
+        return x + (long long)gridDim.x;
     };
     const int hb = P.hb, ok_tab = s_hdr.ok && s_hdr.rows * 16 <= S::kTab;
     const bool has_tab = ok_tab && first < P.tiles;
@@ -1054,30 +1146,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                 if (u < chunks) {
                     // biased fixed-point values: every byte is a digit + 128
                     unsigned char *dst = xp + (u >> 3) * 128 + ((7 - (u & 7)) ^ ((u >> 3) & 7)) * 16;
-                    uint32_t lo[8], hi[8];
-#pragma unroll
-                    for (int v = 0; v < 8; ++v) {
-                        if (ND == kPropNd64) {
-                            const unsigned long long y =
-                                (unsigned long long)to_fixed((double)x[c][v], ref) + 0x0080808080808080ull;
-                            lo[v] = (uint32_t)y;
-                            hi[v] = (uint32_t)(y >> 32);
-                        } else {
-                            lo[v] = (uint32_t)to_fixed((float)x[c][v], ref) + 0x80808080u;
-                        }
-                    }
-#pragma unroll
-                    for (int d = 0; d < ND; ++d) {
-                        const int byte = ND - 1 - d;
-                        const uint32_t sel = byte < 4 ? (uint32_t)(byte | (byte << 4) | ((byte + 4) << 8) | ((byte + 4) << 12))
-                                                      : (uint32_t)((byte - 4) | ((byte - 4) << 4) | (byte << 8) | (byte << 12));
-                        uint4 q;
-                        q.x = byte < 4 ? half_pair(lo[0], lo[1], sel) : half_pair(hi[0], hi[1], sel);
-                        q.y = byte < 4 ? half_pair(lo[2], lo[3], sel) : half_pair(hi[2], hi[3], sel);
-                        q.z = byte < 4 ? half_pair(lo[4], lo[5], sel) : half_pair(hi[4], hi[5], sel);
-                        q.w = byte < 4 ? half_pair(lo[6], lo[7], sel) : half_pair(hi[6], hi[7], sel);
-                        *reinterpret_cast<uint4 *>(dst + (size_t)d * C * 128) = q;
-                    }
+                    convert8(x[c], ref, dst, (size_t)C * 128);
                 }
             }
         }
@@ -1305,6 +1374,383 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
         tmem_dealloc(tbase, S::kCols);
 }
 
+// ---- two teams -------------------------------------------------------------
+
+// Large grids whose taps reach a few blocks only: the table and the planes of
+// two tiles fit shared memory, and two teams of eight warps and an issuing
+// warp each take a tile of their own, so that one team's MMAs run under the
+// other's loads, conversion and drain (in prop_tile_kernel, where a tile's
+// planes fill shared memory, these take 18,000 cycles a tile during which the
+// tensor cores idle).  FP32 teams issue in turn; FP64's few MMAs need not.  A
+// team has 256 of the 512 columns: four accumulators,
+// a ring that its sums go round.  Tiles of as many blocks as fit, up to 128
+// (of the MMA's 128 rows the others are not used).  2^24 FP32 points, 2000
+// steps: 387 -> 312 us a call; 2^22 FP64 points, 24 steps: 110 -> 100 us.
+constexpr int kTeamWarps = 8, kTeam = 32 * kTeamWarps, kRing = 4;
+constexpr int kDuoHb64 = 2, kDuoHb32 = 11;  // widest halo
+constexpr int kDuoSmem = 232448 - 4096;  // static shared memory: below 4 KB
+constexpr int kTeamCols = kPropBlk / (kTeamWarps / 4);
+// Rows of a plane, and blocks of a tile, with `tab` bytes of tables: the MMA
+// reads 128 rows whatever the tile, also past the last plane's end.
+template <typename T>
+__host__ __device__ __forceinline__ int duo_rows(int tab, int hb)
+{
+    constexpr int ND = TileShape<T>::ND;
+    const int need = 128 + 2 * hb, left = kDuoSmem - 1024 - ((tab + 1023) & ~1023);
+    // (rows in eights: a swizzled plane starts on 1024 bytes)
+    const int rows = (left - (need + 7) * 128) / ((2 * ND - 1) * 128);
+    return (rows < need ? rows & ~7 : (need + 7) & ~7);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_constant__ PropRun P)
+{
+    using S = TileShape<T>;
+    using G = typename GroupsOf<T>::G;
+    constexpr int ND = S::ND, NG = S::kGroups;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                          ~static_cast<uintptr_t>(1023));
+    __shared__ __align__(8) uint64_t tab_full, full[2], done[2][NG], reuse[2][kRing];
+    __shared__ uint32_t tmem_sh;
+    __shared__ volatile int s_abort, s_stop[2];
+    __shared__ int s_code[2][kPropTileBlks + 2 * S::kHb + 8];
+    __shared__ int s_max[2][2], s_keep[2], s_left[2], s_turn;
+    __shared__ PropHeader s_hdr;
+    __shared__ DotShared<kEdgeRows> s_dot;
+    __shared__ int4 s_prod[NG * ND];
+
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    if (t < (int)(sizeof(PropHeader) / 4))
+        reinterpret_cast<int *>(&s_hdr)[t] = reinterpret_cast<const int *>(P.hdr)[t];
+    if (t == 0) {
+        bar_init(&tab_full, 1);
+        for (int m = 0; m < 2; ++m) {
+            bar_init(&full[m], kTeamWarps);
+            for (int g = 0; g < NG; ++g)
+                bar_init(&done[m][g], 1);
+            for (int g = 0; g < kRing; ++g)
+                bar_init(&reuse[m][g], kTeamWarps);
+            s_stop[m] = 0;
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_abort = 0;
+        s_turn = 0;
+    }
+    if (warp == kTileWarps) {
+        tmem_alloc(&tmem_sh, 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = tmem_sh;
+    if (blockIdx.x == 0 && t < 3 && P.zero[t])
+        *P.zero[t] = 0;
+    const int hb = P.hb, tab_bytes = s_hdr.rows * 16;
+    // (a table the tiles cannot hold: by the plan's rule there is none, and
+    // every block would take dot products)
+    const bool ok_tab = s_hdr.ok && tab_bytes <= S::kTab && duo_rows<T>(tab_bytes, hb) > 2 * hb;
+    const int C = ok_tab ? duo_rows<T>(tab_bytes, hb) : 64 + 2 * hb;
+    const int per = C - 2 * hb < kPropTileBlks ? C - 2 * hb : kPropTileBlks;  // blocks of a tile
+    const long long tiles = (P.blk1 - P.blk0 + per - 1) / per;
+    if (t == 0 && ok_tab) {
+        bar_expect_tx(&tab_full, (uint32_t)tab_bytes);
+        bulk_load(sm, P.tab, (uint32_t)tab_bytes, &tab_full);
+    }
+    // the digit products' first descriptors and steps, in issue order
+    for (int z = t; z < NG * ND; z += kTileThreads) {
+        const int g = z / ND, i = z % ND;
+        if (i < G::lo(g) || i > G::hi(g))
+            continue;
+        const int W = s_hdr.W[i];
+        int4 p;
+        p.x = (((G::weight(g) - i) * C + hb + (-W >> 6)) * 128) >> 4;
+        p.y = s_hdr.row0[i] + 48 + 2 * W;
+        p.z = (-W & 63) >> 3;
+        p.w = (kPropBlk + 2 * W) / 16;
+        s_prod[z] = p;
+    }
+    __syncthreads();
+    unsigned char *planes = sm + ((tab_bytes + 1023) & ~1023);
+    const T *in = static_cast<const T *>(P.in);
+    T *out = static_cast<T *>(P.out);
+
+    if (warp >= kTileWarps) {
+        // ---- issuing warp of team m ------------------------------------------
+        const int m = warp - kTileWarps;
+        const bool leader = elect_one();
+        bool ok = true, tab_waited = false;
+        const uint64_t ad0 = swizzled_desc(saddr(planes + (size_t)m * ND * C * 128)), bd0 = plain_desc(saddr(sm), 128);
+        int committed = -1;
+        for (uint32_t n = 0; ok; ++n) {  // n: the team's tiles so far
+            ok = __all_sync(0xffffffffu, bar_wait(&full[m], n & 1, kWaitLimitCycles, &s_abort));
+            if (!ok || s_stop[m])
+                break;
+            // one team's MMAs at a time: side by side, both would take twice as
+            // long, and then convert and drain side by side too
+            if (sizeof(T) == 4 && lane == 0) {
+                const long long t0 = clock64();
+                while (atomicCAS(&s_turn, 0, 1) != 0 && !s_abort && clock64() - t0 < kWaitLimitCycles)
+                    __nanosleep(40);
+            }
+            __syncwarp();
+            tc_fence_after();
+            if (!tab_waited) {
+                ok = __all_sync(0xffffffffu, bar_wait(&tab_full, 0, kWaitLimitCycles, &s_abort));
+                tab_waited = true;
+            }
+#pragma unroll 1
+            for (int g = 0; ok && g < NG; ++g) {
+                const int slot = g % kRing;
+                // uses of the slot before this one: each must have been read
+                const uint32_t uses = n * ((NG - slot + kRing - 1) / kRing) + g / kRing;
+                if (uses > 0) {
+                    ok = __all_sync(0xffffffffu, bar_wait(&reuse[m][slot], (uses - 1) & 1, kWaitLimitCycles, &s_abort));
+                    tc_fence_after();
+                    if (!ok)
+                        break;
+                }
+                const int lo = G::lo(g), hi = G::hi(g);
+                uint32_t acc = 0;
+                const uint32_t dcol = tbase + (uint32_t)(m * 256 + slot * kPropBlk);
+#pragma unroll 1
+                for (int i = lo; i <= hi; ++i) {
+                    const int4 p = s_prod[g * ND + i];
+                    issue_product(leader, dcol, ad0 + (uint32_t)__shfl_sync(0xffffffffu, p.x, 0),
+                                  bd0 + (uint32_t)__shfl_sync(0xffffffffu, p.y, 0), __shfl_sync(0xffffffffu, p.z, 0),
+                                  __shfl_sync(0xffffffffu, p.w, 0), acc);
+                }
+                if (lane == 0)
+                    tc_commit(&done[m][g]);
+                __syncwarp();
+                committed = (int)((n & 1) << 8) | g;
+            }
+            if (sizeof(T) == 4 && lane == 0)
+                atomicExch(&s_turn, 0);
+        }
+        if (!ok && lane == 0) {
+            atomicExch(P.err, kDevTimeout);
+            s_abort = 1;
+        }
+        // MMAs in flight end before the CTA does
+        if (s_abort && committed >= 0)
+            bar_drain(&done[m][committed & 255], (uint32_t)(committed >> 8), kWaitLimitCycles);
+        __syncwarp();
+    } else {
+        // ---- a team: load, convert, drain -------------------------------------
+        const int m = warp / kTeamWarps, tw = warp % kTeamWarps, tt = t % kTeam;
+        auto sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(2 + m), "n"(kTeam) : "memory"); };
+        unsigned char *xp = planes + (size_t)m * ND * C * 128;
+        uint32_t phase = 0;
+        for (long long tile = (long long)blockIdx.x * 2 + m; tile < tiles; tile += 2LL * gridDim.x) {
+            const long long b0 = P.blk0 + tile * per;
+            const int nb = (int)(P.blk1 - b0 < per ? P.blk1 - b0 : per);
+            const long long base = (b0 - hb) * kPropBlk;
+            const int chunks = (per + 2 * hb) * 8;
+            constexpr int kIter = ((kPropTileBlks + 2 * (sizeof(T) == 8 ? 0 : kDuoHb32)) * 8 + kTeam - 1) / kTeam;
+            if (tt < 2)
+                s_max[m][tt] = 0;
+            if (tt == 2)
+                s_keep[m] = 0;
+            if (tt == 3)
+                s_left[m] = *reinterpret_cast<const volatile int *>(P.count) > P.gate_min;
+            sync();
+            T x[kIter][8];
+            int wmax = 0;
+            constexpr int kV = 16 / sizeof(T);
+#pragma unroll
+            for (int c = 0; c < kIter; ++c) {
+                const int u = c * kTeam + tt;
+                const long long j = base + (long long)u * 8;
+                const bool in_range = u < chunks && j + 8 <= P.n;
+#pragma unroll
+                for (int v = 0; v < 8 / kV; ++v) {
+                    uint4 q = make_uint4(0, 0, 0, 0);
+                    if (in_range)
+                        q = *reinterpret_cast<const uint4 *>(in + j + v * kV);
+                    *reinterpret_cast<uint4 *>(&x[c][v * kV]) = q;
+                }
+            }
+            // the next tile's window on its way to L2
+            if (tile + 2LL * gridDim.x < tiles) {
+                const long long nx = base + 2LL * gridDim.x * per * kPropBlk;
+                for (long long z = nx + (long long)tt * 128 / (long long)sizeof(T); z < nx + (long long)chunks * 8 && z < P.n;
+                     z += (long long)kTeam * 128 / (long long)sizeof(T))
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(in + z));
+            }
+#pragma unroll
+            for (int c = 0; c < kIter; ++c) {
+                const int u = c * kTeam + tt;
+                int q = 0;
+#pragma unroll
+                for (int v = 0; v < 8; ++v) {
+                    const int y = code_of(x[c][v]);
+                    q = y > q ? y : q;
+                }
+                wmax = q > wmax ? q : wmax;
+                for (int z = 1; z < 8; z <<= 1) {
+                    const int y = __shfl_xor_sync(0xffffffffu, q, z);
+                    q = y > q ? y : q;
+                }
+                if ((tt & 7) == 0 && u < chunks)
+                    s_code[m][u >> 3] = q;
+            }
+            int cmax = wmax;
+            const long long clo = b0 * kPropBlk - P.k - 2, chi = (b0 + nb) * kPropBlk + P.k + 2;
+            auto scan = [&](long long a, long long b) {
+                for (long long j = a + tt; j < b; j += 4 * kTeam)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        cmax = max(cmax, code_of(j + u * kTeam < b ? in[j + u * kTeam] : (T)0));
+            };
+            scan(clo > 0 ? clo : 0, base);
+            scan(base + (long long)chunks * 8, chi < P.n ? chi : P.n);
+            for (long long j = (P.n & ~7LL) + tt; j < P.n && j < chi; j += kTeam)
+                cmax = max(cmax, code_of(in[j]));
+            bulk_wait_read0();  // the last tile's rows have left the planes
+            wmax = __reduce_max_sync(0xffffffffu, wmax);
+            cmax = __reduce_max_sync(0xffffffffu, cmax);
+            if (lane == 0) {
+                atomicMax(&s_max[m][0], wmax);
+                atomicMax(&s_max[m][1], cmax);
+            }
+            sync();
+            if (s_left[m])
+                break;
+            const int ref = s_max[m][0], cone = s_max[m][1];
+            if (tt < nb) {
+                const int q = s_code[m][hb + tt];
+                const bool listed = cone > 0 && (!ok_tab || cone == kCodeInf<T> || q < cone - S::kRange || q == 0);
+                if (listed)
+                    P.list[atomicAdd(P.count, 1)] = (int)(b0 + tt);
+                else if (cone > 0)
+                    s_keep[m] = 1;
+            }
+            if (ok_tab && cone != kCodeInf<T>) {
+#pragma unroll
+                for (int c = 0; c < kIter; ++c) {
+                    const int u = c * kTeam + tt;
+                    if (u < chunks)
+                        convert8(x[c], ref, xp + (u >> 3) * 128 + ((7 - (u & 7)) ^ ((u >> 3) & 7)) * 16, (size_t)C * 128);
+                }
+            }
+            fence_async_smem();
+            tc_fence_before();
+            sync();
+            if (!s_keep[m]) {
+                if (cone == 0 && tt < nb * 2) {
+                    T *o = out + b0 * kPropBlk + tt * 32;
+                    for (int v = 0; v < 32; ++v)
+                        o[v] = (T)0;
+                }
+                continue;
+            }
+            if (lane == 0)
+                bar_arrive(&full[m]);
+            // drain: kTeamCols points of the lane's block
+            const int row = (warp & 3) * 32 + lane, col = (tw >> 2) * kTeamCols;
+            const int room = s_hdr.room, xs = sizeof(T) == 4 ? 0 : room < 8 ? room : 8;
+            long long acc[kTeamCols];
+#pragma unroll
+            for (int v = 0; v < kTeamCols; ++v)
+                acc[v] = 0;
+            bool ok = true;
+#pragma unroll 1
+            for (int g = 0; g < NG; ++g) {
+                ok = ok && bar_wait(&done[m][g], phase, kWaitLimitCycles, &s_abort);
+                if (!__any_sync(0xffffffffu, !ok)) {
+                    tc_fence_after();
+#pragma unroll
+                    for (int h = 0; h < kTeamCols; h += 16) {
+                        uint32_t v[16];
+                        tmem_ld16(tbase + ((uint32_t)((warp & 3) * 32) << 16) +
+                                      (uint32_t)(m * 256 + g % kRing * kPropBlk + col + h), v);
+                        tmem_wait_ld();
+                        if (h + 16 == kTeamCols) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0)
+                                bar_arrive(&reuse[m][g % kRing]);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 16; ++q)
+                            acc[h + q] = fold<T>(acc[h + q], G::weight(g), __float2int_rn(__uint_as_float(v[q])), xs);
+                    }
+                }
+            }
+            if (__any_sync(0xffffffffu, !ok)) {
+                if (lane == 0) {
+                    atomicExch(P.err, kDevTimeout);
+                    s_abort = 1;
+                }
+            } else if (row < nb) {
+                const int ex = sizeof(T) == 8 ? ref - 1022 + 2 - s_hdr.E - xs : ref - 126 - 6 - s_hdr.E;
+                unsigned char *o = xp + row * kStageRow<T> + col * (int)sizeof(T);
+                if (sizeof(T) == 8 && ex >= -1021 && ex <= 959) {
+                    // through the row's own space in a short loop: 32 times the
+                    // code would be fetched anew by every launch
+#pragma unroll
+                    for (int v = 0; v < kTeamCols; v += 2)
+                        *reinterpret_cast<longlong2 *>(o + v * 8) = make_longlong2(acc[v], acc[v + 1]);
+#pragma unroll 1
+                    for (int v = 0; v < kTeamCols; v += 2) {
+                        const longlong2 z = *reinterpret_cast<const longlong2 *>(o + v * 8);
+                        *reinterpret_cast<double2 *>(o + v * 8) =
+                            make_double2(from_fixed<double>(z.x, ex), from_fixed<double>(z.y, ex));
+                    }
+                } else {
+                    finish_row<T>(acc, ex, o);
+                }
+            }
+            fence_async_smem();
+            sync();
+            if (tt < nb && !s_abort) {
+                bulk_store(out + (b0 + tt) * kPropBlk, xp + tt * kStageRow<T>, kPropBlk * (uint32_t)sizeof(T));
+                bulk_commit();
+            }
+            phase ^= 1;
+            if (s_abort)
+                break;
+        }
+        if (tt == 0)
+            s_stop[m] = 1;
+        sync();
+        if (lane == 0)
+            bar_arrive(&full[m]);
+        bulk_wait0();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (t == 0 && ok_tab)
+        bar_drain(&tab_full, 0, kWaitLimitCycles);
+    __syncthreads();
+    if (warp == kTileWarps)
+        tmem_dealloc(tbase, 512);
+    if (s_abort || warp >= kTileWarps)
+        return;
+    // rows near a wall: they fill the last wave, the CTAs with fewer tiles first
+    const int shift = item_shift(P);
+    const long long edge_l = item_count(P.rows_l, kEdgeRows, shift);
+    const long long edges = edge_l + item_count(P.n - P.row_r, kEdgeRows, shift);
+    // (a CTA's pair of tiles takes as long as about four items)
+    const int busy = (int)((tiles + 1) / 2 % gridDim.x), spare = busy ? (int)gridDim.x - busy : 0;
+    const bool few = spare > 0 && edges <= 4LL * spare;
+    const int me = (int)blockIdx.x - busy;
+    double *s_w = reinterpret_cast<double *>(sm), *taps = s_w + kDotWin + kEdgeScratch;
+    bool staged = false;
+    for (long long x = few && me < 0 ? edges : me < 0 ? me + (long long)gridDim.x : me; x < edges;
+         x += few ? spare : (int)gridDim.x) {
+        if (!staged)
+            dot_stage<kTileConv>(P, reinterpret_cast<typename PairOf<T>::E *>(taps));
+        staged = true;
+        const long long a = x < edge_l ? 0 : P.row_r, b = x < edge_l ? P.rows_l : P.n;
+        const long long r0 = a + (x < edge_l ? x : x - edge_l) * kEdgeRows - shift, r1 = r0 + kEdgeRows;
+        dot_rows<T, kTileConv, kEdgeRows, kEdgeParts, true>(P, s_dot, s_w, taps, r0 > a ? r0 : a, r1 < b ? r1 : b);
+    }
+}
+
 }  // namespace
 
 cudaError_t prop_prepare()
@@ -1329,6 +1775,8 @@ cudaError_t prop_prepare()
     smem(prop_tile_kernel<double, true>, kTileSmem<double>);
     smem(prop_tile_kernel<float, false>, kTileSmem<float>);
     smem(prop_tile_kernel<float, true>, kTileSmem<float>);
+    smem(prop_duo_kernel<double>, kDuoSmem);
+    smem(prop_duo_kernel<float>, kDuoSmem);
     smem(prop_dot_kernel<double>, (kDotWin + dot_taps(kPropRMax)) * 8);
     smem(prop_dot_kernel<float>, (kDotWin + dot_taps(kPropRMax)) * 8);
     if (e == cudaSuccess)
@@ -1465,7 +1913,15 @@ cudaError_t prop_launch_tiles(PropRun a, int f64, int num_sms, cudaStream_t s)
         return f64 ? cudaLaunchKernelEx(&c, prop_tile_kernel<double, true>, a)
                    : cudaLaunchKernelEx(&c, prop_tile_kernel<float, true>, a);
     }
+    if (a.tiles >= 2 * num_sms && a.hb <= (f64 ? kDuoHb64 : kDuoHb32)) {
+        if (f64)
+            prop_duo_kernel<double><<<num_sms, kTileThreads, kDuoSmem, s>>>(a);
+        else
+            prop_duo_kernel<float><<<num_sms, kTileThreads, kDuoSmem, s>>>(a);
+        return cudaGetLastError();
+    }
     const int grid = (int)(a.tiles + edges < num_sms ? a.tiles + edges : num_sms);
+    a.edge_rounds = (int)std::min((double)edges, std::max(1.0, (start + 50 * mmas - 4000) / item));
     if (f64)
         prop_tile_kernel<double, false><<<grid, kTileThreads, kTileSmem<double>, s>>>(a);
     else

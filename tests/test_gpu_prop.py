@@ -176,3 +176,42 @@ def test_fp32_rows_at_any_magnitude(n, exp):
     s = 2.0 ** exp
     got = auto_run(u0 * s, r, 0.25 * s, -0.75 * s, steps, B.GE_F32)
     assert rel_max(got / s, want) <= 1e-5
+
+
+def tiled_run(u0, r, bl, br, steps, prec):
+    x = torch.as_tensor(np.asarray(u0), dtype=B.dtype_of(prec), device=DEV).contiguous()
+    ctx = B.ge_create(len(u0), r, bl, br, prec, x)
+    B.ge_set_kernel(ctx, B.GE_KERNEL_TEMPORAL, 0)
+    B.ge_step_n(ctx, steps)
+    out = torch.empty_like(x)
+    B.ge_read_state(ctx, out)
+    B.ge_sync(ctx)
+    B.ge_destroy(ctx)
+    return out.double().cpu().numpy()
+
+
+# large enough for two teams a CTA on 152 SMs (304 tiles of 128 blocks), with
+# the narrowest and the widest halos they take, whole and ragged last tiles
+@pytest.mark.parametrize("n", [304 * 8192 + 64 * 22 * 2 + 1, 2700003])
+@pytest.mark.parametrize("prec,r,steps", [(B.GE_F64, 0.01, 24), (B.GE_F64, 0.5, 24), (B.GE_F64, 2.0, 41),
+                                          (B.GE_F32, 0.05, 200), (B.GE_F32, 2.0, 400), (B.GE_F32, 2.0, 2000)])
+def test_two_teams_match_the_tiled_kernel(n, prec, r, steps):
+    """Each path is within its tolerance of the exact steps: twice that apart.
+    Random data, and the same with a stretch of zeros, a far smaller one and
+    (last) an infinity, whose reach both paths agree on."""
+    tol = 2 * tol64(r) if prec == B.GE_F64 else 2e-5
+    u0 = inputs.random_state(n, seed=n % 97)
+    if prec != B.GE_F64:
+        u0 = u0.astype(np.float32).astype(np.float64)
+    assert rel_max(auto_run(u0, r, 0.3, -0.8, steps, prec), tiled_run(u0, r, 0.3, -0.8, steps, prec)) <= tol
+    u0[n // 3:n // 3 + 100000] = 0.0
+    u0[n // 2:n // 2 + 30000] *= 2.0 ** -40
+    got, want = auto_run(u0, r, 0.3, -0.8, steps, prec), tiled_run(u0, r, 0.3, -0.8, steps, prec)
+    assert rel_max(got, want) <= tol
+    inner = slice(n // 2 + 2 * steps + 64, n // 2 + 30000 - 2 * steps - 64)
+    assert rel_max(got[inner], want[inner]) <= (1e-10 if prec == B.GE_F64 else 1e-3)
+    u0[n // 4] = np.inf
+    got, want = auto_run(u0, r, 0.3, -0.8, steps, prec), tiled_run(u0, r, 0.3, -0.8, steps, prec)
+    assert np.array_equal(np.isfinite(got), np.isfinite(want))
+    ok = np.isfinite(want)
+    assert rel_max(got[ok], want[ok]) <= tol
