@@ -234,6 +234,16 @@ bool tc_shape(const ge_sno *s)
 }
 bool tc_active(const ge_sno *s) { return s->tc && !s->split && tc_shape(s) && s->tc_ready; }
 
+constexpr int kEarlyTiles = 32;
+
+// Whether the tensor-core kernels start early, on R rows: their set-up (4 us of
+// the 9 a kernel takes) hides under the kernel before, but the CTAs that come
+// early take the SMs that are free then, and a long persistent kernel pays for
+// an uneven spread.  Inference of 8 / 100 / 600 / 1200 problems of 1024 points:
+// 93 -> 71, 121 -> 94, 241 -> 237, 447 -> 492 us; training of 8 / 64 / 600:
+// 319 -> 256, 416 -> 343, 1202 -> 1159 us.
+int starts_early(const ge_sno *s, long long R) { return R / 128 <= kEarlyTiles * (long long)s->num_sms ? 1 : 0; }
+
 // Inference with the tensor-core kernels for the truncated DFT, the fused
 // layers and the projection (the mode mixing keeps the mma.sync GEMM).
 ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br, float *out,
@@ -365,13 +375,15 @@ ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const fl
     a.tiles_per_problem = n / 128;
     a.err = s->err;
     a.limit = ge::kWaitLimitCycles;
+    const int early = starts_early(s, R);
+    a.early = early;
     for (int l = 0; l < s->L; ++l) {
         const LayerOff &o = s->lay[l];
         // truncated DFT: vh[b] = F v[b]
         a.out = s->vh[l];
         SNO_TRY(ge::sno_tc_dft(&s->tm_f, &s->tm_v[l], a, s->num_sms, st));
         // per-mode complex mixing: y[b, m] = vh[b, m] Wspec_m
-        const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->y, s->err, ge::kWaitLimitCycles};
+        const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->y, s->err, ge::kWaitLimitCycles, early};
         SNO_TRY(ge::sno_tc_mix(&s->tm_vh[l], &s->tm_wst, x, M, st));
         a.b2_row = l * C;
         a.gelu = l < s->L - 1 ? 1 : 0;
@@ -413,6 +425,8 @@ ge_status backward(ge_sno *s, int B)
     tg.rows = R;
     tg.err = s->err;
     tg.limit = ge::kWaitLimitCycles;
+    const int early = starts_early(s, R);
+    tg.early = early;
     // projection: out = h Q2 + q2; and dhpre = (dout Q2^T) * GELU'(hpre)
     ge::SnoSums q{};
     q.x = s->h;
@@ -435,7 +449,7 @@ ge_status backward(ge_sno *s, int B)
         tg.dw = Gd + s->off_q1;
         tg.db = Gd + s->off_qb1;
         SNO_TRY(ge::sno_tc_grad(&s->tm_v[s->L], &s->tm_dAh, tg, H, s->num_sms, st));
-        const ge::SnoTcMixArgs x{(int)R, 0, C, s->dB, s->err, ge::kWaitLimitCycles};
+        const ge::SnoTcMixArgs x{(int)R, 0, C, s->dB, s->err, ge::kWaitLimitCycles, early};
         SNO_TRY(ge::sno_tc_rows(&s->tm_dAh, &s->tm_q1, x, st));
     } else {
         if ((rc = weight_grad(s, s->v[s->L], C, C, s->dA, H, R, Gd + s->off_q1, Gd + s->off_qb1)) != GE_OK)
@@ -452,6 +466,7 @@ ge_status backward(ge_sno *s, int B)
     ta.tiles_per_problem = n / 128;
     ta.err = s->err;
     ta.limit = ge::kWaitLimitCycles;
+    ta.early = early;
     for (int l = s->L - 1; l >= 0; --l) {
         const LayerOff &o = s->lay[l];
         const void *ws = at(s->wspec, (long long)l * M * 4 * C * C, bf);
@@ -472,7 +487,7 @@ ge_status backward(ge_sno *s, int B)
             ts.drr = Gd + o.rr;
             ts.dri = Gd + o.ri;
             SNO_TRY(ge::sno_tc_grad_spec(&s->tm_vh[l], &s->tm_dy, ts, M, st));
-            const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->dvh, s->err, ge::kWaitLimitCycles};
+            const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->dvh, s->err, ge::kWaitLimitCycles, early};
             SNO_TRY(ge::sno_tc_mix(&s->tm_dy, &s->tm_ws, x, M, st));
             // gradient of v_l, both paths as one layer, times GELU'(pre_{l-1})
             // when v_l is an activation

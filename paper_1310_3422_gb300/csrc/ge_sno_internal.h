@@ -89,6 +89,7 @@ struct SnoTcArgs {
     int *err;               // device error word (GE_ETIMEOUT on a wait that gave up)
     long long limit;        // wait limit in SM cycles
     int keep;               // training forward: also write pre (layer) or hidden layer and pre (projection)
+    int early;              // start under the end of the kernel before (see launch_early)
     const void *dg;         // layer: multiply by GELU' of these BF16 [rows][C], or NULL
 };
 cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s);
@@ -110,6 +111,7 @@ struct SnoTcMixArgs {
     void *y;             // out: BF16 [batch][row_elems]
     int *err;            // device error word
     long long limit;     // wait limit in SM cycles
+    int early;           // as in SnoTcArgs
 };
 cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s);
 cudaError_t sno_tc_rows(const void *map_x, const void *map_b, const SnoTcMixArgs &a, cudaStream_t s);
@@ -126,6 +128,7 @@ struct SnoTcGradArgs {
     float *drr, *dri;    // sno_tc_grad_spec
     int *err;            // device error word
     long long limit;     // wait limit in SM cycles
+    int early;           // as in SnoTcArgs
 };
 cudaError_t sno_tc_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, int cols, int sms,
                         cudaStream_t s);

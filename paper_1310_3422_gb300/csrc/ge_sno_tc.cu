@@ -137,6 +137,17 @@ __device__ __forceinline__ void stage_rows(unsigned char *stg, int lane, const u
             make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
 }
 
+// The kernels of this file start before the one launched before them has
+// finished, and set up (barriers, tensor memory) under its end: nothing
+// before this call may read or write what that kernel does.  It comes after
+// the CTA's tensor memory is allocated, so that the next kernel's CTAs, which
+// it lets in, cannot take it first.
+__device__ __forceinline__ void after_previous()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 constexpr int kTcThreads = 160;
 constexpr int kTileM = 128;
 
@@ -199,14 +210,16 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
         tmem_alloc(&tmem_base_sh, S::kTmemCols);
         tmem_relinquish();
     }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    after_previous();
     for (int i = t; i < N; i += kTcThreads) {
         s_bias[i] = !TRAIN || P.bias ? P.bias[i] : 0.0f;
         // the projection keeps Q2 / 2 (exact): GELU's factor 1/2 moves onto it
         s_q2[i] = MODE == 1 ? 0.5f * P.q2w[i] : 0.0f;
     }
-    tc_fence_before();
     __syncthreads();
-    tc_fence_after();
     const uint32_t tbase = tmem_base_sh;
     const long long my_tiles =
         P.n_tiles > (long long)blockIdx.x ? (P.n_tiles - 1 - (long long)blockIdx.x) / gridDim.x + 1 : 0;
@@ -499,6 +512,7 @@ __global__ void __launch_bounds__(kDftThreads) sno_tc_dft_kernel(const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    after_previous();
     const uint32_t tbase = tmem_base_sh;
     const long long problems = P.n_tiles / P.tiles_per_problem;
     const long long mine = problems > (long long)blockIdx.x ? (problems - 1 - (long long)blockIdx.x) / gridDim.x + 1 : 0;
@@ -651,6 +665,7 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    after_previous();
     const uint32_t tbase = tmem_base_sh;
     if (t == 0) {
         bar_expect_tx(&full, 2 * kMixHalf + 2 * N * 128);
@@ -781,6 +796,7 @@ __global__ void __launch_bounds__(kGradThreads) sno_tc_grad_kernel(const __grid_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    after_previous();
     const uint32_t tbase = tmem_base_sh;
     const long long chunks = (P.rows + 127) / 128;
     const long long mine = chunks > (long long)blockIdx.x ? (chunks - 1 - (long long)blockIdx.x) / gridDim.x + 1 : 0;
@@ -909,6 +925,23 @@ __global__ void __launch_bounds__(kGradThreads) sno_tc_grad_kernel(const __grid_
         tmem_dealloc(tbase, N);
 }
 
+template <typename... Params, typename... Args>
+cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, int threads, int smem, cudaStream_t s, int early,
+                         const Args &...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3((unsigned)threads);
+    c.dynamicSmemBytes = (size_t)smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 template <int MODE, bool TRAIN>
 cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
@@ -962,9 +995,8 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
     const CUtensorMap *b1 = static_cast<const CUtensorMap *>(MODE == 0 ? m.b1 : m.a2);
     const CUtensorMap *o = static_cast<const CUtensorMap *>(MODE == 0 || TRAIN ? m.out : m.a2);
     const CUtensorMap *pre = static_cast<const CUtensorMap *>(TRAIN && m.pre ? m.pre : m.a2);
-    sno_tc_kernel<MODE, TRAIN><<<(int)grid, kTcThreads, S::kSmem, s>>>(*a1, *b1, *static_cast<const CUtensorMap *>(m.a2),
-                                                              *static_cast<const CUtensorMap *>(m.b2), *o, *pre, a);
-    return cudaGetLastError();
+    return launch_early(sno_tc_kernel<MODE, TRAIN>, dim3((unsigned)grid), kTcThreads, S::kSmem, s, a.early, *a1, *b1,
+                        *static_cast<const CUtensorMap *>(m.a2), *static_cast<const CUtensorMap *>(m.b2), *o, *pre, a);
 }
 
 template <int ST>
@@ -999,8 +1031,7 @@ cudaError_t launch_dft(const CUtensorMap &f, const CUtensorMap &v, const SnoTcAr
         grid = problems;
     if (grid < 1)
         return cudaSuccess;
-    sno_tc_dft_kernel<ST><<<(int)grid, kDftThreads, dft_smem(ST), s>>>(f, v, a);
-    return cudaGetLastError();
+    return launch_early(sno_tc_dft_kernel<ST>, dim3((unsigned)grid), kDftThreads, dft_smem(ST), s, a.early, f, v, a);
 }
 
 template <int N>
@@ -1018,9 +1049,8 @@ cudaError_t launch_mix(const void *map_vh, const void *map_wst, const SnoTcMixAr
     if (a.batch == 0)
         return cudaSuccess;
     const dim3 grid((unsigned)((a.batch + 127) / 128), (unsigned)modes);
-    sno_tc_mix_kernel<N><<<grid, kMixThreads, kMixSmem, s>>>(*static_cast<const CUtensorMap *>(map_vh),
-                                                          *static_cast<const CUtensorMap *>(map_wst), a);
-    return cudaGetLastError();
+    return launch_early(sno_tc_mix_kernel<N>, grid, kMixThreads, kMixSmem, s, a.early, *static_cast<const CUtensorMap *>(map_vh),
+                        *static_cast<const CUtensorMap *>(map_wst), a);
 }
 
 template <int KIND>
@@ -1039,9 +1069,8 @@ cudaError_t launch_grad(const void *map_x, const void *map_y, const SnoTcGradArg
         return cudaErrorInvalidValue;
     if (a.rows == 0 || grid.x == 0 || grid.y == 0)
         return cudaSuccess;
-    sno_tc_grad_kernel<KIND><<<grid, kGradThreads, S::kSmem, s>>>(*static_cast<const CUtensorMap *>(map_x),
-                                                                  *static_cast<const CUtensorMap *>(map_y), a);
-    return cudaGetLastError();
+    return launch_early(sno_tc_grad_kernel<KIND>, grid, kGradThreads, S::kSmem, s, a.early, *static_cast<const CUtensorMap *>(map_x),
+                        *static_cast<const CUtensorMap *>(map_y), a);
 }
 
 }  // namespace
