@@ -344,7 +344,7 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
     *taken = 1;
     if (build_only)
         return cudaSuccess;
-    if ((e = cudaMemsetAsync(st->count, 0, 2 * sizeof(int), stream)) != cudaSuccess)
+    if (need[0].tiles && (e = cudaMemsetAsync(st->count, 0, 2 * sizeof(int), stream)) != cudaSuccess)
         return e;
     for (long long i = 0; i <= full; ++i) {
         const Need &w = i == full ? need[needs - 1] : need[i == 0 ? 0 : 1];
