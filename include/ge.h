@@ -157,7 +157,7 @@ ge_status ge_tune(ge_ctx *ctx, int64_t steps, int32_t *best_depth);
  * Saul'yev A runs to the right and B runs to the left (paper node j uses A
  * at parity p iff floor(j/k) + p is even), one thread per confluence unit.
  * With GE_KERNEL_AUTO / GE_KERNEL_TEMPORAL ge_step_n then runs `depth` steps
- * per launch (ge_set_kernel; default 8) on tiles kept in shared memory,
+ * per launch (ge_set_kernel; default 8 to 48 by size) on tiles kept in shared memory,
  * falling back to one launch per step when fewer than 64 units of 2k nodes
  * fit a CTA's shared memory; GE_KERNEL_CANONICAL / GE_KERNEL_ONESTEP run one
  * launch per step.  Both are bit-identical to a serial FP64 evaluation.
@@ -268,9 +268,9 @@ ge_status ge_batch_set_depth(ge_batch *plan, int32_t depth);
 ge_status ge_batch_set_kernel(ge_batch *plan, ge_kernel kernel);
 ge_status ge_batch_get_depth(const ge_batch *plan, int32_t *depth);
 
-/* Tile geometry of later ge_batch_run calls: rows per tile (256, the
- * default, or 128: the tile width W of the 2D TMA box; 0 = 256) and CTAs per
- * SM of the persistent grid (1 .. what fits, 0 = as many as fit; 256-row
+/* Tile geometry of later ge_batch_run calls: rows per tile (256 or 128: the
+ * tile width W of the 2D TMA box; 0 = 256; a new plan starts with the one that
+ * suits its size, as it does with its depth) and CTAs per SM of the persistent grid (1 .. what fits, 0 = as many as fit; 256-row
  * tiles fit 2 per SM, 128-row tiles 4).  The double-float kernel has
  * 256-row tiles only.  Errors: GE_EINVAL (NULL plan, other values). */
 ge_status ge_batch_set_geometry(ge_batch *plan, int32_t tile_rows, int32_t ctas_per_sm);

@@ -42,7 +42,6 @@ ge_status cuda_fail(cudaError_t e, const char *what)
 using ge::kDefaultDepthDf;
 using ge::kDefaultDepthF32;
 using ge::kDefaultDepthF64;
-constexpr int kDefaultDepthSweep = 8;  // width-k steps per launch (k = 16, N = 2^24: 1.41e11 updates/s)
 // Largest r the double-float kernel takes: the right-hand side reaches about
 // (1 + 3r) times the data and must stay far inside the FP32 exponent range.
 constexpr double kDfMaxR = 1048576.0;
@@ -660,7 +659,7 @@ ge_status ge_step_n(ge_ctx *c, int64_t steps)
     ge_status st;
     if (c->width > 1) {
         const bool multi = c->kernel != GE_KERNEL_CANONICAL && c->kernel != GE_KERNEL_ONESTEP;
-        st = run_sweep(c, steps, multi, c->depth ? c->depth : kDefaultDepthSweep);
+        st = run_sweep(c, steps, multi, c->depth ? c->depth : ge::sweep_tb_depth(c->n, c->width, (int)elem_size(c->prec), c->num_sms));
         if (st == GE_OK)
             c->step += steps;
         return st;

@@ -69,6 +69,7 @@ struct ge_batch {
     // tile geometry of the launches (ge_batch_set_geometry, ge_batch_tune):
     // rows per tile (256 or 128) and co-resident CTAs per SM (0: as many as fit)
     int tile_rows = 256, ctas_per_sm = 0;
+    bool shape_set = false;  // depth or geometry chosen by the caller or the tuner
     int blocks_per_sm_128 = 0;
     // one persistent launch per run (plain FP32 plans; ge_batch_set_persistent)
     bool persistent = false;
@@ -112,6 +113,35 @@ void release_batch(ge_batch *b)
     if (b->done)
         cudaFree(b->done);
     delete b;
+}
+
+// Depth and tile height a plan starts with.  Few tiles: a run is a chain of
+// launches, each as long as one tile, so deep ones (64 FP32 problems of up to
+// 65,536 points, 500 steps: 189 -> 142 us; 64 FP64 ones of up to 4096, 300
+// steps: 532 -> 417).  Else 128-row tiles, four to an SM, hide each other's
+// latency better than 256-row ones, two to an SM, at the depth where the
+// redundant halos cost what the launches save (4096 FP32 problems, 2000 steps:
+// 6660 -> 5916 us at 128, 5875 at 96, 6447 at 192; 512 FP64 problems, 500
+// steps: 4971 -> 4803 at 64) -- except FP64 problems shorter than a tile,
+// whose walls the smaller tiles meet more often (4096 of up to 8192 points:
+// 8180 us at 48 rows 256, 7972 at 64).  The compensated and the double-float
+// plans keep the shape they were tuned at.
+void default_shape(const ge_batch *b, int *depth, int *tile_rows)
+{
+    *tile_rows = 256;
+    *depth = b->prec == GE_F64 ? kBatchDefaultDepthF64 : kBatchDefaultDepthF32;
+    if (b->prec == GE_F32_COMP || b->df)
+        return;
+    if ((b->n_rows + 127) / 128 <= 2LL * b->num_sms) {
+        *tile_rows = 128;
+        *depth = 192;
+    } else if (b->prec == GE_F32) {
+        *tile_rows = 128;
+        *depth = 128;
+    } else {
+        *tile_rows = b->n_rows / b->n_problems < 256 ? 256 : 128;
+        *depth = 64;
+    }
 }
 
 int prec_index(ge_precision p) { return p == GE_F64 ? 0 : (p == GE_F32 ? 1 : 2); }
@@ -370,11 +400,11 @@ ge_status ge_batch_create(ge_batch **out, int32_t n_problems, const int64_t *n, 
     b->n_problems = n_problems;
     b->total = total;
     b->n_rows = n_rows;
-    b->depth = prec == GE_F64 ? kBatchDefaultDepthF64 : kBatchDefaultDepthF32;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&b->num_sms, cudaDevAttrMultiProcessorCount, dev);
+    default_shape(b, &b->depth, &b->tile_rows);
     const size_t bytes = (size_t)n_rows * ge::kRowBytes;
     for (int i = 0; i < 2 && e == cudaSuccess; ++i)
         e = cudaMalloc(&b->buf[i], bytes);
@@ -477,6 +507,8 @@ ge_status ge_batch_set_kernel(ge_batch *b, ge_kernel kernel)
             return bcuda(e, "ge_batch_set_kernel: rescale table");
     }
     b->df = df;
+    if (!b->shape_set)
+        default_shape(b, &b->depth, &b->tile_rows);
     if (df)
         b->tile_rows = 256;  // the double-float kernel has the 256-row tile only
     b->R = R;
@@ -493,7 +525,12 @@ ge_status ge_batch_set_depth(ge_batch *b, int32_t depth)
 {
     if (!b || depth < 0 || depth > ge::kMaxTableSteps)
         return bfail(GE_EINVAL, "ge_batch_set_depth: NULL plan or depth outside 0..512");
-    b->depth = depth ? depth : (b->prec == GE_F64 ? kBatchDefaultDepthF64 : kBatchDefaultDepthF32);
+    int rows;
+    if (depth)
+        b->depth = depth;
+    else
+        default_shape(b, &b->depth, &rows);
+    b->shape_set = true;
     return GE_OK;
 }
 
@@ -538,6 +575,7 @@ ge_status ge_batch_set_geometry(ge_batch *b, int32_t tile_rows, int32_t ctas_per
         return bfail(GE_EINVAL, "ge_batch_set_geometry: ctas_per_sm beyond what fits on an SM");
     b->tile_rows = tile_rows;
     b->ctas_per_sm = ctas_per_sm;
+    b->shape_set = true;
     return GE_OK;
 }
 
@@ -671,6 +709,7 @@ ge_status ge_batch_tune(ge_batch *b, const void *u_dev, int64_t steps, int32_t *
     b->depth = best_d;
     b->tile_rows = best_tr;
     b->ctas_per_sm = best_c;
+    b->shape_set = true;
     b->persistent = best_persist;
     if (best_depth)
         *best_depth = best_d;

@@ -256,6 +256,8 @@ cudaError_t launch_sweep_f64(const double *in, double *out, long long n, int par
                              const CanonCoef &c, cudaStream_t s);
 cudaError_t launch_sweep_f32(const float *in, float *out, long long n, int parity, long long k,
                              const CanonCoef &c, cudaStream_t s);
+// Steps per launch for n points of elem_size bytes on sms SMs.
+int sweep_tb_depth(long long n, long long k, int elem_size, int sms);
 // Up to `steps` width-k steps in one launch (tile in shared memory);
 // *done = steps taken, 0 when the width does not fit (use the one-step launch).
 cudaError_t launch_sweep_tb_f64(const double *in, double *out, long long n, int parity, long long k, int steps,

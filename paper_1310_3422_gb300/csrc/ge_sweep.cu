@@ -350,6 +350,15 @@ cudaError_t launch_sweep_t(const Real *in, Real *out, long long n, int parity, l
 // Up to `steps` steps in one launch of sweep_tb_kernel; *done receives the
 // steps taken.  0 when the width leaves too few units per tile (the caller
 // then runs one step with launch_sweep_t).
+//
+// Units of a tile, and the halo of D steps: HU = D + 1 + ceil(D / 2k) units a side.
+long long sweep_units(long long k, int elem_size)
+{
+    const long long units = 227 * 1024 / ((2 * k + 1) * elem_size);
+    return units > 256 ? 256 : units;
+}
+long long sweep_halo(long long k, int d) { return (long long)d + 1 + (d + 2 * k - 1) / (2 * k); }
+
 template <typename Real>
 cudaError_t launch_sweep_tb_t(const Real *in, Real *out, long long n, int parity, long long k, int steps,
                               const CanonCoef &cf, int *done, cudaStream_t s)
@@ -360,14 +369,10 @@ cudaError_t launch_sweep_tb_t(const Real *in, Real *out, long long n, int parity
     SweepCoef<Real> c{(Real)cf.c1, (Real)cf.c2, (Real)cf.c3, (Real)cf.c4,
                       (Real)cf.s0, (Real)cf.s1, (Real)cf.beta_l, (Real)cf.beta_r};
     const long long w = 2 * k;
-    const long long max_smem = 227 * 1024;
-    long long NU = max_smem / ((w + 1) * (long long)sizeof(Real));
-    if (NU > 256)
-        NU = 256;
-    // steps per launch: the halo HU = D + 1 + ceil(D / 2k) units per side
-    // leaves at least half of the tile's units as output
+    const long long NU = sweep_units(k, (int)sizeof(Real));
+    // steps per launch: the halo leaves at least half of the tile's units as output
     int D = steps;
-    auto halo = [&](int d) { return (long long)d + 1 + (d + w - 1) / w; };
+    auto halo = [&](int d) { return sweep_halo(k, d); };
     while (D > 1 && NU - 2 * halo(D) < NU / 2)
         --D;
     if (NU < 64 || NU - 2 * halo(D) < 1)
@@ -400,6 +405,23 @@ cudaError_t launch_sweep_tb_t(const Real *in, Real *out, long long n, int parity
 }
 
 }  // namespace
+
+// Steps per launch without a choice of the caller's.  Where every SM has at
+// most one tile a launch is one tile's chain of steps and costs another two to
+// three steps to start, so the deepest that still fits (FP64, k = 16, 96 steps:
+// n = 2^18 1096 -> 869 us at 48, n = 2^20 1096 -> 999 at 16, where 24 would
+// give some SMs two tiles, 1545); larger grids are bound by the FP64 unit and
+// the halos are work: 8 (n = 2^22: 3288 us, 3683 at 16).
+int sweep_tb_depth(long long n, long long k, int elem_size, int sms)
+{
+    const long long units = sweep_units(k, elem_size);
+    for (int d : {48, 32, 24, 16, 12}) {
+        const long long out = units - 2 * sweep_halo(k, d);
+        if (out >= units / 2 && (n + 1 + k) / (out * 2 * k) + 1 <= sms)
+            return d;
+    }
+    return 8;
+}
 
 cudaError_t launch_sweep_tb_f64(const double *in, double *out, long long n, int parity, long long k, int steps,
                                 const CanonCoef &c, int *done, cudaStream_t s)
