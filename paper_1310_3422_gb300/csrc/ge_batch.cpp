@@ -115,29 +115,30 @@ void release_batch(ge_batch *b)
     delete b;
 }
 
-// Depth and tile height a plan starts with.  Few tiles: a run is a chain of
-// launches, each as long as one tile, so deep ones (64 FP32 problems of up to
-// 65,536 points, 500 steps: 189 -> 142 us; 64 FP64 ones of up to 4096, 300
-// steps: 532 -> 417).  Else 128-row tiles, four to an SM, hide each other's
-// latency better than 256-row ones, two to an SM, at the depth where the
-// redundant halos cost what the launches save (4096 FP32 problems, 2000 steps:
-// 6660 -> 5916 us at 128, 5875 at 96, 6447 at 192; 512 FP64 problems, 500
-// steps: 4971 -> 4803 at 64) -- except FP64 problems shorter than a tile,
-// whose walls the smaller tiles meet more often (4096 of up to 8192 points:
-// 8180 us at 48 rows 256, 7972 at 64).  The compensated and the double-float
-// plans keep the shape they were tuned at.
+// Depth and tile height a plan starts with.  128-row tiles, four to an SM,
+// hide each other's latency better than 256-row ones, two to an SM (4096 FP32
+// problems, 2000 steps: 6660 -> 6353 us) -- except FP64 problems shorter than
+// a tile, whose walls the smaller tiles meet more often (4096 of up to 8192
+// points, 500 steps: 8180 us with 48 steps a launch, 7972 with 64).
+// FP64 launches are as deep as the redundant halos allow (512 problems, 500
+// steps: 4971 -> 4803 us at 64), and with few tiles, where a run is a chain
+// of launches each as long as one tile, deeper (64 problems of up to 4096
+// points, 300 steps: 532 -> 417 us at 192).  FP32 launches keep their 64
+// steps: where a launch ends decides where the scaled form rounds, and FP32
+// results, the surrogate's training targets among them, stay what they were
+// bit for bit (128 steps would take 5916 us; ge_batch_tune finds it).  The
+// compensated and the double-float plans keep the shape they were tuned at.
 void default_shape(const ge_batch *b, int *depth, int *tile_rows)
 {
     *tile_rows = 256;
     *depth = b->prec == GE_F64 ? kBatchDefaultDepthF64 : kBatchDefaultDepthF32;
     if (b->prec == GE_F32_COMP || b->df)
         return;
-    if ((b->n_rows + 127) / 128 <= 2LL * b->num_sms) {
+    if (b->prec == GE_F32) {
+        *tile_rows = 128;
+    } else if ((b->n_rows + 127) / 128 <= 2LL * b->num_sms) {
         *tile_rows = 128;
         *depth = 192;
-    } else if (b->prec == GE_F32) {
-        *tile_rows = 128;
-        *depth = 128;
     } else {
         *tile_rows = b->n_rows / b->n_problems < 256 ? 256 : 128;
         *depth = 64;
