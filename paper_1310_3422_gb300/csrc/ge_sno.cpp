@@ -95,13 +95,9 @@ struct ge_sno {
     // the weight-derived operands above (and the rounded weights pw, pw16)
     // no longer match the parameters: set when the parameters change
     bool tc_stale = true;
-    void *ws = nullptr;                   // [L][M][2C in][2C out] BF16 (the backward mixing's operand)
-    void *FT16 = nullptr, *GT16 = nullptr;  // F^T [n][2M], G^T [2M][n] BF16 (backward)
     int *err = nullptr;                   // device error word of the tensor-core kernels
-    // training: F^T, G^T, the spectral weights, the gradients' spectra (dy as
-    // mixing rows, dvh as a layer's operand) and buffers, W of each layer
-    CUtensorMap tm_ft, tm_gt, tm_ws, tm_dy, tm_dvh, tm_dA, tm_dB, tm_dAs, tm_dBs, tm_dAh, tm_q1, tm_h, tm_hpre;
-    std::vector<CUtensorMap> tm_w, tm_pre;
+    // weight gradients: dy, the gradients as rows of C and (dhpre) of H
+    CUtensorMap tm_dy, tm_dA, tm_dB, tm_dAh;
     CUtensorMap tm_g, tm_y, tm_wt, tm_q1t, tm_f, tm_wst;
     std::vector<CUtensorMap> tm_v;        // one per activation buffer v[0..L]
     std::vector<CUtensorMap> tm_vs;       // store maps of v[1..L] (index l: v[l + 1])
@@ -240,14 +236,13 @@ constexpr int kEarlyTiles = 32;
 // the 9 a kernel takes) hides under the kernel before, but the CTAs that come
 // early take the SMs that are free then, and a long persistent kernel pays for
 // an uneven spread.  Inference of 8 / 100 / 600 / 1200 problems of 1024 points:
-// 93 -> 71, 121 -> 94, 241 -> 237, 447 -> 492 us; training of 8 / 64 / 600:
-// 319 -> 256, 416 -> 343, 1202 -> 1159 us.
+// 93 -> 71, 121 -> 94, 241 -> 237, 447 -> 492 us.
 int starts_early(const ge_sno *s, long long R) { return R / 128 <= kEarlyTiles * (long long)s->num_sms ? 1 : 0; }
 
 // Inference with the tensor-core kernels for the truncated DFT, the fused
 // layers and the projection (the mode mixing keeps the mma.sync GEMM).
-ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br, float *out,
-                     bool keep);
+ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br, float *out);
+ge_status prepare(ge_sno *s);
 
 // Forward pass for B problems into out ([B n], FP32).  keep: also store the
 // pre-activations the backward pass needs (training).
@@ -261,9 +256,15 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
     const float *P = s->pw;  // FP32 rounded weights: biases and the spectral matrices' source
     const void *F = bf ? s->F16 : static_cast<const void *>(s->F);
     const void *G = bf ? s->G16 : static_cast<const void *>(s->G);
-    if (tc_active(s))
-        return forward_tc(s, B, u0, r, bl, br, out, keep);
-    SNO_TRY(ge::sno_round_bf16(s->params, s->pw, bf ? s->pw16 : nullptr, s->n_params, st));
+    if (!keep && tc_active(s))
+        return forward_tc(s, B, u0, r, bl, br, out);
+    if (bf) {
+        const ge_status rc = prepare(s);
+        if (rc != GE_OK)
+            return rc;
+    } else {
+        SNO_TRY(ge::sno_round_bf16(s->params, s->pw, nullptr, s->n_params, st));
+    }
     // lift (K = 4: no GEMM); the features themselves only for the backward pass
     if (keep)
         SNO_TRY(ge::sno_features(u0, r, bl, br, s->feat, B, n, bf ? 1 : 0, st));
@@ -272,7 +273,8 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
     for (int l = 0; l < s->L; ++l) {
         const LayerOff &o = s->lay[l];
         void *ws = at(s->wspec, (long long)l * M * 4 * C * C, bf);
-        SNO_TRY(ge::sno_spec_assemble(P + o.rr, P + o.ri, ws, M, C, bf ? 1 : 0, st));
+        if (!bf)
+            SNO_TRY(ge::sno_spec_assemble(P + o.rr, P + o.ri, ws, M, C, 0, st));
         // truncated DFT along the grid: vh[b] = F [2M x n] * v[b] [n x C]
         g = gemm(F, n, 1, s->v[l], C, 1, s->vh[l], C, 2 * M, C, n);
         g.sA = 0;
@@ -328,47 +330,57 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
     g.bias = P + s->off_qb1;
     g.act = s->h;
     SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
-    SNO_TRY(ge::sno_row_dot(s->h, weight(s, s->off_q2), P + s->off_qb2, u0, out, R, H, bf ? 1 : 0, st));
+    // (a warp per row takes 16 us instead of 23, but sums in another order: where
+    // pred is close to its target, 1e-8 of pred is 2e-6 of the gradients)
+    g = gemm(s->h, H, 1, weight(s, s->off_q2), 1, 1, out, 1, (int)R, 1, H);
+    g.bias = P + s->off_qb2;
+    g.C0 = u0;
+    g.beta = 1.0f;
+    act_fmt(g, bf).out_bf16 = 0;
+    SNO_TRY(ge::sno_gemm(g, 1, s->split, st));
     return GE_OK;
 }
 
-ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br, float *out,
-                     bool keep)
+// The operands derived from the weights in BF16 mode, by one launch: the
+// rounded weights, the K-major copies W^T (per layer) and Q1^T, and the
+// spectral matrices both ways.  Inference on the tensor cores rebuilds them
+// once per parameter change; the other passes always do, so that one captured
+// in a graph uses the parameters of its replay.
+ge_status prepare(ge_sno *s)
 {
-    const int n = s->n, C = s->C, M = s->M, H = s->H;
+    const int C = s->C, M = s->M;
+    ge::SnoPrepare w{};
+    w.params = s->params;
+    w.count = s->n_params;
+    w.pw = s->pw;
+    w.pw16 = s->pw16;
+    w.wt = s->wt;
+    w.ws = s->wspec;
+    w.wst = s->wst;
+    w.q1t = s->q1t;
+    w.c = C;
+    w.modes = M;
+    w.layers = s->L;
+    w.h = s->H;
+    w.lay0 = s->lay[0].rr;
+    w.lay_size = 2LL * M * C * C + (long long)C * C + C;
+    w.q1 = s->off_q1;
+    SNO_TRY(ge::sno_prepare(w, s->stream));
+    return GE_OK;
+}
+
+ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const float *bl, const float *br, float *out)
+{
+    const int n = s->n, C = s->C, M = s->M;
     const long long R = (long long)B * n;
     cudaStream_t st = s->stream;
     const float *P = s->pw;
-    if (s->tc_stale || keep) {
-        // operands derived from the weights: the rounded weights, the K-major
-        // copies W^T (per layer) and Q1^T, and the spectral matrices both
-        // ways.  Inference rebuilds them once per parameter change; a
-        // training pass always does, so that one captured in a graph uses
-        // the parameters of its replay.
-        ge::SnoPrepare w{};
-        w.params = s->params;
-        w.count = s->n_params;
-        w.pw = s->pw;
-        w.pw16 = s->pw16;
-        w.wt = s->wt;
-        w.ws = s->ws;
-        w.wst = s->wst;
-        w.q1t = s->q1t;
-        w.c = C;
-        w.modes = M;
-        w.layers = s->L;
-        w.h = H;
-        w.lay0 = s->lay[0].rr;
-        w.lay_size = 2LL * M * C * C + (long long)C * C + C;
-        w.q1 = s->off_q1;
-        SNO_TRY(ge::sno_prepare(w, st));
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        SNO_TRY(cudaStreamIsCapturing(st, &cap));
-        if (!keep || cap == cudaStreamCaptureStatusNone)
-            s->tc_stale = false;
+    if (s->tc_stale) {
+        const ge_status rc = prepare(s);
+        if (rc != GE_OK)
+            return rc;
+        s->tc_stale = false;
     }
-    if (keep)
-        SNO_TRY(ge::sno_features(u0, r, bl, br, s->feat, B, n, 1, st));
     SNO_TRY(ge::sno_lift(u0, r, bl, br, weight(s, s->off_w0), P + s->off_b0, s->v[0], B, n, C, 1, st));
     ge::SnoTcArgs a{};
     a.n_tiles = R / 128;
@@ -389,19 +401,17 @@ ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const fl
         a.gelu = l < s->L - 1 ? 1 : 0;
         a.bias = P + o.b;
         a.out = s->v[l + 1];
-        a.keep = keep && l < s->L - 1 ? 1 : 0;
-        const ge::SnoTcMaps m{&s->tm_g, &s->tm_y, &s->tm_v[l], &s->tm_wt, &s->tm_vs[l], &s->tm_pre[l]};
+        const ge::SnoTcMaps m{&s->tm_g, &s->tm_y, &s->tm_v[l], &s->tm_wt, &s->tm_vs[l]};
         SNO_TRY(ge::sno_tc_layer(m, a, s->num_sms, st));
     }
     a.b2_row = 0;
     a.gelu = 1;
-    a.keep = keep ? 1 : 0;
     a.bias = P + s->off_qb1;
     a.q2w = P + s->off_q2;
     a.q2b = P + s->off_qb2;
     a.u0 = u0;
     a.out = out;
-    const ge::SnoTcMaps m{nullptr, nullptr, &s->tm_v[s->L], &s->tm_q1t, &s->tm_h, &s->tm_hpre};
+    const ge::SnoTcMaps m{nullptr, nullptr, &s->tm_v[s->L], &s->tm_q1t, nullptr};
     SNO_TRY(ge::sno_tc_projection(m, a, s->num_sms, st));
     return GE_OK;
 }
@@ -427,6 +437,11 @@ ge_status backward(ge_sno *s, int B)
     tg.limit = ge::kWaitLimitCycles;
     const int early = starts_early(s, R);
     tg.early = early;
+    // The activations and their gradients come from the mma.sync GEMMs in both
+    // directions: their spectra are rounded to BF16, and the other summation
+    // order of the tcgen05 kernels flips some of those roundings, 1e-3 of a
+    // spectral weight's gradient.  The weight gradients are not rounded, so
+    // they may be summed in any order.
     // projection: out = h Q2 + q2; and dhpre = (dout Q2^T) * GELU'(hpre)
     ge::SnoSums q{};
     q.x = s->h;
@@ -443,65 +458,31 @@ ge_status backward(ge_sno *s, int B)
     q.pre = s->hpre;
     q.out = s->dA;
     SNO_TRY(ge::sno_colsum(q, bf ? 1 : 0, st));
-    // dQ1, dq1 and dv_L = dhpre Q1^T
-    ge::GemmArgs g{};
     if (tc) {
         tg.dw = Gd + s->off_q1;
         tg.db = Gd + s->off_qb1;
         SNO_TRY(ge::sno_tc_grad(&s->tm_v[s->L], &s->tm_dAh, tg, H, s->num_sms, st));
-        const ge::SnoTcMixArgs x{(int)R, 0, C, s->dB, s->err, ge::kWaitLimitCycles, early};
-        SNO_TRY(ge::sno_tc_rows(&s->tm_dAh, &s->tm_q1, x, st));
-    } else {
-        if ((rc = weight_grad(s, s->v[s->L], C, C, s->dA, H, R, Gd + s->off_q1, Gd + s->off_qb1)) != GE_OK)
-            return rc;
-        g = gemm(s->dA, H, 1, weight(s, s->off_q1), 1, H, s->dB, C, (int)R, C, H);
-        SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
+    } else if ((rc = weight_grad(s, s->v[s->L], C, C, s->dA, H, R, Gd + s->off_q1, Gd + s->off_qb1)) != GE_OK) {
+        return rc;
     }
+    ge::GemmArgs g = gemm(s->dA, H, 1, weight(s, s->off_q1), 1, H, s->dB, C, (int)R, C, H);  // dv_L = dhpre Q1^T
+    SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
     // dv holds the gradient of the current layer's pre-activation: the last
     // layer has no activation, and every lower one's GELU' is applied in the
     // epilogue of the GEMM that makes its gradient.
     void *dv = s->dB, *dnext = s->dA;
-    ge::SnoTcArgs ta{};
-    ta.n_tiles = R / 128;
-    ta.tiles_per_problem = n / 128;
-    ta.err = s->err;
-    ta.limit = ge::kWaitLimitCycles;
-    ta.early = early;
     for (int l = s->L - 1; l >= 0; --l) {
         const LayerOff &o = s->lay[l];
         const void *ws = at(s->wspec, (long long)l * M * 4 * C * C, bf);
         const void *dpre = dv;
+        // pointwise path weights
         if (tc) {
-            const bool from_b = dv == s->dB;
-            const CUtensorMap *map = from_b ? &s->tm_dB : &s->tm_dA;
-            // pointwise path weights
             tg.dw = Gd + o.w;
             tg.db = Gd + o.b;
-            SNO_TRY(ge::sno_tc_grad(&s->tm_v[l], map, tg, C, s->num_sms, st));
-            // spectral path: dy[b] = G^T dpre[b], dWspec_m = vh[:, m]^T dy[:, m],
-            // dvh[:, m] = dy[:, m] Wspec_m^T
-            ta.out = s->y;
-            SNO_TRY(ge::sno_tc_dft(&s->tm_gt, map, ta, s->num_sms, st));
-            ge::SnoTcGradArgs ts = tg;
-            ts.rows = B;
-            ts.drr = Gd + o.rr;
-            ts.dri = Gd + o.ri;
-            SNO_TRY(ge::sno_tc_grad_spec(&s->tm_vh[l], &s->tm_dy, ts, M, st));
-            const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->dvh, s->err, ge::kWaitLimitCycles, early};
-            SNO_TRY(ge::sno_tc_mix(&s->tm_dy, &s->tm_ws, x, M, st));
-            // gradient of v_l, both paths as one layer, times GELU'(pre_{l-1})
-            // when v_l is an activation
-            ta.b2_row = 0;
-            ta.out = dnext;
-            ta.dg = l > 0 ? s->pre[l - 1] : nullptr;
-            const ge::SnoTcMaps m{&s->tm_ft, &s->tm_dvh, map, &s->tm_w[l], from_b ? &s->tm_dAs : &s->tm_dBs, nullptr};
-            SNO_TRY(ge::sno_tc_layer(m, ta, s->num_sms, st));
-            std::swap(dv, dnext);
-            continue;
-        }
-        // pointwise path weights
-        if ((rc = weight_grad(s, s->v[l], C, C, dpre, C, R, Gd + o.w, Gd + o.b)) != GE_OK)
+            SNO_TRY(ge::sno_tc_grad(&s->tm_v[l], dv == s->dB ? &s->tm_dB : &s->tm_dA, tg, C, s->num_sms, st));
+        } else if ((rc = weight_grad(s, s->v[l], C, C, dpre, C, R, Gd + o.w, Gd + o.b)) != GE_OK) {
             return rc;
+        }
         // spectral path: dy[b] = G^T dpre[b]
         g = gemm(G, 1, 2 * M, dpre, C, 1, s->y, C, 2 * M, C, n);
         g.sA = 0;
@@ -509,13 +490,21 @@ ge_status backward(ge_sno *s, int B)
         g.sC = 2LL * M * C;
         SNO_TRY(ge::sno_gemm(act_fmt(g, bf), B, s->split, st));
         // dWspec_m = vh[:, m]^T dy[:, m]  (FP32)
-        g = gemm(s->vh[l], 1, 2LL * M * C, s->y, 2LL * M * C, 1, s->dwspec, 2 * C, 2 * C, 2 * C, B);
-        g.sA = 2 * C;
-        g.sB = 2 * C;
-        g.sC = 4LL * C * C;
-        act_fmt(g, bf).out_bf16 = 0;
-        SNO_TRY(ge::sno_gemm(g, M, s->split, st));
-        SNO_TRY(ge::sno_spec_reduce(s->dwspec, Gd + o.rr, Gd + o.ri, M, C, st));
+        if (tc) {
+            ge::SnoTcGradArgs ts = tg;
+            ts.rows = B;
+            ts.drr = Gd + o.rr;
+            ts.dri = Gd + o.ri;
+            SNO_TRY(ge::sno_tc_grad_spec(&s->tm_vh[l], &s->tm_dy, ts, M, st));
+        } else {
+            g = gemm(s->vh[l], 1, 2LL * M * C, s->y, 2LL * M * C, 1, s->dwspec, 2 * C, 2 * C, 2 * C, B);
+            g.sA = 2 * C;
+            g.sB = 2 * C;
+            g.sC = 4LL * C * C;
+            act_fmt(g, bf).out_bf16 = 0;
+            SNO_TRY(ge::sno_gemm(g, M, s->split, st));
+            SNO_TRY(ge::sno_spec_reduce(s->dwspec, Gd + o.rr, Gd + o.ri, M, C, st));
+        }
         // dvh[:, m] = dy[:, m] Wspec_m^T
         g = gemm(s->y, 2LL * M * C, 1, ws, 1, 2 * C, s->dvh, 2LL * M * C, B, 2 * C, 2 * C);
         g.sA = 2 * C;
@@ -682,9 +671,6 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
     e = e ? e : alloc_bytes(&s->wt, 2LL * layers * C * C);
     e = e ? e : alloc_bytes(&s->q1t, 2LL * H * C);
     e = e ? e : alloc_bytes(&s->wst, 2LL * layers * M * 4 * C * C);
-    e = e ? e : alloc_bytes(&s->ws, 2LL * layers * M * 4 * C * C);
-    e = e ? e : alloc_bytes(&s->FT16, 2 * 2 * M * n);
-    e = e ? e : alloc_bytes(&s->GT16, 2 * 2 * M * n);
     e = e ? e : alloc_bytes(reinterpret_cast<void **>(&s->err), 256);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(s->err, 0, 256, s->stream);
@@ -714,24 +700,10 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
         s->tm_vh.resize(layers);
         for (int l = 0; l < layers && ok; ++l)
             ok = bf16_map(&s->tm_vh[l], s->vh[l], max_batch, 2 * modes * width, 64, 128);
-        // training: the same kernels on the transposed operands and the gradients
-        ok = ok && bf16_map(&s->tm_ft, s->FT16, n, 2 * modes, 2 * modes, 128) &&
-             bf16_map(&s->tm_gt, s->GT16, 2 * modes, n, 64, 2 * modes) &&
-             bf16_map(&s->tm_ws, s->ws, (long long)layers * modes * 2 * width, 2 * width, 64, 128) &&
-             bf16_map(&s->tm_dy, s->y, max_batch, 2 * modes * width, 64, 128) &&
-             bf16_map(&s->tm_dvh, s->dvh, (long long)max_batch * 2 * modes, width, width, 2 * modes) &&
+        // weight gradients
+        ok = ok && bf16_map(&s->tm_dy, s->y, max_batch, 2 * modes * width, 64, 128) &&
              bf16_map(&s->tm_dA, s->dA, R, width, width, 128) && bf16_map(&s->tm_dB, s->dB, R, width, width, 128) &&
-             bf16_map(&s->tm_dAs, s->dA, R, width, 32, 32) && bf16_map(&s->tm_dBs, s->dB, R, width, 32, 32);
-        // dhpre as rows of H, Q1 as stored, the stores of h and the pre-activations
-        ok = ok && bf16_map(&s->tm_dAh, s->dA, R, hidden, 64, 128) &&
-             bf16_map(&s->tm_q1, static_cast<char *>(s->pw16) + 2 * s->off_q1, width, hidden, 64, 64) &&
-             bf16_map(&s->tm_h, s->h, R, hidden, 32, 32) && bf16_map(&s->tm_hpre, s->hpre, R, hidden, 32, 32);
-        s->tm_pre.resize(layers);
-        for (int l = 0; l < layers && ok; ++l)
-            ok = bf16_map(&s->tm_pre[l], s->pre[l], R, width, 32, 32);
-        s->tm_w.resize(layers);
-        for (int l = 0; l < layers && ok; ++l)
-            ok = bf16_map(&s->tm_w[l], static_cast<char *>(s->pw16) + 2 * s->lay[l].w, width, width, width, 64);
+             bf16_map(&s->tm_dAh, s->dA, R, hidden, 64, 128);
         s->tc_ready = ok;
     }
     // DFT bases: F[2m][j] = cos(2 pi m j / n), F[2m+1][j] = -sin(...);
@@ -765,15 +737,10 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
         p[s->off_q1 + i] = (float)rng.uniform(1.0 / std::sqrt((double)C));
     for (long long i = 0; i < H; ++i)
         p[s->off_q2 + i] = (float)rng.uniform(1.0 / std::sqrt((double)H));
-    std::vector<uint16_t> F16(F.size()), G16(Gm.size()), FT16(F.size()), GT16(Gm.size());
+    std::vector<uint16_t> F16(F.size()), G16(Gm.size());
     for (size_t i = 0; i < F.size(); ++i) {
         F16[i] = bf16_bits(F[i]);
         G16[i] = bf16_bits(Gm[i]);
-    }
-    for (int k = 0; k < 2 * modes; ++k)
-        for (int j = 0; j < n; ++j) {
-            FT16[(size_t)j * 2 * modes + k] = F16[(size_t)k * n + j];
-            GT16[(size_t)k * n + j] = G16[(size_t)j * 2 * modes + k];
     }
     e = cudaMemcpyAsync(s->F, F.data(), sizeof(float) * F.size(), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess)
@@ -782,10 +749,6 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
         e = cudaMemcpyAsync(s->F16, F16.data(), 2 * F16.size(), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->G16, G16.data(), 2 * G16.size(), cudaMemcpyHostToDevice, s->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(s->FT16, FT16.data(), 2 * FT16.size(), cudaMemcpyHostToDevice, s->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(s->GT16, GT16.data(), 2 * GT16.size(), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->params, p.data(), sizeof(float) * p.size(), cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess)

@@ -68,13 +68,10 @@ cudaError_t sno_gemm(const GemmArgs &g, int batch, bool split, cudaStream_t s);
 //               MN-major), a2 = v [rows][C] (box 64 x 128, 128-byte swizzle),
 //               b2 = W^T of all layers [L * C][C] (box 64 x 64, 128-byte
 //               swizzle);
-//   projection: a2 = v as above, b2 = Q1^T [H][C] (box 64 x 128);
-//   in training also store maps (box 32 x 32, 64-byte swizzle) of the value
-//   before GELU (pre) and, for the projection, of the hidden layer (out).
+//   projection: a2 = v as above, b2 = Q1^T [H][C] (box 64 x 128).
 struct SnoTcMaps {
     const void *a1, *b1, *a2, *b2;
     const void *out;  // layer: store map of the next activation [rows][C] (box 32 x 32, 64-byte swizzle)
-    const void *pre;  // or NULL
 };
 struct SnoTcArgs {
     long long n_tiles;      // rows / 128
@@ -88,9 +85,7 @@ struct SnoTcArgs {
     void *out;              // layer: next activation, BF16 [rows][C]; projection: FP32 [rows]
     int *err;               // device error word (GE_ETIMEOUT on a wait that gave up)
     long long limit;        // wait limit in SM cycles
-    int keep;               // training forward: also write pre (layer) or hidden layer and pre (projection)
     int early;              // start under the end of the kernel before (see launch_early)
-    const void *dg;         // layer: multiply by GELU' of these BF16 [rows][C], or NULL
 };
 cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s);
 cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s);
@@ -102,8 +97,6 @@ cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a,
 // map_vh over vh [batch rows][2M * 2C] (box 64 x 128, 128-byte swizzle),
 // map_wst over the K-major spectral weights Wspec_m^T of all layers
 // [L * M * 2C][2C] (box 64 x 128); grid = (ceil(batch / 128), modes).
-// sno_tc_rows is the same product with one "mode" and 64 output columns:
-// y [rows][64] = x [rows][128] B^T, B [64][128] (box 64 x 64).
 struct SnoTcMixArgs {
     int batch;           // problems (rows of vh and y)
     int b_row0;          // first row of this layer's block of map_wst (l * M * 2C)
@@ -114,7 +107,6 @@ struct SnoTcMixArgs {
     int early;           // as in SnoTcArgs
 };
 cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s);
-cudaError_t sno_tc_rows(const void *map_x, const void *map_b, const SnoTcMixArgs &a, cudaStream_t s);
 // Weight gradients on the tensor cores, dW = X^T dY over the rows of both:
 //   sno_tc_grad:  X [rows][64] (map_x, box 64 x 128), dY [rows][cols] with
 //       cols = 64 or 128 (map_y, box 64 x 128); adds to dw [64][cols] and
@@ -158,9 +150,6 @@ struct SnoSums {
 long long sno_sum_floats(int cols);
 int sno_sum_tickets(int cols);
 cudaError_t sno_colsum(const SnoSums &a, int bf16, cudaStream_t s);
-// out[i] = u0[i] + q2[0] + sum_j h[i, j] q[j].
-cudaError_t sno_row_dot(const void *h, const void *q, const float *q2, const float *u0, float *out, long long rows, int cols,
-                        int bf16, cudaStream_t s);
 cudaError_t sno_rel_l2(const float *pred, const float *target, void *dpred, float *loss, int n, int batch, int bf16,
                        cudaStream_t s);
 cudaError_t sno_adam(float *p, const float *g, float *m, float *v, long long n, float lr, float b1, float b2,

@@ -562,6 +562,10 @@ __device__ __forceinline__ void epilogue(const GemmArgs &g, int bz, int ks_n, in
 template <bool SPLIT, int MODE>
 __global__ void __launch_bounds__(NT, MODE == 0 ? 1 : 4) gemm_kernel(GemmArgs g)
 {
+    // launched early (launch_gemm): set up under the kernel before, whose results
+    // nothing above this may touch
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     constexpr int NS = (SPLIT || MODE == 2) ? 2 : 1;  // split parts, or pipeline stages
     __shared__ __align__(16) __nv_bfloat16 As[NS][TILE];
     __shared__ __align__(16) __nv_bfloat16 Bs[NS][TILE];
@@ -844,42 +848,6 @@ __global__ void __launch_bounds__(256) colsum_kernel(const SnoSums a)
             v += __shfl_xor_sync(0xffffffffu, v, o);
         if (t == 0)
             *a.wtot = v;
-    }
-}
-
-// out[i] = u0[i] + q2[0] + sum_j h[i, j] q[j], a warp per row.  (As a GEMM
-// with one column: 23 us for 65,536 x 128 BF16, now 16 us.)
-template <typename T, bool V>
-__global__ void __launch_bounds__(256) row_dot_kernel(const T *__restrict__ h, const T *__restrict__ q,
-                                                      const float *__restrict__ q2, const float *__restrict__ u0,
-                                                      float *__restrict__ out, long long rows, int cols)
-{
-    constexpr int E = V ? Chunk<T>::E : 1;
-    const int lane = threadIdx.x & 31;
-    const long long step = (long long)gridDim.x * 8;
-    // the lane's first weights stay in registers (all of them up to 32 E columns)
-    float w[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-        w[e] = lane * E + e < cols ? to_f(q[lane * E + e]) : 0.0f;
-#pragma unroll 4
-    for (long long i = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); i < rows; i += step) {
-        float s = 0.0f;
-        for (int j = lane * E; j < cols; j += 32 * E) {
-            float a[E];
-            if constexpr (V)
-                Chunk<T>::load(h + i * cols + j, a);
-            else
-                a[0] = to_f(h[i * cols + j]);
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                s = fmaf(a[e], j == lane * E ? w[e] : to_f(q[j + e]), s);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0)
-            out[i] = u0[i] + q2[0] + s;
     }
 }
 
@@ -1278,6 +1246,23 @@ int vec_ok(const void *X, long long s_r, long long s_k, int rmax, int kdim, long
 
 }  // namespace
 
+// With programmatic stream serialization: a training pass is a chain of short
+// GEMMs, and a launch costs it 3 to 4 us of idle device.  The results are the
+// same bits.
+static cudaError_t launch_gemm(void (*kernel)(GemmArgs), dim3 grid, cudaStream_t s, const GemmArgs &g)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(NT);
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, g);
+}
+
 cudaError_t sno_gemm(const GemmArgs &g0, int batch, bool split, cudaStream_t s)
 {
     if (g0.M <= 0 || g0.N <= 0 || batch <= 0)
@@ -1301,12 +1286,10 @@ cudaError_t sno_gemm(const GemmArgs &g0, int batch, bool split, cudaStream_t s)
               (batch == 1 || (g.sC % 2 == 0 && g.sC0 % 2 == 0 && g.sDg % 2 == 0 && g.sAct % 2 == 0));
     dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, batch * ks);
     if (g.in_bf16)
-        gemm_kernel<false, 2><<<grid, NT, 0, s>>>(g);
-    else if (split)
-        vec ? gemm_kernel<true, 1><<<grid, NT, 0, s>>>(g) : gemm_kernel<true, 0><<<grid, NT, 0, s>>>(g);
-    else
-        vec ? gemm_kernel<false, 1><<<grid, NT, 0, s>>>(g) : gemm_kernel<false, 0><<<grid, NT, 0, s>>>(g);
-    return cudaGetLastError();
+        return launch_gemm(gemm_kernel<false, 2>, grid, s, g);
+    if (split)
+        return launch_gemm(vec ? gemm_kernel<true, 1> : gemm_kernel<true, 0>, grid, s, g);
+    return launch_gemm(vec ? gemm_kernel<false, 1> : gemm_kernel<false, 0>, grid, s, g);
 }
 
 cudaError_t sno_features(const float *u0, const float *r, const float *bl, const float *br, void *f, int batch, int n,
@@ -1369,20 +1352,6 @@ cudaError_t pick_colsum(const SnoSums &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_row_dot(const void *h, const void *q, const float *q2, const float *u0, float *out, long long rows,
-                           int cols, cudaStream_t s)
-{
-    const T *ht = static_cast<const T *>(h), *qt = static_cast<const T *>(q);
-    const bool v = cols % Chunk<T>::E == 0 && (reinterpret_cast<uintptr_t>(h) & 15) == 0;
-    const int grid = grid_for(rows * 8);
-    if (v)
-        row_dot_kernel<T, true><<<grid, 256, 0, s>>>(ht, qt, q2, u0, out, rows, cols);
-    else
-        row_dot_kernel<T, false><<<grid, 256, 0, s>>>(ht, qt, q2, u0, out, rows, cols);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
 long long sno_sum_floats(int cols) { return (long long)kSumBlocks * (5LL * cols + 1); }
@@ -1391,13 +1360,6 @@ int sno_sum_tickets(int cols) { return (cols + 31) / 32; }
 cudaError_t sno_colsum(const SnoSums &a, int bf16, cudaStream_t s)
 {
     return bf16 ? pick_colsum<__nv_bfloat16>(a, s) : pick_colsum<float>(a, s);
-}
-
-cudaError_t sno_row_dot(const void *h, const void *q, const float *q2, const float *u0, float *out, long long rows, int cols,
-                        int bf16, cudaStream_t s)
-{
-    return bf16 ? launch_row_dot<__nv_bfloat16>(h, q, q2, u0, out, rows, cols, s)
-                : launch_row_dot<float>(h, q, q2, u0, out, rows, cols, s);
 }
 
 cudaError_t sno_rel_l2(const float *pred, const float *target, void *dpred, float *loss, int n, int batch, int bf16,

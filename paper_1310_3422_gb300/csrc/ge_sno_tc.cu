@@ -1,4 +1,5 @@
-// ge_sno_tc.cu -- the surrogate's GEMMs on the fifth-generation
+// ge_sno_tc.cu -- the surrogate's inference GEMMs, and the weight gradients of
+// its training, on the fifth-generation
 // tensor cores: tcgen05.mma with the accumulator in tensor memory (TMEM),
 // operands staged in shared memory by 2D TMA copies, and the epilogue fused.
 // The paper has no counterpart (the surrogate is a deployment variant of the
@@ -11,9 +12,7 @@
 //       inverse truncated DFT, y [2M][C] the mode-mixed spectrum of the
 //       tile's problem, v the tile's activations, W [C][C] the pointwise
 //       weights.  Two products accumulate into one TMEM tile: K = 2M = 32
-//       (G y) and K = C = 64 (v W).  In training it also writes pre; the
-//       layer's backward pass is the same kernel on other operands,
-//       (F^T dvh + dpre W^T) * GELU'(pre of the layer below);
+//       (G y) and K = C = 64 (v W).
 //   projection (MODE 1): out = u0 + q2 + sum_h GELU(v Q1 + q1)_h Q2_h, one
 //       FP32 value per row; the hidden layer (N = H = 128) lives in TMEM
 //       only, and each thread sums its row in a fixed order;
@@ -106,23 +105,9 @@ __device__ __forceinline__ float gelu_hw(float x)
     return 0.5f * x * (1.0f + t);
 }
 
-// Its derivative.
-__device__ __forceinline__ float gelu_grad_hw(float x)
-{
-    float t;
-    asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(x * (kGeluK0 + kGeluK0K1 * x * x)));
-    return 0.5f * (1.0f + t) + 0.5f * x * (1.0f - t * t) * (kGeluK0 + 3.0f * kGeluK0K1 * x * x);
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b)
 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);  // .x = a (low half), .y = b
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
-__device__ __forceinline__ uint32_t half_bf16x2(uint32_t x)
-{
-    const __nv_bfloat162 h = __hmul2(*reinterpret_cast<const __nv_bfloat162 *>(&x), __floats2bfloat162_rn(0.5f, 0.5f));
     return *reinterpret_cast<const uint32_t *>(&h);
 }
 
@@ -151,7 +136,7 @@ __device__ __forceinline__ void after_previous()
 constexpr int kTcThreads = 160;
 constexpr int kTileM = 128;
 
-template <int MODE, bool TRAIN>
+template <int MODE>
 struct TcShape {
     static constexpr int N = MODE == 0 ? 64 : 128;                  // output columns (TMEM columns per stage)
     static constexpr uint32_t kA2 = kTileM * 128;                    // v tile: 128 rows x 64 BF16
@@ -166,24 +151,20 @@ struct TcShape {
     static constexpr int kAccs = MODE == 0 ? 2 : 1;
     static constexpr uint32_t kTmemCols = kAccs * N;
     // layer: per epilogue warp a 2 KB staging buffer of its 32 output rows x
-    // 32 columns (64-byte swizzle), written to global memory by a TMA store;
-    // in training a second one, for the value before GELU, in both modes
-    static constexpr uint32_t kOut = TRAIN ? 8 * 2048 : MODE == 0 ? 4 * 2048 : 0;
+    // 32 columns (64-byte swizzle), written to global memory by a TMA store
+    static constexpr uint32_t kOut = MODE == 0 ? 4 * 2048 : 0;
     static constexpr int kSmem = (int)(2 * kStage + kB2 + kOut + 1024);
 };
 
-// TRAIN: the training epilogues (P.keep, P.dg, no bias); inference keeps its
-// own instance, 8% faster than one that decides at run time.
-template <int MODE, bool TRAIN>
+template <int MODE>
 __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constant__ CUtensorMap tmA1,
                                                             const __grid_constant__ CUtensorMap tmB1,
                                                             const __grid_constant__ CUtensorMap tmA2,
                                                             const __grid_constant__ CUtensorMap tmB2,
                                                             const __grid_constant__ CUtensorMap tmOut,
-                                                            const __grid_constant__ CUtensorMap tmPre,
                                                             const __grid_constant__ SnoTcArgs P)
 {
-    using S = TcShape<MODE, TRAIN>;
+    using S = TcShape<MODE>;
     constexpr int N = S::N;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>(
@@ -215,7 +196,7 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
     tc_fence_after();
     after_previous();
     for (int i = t; i < N; i += kTcThreads) {
-        s_bias[i] = !TRAIN || P.bias ? P.bias[i] : 0.0f;
+        s_bias[i] = P.bias[i];
         // the projection keeps Q2 / 2 (exact): GELU's factor 1/2 moves onto it
         s_q2[i] = MODE == 1 ? 0.5f * P.q2w[i] : 0.0f;
     }
@@ -300,14 +281,6 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
             const int s = (int)(i & 1);
             const long long g = (long long)blockIdx.x + i * gridDim.x;
             const long long row = g * kTileM + warp * 32 + lane;
-            uint4 dg[TRAIN && MODE == 0 ? 8 : 1];
-            if (TRAIN && MODE == 0 && P.dg) {
-                // under the tile's loads and MMAs
-                const uint4 *d = reinterpret_cast<const uint4 *>(P.dg) + row * (N / 8);
-#pragma unroll
-                for (int q = 0; q < (TRAIN && MODE == 0 ? 8 : 1); ++q)
-                    dg[q] = d[q];
-            }
             const bool ok = bar_wait(&mma_done[s], (uint32_t)((i >> 1) & 1), P.limit, &s_abort);
             if (__any_sync(0xffffffffu, !ok)) {
                 if (lane == 0 && !s_abort) {
@@ -335,20 +308,11 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const uint32_t *r = h ? r1 : r0;
-                    uint32_t w[16], keep[16];
+                    uint32_t w[16];
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
                         float a = __uint_as_float(r[2 * c]) + s_bias[32 * h + 2 * c];
                         float b = __uint_as_float(r[2 * c + 1]) + s_bias[32 * h + 2 * c + 1];
-                        if (TRAIN && P.dg) {
-                            const uint4 &x = dg[TRAIN ? 4 * h + (c >> 2) : 0];
-                            const uint32_t y = (c & 3) == 0 ? x.x : (c & 3) == 1 ? x.y : (c & 3) == 2 ? x.z : x.w;
-                            const float2 d = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&y));
-                            a *= gelu_grad_hw(d.x);
-                            b *= gelu_grad_hw(d.y);
-                        } else if (TRAIN && P.keep) {
-                            keep[c] = pack_bf16(a, b);
-                        }
                         if (P.gelu) {
                             a = gelu_hw(a);
                             b = gelu_hw(b);
@@ -360,14 +324,10 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                         bulk_wait_read0();
                     __syncwarp();
                     stage_rows(stg, lane, w);
-                    if (TRAIN && P.keep)
-                        stage_rows(stg + 4 * 2048, lane, keep);
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) {
                         tma_store_2d(&tmOut, stg, 32 * h, (int)row0);
-                        if (TRAIN && P.keep)
-                            tma_store_2d(&tmPre, stg + 4 * 2048, 32 * h, (int)row0);
                         bulk_commit();
                     }
                 }
@@ -389,7 +349,6 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                     tmem_ld32(taddr + 64 * h, r[0]);
                     tmem_ld32(taddr + 64 * h + 32, r[1]);
                     tmem_wait_ld();
-                    uint32_t wp[TRAIN ? 2 : 1][16], wh[TRAIN ? 2 : 1][16];
 #pragma unroll
                     for (int c = 0; c < 64; c += 2) {
                         const int col = 64 * h + c;
@@ -403,35 +362,7 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
                         float t0, t1;
                         asm("tanh.approx.f32 %0, %1;" : "=f"(t0) : "f"(af.x));
                         asm("tanh.approx.f32 %0, %1;" : "=f"(t1) : "f"(af.y));
-                        uint64_t x2 = f2_fma(x, f2(t0, t1), x);  // 2 GELU(x)
-                        if (TRAIN) {
-                            // h is stored in BF16, and the output is the product
-                            // with what is stored (the backward pass uses it)
-                            const float2 xf = f2_split(x), hf = f2_split(x2);
-                            const uint32_t hb = pack_bf16(hf.x, hf.y);
-                            wp[TRAIN ? c >> 5 : 0][(c & 31) >> 1] = pack_bf16(xf.x, xf.y);
-                            wh[TRAIN ? c >> 5 : 0][(c & 31) >> 1] = half_bf16x2(hb);
-                            x2 = f2(__uint_as_float(hb << 16), __uint_as_float(hb & 0xFFFF0000u));
-                        }
-                        part[(c >> 1) & 3] = f2_fma(x2, f2(wq.x, wq.y), part[(c >> 1) & 3]);
-                    }
-                    if (TRAIN) {
-                        unsigned char *stg = sm + 2 * S::kStage + S::kB2 + warp * 2048;
-#pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            if (lane == 0)
-                                bulk_wait_read0();
-                            __syncwarp();
-                            stage_rows(stg, lane, wh[TRAIN ? q : 0]);
-                            stage_rows(stg + 4 * 2048, lane, wp[TRAIN ? q : 0]);
-                            fence_async_smem();
-                            __syncwarp();
-                            if (lane == 0) {
-                                tma_store_2d(&tmOut, stg, 64 * h + 32 * q, (int)(g * kTileM + warp * 32));
-                                tma_store_2d(&tmPre, stg + 4 * 2048, 64 * h + 32 * q, (int)(g * kTileM + warp * 32));
-                                bulk_commit();
-                            }
-                        }
+                        part[(c >> 1) & 3] = f2_fma(f2_fma(x, f2(t0, t1), x), f2(wq.x, wq.y), part[(c >> 1) & 3]);
                     }
                 }
                 const float2 accf = f2_split(f2_add(f2_add(part[0], part[1]), f2_add(part[2], part[3])));
@@ -445,8 +376,8 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
             }
         }
     }
-    // the output stores have landed before the CTA exits
-    if ((MODE == 0 || TRAIN) && warp < 4 && lane == 0)
+    // the layer's output stores have landed before the CTA exits
+    if (MODE == 0 && warp < 4 && lane == 0)
         bulk_wait0();
     tc_fence_before();
     __syncthreads();
@@ -471,7 +402,7 @@ __global__ void __launch_bounds__(kTcThreads) sno_tc_kernel(const __grid_constan
 // the MMAs, commits); two accumulators, so the next problem's MMAs run
 // under the previous one's write-out.  Bounded waits as in sno_tc_kernel.
 // Two stages let four CTAs share an SM, the choice for many problems; with at
-// most one problem per SM (a training batch) a CTA is alone and the latency
+// most one problem per SM a CTA is alone and the latency
 // of its loads counts, so all 8 chunks of 1024 points are in flight (64 problems: 10.9 -> 9.8 us).
 constexpr int kDftThreads = 64;
 constexpr uint32_t kDftAtom = 32 * 128;              // F rows of one 64-point half of a chunk
@@ -628,7 +559,7 @@ __global__ void __launch_bounds__(kDftThreads) sno_tc_dft_kernel(const __grid_co
 // the [2C][2C] real form of the complex mode weights.  A CTA takes 128
 // problems of one mode: A = those problems' vh[., m] rows (K-major, two
 // 64-wide 128-byte-swizzled boxes), B = Wspec_m^T [N][K] (K-major, written so
-// by sno_prepare; Wspec_m itself in the backward pass), one 128 x 128 FP32
+// by sno_prepare), one 128 x 128 FP32
 // accumulator in TMEM after 8 MMAs of K = 16.  Thread 0 issues the four loads
 // and the MMAs; the four warps then read back their 32 rows each and write
 // y[b, m] as BF16 (rows past the batch are not written).
@@ -636,12 +567,11 @@ constexpr int kMixThreads = 128;
 constexpr uint32_t kMixHalf = 128 * 128;  // one 64-wide box of 128 rows
 constexpr int kMixSmem = (int)(4 * kMixHalf) + 1024;
 
-template <int N>
 __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                  const __grid_constant__ CUtensorMap tmB,
                                                                  const __grid_constant__ SnoTcMixArgs P)
 {
-    constexpr uint32_t idesc = idesc_bf16(128, N);
+    constexpr uint32_t idesc = idesc_bf16(128, 128);
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -668,7 +598,7 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
     after_previous();
     const uint32_t tbase = tmem_base_sh;
     if (t == 0) {
-        bar_expect_tx(&full, 2 * kMixHalf + 2 * N * 128);
+        bar_expect_tx(&full, 4 * kMixHalf);
         tma_2d(sa, &tmA, m * 128, row0, &full);
         tma_2d(sa + kMixHalf, &tmA, m * 128 + 64, row0, &full);
         tma_2d(sb, &tmB, 0, P.b_row0 + m * 128, &full);
@@ -701,9 +631,9 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
         tc_fence_after();
         const int b = row0 + warp * 32 + lane;
         uint4 *dst = reinterpret_cast<uint4 *>(static_cast<unsigned char *>(P.y) +
-                                               ((long long)b * P.row_elems + (long long)m * N) * 2);
+                                               ((long long)b * P.row_elems + (long long)m * 128) * 2);
 #pragma unroll
-        for (int h = 0; h < N / 32; ++h) {
+        for (int h = 0; h < 4; ++h) {
             uint32_t r[32];
             tmem_ld32(tbase + ((uint32_t)(warp * 32) << 16) + (uint32_t)(32 * h), r);
             tmem_wait_ld();
@@ -942,18 +872,18 @@ cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, int threads, int 
     return cudaLaunchKernelEx(&c, kernel, args...);
 }
 
-template <int MODE, bool TRAIN>
+template <int MODE>
 cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
-    using S = TcShape<MODE, TRAIN>;
+    using S = TcShape<MODE>;
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(sno_tc_kernel<MODE, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(sno_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              S::kSmem);
         // the largest shared-memory carve-out, so that as many CTAs fit as
         // TMEM allows (3 layer CTAs of 74 KB need about 225 KB)
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(sno_tc_kernel<MODE, TRAIN>, cudaFuncAttributePreferredSharedMemoryCarveout,
+            e = cudaFuncSetAttribute(sno_tc_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                      cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess)
             return e;
@@ -966,7 +896,7 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
     if (per_sm == 0) {
         cudaFuncAttributes fa{};
         int dev = 0, sm_bytes = 0, reserve = 0;
-        cudaError_t e = cudaFuncGetAttributes(&fa, sno_tc_kernel<MODE, TRAIN>);
+        cudaError_t e = cudaFuncGetAttributes(&fa, sno_tc_kernel<MODE>);
         if (e == cudaSuccess)
             e = cudaGetDevice(&dev);
         if (e == cudaSuccess)
@@ -987,16 +917,15 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
         grid = a.n_tiles;
     if (grid < 1)
         return cudaSuccess;
-    if (!m.a2 || !m.b2 || (MODE == 0 && (!m.a1 || !m.b1 || !m.out)) || (TRAIN && a.keep && (!m.out || !m.pre)))
+    if (!m.a2 || !m.b2 || (MODE == 0 && (!m.a1 || !m.b1 || !m.out)))
         return cudaErrorInvalidValue;
     // the projection has no first product and no output map: those
     // parameters repeat a2
     const CUtensorMap *a1 = static_cast<const CUtensorMap *>(MODE == 0 ? m.a1 : m.a2);
     const CUtensorMap *b1 = static_cast<const CUtensorMap *>(MODE == 0 ? m.b1 : m.a2);
-    const CUtensorMap *o = static_cast<const CUtensorMap *>(MODE == 0 || TRAIN ? m.out : m.a2);
-    const CUtensorMap *pre = static_cast<const CUtensorMap *>(TRAIN && m.pre ? m.pre : m.a2);
-    return launch_early(sno_tc_kernel<MODE, TRAIN>, dim3((unsigned)grid), kTcThreads, S::kSmem, s, a.early, *a1, *b1,
-                        *static_cast<const CUtensorMap *>(m.a2), *static_cast<const CUtensorMap *>(m.b2), *o, *pre, a);
+    const CUtensorMap *o = static_cast<const CUtensorMap *>(MODE == 0 ? m.out : m.a2);
+    return launch_early(sno_tc_kernel<MODE>, dim3((unsigned)grid), kTcThreads, S::kSmem, s, a.early, *a1, *b1,
+                        *static_cast<const CUtensorMap *>(m.a2), *static_cast<const CUtensorMap *>(m.b2), *o, a);
 }
 
 template <int ST>
@@ -1034,24 +963,6 @@ cudaError_t launch_dft(const CUtensorMap &f, const CUtensorMap &v, const SnoTcAr
     return launch_early(sno_tc_dft_kernel<ST>, dim3((unsigned)grid), kDftThreads, dft_smem(ST), s, a.early, f, v, a);
 }
 
-template <int N>
-cudaError_t launch_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s)
-{
-    static bool ready = false;
-    if (!ready) {
-        cudaError_t e = cudaFuncSetAttribute(sno_tc_mix_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMixSmem);
-        if (e != cudaSuccess)
-            return e;
-        ready = true;
-    }
-    if (!map_vh || !map_wst || modes < 1 || a.batch < 0)
-        return cudaErrorInvalidValue;
-    if (a.batch == 0)
-        return cudaSuccess;
-    const dim3 grid((unsigned)((a.batch + 127) / 128), (unsigned)modes);
-    return launch_early(sno_tc_mix_kernel<N>, grid, kMixThreads, kMixSmem, s, a.early, *static_cast<const CUtensorMap *>(map_vh),
-                        *static_cast<const CUtensorMap *>(map_wst), a);
-}
 
 template <int KIND>
 cudaError_t launch_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, dim3 grid, cudaStream_t s)
@@ -1077,12 +988,12 @@ cudaError_t launch_grad(const void *map_x, const void *map_y, const SnoTcGradArg
 
 cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
-    return a.keep || a.dg || !a.bias ? launch_tc<0, true>(m, a, sms, s) : launch_tc<0, false>(m, a, sms, s);
+    return launch_tc<0>(m, a, sms, s);
 }
 
 cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
 {
-    return a.keep ? launch_tc<1, true>(m, a, sms, s) : launch_tc<1, false>(m, a, sms, s);
+    return launch_tc<1>(m, a, sms, s);
 }
 
 cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a, int sms, cudaStream_t s)
@@ -1095,12 +1006,20 @@ cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a,
 
 cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s)
 {
-    return launch_mix<128>(map_vh, map_wst, a, modes, s);
-}
-
-cudaError_t sno_tc_rows(const void *map_x, const void *map_b, const SnoTcMixArgs &a, cudaStream_t s)
-{
-    return launch_mix<64>(map_x, map_b, a, 1, s);
+    static bool ready = false;
+    if (!ready) {
+        cudaError_t e = cudaFuncSetAttribute(sno_tc_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMixSmem);
+        if (e != cudaSuccess)
+            return e;
+        ready = true;
+    }
+    if (!map_vh || !map_wst || modes < 1 || a.batch < 0)
+        return cudaErrorInvalidValue;
+    if (a.batch == 0)
+        return cudaSuccess;
+    const dim3 grid((unsigned)((a.batch + 127) / 128), (unsigned)modes);
+    return launch_early(sno_tc_mix_kernel, grid, kMixThreads, kMixSmem, s, a.early, *static_cast<const CUtensorMap *>(map_vh),
+                        *static_cast<const CUtensorMap *>(map_wst), a);
 }
 
 cudaError_t sno_tc_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, int cols, int sms, cudaStream_t s)

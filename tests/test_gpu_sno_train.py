@@ -1,4 +1,4 @@
-"""Training on the tcgen05 path against the mma.sync path.
+"""Training with the weight gradients on tcgen05 against the mma.sync path.
 
 Both round the same values to BF16 and accumulate in FP32, so the gradients
 differ by the order of the sums and by BF16 roundings that fall the other way
