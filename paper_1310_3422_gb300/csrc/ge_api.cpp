@@ -397,10 +397,12 @@ void release(ge_ctx *c)
 {
     if (!c)
         return;
-    if (c->buf[0] && c->pooled)
-        cudaFreeAsync(c->buf[0], c->stream);  // holds everything
-    else if (c->buf[0])
+    // buf[0] holds everything; a caller may have destroyed its stream already
+    if (c->buf[0] && !(c->pooled && cudaFreeAsync(c->buf[0], c->stream) == cudaSuccess)) {
+        if (c->pooled)
+            cudaGetLastError();
         cudaFree(c->buf[0]);
+    }
     delete c;
 }
 
