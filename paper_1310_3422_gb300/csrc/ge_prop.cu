@@ -1207,8 +1207,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                             acc = 1;
                         }
                     }
-                    if (lane == 0)
-                        tc_commit(&done[g]);
+                    tc_commit_if(leader, &done[g]);
                     __syncwarp();
                 }
                 if (!ok && lane == 0) {
@@ -1521,8 +1520,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
                                   bd0 + (uint32_t)__shfl_sync(0xffffffffu, p.y, 0), __shfl_sync(0xffffffffu, p.z, 0),
                                   __shfl_sync(0xffffffffu, p.w, 0), acc);
                 }
-                if (lane == 0)
-                    tc_commit(&done[m][g]);
+                tc_commit_if(leader, &done[m][g]);
                 __syncwarp();
                 committed = (int)((n & 1) << 8) | g;
             }

@@ -145,6 +145,18 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar)
                  : "memory");
 }
 
+// The same from a converged warp, by the lane that issued the MMAs (tc_mma_if):
+// a commit tracks its own thread's only.
+__device__ __forceinline__ void tc_commit_if(bool issue, uint64_t *bar)
+{
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(saddr(bar)),
+        "r"((uint32_t)issue)
+        : "memory");
+}
+
 // 32 consecutive FP32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
 {
