@@ -324,6 +324,9 @@ __device__ __forceinline__ bool tb_tiles(const CUtensorMap *tmap, const TbParams
     // takes the next position while the current tile is computed
     long long k = blockIdx.x;
     if (t == 0 && k < P.n_tiles) {
+        // the buffer may hold the last round's output rows (the caller's
+        // barrier has ordered their threads before this one)
+        fence_proxy_async_smem();
         mbar_arrive_expect_tx(&mbar[it & 1], kTileBytes);
         tma_load_rows(tiles + (it & 1) * kTileBytes, tmap, &mbar[it & 1], (int)(queue_tile(k, P.n_tiles) * ur - hr));
     }

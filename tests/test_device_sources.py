@@ -31,3 +31,13 @@ def test_a_commit_comes_from_the_lane_that_issued_the_products(kernel):
     body = dict(functions(code("ge_prop.cu")))[kernel]
     assert re.search(r"bool leader = elect_one\(\)", body)
     assert re.findall(r"\btc_commit\w*\(\w+", body) == ["tc_commit_if(leader"]
+
+
+def test_a_tile_buffer_is_fenced_before_tma_writes_it_again():
+    """The rounds of a launch use the same two buffers, which threads wrote and
+    read before: a proxy fence between those accesses and the copy, at every load."""
+    loads = [m.start() for m in re.finditer(r"\btma_load_rows\(", code("ge_tb.cu"))]
+    assert len(loads) == 2
+    for at in loads:
+        before = code("ge_tb.cu")[:at]
+        assert re.search(r"fence_proxy_async_smem\(\);\s*mbar_arrive_expect_tx\([^;]*\);\s*$", before)
