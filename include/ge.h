@@ -208,7 +208,11 @@ ge_status ge_sync(ge_ctx *ctx);
  * Errors: GE_EINVAL (NULL ctx, cycles < 0). */
 ge_status ge_debug_stall(ge_ctx *ctx, int64_t cycles);
 
-/* Release the context and its buffers (after finishing its stream's work).
+/* Release the context and its buffers, after waiting for the device: work of
+ * its stream, and of graphs captured from it that run elsewhere, ends first.
+ * The stream itself is not used and may have been destroyed.  Contexts of up
+ * to 64 MB come from a pool that keeps at most as much per device for the
+ * next ones, and none once an allocation of the library fails.
  * NULL is a no-op. */
 void ge_destroy(ge_ctx *ctx);
 

@@ -344,12 +344,12 @@ ge_status run_canonical(ge_ctx *c, int64_t steps)
 
 // A context's memory, from a pool of its own per device: cudaMalloc and
 // cudaFree of 20 MB took 125 us of a one-shot solve's 495.  The pool keeps at
-// most kPoolKeep bytes between contexts, and none when an allocation fails
-// (it is trimmed, and the allocation tried again); larger contexts, and
-// streams that are being captured, use cudaMalloc.
+// most kPoolKeep bytes between contexts, and none once an allocation of the
+// library fails (it is trimmed, and the allocation tried again); larger
+// contexts, and streams that are being captured, use cudaMalloc.
 constexpr size_t kPoolKeep = (size_t)64 << 20;
 
-cudaMemPool_t ctx_pool(int device)
+cudaMemPool_t ctx_pool(int device, bool make)
 {
     static std::mutex lock;
     static cudaMemPool_t pool[64];
@@ -357,7 +357,7 @@ cudaMemPool_t ctx_pool(int device)
     if (device < 0 || device >= 64)
         return nullptr;
     std::lock_guard<std::mutex> hold(lock);
-    if (!tried[device]) {
+    if (!tried[device] && make) {
         tried[device] = true;
         cudaMemPoolProps p{};
         p.allocType = cudaMemAllocationTypePinned;
@@ -379,29 +379,40 @@ cudaMemPool_t ctx_pool(int device)
 cudaError_t ctx_alloc(ge_ctx *c, char **mem, size_t bytes)
 {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    cudaMemPool_t pool = bytes <= kPoolKeep ? ctx_pool(c->device) : nullptr;
+    cudaMemPool_t pool = bytes <= kPoolKeep ? ctx_pool(c->device, true) : nullptr;
     if (pool && cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
-        for (int again = 0; again < 2; ++again) {
-            if (cudaMallocFromPoolAsync(reinterpret_cast<void **>(mem), bytes, pool, c->stream) == cudaSuccess) {
-                c->pooled = true;
-                return cudaSuccess;
-            }
-            cudaGetLastError();
-            cudaMemPoolTrimTo(pool, 0);
+        if (cudaMallocFromPoolAsync(reinterpret_cast<void **>(mem), bytes, pool, c->stream) == cudaSuccess) {
+            c->pooled = true;
+            return cudaSuccess;
         }
+        cudaGetLastError();
     }
-    return cudaMalloc(reinterpret_cast<void **>(mem), bytes);
+    return ge::device_malloc(reinterpret_cast<void **>(mem), bytes);
 }
 
-void release(ge_ctx *c)
+// The context's memory is one allocation, buf[0].  Its stream's work, and a
+// graph captured from it that runs on any other stream, may still use it:
+// cudaFree waits for the device, but not for memory from a pool, so that is
+// waited for here, on the context's device and without touching its stream
+// (the caller may have destroyed it).  idle: nothing of the context can be
+// running, and its stream is the caller's of this very call.
+void release(ge_ctx *c, bool idle = false)
 {
     if (!c)
         return;
-    // buf[0] holds everything; a caller may have destroyed its stream already
-    if (c->buf[0] && !(c->pooled && cudaFreeAsync(c->buf[0], c->stream) == cudaSuccess)) {
-        if (c->pooled)
+    if (c->buf[0] && c->pooled && idle) {
+        if (cudaFreeAsync(c->buf[0], c->stream) != cudaSuccess)
             cudaGetLastError();
-        cudaFree(c->buf[0]);
+    } else if (c->buf[0]) {
+        int dev = c->device;
+        cudaGetDevice(&dev);
+        if (dev != c->device)
+            cudaSetDevice(c->device);
+        // (memory that may be in use is never given back)
+        if (!c->pooled || cudaDeviceSynchronize() == cudaSuccess)
+            cudaFree(c->buf[0]);
+        if (dev != c->device)
+            cudaSetDevice(dev);
     }
     delete c;
 }
@@ -422,6 +433,20 @@ cudaError_t side_stream(int device, cudaStream_t *s)
 }
 
 }  // namespace
+
+cudaError_t ge::device_malloc(void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    int dev = 0;
+    if (e != cudaErrorMemoryAllocation || cudaGetDevice(&dev) != cudaSuccess)
+        return e;
+    cudaMemPool_t pool = ctx_pool(dev, false);
+    if (!pool)
+        return e;
+    cudaGetLastError();
+    cudaMemPoolTrimTo(pool, 0);
+    return cudaMalloc(p, bytes);
+}
 
 extern "C" {
 
@@ -581,7 +606,7 @@ ge_status ge_tune(ge_ctx *c, int64_t steps, int32_t *best_depth)
     const size_t bytes = (size_t)c->n * elem_size(c->prec);
     void *saved = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    cudaError_t e = cudaMalloc(&saved, bytes);
+    cudaError_t e = ge::device_malloc(&saved, bytes);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(saved, c->buf[c->cur], bytes, cudaMemcpyDeviceToDevice, c->stream);
     if (e == cudaSuccess)
@@ -779,7 +804,6 @@ void ge_destroy(ge_ctx *c)
 {
     if (!c)
         return;
-    cudaStreamSynchronize(c->stream);
     release(c);
 }
 
@@ -834,7 +858,7 @@ ge_status ge_solve(int64_t n, double r, double beta_l, double beta_r, ge_precisi
     }
     if (st == GE_OK)
         st = ge_sync(c);
-    ge_destroy(c);
+    release(c, st == GE_OK);
     return st;
 }
 

@@ -408,13 +408,13 @@ ge_status ge_batch_create(ge_batch **out, int32_t n_problems, const int64_t *n, 
     default_shape(b, &b->depth, &b->tile_rows);
     const size_t bytes = (size_t)n_rows * ge::kRowBytes;
     for (int i = 0; i < 2 && e == cudaSuccess; ++i)
-        e = cudaMalloc(&b->buf[i], bytes);
+        e = ge::device_malloc(&b->buf[i], bytes);
     if (e == cudaSuccess)
-        e = cudaMalloc(reinterpret_cast<void **>(&b->row_pid), row_pid.size() * sizeof(int));
+        e = ge::device_malloc(reinterpret_cast<void **>(&b->row_pid), row_pid.size() * sizeof(int));
     if (e == cudaSuccess)
-        e = cudaMalloc(reinterpret_cast<void **>(&b->desc), desc.size() * sizeof(ge::BatchDesc));
+        e = ge::device_malloc(reinterpret_cast<void **>(&b->desc), desc.size() * sizeof(ge::BatchDesc));
     if (e == cudaSuccess)
-        e = cudaMalloc(reinterpret_cast<void **>(&b->err), 256);
+        e = ge::device_malloc(reinterpret_cast<void **>(&b->err), 256);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(b->row_pid, row_pid.data(), row_pid.size() * sizeof(int), cudaMemcpyHostToDevice,
                             b->stream);
@@ -433,9 +433,9 @@ ge_status ge_batch_create(ge_batch **out, int32_t n_problems, const int64_t *n, 
         const int R = (int)std::floor(headroom / std::log2(1.0 + 2.0 * r_max));
         b->R = R < 1 ? 1 : (R > ge::kMaxTableSteps ? ge::kMaxTableSteps : R);
         b->Q = (ge::kMaxTableSteps + b->R - 1) / b->R;
-        e = cudaMalloc(reinterpret_cast<void **>(&b->exps), (size_t)n_problems * b->Q * sizeof(short));
+        e = ge::device_malloc(reinterpret_cast<void **>(&b->exps), (size_t)n_problems * b->Q * sizeof(short));
         if (e == cudaSuccess)
-            e = cudaMalloc(&b->endf, (size_t)kEndfSlots * n_problems * 8);
+            e = ge::device_malloc(&b->endf, (size_t)kEndfSlots * n_problems * 8);
         if (e == cudaSuccess)
             e = ge::batch_exps(b->desc, n_problems, b->R, b->Q, scale_mode(b), b->exps, b->stream);
     }
@@ -489,7 +489,7 @@ ge_status ge_batch_set_kernel(ge_batch *b, ge_kernel kernel)
     // launches in flight still read the scaled form's tables
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e == cudaSuccess && df && !b->df_codes)
-        e = cudaMalloc(reinterpret_cast<void **>(&b->df_codes), (size_t)b->n_problems * sizeof(int));
+        e = ge::device_malloc(reinterpret_cast<void **>(&b->df_codes), (size_t)b->n_problems * sizeof(int));
     if (e == cudaSuccess && df && b->df_blocks_per_sm < 1)
         e = ge::tbb_df_occupancy(&b->df_blocks_per_sm);
     if (e != cudaSuccess)
@@ -503,7 +503,7 @@ ge_status ge_batch_set_kernel(ge_batch *b, ge_kernel kernel)
     if (Q > b->Q) {
         cudaFree(b->exps);
         b->exps = nullptr;
-        e = cudaMalloc(reinterpret_cast<void **>(&b->exps), (size_t)b->n_problems * Q * sizeof(short));
+        e = ge::device_malloc(reinterpret_cast<void **>(&b->exps), (size_t)b->n_problems * Q * sizeof(short));
         if (e != cudaSuccess)
             return bcuda(e, "ge_batch_set_kernel: rescale table");
     }
@@ -596,7 +596,7 @@ ge_status ge_batch_set_persistent(ge_batch *b, int32_t on)
     if (!b || (on != 0 && on != 1))
         return bfail(GE_EINVAL, "ge_batch_set_persistent: NULL plan or value not 0/1");
     if (on && !b->done) {
-        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&b->done), sizeof(int) * (size_t)(b->n_rows + 1));
+        cudaError_t e = ge::device_malloc(reinterpret_cast<void **>(&b->done), sizeof(int) * (size_t)(b->n_rows + 1));
         if (e != cudaSuccess)
             return bcuda(e, "ge_batch_set_persistent");
     }

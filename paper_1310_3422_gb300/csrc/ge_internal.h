@@ -339,6 +339,10 @@ cudaError_t tb_run(const TbTarget &t, const TbParams &base, double growth_lo, bo
 bool tb_plan_rounds(const TbTarget &t, const TbParams &base, double growth_lo, int prec, int cur, int p_first,
                     long long n_mid, bool entry, bool exit, int depth, TbRounds *out);
 
+// cudaMalloc; when the device is out of memory, once more without what the
+// contexts' pool keeps.
+cudaError_t device_malloc(void **p, size_t bytes);
+
 // Record the calling thread's last-failure text (read by ge_last_error()).
 void set_last_error(const char *msg);
 

@@ -621,13 +621,13 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
 
     const long long R = (long long)max_batch * n;
     auto alloc = [&](float **p, long long count) -> cudaError_t {
-        cudaError_t e = cudaMalloc(reinterpret_cast<void **>(p), sizeof(float) * (count > 0 ? count : 1));
+        cudaError_t e = ge::device_malloc(reinterpret_cast<void **>(p), sizeof(float) * (count > 0 ? count : 1));
         if (e == cudaSuccess)
             s->allocs.push_back(*p);
         return e;
     };
     auto alloc_bytes = [&](void **p, long long bytes) -> cudaError_t {
-        cudaError_t e = cudaMalloc(p, (size_t)(bytes > 16 ? bytes : 16));
+        cudaError_t e = ge::device_malloc(p, (size_t)(bytes > 16 ? bytes : 16));
         if (e == cudaSuccess)
             s->allocs.push_back(*p);
         return e;
