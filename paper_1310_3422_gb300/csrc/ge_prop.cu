@@ -1105,9 +1105,12 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                 if ((t & 7) == 0 && u < chunks)
                     s_code[u >> 3] = m;
             }
-            // the rest of the cone: everything that reaches the tile's blocks in k steps
+            // the rest of the cone: everything that reaches the tile's blocks in
+            // k steps, the walls included (tiles leave out what a wall adds
+            // beyond the rows near it, so it counts against their own values)
             int cmax = wmax;
             const long long clo = b0 * kPropBlk - P.k - 2, chi = (b0 + nb) * kPropBlk + P.k + 2;
+            cmax = max(cmax, max(clo <= 0 ? P.wall_l : 0, chi >= P.n ? P.wall_r : 0));
             auto scan = [&](long long a, long long b) {
                 for (long long j = a + t; j < b; j += 4 * kTileConv)
 #pragma unroll
@@ -1594,8 +1597,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
                 if ((tt & 7) == 0 && u < chunks)
                     s_code[m][u >> 3] = q;
             }
+            // the rest of the cone, the walls included
             int cmax = wmax;
             const long long clo = b0 * kPropBlk - P.k - 2, chi = (b0 + nb) * kPropBlk + P.k + 2;
+            cmax = max(cmax, max(clo <= 0 ? P.wall_l : 0, chi >= P.n ? P.wall_r : 0));
             auto scan = [&](long long a, long long b) {
                 for (long long j = a + tt; j < b; j += 4 * kTeam)
 #pragma unroll

@@ -97,6 +97,7 @@ struct PropRun {
     double r, omr, x1, x2, xs;  // entry and exit coefficients
     double fl, fr;              // r beta_l, r beta_r
     double bl, br;
+    int wall_l, wall_r;         // exponent codes of what the walls add (tiles: see code_of)
     int k, p0, pr;              // block steps, start parity, start parity seen from the right wall
     int entry, exit;
     int R;                      // reach of the FP64 taps

@@ -150,6 +150,17 @@ unsigned long long fraction(double hi, double lo)
     return v < 0.0 ? (unsigned long long)w - (unsigned long long)-v : (unsigned long long)w + (unsigned long long)v;
 }
 
+// Exponent code (code_of in ge_prop.cu: 0 for zero, else the biased exponent
+// of the state's type, at least 1) of what a wall adds to a right-hand side.
+int wall_code(double beta, double r, int f64)
+{
+    if (beta == 0.0)
+        return 0;
+    int e = 0;
+    std::frexp(beta * std::max(1.0, r), &e);
+    return f64 ? std::min(std::max(e + 1022, 1), 2046) : std::min(std::max(e + 126, 1), 254);
+}
+
 // Build an operator's arrays: a short chain step by step, then binary powering.
 cudaError_t build_set(PropState *st, const PropTarget &t, PropSet &s, int pr, int hb, cudaStream_t stream)
 {
@@ -362,6 +373,8 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
         a.fr = r * t.beta_r;
         a.bl = t.beta_l;
         a.br = t.beta_r;
+        a.wall_l = wall_code(t.beta_l, r, t.f64);
+        a.wall_r = wall_code(t.beta_r, r, t.f64);
         a.k = s.k;
         a.p0 = p0;
         a.pr = pr;

@@ -215,3 +215,27 @@ def test_two_teams_match_the_tiled_kernel(n, prec, r, steps):
     assert np.array_equal(np.isfinite(got), np.isfinite(want))
     ok = np.isfinite(want)
     assert rel_max(got[ok], want[ok]) <= tol
+
+
+# dot products only; split tiles; whole tiles; and, FP32, two teams a CTA
+@pytest.mark.parametrize("n", [5000, 40001, 1300001])
+@pytest.mark.parametrize("prec,r,steps", [(B.GE_F64, 2.0, 700), (B.GE_F64, 0.7, 2001), (B.GE_F32, 2.0, 2000),
+                                          (B.GE_F32, 4.0, 1800), (B.GE_F32_COMP, 2.0, 2001)])
+def test_a_hot_wall_beside_a_quiet_field(n, prec, r, steps):
+    """What a wall sends into a field of zeros, and into one far below it,
+    arrives block by block down to 2^-86 of the wall value (ge.h: 2^-100; the
+    last standard deviation is cut off with the taps): within the FP64 (1e-10,
+    as above) and FP32 tolerances of each block's largest value."""
+    tol, far = (1e-10, 2.0 ** -86) if prec == B.GE_F64 else (1e-5, 2.0 ** -86)
+    for ground in (0.0, 2.0 ** -60):
+        for left, right in ((1.0, 0.0), (0.0, -1.0)):
+            u0 = ground * np.sin(np.arange(n) * 0.01)
+            u0 = u0.astype(np.float32).astype(np.float64)
+            want = oracle.run(u0, r, left, right, steps)
+            got = auto_run(u0, r, left, right, steps, prec)
+            rows = min(n, 64 * 64)
+            for a in range(0, rows, 64):
+                part = slice(a, a + 64) if left else slice(n - 64 - a, n - a)
+                big = np.max(np.abs(want[part]))
+                if big > far:
+                    assert np.max(np.abs(got[part] - want[part])) <= tol * big, (ground, left, a)
