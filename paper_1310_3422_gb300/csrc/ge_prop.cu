@@ -441,7 +441,7 @@ __global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, cons
     extern __shared__ long long q[];  // [2][kPropQ]
     constexpr int kQ = kPropQ, kMid = kPropRMax + 6;
     __shared__ long long s_sum[2];
-    __shared__ float s_abs[32];
+    __shared__ float s_abs[32][2];
     __shared__ int s_W[8], s_row0[8];
     __shared__ int s_ok;
     const int t = threadIdx.x, RX = R + 4;
@@ -457,17 +457,23 @@ __global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, cons
         float m = 0.0f;
         for (int i = t; i < count; i += 1024)
             m += fabsf((float)x[2 * i]);
+        // the phases alternate over the threads
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
+        for (int o = 16; o > 1; o >>= 1)
             m += __shfl_xor_sync(0xffffffffu, m, o);
-        if ((t & 31) == 0)
-            s_abs[t >> 5] = m;
+        if ((t & 31) < 2)
+            s_abs[t >> 5][t & 1] = m;
     }
     __syncthreads();
-    float abs_sum = s_abs[t & 31];
+    float row_abs[2];  // sums of magnitudes of the two phases' rows
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        abs_sum += __shfl_xor_sync(0xffffffffu, abs_sum, o);  // of both phases: twice a row's
+    for (int p = 0; p < 2; ++p) {
+        row_abs[p] = s_abs[t & 31][p];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            row_abs[p] += __shfl_xor_sync(0xffffffffu, row_abs[p], o);
+    }
+    const float abs_sum = row_abs[0] + row_abs[1];  // twice a row's
     // 126 / max in [2^(ex - 1), 2^ex): the quotient's exponent, one less to be safe of its rounding
     int ex, es;
     frexpf(125.99f / (float)__longlong_as_double((long long)*x_max), &ex);
@@ -492,10 +498,14 @@ __global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, cons
     }
     __syncthreads();
     // the rows' sum is exactly 1, so a constant stays what it is: the taps
-    // share what rounding left in proportion (put on one tap it would be
-    // white noise next to the smoothed field), the middle one takes the rest
+    // share what rounding left in proportion to their magnitudes (put on one
+    // tap it would be white noise next to the smoothed field; in proportion
+    // to the taps themselves, which at large r are of both signs and sum to
+    // far less than their magnitudes, it changed each by up to r 2^-53 of
+    // itself), the middle one takes the rest
     const float unit = __int_as_float((127 - E) << 23);
-    const float miss[2] = {(float)((1LL << E) - s_sum[0]) * unit, (float)((1LL << E) - s_sum[1]) * unit};
+    const float miss[2] = {(float)((1LL << E) - s_sum[0]) * unit / row_abs[0],
+                           (float)((1LL << E) - s_sum[1]) * unit / row_abs[1]};
     __syncthreads();
     if (t < 2)
         s_sum[t] = 0;
@@ -505,7 +515,7 @@ __global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, cons
         long long v = 0;
         if (i < count) {
             v = q[phase * kQ + kMid + d];
-            v += __float2ll_rn((float)v * miss[phase]);
+            v += __float2ll_rn(fabsf((float)v) * miss[phase]);
             q[phase * kQ + kMid + d] = v;
         }
         add_sum(phase, v);

@@ -1,0 +1,72 @@
+"""Errors of composed steps (GE_KERNEL_AUTO) against the steps evaluated in
+extended precision (numpy.longdouble: 64 or 113 bits), beside those of the
+tiled kernel, which takes the same steps one by one."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1310_3422_gb300 import binding as B
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+LD = np.longdouble
+SLACK = 1.25
+
+
+def exact(u0, r, bl, br, steps):
+    """Steps of parity 0, 1, 0, ... of the rows of u0: (I + r G_p) u' = (I - r G_1-p) u + r walls."""
+    u, r = np.array(u0, dtype=LD), LD(r)
+    n = u.shape[-1]
+    for s in range(steps):
+        p = s & 1
+        w = (1 - r) * u
+        a, b = slice(1 - p, n - ((n - 1 + p) & 1), 2), slice(2 - p, n - ((n - 1 + p) & 1), 2)
+        w[..., a] += r * u[..., b]
+        w[..., b] += r * u[..., a]
+        w[..., 0] += r * LD(bl)
+        w[..., -1] += r * LD(br)
+        u = w / (1 + r)
+        a, b = slice(p, n - ((n - p) & 1), 2), slice(p + 1, n - ((n - p) & 1), 2)
+        u[..., a] = ((1 + r) * w[..., a] + r * w[..., b]) / (1 + 2 * r)
+        u[..., b] = ((1 + r) * w[..., b] + r * w[..., a]) / (1 + 2 * r)
+    return u
+
+
+def run(u0, r, bl, br, steps, kernel, prec=B.GE_F64):
+    x = torch.as_tensor(np.asarray(u0), dtype=B.dtype_of(prec), device=DEV).contiguous()
+    ctx = B.ge_create(len(u0), r, bl, br, prec, x)
+    B.ge_set_kernel(ctx, kernel, 0)
+    B.ge_step_n(ctx, steps)
+    out = torch.empty_like(x)
+    B.ge_read_state(ctx, out)
+    B.ge_sync(ctx)
+    B.ge_destroy(ctx)
+    return out.cpu().numpy()
+
+
+def rms_errors(u0, r, bl, br, steps, prec, parts=None):
+    """RMS error of both kernels over the rows of u0, divided by the exact
+    field's RMS there (over `parts` of a row)."""
+    want = exact(u0, r, bl, br, steps)
+    parts = parts or slice(None)
+    norm = np.sqrt(np.mean(want[:, parts] ** 2))
+    return [float(np.sqrt(np.mean([np.mean((run(u, r, bl, br, steps, kernel, prec)[parts] - w[parts]) ** 2)
+                                   for u, w in zip(u0, want)])) / norm)
+            for kernel in (B.GE_KERNEL_AUTO, B.GE_KERNEL_TEMPORAL)]
+
+
+def rough(seeds, n, dtype=np.float64):
+    return np.stack([np.random.default_rng(s).standard_normal(n) for s in range(seeds)]).astype(dtype).astype(np.float64)
+
+
+# r far above any the other tests take: taps of both signs, up to r / 2; dot
+# products only, and tiles
+@pytest.mark.parametrize("n", [1024, 12000])
+@pytest.mark.parametrize("r", [30.0, 1000.0, 1e6])
+@pytest.mark.parametrize("prec,steps", [(B.GE_F64, 24), (B.GE_F64, 150), (B.GE_F32, 150), (B.GE_F32_COMP, 150)])
+def test_large_mesh_ratios(n, r, prec, steps):
+    """Composed steps err no more than steps one by one, up to the scatter of
+    one rough field's error (a few hundred independent samples: 1.25)."""
+    u0 = rough(1, n, np.float64 if prec == B.GE_F64 else np.float32)
+    auto, tiled = rms_errors(u0, r, 0.3, -0.8, steps, prec)
+    assert auto <= SLACK * tiled, (auto, tiled)
