@@ -743,24 +743,13 @@ __device__ __forceinline__ float pow2<float>(int e)
     return __int_as_float((e + 127) << 23);
 }
 
-// z 2^e rounded to nearest even, for a normal result.  FP64 on the integer
-// pipes: the conversion instruction runs on the FP64 unit.
+// z 2^e rounded to nearest even, for a normal result.
 template <typename T>
 __device__ __forceinline__ T from_fixed(long long z, int e);
 template <>
 __device__ __forceinline__ double from_fixed<double>(long long z, int e)
 {
-    const unsigned long long m = (unsigned long long)(z < 0 ? -z : z);
-    const int lead = __clzll((long long)m);                 // 2 .. 63 (64 for zero)
-    const unsigned long long w = m << (lead & 63);          // leading one at bit 63
-    unsigned long long f = w >> 11;
-    const unsigned low = (unsigned)w & 0x7ff;
-    f += (low > 0x400 || (low == 0x400 && (f & 1))) ? 1 : 0;
-    // exponent field of 2^(63 - lead + e), less the leading one's own unit
-    f += (unsigned long long)(unsigned)(1023 + 62 - lead + e) << 52;
-    if (m == 0)
-        f = 0;
-    return __longlong_as_double((long long)(f | ((unsigned long long)z & 0x8000000000000000ull)));
+    return fixed_to_double(z, e);
 }
 template <>
 __device__ __forceinline__ float from_fixed<float>(long long z, int e)

@@ -94,7 +94,7 @@ struct PropRun {
     const void *in;
     void *out;
     long long n;
-    double r, omr, x1, x2, xs;  // entry and exit coefficients
+    double r, x2, xs;           // entry and exit coefficients
     double fl, fr;              // r beta_l, r beta_r
     double bl, br;
     int wall_l, wall_r;         // exponent codes of what the walls add (tiles: see code_of)

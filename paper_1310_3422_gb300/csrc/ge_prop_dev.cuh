@@ -15,11 +15,65 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+// z 2^e rounded to nearest even, for a normal result, on the integer pipes
+// (the conversion instruction runs on the FP64 unit).
+__device__ __forceinline__ double fixed_to_double(long long z, int e)
+{
+    const unsigned long long m = (unsigned long long)(z < 0 ? -z : z);
+    const int lead = __clzll((long long)m);                 // 1 .. 63 (64 for zero)
+    const unsigned long long w = m << (lead & 63);          // leading one at bit 63
+    unsigned long long f = w >> 11;
+    const unsigned low = (unsigned)w & 0x7ff;
+    f += (low > 0x400 || (low == 0x400 && (f & 1))) ? 1 : 0;
+    // exponent field of 2^(63 - lead + e), less the leading one's own unit
+    f += (unsigned long long)(unsigned)(1023 + 62 - lead + e) << 52;
+    if (m == 0)
+        f = 0;
+    return __longlong_as_double((long long)(f | ((unsigned long long)z & 0x8000000000000000ull)));
+}
+
+// The sum over a warp of P (1 or 2) values a lane, each to 2^-57 of the
+// largest, rounded once.  As integers relative to the largest exponent, by
+// three reductions of 27 bits each: FP64 additions in a tree round at each of
+// its five levels, which was half of a short row's error (24 steps of rough
+// data at r = 1: 1.3e-16 where the steps one by one err 1.1e-16), and take
+// the FP64 unit 19 cycles each.  Sums that are not finite, or that could
+// overflow or be subnormal, take the tree.
+template <int P>
+__device__ __forceinline__ double warp_sum_rounded_once(const double (&v)[P])
+{
+    static_assert(P == 1 || P == 2, "the sum of 32 P integers below 2^57 stays below 2^63");
+    unsigned code = 0;
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+        code = max(code, ((unsigned)__double2hiint(v[p]) >> 20) & 0x7ff);
+    const int ref = (int)__reduce_max_sync(0xffffffffu, code);
+    if (ref < 64 || ref >= 2040)
+        return warp_sum(P == 2 ? v[0] + v[P - 1] : v[0]);
+    unsigned long long y = 0;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        const unsigned long long u = (unsigned long long)__double_as_longlong(v[p]);
+        const int e = (int)(u >> 52) & 0x7ff;
+        unsigned long long m = (u & 0x000fffffffffffffull) | (e ? 0x0010000000000000ull : 0);
+        // v = m 2^(e - 1075) = (m 2^(e - ref + 4)) 2^(ref - 1079)
+        const int sh = (e ? e : 1) - ref + 4, n = -sh < 60 ? -sh : 60;
+        m = sh >= 0 ? m << sh : (m + (1ull << (n - 1))) >> n;
+        // (biased: 32 P times 2^59 / P is 2^64, no part of the sum)
+        y += (1ull << 59) / P + ((long long)u < 0 ? 0 - m : m);
+    }
+    const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)y & 0x7ffffffu);
+    const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(y >> 27) & 0x7ffffffu);
+    const unsigned c = __reduce_add_sync(0xffffffffu, (unsigned)(y >> 54));
+    return fixed_to_double((long long)(a + ((unsigned long long)b << 27) + ((unsigned long long)c << 54)), ref - 1079);
+}
+
 // ---- reading the state ---------------------------------------------------
 
-// Point j's right-hand side w = (1 - r) u + r u_partner (+ the wall terms),
-// the groups those of parity 1 - p0 -- or the value itself after the first
-// operator, when the buffer holds w.
+// Point j's right-hand side w = u + r (u_partner - u) (+ the wall terms), the
+// groups those of parity 1 - p0 -- or the value itself after the first
+// operator, when the buffer holds w.  (As (1 - r) u + r u_partner it would
+// take the rounding of 1 - r, the same in every row, and of the first product.)
 template <typename T>
 __device__ __forceinline__ double load_w(const PropRun &P, long long j)
 {
@@ -28,9 +82,7 @@ __device__ __forceinline__ double load_w(const PropRun &P, long long j)
     if (!P.entry)
         return u;
     const long long m = ((j + 1 - P.p0) & 1) ? j - 1 : j + 1;
-    double w = P.omr * u;
-    if (m >= 0 && m < P.n)
-        w = fma(P.r, (double)in[m], w);
+    double w = fma(P.r, (m >= 0 && m < P.n ? (double)in[m] : 0.0) - u, u);
     if (j == 0)
         w += P.fl;
     if (j == P.n - 1)
@@ -370,18 +422,18 @@ __device__ __forceinline__ void dot_rows(const PropRun &P, DotShared<ROWS> &sh, 
             s_w[kDotWin + z * 32 + lane] = s;
             continue;
         }
-        s = warp_sum(s);
+        s = warp_sum_rounded_once<1>({s});
         if (lane == 0)
             sh.row[q] = sh.bad[q] ? s + __longlong_as_double(0x7ff8000000000000ll) : s;
     }
     sync();
     if (PARTS > 1) {
         for (int q = warp; q < (int)(hi - lo); q += NT / 32) {
-            double s = s_w[kDotWin + q * PARTS * 32 + lane];
+            double v[PARTS];
 #pragma unroll
-            for (int p = 1; p < PARTS; ++p)
-                s += s_w[kDotWin + (q * PARTS + p) * 32 + lane];
-            s = warp_sum(s);
+            for (int p = 0; p < PARTS; ++p)
+                v[p] = s_w[kDotWin + (q * PARTS + p) * 32 + lane];
+            const double s = warp_sum_rounded_once(v);
             if (lane == 0)
                 sh.row[q] = sh.bad[q] ? s + __longlong_as_double(0x7ff8000000000000ll) : s;
         }
@@ -392,7 +444,8 @@ __device__ __forceinline__ void dot_rows(const PropRun &P, DotShared<ROWS> &sh, 
         double v = sh.row[i - lo];
         if (P.exit) {
             const long long m = ((i + pe) & 1) ? i - 1 : i + 1;
-            v = (m >= 0 && m < P.n) ? fma(P.x2, sh.row[m - lo], P.x1 * v) : P.xs * v;
+            // (x1 + x2 = 1)
+            v = (m >= 0 && m < P.n) ? fma(P.x2, sh.row[m - lo] - v, v) : P.xs * v;
         }
         static_cast<T *>(P.out)[i] = (T)v;
     }

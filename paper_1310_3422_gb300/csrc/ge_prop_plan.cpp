@@ -338,7 +338,7 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
         w.build = !s->valid;
         s->used = ++st->clock;
     }
-    const double x1 = (1.0 + r) / det, x2 = r / det;
+    const double x2 = r / det;
     for (int i = 0; i < needs; ++i) {
         Need &w = need[i];
         w.hb = halo_blocks(r, w.k, t.f64);
@@ -365,8 +365,6 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
         a.out = t.buf[*cur ^ 1];
         a.n = t.n;
         a.r = r;
-        a.omr = 1.0 - r;
-        a.x1 = x1;
         a.x2 = x2;
         a.xs = 1.0 / (1.0 + r);
         a.fl = r * t.beta_l;
