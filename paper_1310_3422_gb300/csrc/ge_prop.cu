@@ -1398,9 +1398,10 @@ __host__ __device__ __forceinline__ int duo_rows(int tab, int hb)
 {
     constexpr int ND = TileShape<T>::ND;
     const int need = 128 + 2 * hb, left = kDuoSmem - 1024 - ((tab + 1023) & ~1023);
-    // (rows in eights: a swizzled plane starts on 1024 bytes)
-    const int rows = (left - (need + 7) * 128) / ((2 * ND - 1) * 128);
-    return (rows < need ? rows & ~7 : (need + 7) & ~7);
+    // (in eights, both the rows there are and the rows there could be use of:
+    // a swizzled plane starts on 1024 bytes)
+    const int rows = (left - (need + 7) * 128) / ((2 * ND - 1) * 128) & ~7, most = (need + 7) & ~7;
+    return rows < most ? rows : most;
 }
 
 template <typename T>

@@ -239,3 +239,12 @@ def test_a_hot_wall_beside_a_quiet_field(n, prec, r, steps):
                 big = np.max(np.abs(want[part]))
                 if big > far:
                     assert np.max(np.abs(got[part] - want[part])) <= tol * big, (ground, left, a)
+
+
+@pytest.mark.parametrize("r,steps", [(7.5, 670), (12.0, 640), (16.0, 690)])
+def test_two_teams_with_the_largest_tables(r, steps):
+    """The widest halo of two FP32 teams with taps that reach as far as the
+    steps do: the tables leave the planes the least room."""
+    n = 304 * 8192 + 64 * 22 * 2 + 1
+    u0 = inputs.random_state(n, seed=7).astype(np.float32).astype(np.float64)
+    assert rel_max(auto_run(u0, r, 0.3, -0.8, steps, B.GE_F32), tiled_run(u0, r, 0.3, -0.8, steps, B.GE_F32)) <= 2e-5
