@@ -66,13 +66,24 @@ typedef enum {
                                 parity and kept by the context, applied in one
                                 pass on the tensor cores (values and taps cut
                                 into digits whose products sum exactly; FP64:
-                                values to 2^-54 and taps to 2^-62 of the
-                                largest of 8192 neighbours, one rounding a
-                                pass) and as FP64 dot products near the walls
-                                and wherever a block of 64 points lies below
-                                2^-16 (FP32: 2^-10) of the values that reach
-                                it, down to 2^-100 of those.  The same scheme,
-                                reassociated; width k = 1; r in [1e-6, 1e6] */
+                                values to 2^-63 and taps to 2^-62 of the
+                                largest of up to 8192 neighbours, FP32: 2^-31
+                                and 2^-39; one rounding a pass) and as dot
+                                products near the walls and in the blocks of
+                                64 points that would keep fewer digits so than
+                                step by step: those whose values lie below
+                                2^-8 (FP32: 2^-5; less where the taps smooth
+                                more) of the values that reach them, or whose
+                                results need more bits than the sums have; the
+                                dot products keep them down to 2^-100 of what
+                                reaches them.  Each tap of more than 31 steps
+                                carries a few FP64 roundings (2^-53 of itself).
+                                The same scheme, reassociated, with errors no
+                                larger than its steps one by one; width k = 1;
+                                r in [1e-6, 1e6].  A context keeps six
+                                operators, a call takes up to three; while
+                                live CUDA graphs hold them all, other calls go
+                                step by step */
     GE_KERNEL_CANONICAL = 1, /* one launch per step; Eqs. (cc)/(dd), (aa)/(bb)
                                 evaluated literally with fused multiply-adds
                                 in the order the equations print their terms

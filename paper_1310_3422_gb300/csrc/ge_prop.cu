@@ -10,10 +10,14 @@
 // while a sum stays below 2^24, and the accumulators of equal weight i + j
 // (value digit j, tap digit i) join as 64-bit integers.  So a tile's result
 // is the exact fixed-point sum, rounded once.
-//   FP64: values to 2^-54 of the tile's largest, 7 digits; taps to about
-//     2^-62, 7 digits; the 34 products with i + j <= 7 (the rest is below
+//   FP64: values to 2^-62 of the tile's largest, 8 digits; taps to about
+//     2^-62, 7 digits; the 35 products with i + j <= 7 (the rest is below
 //     2^-64 of the largest value).
 //   FP32: values to 2^-30, taps to about 2^-39, 4 digits each, 10 products.
+// (FP64 values in seven digits, 2^-54, were 14 % faster on large grids: 2^24
+// points, r = 2, 2000 steps, 2.09 ms, now 2.42.  But a stretch of rough data
+// 2^-8 of its neighbours erred 146 times as much as step by step, 24 steps at
+// r = 1; now 0.7 times.)
 // Step by step the same k steps cost k multiply-adds a point on the FP64 (or
 // FP32) pipes; composed they cost the taps' width times the products on the
 // tensor cores, and the width grows with sqrt(k) only.
@@ -435,7 +439,7 @@ __device__ __forceinline__ long long fixed_of(double x, int E)
 }
 
 __global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, const unsigned long long *x_max, int R,
-                                                           int nd, int hb_max, int tab_cap, unsigned char *tab,
+                                                           int nd, int comp, int hb_max, int tab_cap, unsigned char *tab,
                                                            PropHeader *hdr)
 {
     extern __shared__ long long q[];  // [2][kPropQ]
@@ -559,7 +563,14 @@ __global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, cons
         }
         s_ok = ok;
         hdr->E = E;
-        hdr->room = 62 - es - E;
+        // What the digits drop (products of the next weight, of N taps) has a
+        // root mean square of 2^-10 sqrt(N) units of the sums, FP32 2^-1.3
+        // sqrt(N).  FP64: N grows with the taps' scale, and a block's results
+        // are kept to 2^-54 of their largest.  FP32: to 2^-22 (the compensated
+        // kernel's 2^-23; wide taps smooth out more of its early roundings),
+        // where the steps one by one err as much.  Rows of far larger
+        // magnitudes than their sum (large r) cancel, also step by step.
+        hdr->keep = es >= 2 ? 0 : nd == kPropNd64 ? (E + 38) >> 1 : comp && E < 38 ? 34 : 33;
         hdr->ok = ok;
         hdr->rows = rows;
         for (int j = 0; j < nd; ++j) {
@@ -616,19 +627,21 @@ __global__ void __launch_bounds__(256) prop_dot_kernel(const __grid_constant__ P
 
 // ---- tiles on the tensor cores -------------------------------------------
 
-// Blocks whose values all lie below 2^-kRange of the largest value they
-// depend on go to the dot products: the fixed-point sum would leave them too
-// few digits of their own.
+// Blocks whose values all lie below 2^-P.range of the largest value of the
+// window go to the dot products: the fixed-point sum would leave them too few
+// digits of their own.  So do those below 2^-kFar of the largest value that
+// reaches them at all: what lies beyond the window counts with taps that the
+// digits leave out, 2^-64 (FP32: 2^-39) of the sum in all.
 template <typename T>
 struct TileShape;
 template <>
 struct TileShape<double> {
-    static constexpr int ND = kPropNd64, kHb = kPropHb64, kTab = kPropTab64, kRange = 16;
+    static constexpr int ND = kPropNd64, NV = kPropNv64, kHb = kPropHb64, kTab = kPropTab64, kFar = 10;
     static constexpr int kGroups = 9, kCols = 512;
 };
 template <>
 struct TileShape<float> {
-    static constexpr int ND = kPropNd32, kHb = kPropHb32, kTab = kPropTab32, kRange = 10;
+    static constexpr int ND = kPropNd32, NV = kPropNv32, kHb = kPropHb32, kTab = kPropTab32, kFar = 10;
     static constexpr int kGroups = 4, kCols = 256;
 };
 
@@ -639,23 +652,26 @@ struct TileShape<float> {
 // further on, and every eight rows of a piece cover all banks.  (The same
 // plane unswizzled, rows of 16 bytes, took 85 to 90 cycles an MMA.)
 template <typename T>
-constexpr int kPlaneRows = kPropTileBlks + 2 * TileShape<T>::kHb;
+constexpr int kPlaneRows = sizeof(T) == 8 ? kPropRows64 : kPropTileBlks + 2 * TileShape<T>::kHb;
+// (the MMA reads 128 rows from wherever a window starts: past the last plane's
+// end in a tile of fewer blocks)
 template <typename T>
-constexpr int kTileSmem = TileShape<T>::kTab + TileShape<T>::ND * kPlaneRows<T> * 128 + 1024;
+constexpr int kTileSmem = TileShape<T>::kTab + (TileShape<T>::NV * kPlaneRows<T> + kPropTileBlks + 2 * TileShape<T>::kHb - kPlaneRows<T>) * 128 + 1024;
 // The finished rows leave through the planes' space, padded so that the lanes
 // (a row each) write different banks.
 template <typename T>
 constexpr int kStageRow = kPropBlk * (int)sizeof(T) + 16;
 
-static_assert(kTileSmem<double> <= 232448 - 2048 && kTileSmem<float> <= 232448 - 2048, "tile exceeds shared memory");
+static_assert(kTileSmem<double> <= 232448 - 2560 && kTileSmem<float> <= 232448 - 2560, "tile exceeds shared memory");
 
 // Digit products of each accumulator, in issue order: sum g holds the products
-// of weight(g) whose tap digit lies in [lo(g), hi(g)].  FP64's weight 4 takes
+// of weight(g) whose tap digit lies in [lo(g), hi(g)], the value digit being
+// weight(g) less that.  FP64's weight 4 takes
 // two sums so that each stays exact; its first and last sum share one
 // accumulator (512 columns hold eight).
 struct Groups64 {
     __host__ __device__ static constexpr int weight(int g) { return g <= 3 ? 7 - g : 8 - g; }
-    __host__ __device__ static constexpr int lo(int g) { return g == 0 ? 1 : g == 4 ? 3 : 0; }
+    __host__ __device__ static constexpr int lo(int g) { return g == 4 ? 3 : 0; }
     __host__ __device__ static constexpr int hi(int g) { return g == 0 ? 6 : g == 3 ? 2 : weight(g); }
 };
 struct Groups32 {
@@ -691,8 +707,25 @@ __device__ __forceinline__ int code_of(float x)
 template <typename T>
 constexpr int kCodeInf = sizeof(T) == 8 ? 2047 : 255;
 
-// round(x 2^(kVal - e)) for |x| < 2^e, e = code - bias + 1 of the tile's
-// largest value; `ref` is that largest code.
+// Whether a tile leaves a block to dot products for its values: the code of
+// its largest, of the window's and of the cone's.
+template <typename T>
+__device__ __forceinline__ bool values_too_small(const PropRun &P, int q, int ref, int cone)
+{
+    return cone == kCodeInf<T> || q == 0 || q < ref - P.range || q < cone - TileShape<T>::kFar;
+}
+
+// Whether it does for its results: bits[0] those of block `row`'s largest sum.
+__device__ __forceinline__ bool results_too_small(const PropRun &P, const int *bits, int row, int rows, int keep)
+{
+    int b = bits[row];
+    if (P.near)
+        b = max(b, max(row > 0 ? bits[row - 1] : 0, row + 1 < rows ? bits[row + 1] : 0));
+    return b < keep;
+}
+
+// round(x 2^(62 - e)), FP32 round(x 2^(30 - e)), for |x| < 2^e, e = code -
+// bias + 1 of the tile's largest value; `ref` is that largest code.
 __device__ __forceinline__ long long to_fixed(double x, int ref)
 {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
@@ -700,8 +733,8 @@ __device__ __forceinline__ long long to_fixed(double x, int ref)
     unsigned long long m = u & 0x000fffffffffffffull;
     if (e)
         m |= 0x0010000000000000ull;
-    // x = m 2^(ec - 1075), 2^e_tile = 2^(ref - 1022): shift by ec - ref + 1
-    const int sh = (e ? e : 1) - ref + 1;
+    // x = m 2^(ec - 1075), 2^e_tile = 2^(ref - 1022): shift by ec - ref + 9
+    const int sh = (e ? e : 1) - ref + 9;
     if (sh >= 0) {
         m <<= sh;
     } else {
@@ -757,6 +790,13 @@ __device__ __forceinline__ float from_fixed<float>(long long z, int e)
     return z ? add_exponent((float)z, e) : 0.0f;
 }
 
+// Whether from_fixed takes every 64-bit integer times 2^e.
+template <typename T>
+__device__ __forceinline__ bool plain_exponent(int e)
+{
+    return sizeof(T) == 8 ? e >= -1021 && e <= 959 : e >= -125 && e <= 63;
+}
+
 // Two digits as FP16: bytes b of two biased values to (b - 128).
 __device__ __forceinline__ uint32_t half_pair(uint32_t a, uint32_t b, uint32_t sel)
 {
@@ -786,12 +826,12 @@ constexpr uint32_t kIdescF16 = (1u << 4) | ((uint32_t)(kPropBlk >> 3) << 17) | (
 template <typename T>
 __device__ __forceinline__ void convert8(const T (&x)[8], int ref, unsigned char *dst, size_t plane)
 {
-    constexpr int ND = TileShape<T>::ND;
+    constexpr int NV = TileShape<T>::NV;
     uint32_t lo[8], hi[8];
 #pragma unroll
     for (int v = 0; v < 8; ++v) {
-        if (ND == kPropNd64) {
-            const unsigned long long y = (unsigned long long)to_fixed((double)x[v], ref) + 0x0080808080808080ull;
+        if (NV == kPropNv64) {
+            const unsigned long long y = (unsigned long long)to_fixed((double)x[v], ref) + 0x8080808080808080ull;
             lo[v] = (uint32_t)y;
             hi[v] = (uint32_t)(y >> 32);
         } else {
@@ -799,8 +839,8 @@ __device__ __forceinline__ void convert8(const T (&x)[8], int ref, unsigned char
         }
     }
 #pragma unroll
-    for (int d = 0; d < ND; ++d) {
-        const int byte = ND - 1 - d;
+    for (int d = 0; d < NV; ++d) {
+        const int byte = NV - 1 - d;
         const uint32_t sel = byte < 4 ? (uint32_t)(byte | (byte << 4) | ((byte + 4) << 8) | ((byte + 4) << 12))
                                       : (uint32_t)((byte - 4) | ((byte - 4) << 4) | (byte << 8) | (byte << 12));
         uint4 q;
@@ -812,23 +852,81 @@ __device__ __forceinline__ void convert8(const T (&x)[8], int ref, unsigned char
     }
 }
 
-// One sum's value into a point's 64-bit accumulator (weight w; units: see the drain).
-template <typename T>
-__device__ __forceinline__ long long fold(long long acc, int w, int z, int xs)
+// The accumulators of a row's points: 64-bit sums in units of weight 5 (FP32:
+// weight 3), and for FP64 the next 16 bits of each (weights 6 and 7), two to a
+// register.
+template <typename T, int N>
+struct Sums {
+    long long hi[N] = {};
+    uint32_t low[sizeof(T) == 8 ? N / 2 : 1] = {};
+    // one digit sum of weight w (FP64: 7 first, then 6)
+    __device__ __forceinline__ void fold(int v, int w, int z)
+    {
+        if (sizeof(T) == 4) {
+            hi[v] += (long long)z << (8 * (3 - (w < 4 ? w : 3)));
+        } else if (w >= 6) {
+            const long long s = w == 7 ? (long long)z : hi[v] + ((long long)z << 8);
+            if (w == 6) {
+                low[v / 2] |= ((uint32_t)s & 0xffff) << (v & 1) * 16;
+                hi[v] = s >> 16;
+            } else {
+                hi[v] = s;
+            }
+        } else {
+            hi[v] += (long long)z << (8 * (5 - w));
+        }
+    }
+    __device__ __forceinline__ int last(int v) const { return (int)(low[v / 2] >> (v & 1) * 16) & 0xffff; }
+    // bits of the largest
+    __device__ __forceinline__ int bits() const
+    {
+        unsigned long long m = 0;
+#pragma unroll
+        for (int v = 0; v < N; ++v)
+            m |= (unsigned long long)(hi[v] ^ (hi[v] >> 63));
+        return 64 - __clzll((long long)m);
+    }
+};
+
+// A sum and its 16 low bits, the sum of `bits` bits or fewer, as one integer
+// times 2^-shift.
+__device__ __forceinline__ int join_shift(int bits) { return bits < 46 ? 16 : 62 - bits; }
+__device__ __forceinline__ long long join(long long hi, int low, int shift)
 {
-    if (sizeof(T) == 8)
-        return w == 7   ? (long long)z
-               : w == 6 ? ((acc + ((long long)z << 8) + (0x8000 >> xs)) >> (16 - xs))
-                        : acc + ((long long)z << (8 * (5 - (w < 6 ? w : 5)) + xs));
-    return acc + ((long long)z << (8 * (3 - (w < 4 ? w : 3))));
+    return (long long)((unsigned long long)hi << shift) + (low >> (16 - shift));
+}
+
+// out = (hi + low 2^-16) 2^ex, rounded once (FP32: no low part).
+template <typename T>
+__device__ __forceinline__ T finish_point(long long hi, int low, int ex, bool plain)
+{
+    long long z = hi;
+    if (sizeof(T) == 8) {
+        const int shift = join_shift(64 - __clzll(hi ^ (hi >> 63)));
+        z = join(hi, low, shift);
+        if (plain)
+            return from_fixed<T>(z, ex - shift);
+        // near the ends of the exponent range
+        return (T)z * pow2<T>(ex / 2) * pow2<T>(ex - ex / 2 - shift);
+    }
+    return plain ? from_fixed<T>(z, ex) : (T)z * pow2<T>(ex / 2) * pow2<T>(ex - ex / 2);
+}
+// The exponent of a tile's sums, and whether finish_point's results are normal
+// whatever the sum: FP64 2^ex = 2^(e + 2 - E), FP32 2^(e - 6 - E), 2^e above
+// the tile's largest value (code `ref`).
+template <typename T>
+__device__ __forceinline__ int sum_exponent(int ref, int E) { return sizeof(T) == 8 ? ref - 1022 + 2 - E : ref - 126 - 6 - E; }
+template <typename T>
+__device__ __forceinline__ bool plain_sums(int ex)
+{
+    return plain_exponent<T>(ex) && (sizeof(T) == 4 || plain_exponent<T>(ex - 16));
 }
 
 // N finished points of a row to the staging buffer: out = acc 2^ex.
 template <typename T, int N>
 __device__ __forceinline__ void finish_row(const long long (&acc)[N], int ex, unsigned char *o)
 {
-    const bool plain = sizeof(T) == 8 ? ex >= -1021 && ex <= 959 : ex >= -125 && ex <= 63;
-    if (plain) {
+    if (plain_exponent<T>(ex)) {
 #pragma unroll
         for (int v = 0; v < N; v += 16 / sizeof(T)) {
             T y[16 / sizeof(T)];
@@ -896,7 +994,9 @@ static_assert((kDotWin + kEdgeScratch + dot_taps(kPropR64Max)) * 8 <= kTileSmem<
 // 100,003, k = 1999, FP64 takes 4 CTAs a tile, 68 -> 49 us a call (8: 57, 2:
 // 59); n = 500,000 takes 2, 82 -> 67 us; n = 300,001, FP32, two operators:
 // 100 -> 82 us.
+template <typename T>
 constexpr int kPartHigh = kPropTileBlks * kPropBlk * 8;  // bytes of a CTA's sums [64 points][128 blocks]; FP64: 16 last bits follow
+static_assert(kPartHigh<double> / 8 * 10 <= kPropTab64 && kPartHigh<float> <= kPropTab32, "the sums fit the tables' space");
 // One partial sum from each CTA of the cluster, and for FP64 its last bits.
 template <typename T, int C>
 __device__ __forceinline__ void add_parts(uint32_t addr, uint32_t addr_low, long long &hi, int &low)
@@ -940,9 +1040,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
     __shared__ __align__(8) uint64_t tab_full, done[S::kGroups], reuse;
     __shared__ uint32_t tmem_sh;
     __shared__ volatile int s_abort;
-    __shared__ int s_code[kPropTileBlks + 2 * S::kHb + 8];
+    __shared__ int s_code[C + 8];
     __shared__ int s_max[2];  // largest code: the window, the whole cone
     __shared__ int s_keep;    // blocks the tile itself answers
+    __shared__ int s_bits[kPropTileBlks];  // bits of each block's largest sum
     __shared__ int s_left;
     __shared__ PropHeader s_hdr;
     __shared__ DotShared<kEdgeRows> s_dot;
@@ -991,7 +1092,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
             return x + spare < P.tiles + early ? x + spare : P.tiles + early + (long long)blockIdx.x;
         return x + (long long)gridDim.x;
     };
-    const int hb = P.hb, ok_tab = s_hdr.ok && s_hdr.rows * 16 <= S::kTab;
+    const int hb = P.hb, per = P.per, ok_tab = s_hdr.ok && s_hdr.rows * 16 <= S::kTab;
     const bool has_tab = ok_tab && first < P.tiles;
     if (t == 0 && has_tab) {
         bar_expect_tx(&tab_full, (uint32_t)s_hdr.rows * 16);
@@ -1046,11 +1147,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
             }
             continue;
         }
-        const long long b0 = P.blk0 + tile * kPropTileBlks;       // first output block
-        const int nb = (int)(P.blk1 - b0 < kPropTileBlks ? P.blk1 - b0 : kPropTileBlks);
+        const long long b0 = P.blk0 + tile * per;                 // first output block
+        const int nb = (int)(P.blk1 - b0 < per ? P.blk1 - b0 : per);
         const long long base = (b0 - hb) * kPropBlk;              // first point of the window
-        const int chunks = (kPropTileBlks + 2 * hb) * 8;          // 8 points each
-        constexpr int kIter = ((kPropTileBlks + 2 * S::kHb) * 8 + kTileConv - 1) / kTileConv;
+        const int chunks = (per + 2 * hb) * 8;                    // 8 points each
+        constexpr int kIter = (C * 8 + kTileConv - 1) / kTileConv;
         if (t < 2)
             s_max[t] = 0;
         if (t == 2)
@@ -1081,7 +1182,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
             }
             // the next tile's window on its way to L2
             if (!SPLIT && tile + gridDim.x < P.tiles) {
-                const long long nx = base + (long long)gridDim.x * kPropTileBlks * kPropBlk + (long long)t * 128 / sizeof(T);
+                const long long nx = base + (long long)gridDim.x * per * kPropBlk + (long long)t * 128 / sizeof(T);
                 for (long long z = nx; z < nx - (long long)t * 128 / sizeof(T) + (long long)chunks * 8 && z < P.n;
                      z += (long long)kTileConv * 128 / sizeof(T))
                     asm volatile("prefetch.global.L2 [%0];" ::"l"(in + z));
@@ -1133,9 +1234,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
         if (!SPLIT && s_left)
             break;
         const int ref = s_max[0], cone = s_max[1];
+        bool listed = false;  // block t
         if (t < nb) {
-            const int q = s_code[hb + t];
-            const bool listed = cone > 0 && (!ok_tab || cone == kCodeInf<T> || q < cone - S::kRange || q == 0);
+            s_bits[t] = 0;
+            listed = cone > 0 && (!ok_tab || values_too_small<T>(P, s_code[hb + t], ref, cone));
             if (listed && rank == 0)
                 P.list[atomicAdd(P.count, 1)] = (int)(b0 + t);
             else if (!listed && cone > 0)
@@ -1183,31 +1285,9 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
 #pragma unroll 1
                     for (int i = lo; i <= hi; ++i) {
                         const int4 p = s_prod[g * ND + i];
-                        const int q = __shfl_sync(0xffffffffu, p.z, 0), end = __shfl_sync(0xffffffffu, p.w, 0);
-                        uint64_t ad = ad0 + (uint32_t)__shfl_sync(0xffffffffu, p.x, 0);
-                        uint64_t bd = bd0 + (uint32_t)__shfl_sync(0xffffffffu, p.y, 0);
-                        const uint64_t a0 = (uint64_t)(6 - q), a1 = (uint64_t)(6 - ((q + 2) & 7) + ((q + 2) & 8)),
-                                       a2 = (uint64_t)(6 - ((q + 4) & 7) + ((q + 4) & 8)),
-                                       a3 = (uint64_t)(6 - ((q + 6) & 7) + ((q + 6) & 8));
-                        int s = 0;
-#pragma unroll 1
-                        for (; s + 4 <= end; s += 4) {
-                            tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, acc);
-                            tc_mma_if(leader, dcol, ad + a1, bd - 16, kIdescF16, 1);
-                            tc_mma_if(leader, dcol, ad + a2, bd - 32, kIdescF16, 1);
-                            tc_mma_if(leader, dcol, ad + a3, bd - 48, kIdescF16, 1);
-                            acc = 1;
-                            ad += 8;
-                            bd -= 64;
-                        }
-                        if (s < end) {
-                            tc_mma_if(leader, dcol, ad + a0, bd, kIdescF16, SPLIT ? acc : 1);
-                            if (s + 1 < end)
-                                tc_mma_if(leader, dcol, ad + a1, bd - 16, kIdescF16, 1);
-                            if (s + 2 < end)
-                                tc_mma_if(leader, dcol, ad + a2, bd - 32, kIdescF16, 1);
-                            acc = 1;
-                        }
+                        issue_product(leader, dcol, ad0 + (uint32_t)__shfl_sync(0xffffffffu, p.x, 0),
+                                      bd0 + (uint32_t)__shfl_sync(0xffffffffu, p.y, 0), __shfl_sync(0xffffffffu, p.z, 0),
+                                      __shfl_sync(0xffffffffu, p.w, 0), acc);
                     }
                     tc_commit_if(leader, &done[g]);
                     __syncwarp();
@@ -1221,13 +1301,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
         } else if (keep) {
             // drain: kTileCols columns (points of a block) of the lane's block
             const int row = (warp & 3) * 32 + lane, col = (warp >> 2) * kTileCols;
-            // units of the sums: weight 5 (FP32: 3), and up to 8 bits below
-            // where the taps' scale leaves the 64-bit sum that room
-            const int room = s_hdr.room, xs = sizeof(T) == 4 ? 0 : room < 8 ? room : 8;
-            long long acc[kTileCols], low[SPLIT && sizeof(T) == 8 ? kTileCols : 1];
-#pragma unroll
-            for (int v = 0; v < kTileCols; ++v)
-                acc[v] = 0;
+            Sums<T, kTileCols> acc;
             bool ok = true;
 #pragma unroll
             for (int g = 0; g < S::kGroups; ++g) {
@@ -1248,19 +1322,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
 #pragma unroll
                     for (int q = 0; q < kTileCols; ++q) {
                         const int z = mine ? __float2int_rn(__uint_as_float(v[q])) : 0;
-                        if (SPLIT && ND == kPropNd64) {
-                            // weights 7 and 6 apart: their last bits are rounded off the whole sum
-                            if (w >= 6)
-                                low[SPLIT && sizeof(T) == 8 ? q : 0] =
-                                    w == 7 ? (long long)z : low[SPLIT && sizeof(T) == 8 ? q : 0] + ((long long)z << 8);
-                            else
-                                acc[q] += (long long)z << (8 * (5 - (w < 6 ? w : 5)) + xs);
-                        } else if (ND == kPropNd64)
-                            acc[q] = w == 7   ? (long long)z
-                                     : w == 6 ? ((acc[q] + ((long long)z << 8) + (0x8000 >> xs)) >> (16 - xs))
-                                              : acc[q] + ((long long)z << (8 * (5 - (w < 6 ? w : 5)) + xs));
-                        else
-                            acc[q] += (long long)z << (8 * (3 - (w < 4 ? w : 3)));
+                        acc.fold(q, w, z);
                     }
                 }
             }
@@ -1273,32 +1335,22 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
 #pragma unroll
                 for (int v = 0; v < kTileCols; ++v) {
                     const int at = (col + v) * kPropTileBlks + row;
-                    if (sizeof(T) == 8) {
-                        const long long l = low[SPLIT && sizeof(T) == 8 ? v : 0];
-                        acc[v] += l >> (16 - xs);
-                        reinterpret_cast<unsigned short *>(sm + kPartHigh)[at] = (unsigned short)(l & ((1 << (16 - xs)) - 1));
-                    }
-                    reinterpret_cast<long long *>(sm)[at] = acc[v];
+                    if (sizeof(T) == 8)
+                        reinterpret_cast<unsigned short *>(sm + kPartHigh<T>)[at] = (unsigned short)acc.last(v);
+                    reinterpret_cast<long long *>(sm)[at] = acc.hi[v];
                 }
-            } else if (row < nb) {
-                // out = acc 2^x: FP64 x = e + 2 - E - xs, FP32 x = e - 6 - E, 2^e above the tile's largest value
-                const int ex = sizeof(T) == 8 ? ref - 1022 + 2 - s_hdr.E - xs : ref - 126 - 6 - s_hdr.E;
+            } else if (!SPLIT && row < nb) {
+                const int ex = sum_exponent<T>(ref, s_hdr.E);
+                const bool plain = plain_sums<T>(ex);
                 unsigned char *o = xp + row * kStageRow<T> + col * (int)sizeof(T);
-                const bool plain = sizeof(T) == 8 ? ex >= -1021 && ex <= 959 : ex >= -125 && ex <= 63;
-                const T s1 = pow2<T>(ex / 2), s2 = pow2<T>(ex - ex / 2);
-                if (plain) {
+                atomicMax(&s_bits[row], acc.bits());
 #pragma unroll
-                    for (int v = 0; v < kTileCols; v += 16 / sizeof(T)) {
-                        T y[16 / sizeof(T)];
+                for (int v = 0; v < kTileCols; v += 16 / sizeof(T)) {
+                    T y[16 / sizeof(T)];
 #pragma unroll
-                        for (int z = 0; z < (int)(16 / sizeof(T)); ++z)
-                            y[z] = from_fixed<T>(acc[v + z], ex);
-                        *reinterpret_cast<uint4 *>(o + v * sizeof(T)) = *reinterpret_cast<const uint4 *>(y);
-                    }
-                } else {  // near the ends of the exponent range
-#pragma unroll
-                    for (int v = 0; v < kTileCols; ++v)
-                        reinterpret_cast<volatile T *>(o)[v] = (T)acc[v] * s1 * s2;
+                    for (int z = 0; z < (int)(16 / sizeof(T)); ++z)
+                        y[z] = finish_point<T>(acc.hi[v + z], sizeof(T) == 8 ? acc.last(v + z) : 0, ex, plain);
+                    *reinterpret_cast<uint4 *>(o + v * sizeof(T)) = *reinterpret_cast<const uint4 *>(y);
                 }
             }
             if (!SPLIT) {
@@ -1309,6 +1361,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                 if (t < nb && !s_abort) {
                     bulk_store(out + (b0 + t) * kPropBlk, xp + t * kStageRow<T>, kPropBlk * (uint32_t)sizeof(T));
                     bulk_commit();
+                    if (!listed && results_too_small(P, s_bits, t, nb, s_hdr.keep))
+                        P.list[atomicAdd(P.count, 1)] = (int)(b0 + t);
                 }
             }
         } else if (cone == 0 && rank == 0) {
@@ -1323,10 +1377,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
             __syncwarp();
             cluster_sync();
             if (keep && warp < kTileWarps) {
-                const int share = kPropBlk / ctas, room = s_hdr.room, xs = sizeof(T) == 4 ? 0 : room < 8 ? room : 8;
-                const int ex = sizeof(T) == 8 ? ref - 1022 + 2 - s_hdr.E - xs : ref - 126 - 6 - s_hdr.E;
-                const bool plain = sizeof(T) == 8 ? ex >= -1021 && ex <= 959 : ex >= -125 && ex <= 63;
-                const T s1 = pow2<T>(ex / 2), s2 = pow2<T>(ex - ex / 2);
+                const int share = kPropBlk / ctas, ex = sum_exponent<T>(ref, s_hdr.E);
+                const bool plain = plain_sums<T>(ex);
                 // a warp reads 32 blocks' sums of one point (contiguous: reads
                 // from another CTA's memory cost by the piece)
 #pragma unroll 2
@@ -1335,7 +1387,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                     if (row >= nb)
                         continue;
                     const uint32_t cell = (uint32_t)(col * kPropTileBlks + row), at = saddr(sm) + cell * 8,
-                                   at_low = saddr(sm) + kPartHigh + cell * 2;
+                                   at_low = saddr(sm) + kPartHigh<T> + cell * 2;
                     long long z;
                     int low;
                     if (ctas == 2)
@@ -1344,17 +1396,22 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
                         add_parts<T, 4>(at, at_low, z, low);
                     else
                         add_parts<T, 8>(at, at_low, z, low);
-                    if (sizeof(T) == 8)
-                        z += (low + (0x8000 >> xs)) >> (16 - xs);
-                    T *o = out + (b0 + row) * kPropBlk + col;
-                    if (plain)
-                        *o = from_fixed<T>(z, ex);
-                    else
-                        *reinterpret_cast<volatile T *>(o) = (T)z * s1 * s2;
+                    z += low >> 16;
+                    atomicMax(&s_bits[row], 64 - __clzll(z ^ (z >> 63)));
+                    out[(b0 + row) * kPropBlk + col] = finish_point<T>(z, low & 0xffff, ex, plain);
+                }
+                // the blocks' largest sums, of every CTA's points, to the first
+                asm volatile("bar.sync 1, %0;" ::"n"(kTileConv) : "memory");
+                if (t < nb && rank != 0) {
+                    uint32_t at;
+                    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(saddr(&s_bits[t])), "r"(0));
+                    asm volatile("red.relaxed.cluster.shared::cluster.max.s32 [%0], %1;" ::"r"(at), "r"(s_bits[t]) : "memory");
                 }
             }
             __syncwarp();
             cluster_sync();
+            if (keep && rank == 0 && t < nb && !listed && !s_abort && results_too_small(P, s_bits, t, nb, s_hdr.keep))
+                P.list[atomicAdd(P.count, 1)] = (int)(b0 + t);
         }
         if (keep)
             phase ^= 1;
@@ -1377,39 +1434,40 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
 
 // ---- two teams -------------------------------------------------------------
 
-// Large grids whose taps reach a few blocks only: the table and the planes of
-// two tiles fit shared memory, and two teams of eight warps and an issuing
+// Large FP32 grids whose taps reach a few blocks only: the table and the planes
+// of two tiles fit shared memory, and two teams of eight warps and an issuing
 // warp each take a tile of their own, so that one team's MMAs run under the
 // other's loads, conversion and drain (in prop_tile_kernel, where a tile's
 // planes fill shared memory, these take 18,000 cycles a tile during which the
-// tensor cores idle).  FP32 teams issue in turn; FP64's few MMAs need not.  A
-// team has 256 of the 512 columns: four accumulators,
-// a ring that its sums go round.  Tiles of as many blocks as fit, up to 128
-// (of the MMA's 128 rows the others are not used).  2^24 FP32 points, 2000
-// steps: 387 -> 312 us a call; 2^22 FP64 points, 24 steps: 110 -> 100 us.
+// tensor cores idle).  The teams issue in turn.  A team has 256 of the 512
+// columns: four accumulators, a ring that its sums go round.  Tiles of as many
+// blocks as fit, up to 128 (of the MMA's 128 rows the others are not used).
+// 2^24 points, 2000 steps: 387 -> 312 us a call.  (FP64: the eight planes of
+// two tiles leave each 94 blocks where prop_tile_kernel's have 126: 2^22
+// points, 24 steps, 138 us, 114 there.)
 constexpr int kTeamWarps = 8, kTeam = 32 * kTeamWarps, kRing = 4;
-constexpr int kDuoHb64 = 2, kDuoHb32 = 11;  // widest halo
+constexpr int kDuoHb = 11;               // widest halo
 constexpr int kDuoSmem = 232448 - 4096;  // static shared memory: below 4 KB
 constexpr int kTeamCols = kPropBlk / (kTeamWarps / 4);
 // Rows of a plane, and blocks of a tile, with `tab` bytes of tables: the MMA
 // reads 128 rows whatever the tile, also past the last plane's end.
-template <typename T>
 __host__ __device__ __forceinline__ int duo_rows(int tab, int hb)
 {
-    constexpr int ND = TileShape<T>::ND;
+    constexpr int NV = kPropNv32;
     const int need = 128 + 2 * hb, left = kDuoSmem - 1024 - ((tab + 1023) & ~1023);
     // (in eights, both the rows there are and the rows there could be use of:
     // a swizzled plane starts on 1024 bytes)
-    const int rows = (left - (need + 7) * 128) / ((2 * ND - 1) * 128) & ~7, most = (need + 7) & ~7;
+    const int rows = (left - (need + 7) * 128) / ((2 * NV - 1) * 128) & ~7,
+              most = (need + 7) & ~7;
     return rows < most ? rows : most;
 }
 
-template <typename T>
 __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_constant__ PropRun P)
 {
+    using T = float;
     using S = TileShape<T>;
     using G = typename GroupsOf<T>::G;
-    constexpr int ND = S::ND, NG = S::kGroups;
+    constexpr int ND = S::ND, NV = S::NV, NG = S::kGroups;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *sm = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                           ~static_cast<uintptr_t>(1023));
@@ -1418,6 +1476,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
     __shared__ volatile int s_abort, s_stop[2];
     __shared__ int s_code[2][kPropTileBlks + 2 * S::kHb + 8];
     __shared__ int s_max[2][2], s_keep[2], s_left[2], s_turn;
+    __shared__ int s_bits[2][kPropTileBlks];
     __shared__ PropHeader s_hdr;
     __shared__ DotShared<kEdgeRows> s_dot;
     __shared__ int4 s_prod[NG * ND];
@@ -1452,8 +1511,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
     const int hb = P.hb, tab_bytes = s_hdr.rows * 16;
     // (a table the tiles cannot hold: by the plan's rule there is none, and
     // every block would take dot products)
-    const bool ok_tab = s_hdr.ok && tab_bytes <= S::kTab && duo_rows<T>(tab_bytes, hb) > 2 * hb;
-    const int C = ok_tab ? duo_rows<T>(tab_bytes, hb) : 64 + 2 * hb;
+    const bool ok_tab = s_hdr.ok && tab_bytes <= S::kTab && duo_rows(tab_bytes, hb) > 2 * hb;
+    const int C = ok_tab ? duo_rows(tab_bytes, hb) : 64 + 2 * hb;
     const int per = C - 2 * hb < kPropTileBlks ? C - 2 * hb : kPropTileBlks;  // blocks of a tile
     const long long tiles = (P.blk1 - P.blk0 + per - 1) / per;
     if (t == 0 && ok_tab) {
@@ -1483,7 +1542,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
         const int m = warp - kTileWarps;
         const bool leader = elect_one();
         bool ok = true, tab_waited = false;
-        const uint64_t ad0 = swizzled_desc(saddr(planes + (size_t)m * ND * C * 128)), bd0 = plain_desc(saddr(sm), 128);
+        const uint64_t ad0 = swizzled_desc(saddr(planes + (size_t)m * NV * C * 128)), bd0 = plain_desc(saddr(sm), 128);
         int committed = -1;
         for (uint32_t n = 0; ok; ++n) {  // n: the team's tiles so far
             ok = __all_sync(0xffffffffu, bar_wait(&full[m], n & 1, kWaitLimitCycles, &s_abort));
@@ -1491,7 +1550,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
                 break;
             // one team's MMAs at a time: side by side, both would take twice as
             // long, and then convert and drain side by side too
-            if (sizeof(T) == 4 && lane == 0) {
+            if (lane == 0) {
                 const long long t0 = clock64();
                 while (atomicCAS(&s_turn, 0, 1) != 0 && !s_abort && clock64() - t0 < kWaitLimitCycles)
                     __nanosleep(40);
@@ -1527,7 +1586,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
                 __syncwarp();
                 committed = (int)((n & 1) << 8) | g;
             }
-            if (sizeof(T) == 4 && lane == 0)
+            if (lane == 0)
                 atomicExch(&s_turn, 0);
         }
         if (!ok && lane == 0) {
@@ -1542,14 +1601,14 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
         // ---- a team: load, convert, drain -------------------------------------
         const int m = warp / kTeamWarps, tw = warp % kTeamWarps, tt = t % kTeam;
         auto sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(2 + m), "n"(kTeam) : "memory"); };
-        unsigned char *xp = planes + (size_t)m * ND * C * 128;
+        unsigned char *xp = planes + (size_t)m * NV * C * 128;
         uint32_t phase = 0;
         for (long long tile = (long long)blockIdx.x * 2 + m; tile < tiles; tile += 2LL * gridDim.x) {
             const long long b0 = P.blk0 + tile * per;
             const int nb = (int)(P.blk1 - b0 < per ? P.blk1 - b0 : per);
             const long long base = (b0 - hb) * kPropBlk;
             const int chunks = (per + 2 * hb) * 8;
-            constexpr int kIter = ((kPropTileBlks + 2 * (sizeof(T) == 8 ? 0 : kDuoHb32)) * 8 + kTeam - 1) / kTeam;
+            constexpr int kIter = ((kPropTileBlks + 2 * kDuoHb) * 8 + kTeam - 1) / kTeam;
             if (tt < 2)
                 s_max[m][tt] = 0;
             if (tt == 2)
@@ -1622,9 +1681,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
             if (s_left[m])
                 break;
             const int ref = s_max[m][0], cone = s_max[m][1];
+            bool listed = false;  // block tt
             if (tt < nb) {
-                const int q = s_code[m][hb + tt];
-                const bool listed = cone > 0 && (!ok_tab || cone == kCodeInf<T> || q < cone - S::kRange || q == 0);
+                s_bits[m][tt] = 0;
+                listed = cone > 0 && (!ok_tab || values_too_small<T>(P, s_code[m][hb + tt], ref, cone));
                 if (listed)
                     P.list[atomicAdd(P.count, 1)] = (int)(b0 + tt);
                 else if (cone > 0)
@@ -1653,11 +1713,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
                 bar_arrive(&full[m]);
             // drain: kTeamCols points of the lane's block
             const int row = (warp & 3) * 32 + lane, col = (tw >> 2) * kTeamCols;
-            const int room = s_hdr.room, xs = sizeof(T) == 4 ? 0 : room < 8 ? room : 8;
-            long long acc[kTeamCols];
-#pragma unroll
-            for (int v = 0; v < kTeamCols; ++v)
-                acc[v] = 0;
+            Sums<T, kTeamCols> acc;
             bool ok = true;
 #pragma unroll 1
             for (int g = 0; g < NG; ++g) {
@@ -1678,7 +1734,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
                         }
 #pragma unroll
                         for (int q = 0; q < 16; ++q)
-                            acc[h + q] = fold<T>(acc[h + q], G::weight(g), __float2int_rn(__uint_as_float(v[q])), xs);
+                            acc.fold(h + q, G::weight(g), __float2int_rn(__uint_as_float(v[q])));
                     }
                 }
             }
@@ -1688,29 +1744,16 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
                     s_abort = 1;
                 }
             } else if (row < nb) {
-                const int ex = sizeof(T) == 8 ? ref - 1022 + 2 - s_hdr.E - xs : ref - 126 - 6 - s_hdr.E;
-                unsigned char *o = xp + row * kStageRow<T> + col * (int)sizeof(T);
-                if (sizeof(T) == 8 && ex >= -1021 && ex <= 959) {
-                    // through the row's own space in a short loop: 32 times the
-                    // code would be fetched anew by every launch
-#pragma unroll
-                    for (int v = 0; v < kTeamCols; v += 2)
-                        *reinterpret_cast<longlong2 *>(o + v * 8) = make_longlong2(acc[v], acc[v + 1]);
-#pragma unroll 1
-                    for (int v = 0; v < kTeamCols; v += 2) {
-                        const longlong2 z = *reinterpret_cast<const longlong2 *>(o + v * 8);
-                        *reinterpret_cast<double2 *>(o + v * 8) =
-                            make_double2(from_fixed<double>(z.x, ex), from_fixed<double>(z.y, ex));
-                    }
-                } else {
-                    finish_row<T>(acc, ex, o);
-                }
+                atomicMax(&s_bits[m][row], acc.bits());
+                finish_row<T>(acc.hi, sum_exponent<T>(ref, s_hdr.E), xp + row * kStageRow<T> + col * (int)sizeof(T));
             }
             fence_async_smem();
             sync();
             if (tt < nb && !s_abort) {
                 bulk_store(out + (b0 + tt) * kPropBlk, xp + tt * kStageRow<T>, kPropBlk * (uint32_t)sizeof(T));
                 bulk_commit();
+                if (!listed && results_too_small(P, s_bits[m], tt, nb, s_hdr.keep))
+                    P.list[atomicAdd(P.count, 1)] = (int)(b0 + tt);
             }
             phase ^= 1;
             if (s_abort)
@@ -1778,8 +1821,7 @@ cudaError_t prop_prepare()
     smem(prop_tile_kernel<double, true>, kTileSmem<double>);
     smem(prop_tile_kernel<float, false>, kTileSmem<float>);
     smem(prop_tile_kernel<float, true>, kTileSmem<float>);
-    smem(prop_duo_kernel<double>, kDuoSmem);
-    smem(prop_duo_kernel<float>, kDuoSmem);
+    smem(prop_duo_kernel, kDuoSmem);
     smem(prop_dot_kernel<double>, (kDotWin + dot_taps(kPropRMax)) * 8);
     smem(prop_dot_kernel<float>, (kDotWin + dot_taps(kPropRMax)) * 8);
     if (e == cudaSuccess)
@@ -1822,10 +1864,11 @@ cudaError_t prop_launch_finish(const PropLevel &a, const PropFinish &f, cudaStre
     return cudaGetLastError();
 }
 
-cudaError_t prop_launch_digits(const PropSet &set, const PropFinish &f, int R, int f64, int hb_max, cudaStream_t s)
+cudaError_t prop_launch_digits(const PropSet &set, const PropFinish &f, int R, int prec, int hb_max, cudaStream_t s)
 {
-    prop_digits_kernel<<<1, 1024, 2 * kPropQ * 8, s>>>(f.x, f.x_max, R, f64 ? kPropNd64 : kPropNd32, hb_max,
-                                                                    f64 ? kPropTab64 : kPropTab32, set.tab, set.hdr);
+    prop_digits_kernel<<<1, 1024, 2 * kPropQ * 8, s>>>(f.x, f.x_max, R, prec == 0 ? kPropNd64 : kPropNd32,
+                                                                    prec == 2, hb_max,
+                                                                    prec == 0 ? kPropTab64 : kPropTab32, set.tab, set.hdr);
     return cudaGetLastError();
 }
 
@@ -1871,7 +1914,7 @@ cudaError_t prop_launch_tiles(PropRun a, int f64, int num_sms, cudaStream_t s)
     // on this device: loading and converting a tile, an MMA, finishing it, an
     // item of wall rows; a digit's reach is on average 0.62 of the halo).
     int best = 1, split_grid = 0;
-    const double mmas = (f64 ? 34.0 : 10.0) * (4 + 5 * a.hb), start = f64 ? 15500 : 11000;
+    const double mmas = (f64 ? 35.0 : 10.0) * (4 + 5 * a.hb), start = f64 ? 15500 : 11000;
     const double item = f64 ? 7000 + 16.0 * a.R : 6500 + 6.0 * a.R;
     if (a.tiles < num_sms) {
         const double rounds = std::ceil((double)edges / (double)(num_sms - a.tiles));
@@ -1916,11 +1959,8 @@ cudaError_t prop_launch_tiles(PropRun a, int f64, int num_sms, cudaStream_t s)
         return f64 ? cudaLaunchKernelEx(&c, prop_tile_kernel<double, true>, a)
                    : cudaLaunchKernelEx(&c, prop_tile_kernel<float, true>, a);
     }
-    if (a.tiles >= 2 * num_sms && a.hb <= (f64 ? kDuoHb64 : kDuoHb32)) {
-        if (f64)
-            prop_duo_kernel<double><<<num_sms, kTileThreads, kDuoSmem, s>>>(a);
-        else
-            prop_duo_kernel<float><<<num_sms, kTileThreads, kDuoSmem, s>>>(a);
+    if (!f64 && a.tiles >= 2 * num_sms && a.hb <= kDuoHb) {
+        prop_duo_kernel<<<num_sms, kTileThreads, kDuoSmem, s>>>(a);
         return cudaGetLastError();
     }
     const int grid = (int)(a.tiles + edges < num_sms ? a.tiles + edges : num_sms);

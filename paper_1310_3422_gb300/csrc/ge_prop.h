@@ -25,13 +25,16 @@ namespace ge {
 // Most taps kept per side (FP32; an FP64 context keeps up to kPropR64Max).
 constexpr int kPropRMax = 1536, kPropR64Max = 704;
 // Points of one block (columns of the accumulator) and blocks of a tile (its
-// rows, the 128 lanes of tensor memory).
+// rows, the 128 lanes of tensor memory).  FP64: with its halo a tile has 128,
+// the rows of a plane of digits that leave room for eight of them, and that
+// 512 threads load in two turns.
 constexpr int kPropBlk = 64;
-constexpr int kPropTileBlks = 128;
-// Digits (base 256) of a value and of a tap: FP64 and FP32 storage.
+constexpr int kPropTileBlks = 128, kPropRows64 = 128;
+// Digits (base 256) of a tap and of a value: FP64 and FP32 storage.
 constexpr int kPropNd64 = 7, kPropNd32 = 4;
-// Bytes of the tap tables in shared memory.
-constexpr int kPropTab64 = 96 * 1024, kPropTab32 = 136 * 1024;
+constexpr int kPropNv64 = 8, kPropNv32 = 4;
+// Bytes of the tap tables in shared memory (FP64: at most 93,824 by the plan's rule).
+constexpr int kPropTab64 = 93 * 1024, kPropTab32 = 136 * 1024;
 // Halo blocks a tile may have on each side.
 constexpr int kPropHb64 = 8, kPropHb32 = 16;
 
@@ -40,7 +43,7 @@ struct PropHeader {
     int E;         // a tap is its integer times 2^-E
     int ok;        // 0: the tables do not fit (never, by the plan's rule): every block takes the dot products
     int rows;      // 16-byte rows in all tables
-    int room;      // bits by which a row's sum of magnitudes at scale 2^E stays below 2^62
+    int keep;      // bits the largest sum of a block needs to be the tile's answer
     int W[8];      // reach of digit i's table: its taps beyond |d| = W are zero
     int row0[8];   // first row of digit i's table
 };
@@ -106,9 +109,13 @@ struct PropRun {
     const unsigned char *tab;
     const PropHeader *hdr;
     int *err;
-    // tiles: blocks [blk0, blk1) in tiles of kPropTileBlks, hb halo blocks per side
+    // tiles: blocks [blk0, blk1) in tiles of `per`, hb halo blocks per side
     long long blk0, blk1, tiles;
-    int hb;
+    int per, hb;
+    // a block is left to dot products when its values lie below 2^-range of
+    // the largest of the tile's window, or when its results (and those of
+    // `near` blocks a side) are too far below that (PropHeader::keep)
+    int range, near;
     // dot products: rows [0, rows_l) and [row_r, n), and the listed blocks
     long long rows_l, row_r;
     int *list, *count, *count_next;
@@ -148,7 +155,7 @@ cudaError_t prop_launch_short(double *e, double *el, double *h, double *hl, int 
                               cudaStream_t s);
 cudaError_t prop_launch_level(const PropLevel &a, cudaStream_t s);
 cudaError_t prop_launch_finish(const PropLevel &a, const PropFinish &f, cudaStream_t s);
-cudaError_t prop_launch_digits(const PropSet &set, const PropFinish &f, int R, int f64, int hb_max, cudaStream_t s);
+cudaError_t prop_launch_digits(const PropSet &set, const PropFinish &f, int R, int prec, int hb_max, cudaStream_t s);
 cudaError_t prop_launch_tiles(PropRun a, int f64, int num_sms, cudaStream_t s);
 cudaError_t prop_launch_dots(const PropRun &a, int f64, int grid, cudaStream_t s);
 cudaError_t prop_prepare();  // per-device kernel attributes

@@ -71,6 +71,24 @@ int halo_blocks(double r, int k, int f64)
     return std::min(hb, f64 ? kPropHb64 : kPropHb32);
 }
 
+// Which blocks of a tile are left to dot products (PropRun::range, near).
+// Values are held to 2^-63 (FP32: 2^-31) of 2^e, the power of two above the
+// window's largest, and the rounding of that is smoothed as the values are:
+// for taps of standard deviation d its root mean square shrinks by S =
+// (2 sqrt(pi) d)^-1/2.  `range` keeps it below 2^-54 (2^-25) of a block's
+// largest value, which storing the result may cost as well.
+//   Past d = 48 points the steps one by one give a block the errors of the
+// blocks beside it (where a smooth field crosses zero, say), and its results
+// are looked at together with theirs.
+void tile_range(double r, int k, int f64, int *range, int *near)
+{
+    const double d = std::sqrt(2.0 * r * (double)k);
+    const bool bell = k >= 16.0 * r;
+    const double s2 = bell ? std::min(1.0, 1.0 / (3.5449 * d)) : 1.0;
+    *range = (f64 ? 8 : 5) + (int)std::floor(-0.5 * std::log2(s2));
+    *near = bell && d >= 48.0 ? 1 : 0;
+}
+
 }  // namespace
 
 size_t prop_bytes(long long n, int f64) { return Sizes(n, f64).total(); }
@@ -257,7 +275,7 @@ cudaError_t build_set(PropState *st, const PropTarget &t, PropSet &s, int pr, in
     }
     e = prop_launch_finish(a, f, stream);
     if (e == cudaSuccess && f.x)
-        e = prop_launch_digits(s, f, a.R1, t.f64, hb, stream);
+        e = prop_launch_digits(s, f, a.R1, t.prec, hb, stream);
     return e;
 }
 
@@ -394,7 +412,9 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
             a.hb = w.hb;
             a.blk0 = a.hb;
             a.blk1 = t.n / kPropBlk - a.hb;
-            a.tiles = (a.blk1 - a.blk0 + kPropTileBlks - 1) / kPropTileBlks;
+            a.per = t.f64 ? kPropRows64 - 2 * a.hb : kPropTileBlks;
+            a.tiles = (a.blk1 - a.blk0 + a.per - 1) / a.per;
+            tile_range(r, s.k, t.f64, &a.range, &a.near);
             a.rows_l = a.blk0 * kPropBlk;
             a.row_r = a.blk1 * kPropBlk;
             // listed blocks past which the whole grid step by step is sooner

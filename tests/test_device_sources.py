@@ -50,31 +50,26 @@ def test_two_teams_fit_shared_memory(tmp_path):
     within the block's shared memory."""
     header = re.findall(r"constexpr int kProp[^;]*;", code("ge_prop.h"))
     text = code("ge_prop.cu")
-    shapes = re.search(r"template <typename T>\s*struct TileShape;.*?struct TileShape<float> \{.*?\};", text, re.S).group(0)
     consts = re.findall(r"constexpr int kDuo[^;]*;", text)
-    rows = re.search(r"template <typename T>\s*__host__ __device__ __forceinline__ int duo_rows.*?\n\}", text, re.S).group(0)
+    rows = re.search(r"__host__ __device__ __forceinline__ int duo_rows.*?\n\}", text, re.S).group(0)
     src = tmp_path / "duo.cpp"
-    src.write_text("#include <cstdio>\n#define __host__\n#define __device__\n#define __forceinline__ inline\n" + "\n".join(
-        header) + "\n" + shapes + "\n" + "\n".join(consts) + "\n" + rows + """
-template <typename T> int check(int widest, int most)
+    src.write_text("#include <cstdio>\n#define __host__\n#define __device__\n#define __forceinline__ inline\n"
+                   + "\n".join(header + consts) + "\n" + rows + """
+int main()
 {
     int bad = 0;
-    for (int hb = 1; hb <= widest; ++hb)
-        for (int tab = 0; tab <= most; tab += 16) {
-            const int C = duo_rows<T>(tab, hb);
+    for (int hb = 1; hb <= kDuoHb; ++hb)
+        for (int tab = 0; tab <= kPropTab32; tab += 16) {
+            const int C = duo_rows(tab, hb);
             if (C <= 2 * hb)
                 continue;  // the kernel leaves such a table to dot products
             const int left = kDuoSmem - 1024 - (tab + 1023) / 1024 * 1024;
-            const int used = ((2 * PLANES - 1) * C + 128 + 2 * hb) * 128;
-            if (C % 8 || used > left)
-                if (!bad++)
-                    std::printf("halo %d, %d bytes of tables: %d rows, %d of %d bytes\\n", hb, tab, C, used, left);
+            const int used = ((2 * kPropNv32 - 1) * C + 128 + 2 * hb) * 128;
+            if ((C % 8 || used > left) && !bad++)
+                std::printf("halo %d, %d bytes of tables: %d rows, %d of %d bytes\\n", hb, tab, C, used, left);
         }
-    return bad;
+    return bad ? 1 : 0;
 }
-""".replace("PLANES", "(sizeof(T) == 8 ? %s : %s)" % (
-        ("TileShape<double>::NV", "TileShape<float>::NV") if "NV =" in shapes else ("TileShape<double>::ND", "TileShape<float>::ND"))) + """
-int main() { return check<double>(kDuoHb64, kPropTab64) + check<float>(kDuoHb32, kPropTab32) ? 1 : 0; }
 """)
     exe = tmp_path / "duo"
     subprocess.run(["g++", "-std=c++17", "-O1", str(src), "-o", str(exe)], check=True)

@@ -48,7 +48,7 @@ def rms_errors(u0, r, bl, br, steps, prec, parts=None):
     """RMS error of both kernels over the rows of u0, divided by the exact
     field's RMS there (over `parts` of a row)."""
     want = exact(u0, r, bl, br, steps)
-    parts = parts or slice(None)
+    parts = slice(None) if parts is None else parts
     norm = np.sqrt(np.mean(want[:, parts] ** 2))
     return [float(np.sqrt(np.mean([np.mean((run(u, r, bl, br, steps, kernel, prec)[parts] - w[parts]) ** 2)
                                    for u, w in zip(u0, want)])) / norm)
@@ -83,3 +83,23 @@ def test_short_rows_of_rough_data(r, steps):
     6 % in its root for either kernel, 1.1."""
     auto, tiled = rms_errors(rough(16, 1024), r, 0.3, -0.8, steps, B.GE_F64)
     assert auto <= 1.1 * tiled, (auto, tiled)
+
+
+# either side of where blocks go to dot products instead: by their values
+# (2^-8 to 2^-12 of their neighbours', FP32 2^-5 to 2^-9), by their results
+@pytest.mark.parametrize("level", [2, 4, 5, 6, 7, 8, 9, 10, 12, 16, 24])
+@pytest.mark.parametrize("prec,r,steps", [(B.GE_F64, 1.0, 24), (B.GE_F64, 0.5, 100), (B.GE_F64, 2.0, 300),
+                                          (B.GE_F32, 1.0, 150), (B.GE_F32, 4.0, 400), (B.GE_F32_COMP, 1.0, 150),
+                                          (B.GE_F32_COMP, 4.0, 400)])
+def test_quiet_stretches_keep_their_precision(prec, r, steps, level):
+    """Stretches of rough data 2^-level of the data around them: within them
+    (14 standard deviations of the taps from their ends) composed steps err no
+    more than steps one by one, relative to the stretch's own field."""
+    u0 = rough(1, 20000, np.float64 if prec == B.GE_F64 else np.float32)
+    inner = np.zeros(20000, bool)
+    margin = int(14 * np.sqrt(2 * r * steps)) + 10
+    for a in (6000, 13000):
+        u0[:, a:a + 3000] *= 2.0 ** -level
+        inner[a + margin:a + 3000 - margin] = True
+    auto, tiled = rms_errors(u0, r, 0.3, -0.8, steps, prec, inner)
+    assert auto <= SLACK * tiled, (auto, tiled)
