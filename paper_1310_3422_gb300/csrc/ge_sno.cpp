@@ -89,6 +89,7 @@ struct ge_sno {
     bool tc = true;                       // use it where the shape allows
     bool tc_ready = false;                // tensor maps encoded
     int num_sms = 0;
+    ge::SnoTcGrid grid{};                 // launch sizes of the tensor-core kernels
     void *wt = nullptr;                   // [L][C out][C in] BF16
     void *q1t = nullptr;                  // [H][C] BF16
     void *wst = nullptr;                  // [L][M][2C out][2C in] BF16 (K-major spectral weights)
@@ -393,7 +394,7 @@ ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const fl
         const LayerOff &o = s->lay[l];
         // truncated DFT: vh[b] = F v[b]
         a.out = s->vh[l];
-        SNO_TRY(ge::sno_tc_dft(&s->tm_f, &s->tm_v[l], a, s->num_sms, st));
+        SNO_TRY(ge::sno_tc_dft(&s->tm_f, &s->tm_v[l], a, s->grid, st));
         // per-mode complex mixing: y[b, m] = vh[b, m] Wspec_m
         const ge::SnoTcMixArgs x{B, l * M * 2 * C, 2LL * M * C, s->y, s->err, ge::kWaitLimitCycles, early};
         SNO_TRY(ge::sno_tc_mix(&s->tm_vh[l], &s->tm_wst, x, M, st));
@@ -402,7 +403,7 @@ ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const fl
         a.bias = P + o.b;
         a.out = s->v[l + 1];
         const ge::SnoTcMaps m{&s->tm_g, &s->tm_y, &s->tm_v[l], &s->tm_wt, &s->tm_vs[l]};
-        SNO_TRY(ge::sno_tc_layer(m, a, s->num_sms, st));
+        SNO_TRY(ge::sno_tc_layer(m, a, s->grid, st));
     }
     a.b2_row = 0;
     a.gelu = 1;
@@ -412,7 +413,7 @@ ge_status forward_tc(ge_sno *s, int B, const float *u0, const float *r, const fl
     a.u0 = u0;
     a.out = out;
     const ge::SnoTcMaps m{nullptr, nullptr, &s->tm_v[s->L], &s->tm_q1t, nullptr};
-    SNO_TRY(ge::sno_tc_projection(m, a, s->num_sms, st));
+    SNO_TRY(ge::sno_tc_projection(m, a, s->grid, st));
     return GE_OK;
 }
 
@@ -682,6 +683,10 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
     if (e != cudaSuccess) {
         release_sno(s);
         return scuda(e, "ge_sno_create: device allocation");
+    }
+    if (tc_shape(s) && (e = ge::sno_tc_prepare(&s->grid, s->num_sms)) != cudaSuccess) {
+        release_sno(s);
+        return scuda(e, "ge_sno_create: tensor-core kernels");
     }
     if (tc_shape(s)) {
         // tensor maps of the tensor-core path (BF16 views of the buffers)

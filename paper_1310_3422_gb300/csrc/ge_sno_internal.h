@@ -87,12 +87,20 @@ struct SnoTcArgs {
     long long limit;        // wait limit in SM cycles
     int early;              // start under the end of the kernel before (see launch_early)
 };
-cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s);
-cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s);
+// What a model keeps of its device: the SMs, and each persistent kernel's
+// co-resident CTAs.  sno_tc_prepare fills it and sets, on the current device,
+// the attributes of every kernel below (they belong to the device, so each
+// model's creation sets them).
+struct SnoTcGrid {
+    int sms, layer, projection, dft2, dft8;
+};
+cudaError_t sno_tc_prepare(SnoTcGrid *g, int sms);
+cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, const SnoTcGrid &g, cudaStream_t s);
+cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, const SnoTcGrid &g, cudaStream_t s);
 // Truncated DFT vh[b] = F v[b] on the tensor cores (2M = 32, C = 64; map_f:
 // F [2M][n] BF16, box 64 x 32, 128-byte swizzle; map_v: the activation map of
 // the layer kernel); writes a.out = vh, BF16 [batch][2M][C].
-cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a, int sms, cudaStream_t s);
+cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a, const SnoTcGrid &g, cudaStream_t s);
 // Mode mixing y[b, m] = vh[b, m] Wspec_m on the tensor cores (2C = 128):
 // map_vh over vh [batch rows][2M * 2C] (box 64 x 128, 128-byte swizzle),
 // map_wst over the K-major spectral weights Wspec_m^T of all layers

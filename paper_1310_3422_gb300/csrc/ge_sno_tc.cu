@@ -872,47 +872,42 @@ cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, int threads, int 
     return cudaLaunchKernelEx(&c, kernel, args...);
 }
 
+// Dynamic shared memory a kernel may take, on the current device, and (where
+// per_sm is given) its co-resident CTAs per SM: what shared memory holds at
+// the largest carve-out (the kernel's static and dynamic bytes plus the
+// driver's reserve per CTA), what the registers hold, and at most `most`, so
+// that their TMEM columns (512 per SM) all fit.
+template <typename... Params>
+cudaError_t prepare_kernel(void (*kernel)(Params...), int threads, int smem, int most, int *per_sm)
+{
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess || !per_sm)
+        return e;
+    cudaFuncAttributes fa{};
+    int dev = 0, sm_bytes = 0, reserve = 0;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess)
+        e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess)
+        e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&reserve, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (e != cudaSuccess)
+        return e;
+    const int fit = sm_bytes / (smem + (int)fa.sharedSizeBytes + reserve),
+              regs = 65536 / ((fa.numRegs + 7) / 8 * 8 * threads);
+    *per_sm = fit < regs ? fit : regs;
+    *per_sm = *per_sm < most ? *per_sm : most;
+    return *per_sm < 1 ? cudaErrorInvalidConfiguration : cudaSuccess;
+}
+
 template <int MODE>
-cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
+cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int ctas, cudaStream_t s)
 {
     using S = TcShape<MODE>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(sno_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             S::kSmem);
-        // the largest shared-memory carve-out, so that as many CTAs fit as
-        // TMEM allows (3 layer CTAs of 74 KB need about 225 KB)
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(sno_tc_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess)
-            return e;
-        attr_set = true;
-    }
-    // co-resident CTAs per SM: what shared memory holds (the kernel's static
-    // and dynamic bytes plus the driver's reserve per CTA), capped so that
-    // their TMEM columns (at most 512 per SM) all fit
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        cudaFuncAttributes fa{};
-        int dev = 0, sm_bytes = 0, reserve = 0;
-        cudaError_t e = cudaFuncGetAttributes(&fa, sno_tc_kernel<MODE>);
-        if (e == cudaSuccess)
-            e = cudaGetDevice(&dev);
-        if (e == cudaSuccess)
-            e = cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        if (e == cudaSuccess)
-            e = cudaDeviceGetAttribute(&reserve, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-        if (e != cudaSuccess)
-            return e;
-        int fit = sm_bytes / (S::kSmem + (int)fa.sharedSizeBytes + reserve);
-        const int tmem_cap = 512 / (int)S::kTmemCols, reg_cap = 65536 / ((fa.numRegs + 7) / 8 * 8 * kTcThreads);
-        per_sm = fit < tmem_cap ? fit : tmem_cap;
-        per_sm = per_sm < reg_cap ? per_sm : reg_cap;
-        if (per_sm < 1)
-            return cudaErrorInvalidConfiguration;
-    }
-    long long grid = (long long)sms * per_sm;
+    long long grid = ctas;
     if (grid > a.n_tiles)
         grid = a.n_tiles;
     if (grid < 1)
@@ -929,33 +924,10 @@ cudaError_t launch_tc(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStrea
 }
 
 template <int ST>
-cudaError_t launch_dft(const CUtensorMap &f, const CUtensorMap &v, const SnoTcArgs &a, int sms, cudaStream_t s)
+cudaError_t launch_dft(const CUtensorMap &f, const CUtensorMap &v, const SnoTcArgs &a, int ctas, cudaStream_t s)
 {
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(sno_tc_dft_kernel<ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, dft_smem(ST));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(sno_tc_dft_kernel<ST>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     cudaSharedmemCarveoutMaxShared);
-        cudaFuncAttributes fa{};
-        int dev = 0, sm_bytes = 0, reserve = 0;
-        if (e == cudaSuccess)
-            e = cudaFuncGetAttributes(&fa, sno_tc_dft_kernel<ST>);
-        if (e == cudaSuccess)
-            e = cudaGetDevice(&dev);
-        if (e == cudaSuccess)
-            e = cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-        if (e == cudaSuccess)
-            e = cudaDeviceGetAttribute(&reserve, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-        if (e != cudaSuccess)
-            return e;
-        const int fit = sm_bytes / (dft_smem(ST) + (int)fa.sharedSizeBytes + reserve);
-        per_sm = fit < 4 ? fit : 4;  // 128 TMEM columns each
-        if (per_sm < 1)
-            return cudaErrorInvalidConfiguration;
-    }
     const long long problems = a.n_tiles / a.tiles_per_problem;
-    long long grid = (long long)sms * per_sm;
+    long long grid = ctas;
     if (grid > problems)
         grid = problems;
     if (grid < 1)
@@ -963,19 +935,10 @@ cudaError_t launch_dft(const CUtensorMap &f, const CUtensorMap &v, const SnoTcAr
     return launch_early(sno_tc_dft_kernel<ST>, dim3((unsigned)grid), kDftThreads, dft_smem(ST), s, a.early, f, v, a);
 }
 
-
 template <int KIND>
 cudaError_t launch_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, dim3 grid, cudaStream_t s)
 {
     using S = GradShape<KIND>;
-    static bool ready = false;
-    if (!ready) {
-        cudaError_t e =
-            cudaFuncSetAttribute(sno_tc_grad_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
-        if (e != cudaSuccess)
-            return e;
-        ready = true;
-    }
     if (!map_x || !map_y || a.rows < 0 || a.rows > 0x7FFFFF00LL)
         return cudaErrorInvalidValue;
     if (a.rows == 0 || grid.x == 0 || grid.y == 0)
@@ -986,33 +949,49 @@ cudaError_t launch_grad(const void *map_x, const void *map_y, const SnoTcGradArg
 
 }  // namespace
 
-cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
+cudaError_t sno_tc_prepare(SnoTcGrid *g, int sms)
 {
-    return launch_tc<0>(m, a, sms, s);
+    int layer = 0, projection = 0, dft2 = 0, dft8 = 0;
+    auto tmem = [](uint32_t cols) { return 512 / (int)cols; };
+    cudaError_t e = prepare_kernel(sno_tc_kernel<0>, kTcThreads, TcShape<0>::kSmem, tmem(TcShape<0>::kTmemCols), &layer);
+    if (e == cudaSuccess)
+        e = prepare_kernel(sno_tc_kernel<1>, kTcThreads, TcShape<1>::kSmem, tmem(TcShape<1>::kTmemCols), &projection);
+    if (e == cudaSuccess)
+        e = prepare_kernel(sno_tc_dft_kernel<2>, kDftThreads, dft_smem(2), tmem(128), &dft2);
+    if (e == cudaSuccess)
+        e = prepare_kernel(sno_tc_dft_kernel<8>, kDftThreads, dft_smem(8), tmem(128), &dft8);
+    if (e == cudaSuccess)
+        e = prepare_kernel(sno_tc_mix_kernel, kMixThreads, kMixSmem, 0, nullptr);
+    if (e == cudaSuccess)
+        e = prepare_kernel(sno_tc_grad_kernel<0>, kGradThreads, GradShape<0>::kSmem, 0, nullptr);
+    if (e == cudaSuccess)
+        e = prepare_kernel(sno_tc_grad_kernel<1>, kGradThreads, GradShape<1>::kSmem, 0, nullptr);
+    if (e == cudaSuccess)
+        e = prepare_kernel(sno_tc_grad_kernel<2>, kGradThreads, GradShape<2>::kSmem, 0, nullptr);
+    *g = {sms, sms * layer, sms * projection, sms * dft2, sms * dft8};
+    return e;
 }
 
-cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, int sms, cudaStream_t s)
+cudaError_t sno_tc_layer(const SnoTcMaps &m, const SnoTcArgs &a, const SnoTcGrid &g, cudaStream_t s)
 {
-    return launch_tc<1>(m, a, sms, s);
+    return launch_tc<0>(m, a, g.layer, s);
 }
 
-cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a, int sms, cudaStream_t s)
+cudaError_t sno_tc_projection(const SnoTcMaps &m, const SnoTcArgs &a, const SnoTcGrid &g, cudaStream_t s)
+{
+    return launch_tc<1>(m, a, g.projection, s);
+}
+
+cudaError_t sno_tc_dft(const void *map_f, const void *map_v, const SnoTcArgs &a, const SnoTcGrid &g, cudaStream_t s)
 {
     if (!map_f || !map_v || a.tiles_per_problem < 1)
         return cudaErrorInvalidValue;
     const CUtensorMap &f = *static_cast<const CUtensorMap *>(map_f), &v = *static_cast<const CUtensorMap *>(map_v);
-    return a.n_tiles / a.tiles_per_problem <= sms ? launch_dft<8>(f, v, a, sms, s) : launch_dft<2>(f, v, a, sms, s);
+    return a.n_tiles / a.tiles_per_problem <= g.sms ? launch_dft<8>(f, v, a, g.dft8, s) : launch_dft<2>(f, v, a, g.dft2, s);
 }
 
 cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s)
 {
-    static bool ready = false;
-    if (!ready) {
-        cudaError_t e = cudaFuncSetAttribute(sno_tc_mix_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMixSmem);
-        if (e != cudaSuccess)
-            return e;
-        ready = true;
-    }
     if (!map_vh || !map_wst || modes < 1 || a.batch < 0)
         return cudaErrorInvalidValue;
     if (a.batch == 0)

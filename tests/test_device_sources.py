@@ -75,3 +75,15 @@ int main()
     subprocess.run(["g++", "-std=c++17", "-O1", str(src), "-o", str(exe)], check=True)
     res = subprocess.run([str(exe)], capture_output=True, text=True)
     assert res.returncode == 0, res.stdout
+
+
+def test_kernel_attributes_are_set_for_every_model():
+    """The attributes a launch needs belong to a device: set once a process,
+    a model on the next device would fail at its first launch."""
+    text = code("ge_sno_tc.cu")
+    assert not re.search(r"\bstatic\s+(bool|int)\b", text)
+    assert len(re.findall(r"cudaFuncAttributeMaxDynamicSharedMemorySize", text)) == 1
+    kernels = {name for name, _ in functions(text)}
+    prepared = re.search(r"cudaError_t sno_tc_prepare.*?\n\}", text, re.S).group(0)
+    assert kernels and kernels == set(re.findall(r"prepare_kernel\((\w+)", prepared))
+    assert "sno_tc_prepare(&s->grid" in code("ge_sno.cpp")
