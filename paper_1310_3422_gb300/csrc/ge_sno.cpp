@@ -84,6 +84,7 @@ struct ge_sno {
     float *dvh = nullptr;                 // [B][2M][C]
     float *sums = nullptr;                // column sums' scratch, and their blocks' counts (zero between launches)
     int *sum_tickets = nullptr;
+    float *bias_parts[2] = {nullptr, nullptr};  // tensor-core bias gradients: a layer's, the projection's
     // tensor-core inference path (ge_sno_tc.cu; plain mode, C = 64, 2M = 32,
     // H = 128, n a multiple of 128): transposed B operands and tensor maps
     bool tc = true;                       // use it where the shape allows
@@ -430,7 +431,7 @@ ge_status backward(ge_sno *s, int B)
     float *Gd = s->grads;
     ge_status rc;
     const bool tc = tc_active(s);
-    if (tc)  // sno_tc_grad adds to its results
+    if (tc)  // sno_tc_grad adds to dw
         SNO_TRY(cudaMemsetAsync(Gd, 0, sizeof(float) * s->n_params, st));
     ge::SnoTcGradArgs tg{};
     tg.rows = R;
@@ -461,7 +462,7 @@ ge_status backward(ge_sno *s, int B)
     SNO_TRY(ge::sno_colsum(q, bf ? 1 : 0, st));
     if (tc) {
         tg.dw = Gd + s->off_q1;
-        tg.db = Gd + s->off_qb1;
+        tg.part = s->bias_parts[1];
         SNO_TRY(ge::sno_tc_grad(&s->tm_v[s->L], &s->tm_dAh, tg, H, s->num_sms, st));
     } else if ((rc = weight_grad(s, s->v[s->L], C, C, s->dA, H, R, Gd + s->off_q1, Gd + s->off_qb1)) != GE_OK) {
         return rc;
@@ -479,7 +480,7 @@ ge_status backward(ge_sno *s, int B)
         // pointwise path weights
         if (tc) {
             tg.dw = Gd + o.w;
-            tg.db = Gd + o.b;
+            tg.part = s->bias_parts[0];
             SNO_TRY(ge::sno_tc_grad(&s->tm_v[l], dv == s->dB ? &s->tm_dB : &s->tm_dA, tg, C, s->num_sms, st));
         } else if ((rc = weight_grad(s, s->v[l], C, C, dpre, C, R, Gd + o.w, Gd + o.b)) != GE_OK) {
             return rc;
@@ -496,6 +497,11 @@ ge_status backward(ge_sno *s, int B)
             ts.rows = B;
             ts.drr = Gd + o.rr;
             ts.dri = Gd + o.ri;
+            // (the projection's with the last layer's, the first to come)
+            const int ctas = ge::sno_tc_grad_ctas(R, s->num_sms);
+            ts.bias[0] = {s->bias_parts[0], ctas, C, Gd + o.b};
+            if (l == s->L - 1)
+                ts.bias[1] = {s->bias_parts[1], ctas, H, Gd + s->off_qb1};
             SNO_TRY(ge::sno_tc_grad_spec(&s->tm_vh[l], &s->tm_dy, ts, M, st));
         } else {
             g = gemm(s->vh[l], 1, 2LL * M * C, s->y, 2LL * M * C, 1, s->dwspec, 2 * C, 2 * C, 2 * C, B);
@@ -683,6 +689,14 @@ ge_status ge_sno_create(ge_sno **out, int32_t n, int32_t width, int32_t modes, i
     if (e != cudaSuccess) {
         release_sno(s);
         return scuda(e, "ge_sno_create: device allocation");
+    }
+    if (tc_shape(s)) {
+        e = alloc(&s->bias_parts[0], (long long)s->num_sms * C);
+        e = e ? e : alloc(&s->bias_parts[1], (long long)s->num_sms * H);
+        if (e != cudaSuccess) {
+            release_sno(s);
+            return scuda(e, "ge_sno_create: device allocation");
+        }
     }
     if (tc_shape(s) && (e = ge::sno_tc_prepare(&s->grid, s->num_sms)) != cudaSuccess) {
         release_sno(s);

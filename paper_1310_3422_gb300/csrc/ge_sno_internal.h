@@ -117,19 +117,28 @@ struct SnoTcMixArgs {
 cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixArgs &a, int modes, cudaStream_t s);
 // Weight gradients on the tensor cores, dW = X^T dY over the rows of both:
 //   sno_tc_grad:  X [rows][64] (map_x, box 64 x 128), dY [rows][cols] with
-//       cols = 64 or 128 (map_y, box 64 x 128); adds to dw [64][cols] and
-//       the column sums of dY to db [cols] (both 16-byte aligned).
+//       cols = 64 or 128 (map_y, box 64 x 128); adds to dw [64][cols] (16-byte
+//       aligned) and writes each CTA's column sums of its rows of dY to part
+//       [sno_tc_grad_ctas(rows, sms)][cols].
 //   sno_tc_grad_spec:  per mode m, X and dY the columns 128 m .. 128 m + 127
 //       of vh and dy [rows][2M * C] (same boxes); writes dRr and dRi
-//       [modes][C out][C in], C = 64.
+//       [modes][C out][C in], C = 64; and adds up to two such sets of parts.
+struct SnoBiasParts {
+    const float *part;   // [ctas][cols], cols a multiple of 16 (0: none)
+    int ctas, cols;
+    float *out;          // [cols], 16-byte aligned
+};
 struct SnoTcGradArgs {
     long long rows;
-    float *dw, *db;      // sno_tc_grad
+    float *dw, *part;    // sno_tc_grad
     float *drr, *dri;    // sno_tc_grad_spec
+    SnoBiasParts bias[2];
+    int modes;           // set by sno_tc_grad_spec
     int *err;            // device error word
     long long limit;     // wait limit in SM cycles
     int early;           // as in SnoTcArgs
 };
+int sno_tc_grad_ctas(long long rows, int sms);
 cudaError_t sno_tc_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, int cols, int sms,
                         cudaStream_t s);
 cudaError_t sno_tc_grad_spec(const void *map_vh, const void *map_dy, const SnoTcGradArgs &a, int modes,

@@ -665,9 +665,13 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
 //   KIND 0 / 1: X [rows][64], dY [rows][64 / 128].  The instruction has 128
 //       rows of A and X gives 64: the others come from a constant tile whose
 //       first column is 1 (the second atom of A, at its own stride), so that
-//       accumulator row 64 is the column sum of dY, the bias gradient.
+//       accumulator row 64 is the column sum of dY, the bias gradient.  Each
+//       CTA stores its own; they are added in a fixed order, so that it is the
+//       same from run to run, by the next KIND 2 launch.  (By the last CTA to
+//       finish: 3 to 6 us a launch.)
 //   KIND 2: one CTA per mode, X and dY [rows = problems][128]; D = X^T dY is
-//       folded to the complex weights' gradients before it is stored.
+//       folded to the complex weights' gradients before it is stored.  A
+//       few more CTAs add the bias parts meanwhile.
 // Bound by the latency of the loads and of the adds (16 MB in KIND 0: 2.4 us
 // at the copy rate).  65,536 rows, cold caches: KIND 0 takes 11.1 us, KIND 1
 // 12.9 us; as mma.sync tiles with split K, a column-sum pass and a memset
@@ -689,6 +693,31 @@ __device__ __forceinline__ void red_add4(float *p, float a, float b, float c, fl
     asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
+// Columns 16 c .. 16 c + 15 of the parts [ctas][cols] of a bias gradient, added
+// in a fixed order by 128 threads: thread (k, j) takes CTAs k, k + 32, ..., so
+// that all loads are in flight at once.
+__device__ __forceinline__ void add_bias_parts(const SnoBiasParts &b, int c, float4 (&sh)[128])
+{
+    const int t = threadIdx.x, at = 4 * c + t % 4;
+    const float4 *part = reinterpret_cast<const float4 *>(b.part);
+    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 5
+    for (int i = t / 4; i < b.ctas; i += 32) {
+        const float4 x = __ldcg(part + i * (b.cols / 4) + at);
+        v.x += x.x, v.y += x.y, v.z += x.z, v.w += x.w;
+    }
+    sh[t] = v;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (t < 4) {
+#pragma unroll 8
+        for (int k = 1; k < 32; ++k) {
+            const float4 x = sh[4 * k + t];
+            v.x += x.x, v.y += x.y, v.z += x.z, v.w += x.w;
+        }
+        reinterpret_cast<float4 *>(b.out)[at] = v;
+    }
+}
+
 template <int KIND>
 __global__ void __launch_bounds__(kGradThreads) sno_tc_grad_kernel(const __grid_constant__ CUtensorMap tmX,
                                                                    const __grid_constant__ CUtensorMap tmY,
@@ -705,6 +734,16 @@ __global__ void __launch_bounds__(kGradThreads) sno_tc_grad_kernel(const __grid_
     __shared__ uint32_t tmem_base_sh;
     __shared__ volatile int s_abort;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    if constexpr (KIND == 2) {
+        if ((int)blockIdx.y >= P.modes) {
+            __shared__ float4 sh[128];
+            const int c = (int)blockIdx.y - P.modes, first = P.bias[0].cols / 16;
+            after_previous();
+            if (t < 128)
+                add_bias_parts(P.bias[c < first ? 0 : 1], c < first ? c : c - first, sh);
+            return;
+        }
+    }
     if (t == 0) {
         for (int s = 0; s < ST; ++s) {
             bar_init(&full[s], 1);
@@ -834,18 +873,23 @@ __global__ void __launch_bounds__(kGradThreads) sno_tc_grad_kernel(const __grid_
                         dst[o * 64 + row] = h < 2 ? v + w : v - w;
                     }
                 }
-        } else if (ok && warp < 3) {
-            float *dst = row < 64 ? P.dw + row * N : P.db;
-            for (int h = 0; h < N / 32; ++h) {
-                uint32_t r[32];
-                tmem_ld32(taddr + 32 * h, r);
-                tmem_wait_ld();
-                if (row <= 64)
+        } else {
+            if (ok && warp < 3)
+                for (int h = 0; h < N / 32; ++h) {
+                    uint32_t r[32];
+                    tmem_ld32(taddr + 32 * h, r);
+                    tmem_wait_ld();
+                    float *dst = (row < 64 ? P.dw + row * N : P.part + (long long)blockIdx.x * N) + 32 * h;
 #pragma unroll
-                    for (int c = 0; c < 32; c += 4)
-                        red_add4(dst + 32 * h + c, __uint_as_float(r[c]), __uint_as_float(r[c + 1]),
-                                 __uint_as_float(r[c + 2]), __uint_as_float(r[c + 3]));
-            }
+                    for (int c = 0; c < 32; c += 4) {
+                        const float4 v = make_float4(__uint_as_float(r[c]), __uint_as_float(r[c + 1]),
+                                                     __uint_as_float(r[c + 2]), __uint_as_float(r[c + 3]));
+                        if (row < 64)
+                            red_add4(dst + c, v.x, v.y, v.z, v.w);
+                        else if (row == 64)
+                            *reinterpret_cast<float4 *>(dst + c) = v;
+                    }
+                }
         }
     }
     tc_fence_before();
@@ -1001,18 +1045,26 @@ cudaError_t sno_tc_mix(const void *map_vh, const void *map_wst, const SnoTcMixAr
                         *static_cast<const CUtensorMap *>(map_wst), a);
 }
 
+int sno_tc_grad_ctas(long long rows, int sms)
+{
+    const long long chunks = (rows + 127) / 128, per = (chunks + sms - 1) / sms;
+    return (int)(per > 0 ? (chunks + per - 1) / per : 0);
+}
+
 cudaError_t sno_tc_grad(const void *map_x, const void *map_y, const SnoTcGradArgs &a, int cols, int sms, cudaStream_t s)
 {
     if (cols != 64 && cols != 128)
         return cudaErrorInvalidValue;
-    const long long chunks = (a.rows + 127) / 128, per = (chunks + sms - 1) / sms;
-    const dim3 grid((unsigned)(per > 0 ? (chunks + per - 1) / per : 0), 1);
+    const dim3 grid((unsigned)sno_tc_grad_ctas(a.rows, sms), 1);
     return cols == 64 ? launch_grad<0>(map_x, map_y, a, grid, s) : launch_grad<1>(map_x, map_y, a, grid, s);
 }
 
 cudaError_t sno_tc_grad_spec(const void *map_vh, const void *map_dy, const SnoTcGradArgs &a, int modes, cudaStream_t s)
 {
-    return launch_grad<2>(map_vh, map_dy, a, dim3(1, (unsigned)modes), s);
+    SnoTcGradArgs b = a;
+    b.modes = modes;
+    const unsigned extra = (unsigned)(a.bias[0].cols + a.bias[1].cols) / 16;
+    return launch_grad<2>(map_vh, map_dy, b, dim3(1, (unsigned)modes + extra), s);
 }
 
 }  // namespace ge
