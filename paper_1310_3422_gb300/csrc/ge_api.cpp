@@ -414,6 +414,8 @@ void release(ge_ctx *c, bool idle = false)
         if (dev != c->device)
             cudaSetDevice(dev);
     }
+    if (c->prop.pins)
+        c->prop.pins->drop();
     delete c;
 }
 
@@ -485,8 +487,12 @@ ge_status ge_create(ge_ctx **out, int64_t n, double r, double beta_l, double bet
         return fail(GE_EINVAL, "ge_create: n = %lld is too large", (long long)n);
 
     ge_ctx *c = new (std::nothrow) ge_ctx();
-    if (!c)
+    if (c)
+        c->prop.pins = ge::PropPins::make();
+    if (!c || !c->prop.pins) {
+        release(c);
         return fail(GE_ENOMEM, "ge_create: host allocation failed");
+    }
     c->n = n;
     c->r = r;
     c->beta_l = beta_l;

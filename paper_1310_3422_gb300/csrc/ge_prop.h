@@ -15,6 +15,7 @@
 // reached by a reflection off both walls.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime_api.h>
 
@@ -58,16 +59,33 @@ struct PropSet {
     // host-side key and state
     int k, p0, entry, exit;
     int valid;          // arrays are written by work already on the stream
-    int pinned;         // a captured graph reads them
     long long used;
 };
 
 constexpr int kPropSets = 6;
 
+// Which operators captured graphs read: a count each, held by the graphs (and
+// whatever is instantiated from them) as user objects, which CUDA gives back
+// when the last of them is gone.  That may be after the context is, so the
+// counts have an owner count of their own.
+struct PropPins {
+    struct Slot {
+        std::atomic<int> graphs{0};
+        PropPins *owner = nullptr;
+    } slot[kPropSets];
+    std::atomic<int> owners{1};
+    static PropPins *make();  // NULL: out of memory
+    void drop();              // one owner less
+    // The graph that `stream` is being captured into reads operator i.
+    void pin(int i, cudaStream_t stream);
+    bool pinned(int i) const { return slot[i].graphs.load(std::memory_order_acquire) > 0; }
+};
+
 // Per-context state.
 struct PropState {
     void *mem = nullptr;          // one allocation for everything below
     PropSet set[kPropSets];
+    PropPins *pins = nullptr;
     double *scratch[2];           // the chain's ping-pong arrays (e, h)
     double *x = nullptr;          // rows for the digits, and the word of their largest
     int *list = nullptr;          // blocks that need dot products

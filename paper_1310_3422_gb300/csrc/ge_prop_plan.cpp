@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <new>
 
 namespace ge {
 
@@ -90,6 +91,47 @@ void tile_range(double r, int k, int f64, int *range, int *near)
 }
 
 }  // namespace
+
+PropPins *PropPins::make()
+{
+    PropPins *p = new (std::nothrow) PropPins();
+    for (int i = 0; p && i < kPropSets; ++i)
+        p->slot[i].owner = p;
+    return p;
+}
+
+void PropPins::drop()
+{
+    if (owners.fetch_sub(1, std::memory_order_acq_rel) == 1)
+        delete this;
+}
+
+void PropPins::pin(int i, cudaStream_t stream)
+{
+    Slot *s = &slot[i];
+    s->graphs.fetch_add(1, std::memory_order_relaxed);
+    owners.fetch_add(1, std::memory_order_relaxed);
+    // (called from a thread of CUDA's, where no CUDA call is allowed)
+    cudaHostFn_t gone = [](void *p) {
+        Slot *s = static_cast<Slot *>(p);
+        PropPins *owner = s->owner;
+        s->graphs.fetch_sub(1, std::memory_order_release);
+        owner->drop();
+    };
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    cudaUserObject_t object = nullptr;
+    bool held = cudaStreamGetCaptureInfo(stream, &cap, nullptr, &graph, nullptr, nullptr, nullptr) == cudaSuccess && graph &&
+                cudaUserObjectCreate(&object, s, gone, 1, cudaUserObjectNoDestructorSync) == cudaSuccess;
+    if (held && cudaGraphRetainUserObject(graph, object, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+        s->graphs.fetch_add(1, std::memory_order_relaxed);
+        owners.fetch_add(1, std::memory_order_relaxed);
+        cudaUserObjectRelease(object, 1);
+        held = false;
+    }
+    if (!held)
+        cudaGetLastError();  // the operator stays the graph's for the context's life
+}
 
 size_t prop_bytes(long long n, int f64) { return Sizes(n, f64).total(); }
 
@@ -331,30 +373,38 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
         for (PropSet &s : st->set)
             if (holds(s, need[i]))
                 need[i].set = &s;
+    // a slot for each of the others, the least recently used: all of them
+    // before any is given up
     for (int i = 0; i < needs; ++i) {
-        Need &w = need[i];
-        PropSet *s = w.set;
-        if (!s) {
-            for (PropSet &c : st->set) {
-                bool taken_here = c.pinned;
-                for (int j = 0; j < needs; ++j)
-                    taken_here = taken_here || need[j].set == &c;
-                if (!taken_here && (!s || c.used < s->used))
-                    s = &c;
-            }
-            if (!s)
-                return cudaSuccess;  // every slot belongs to a captured graph
-            s->k = w.k;
-            s->p0 = p0;
-            s->entry = w.entry;
-            s->exit = w.exit;
-            s->valid = 0;
-            w.set = s;
+        if (need[i].set)
+            continue;
+        PropSet *s = nullptr;
+        for (int z = 0; z < kPropSets; ++z) {
+            PropSet &c = st->set[z];
+            bool taken_here = st->pins->pinned(z);
+            for (int j = 0; j < needs; ++j)
+                taken_here = taken_here || need[j].set == &c;
+            if (!taken_here && (!s || c.used < s->used))
+                s = &c;
+        }
+        if (!s)
+            return cudaSuccess;  // every slot belongs to a captured graph
+        need[i].set = s;
+        need[i].build = true;
+    }
+    for (int i = 0; i < needs; ++i) {
+        PropSet &s = *need[i].set;
+        if (need[i].build) {
+            s.k = need[i].k;
+            s.p0 = p0;
+            s.entry = need[i].entry;
+            s.exit = need[i].exit;
+            s.valid = 0;
         }
         // arrays written inside a capture exist only once that graph runs:
         // outside one they count as missing
-        w.build = !s->valid;
-        s->used = ++st->clock;
+        need[i].build = !s.valid;
+        s.used = ++st->clock;
     }
     const double x2 = r / det;
     for (int i = 0; i < needs; ++i) {
@@ -366,7 +416,7 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
         if (w.build && (e = build_set(st, t, *w.set, pr, w.hb, stream)) != cudaSuccess)
             return e;
         if (capturing)
-            w.set->pinned = 1;
+            st->pins->pin((int)(w.set - st->set), stream);
         else
             w.set->valid = 1;
     }
