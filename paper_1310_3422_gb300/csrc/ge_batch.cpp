@@ -69,7 +69,7 @@ struct ge_batch {
     // tile geometry of the launches (ge_batch_set_geometry, ge_batch_tune):
     // rows per tile (256 or 128) and co-resident CTAs per SM (0: as many as fit)
     int tile_rows = 256, ctas_per_sm = 0;
-    bool shape_set = false;  // depth or geometry chosen by the caller or the tuner
+    bool depth_set = false, rows_set = false;  // chosen by the caller or the tuner
     int blocks_per_sm_128 = 0;
     // one persistent launch per run (plain FP32 plans; ge_batch_set_persistent)
     bool persistent = false;
@@ -508,8 +508,12 @@ ge_status ge_batch_set_kernel(ge_batch *b, ge_kernel kernel)
             return bcuda(e, "ge_batch_set_kernel: rescale table");
     }
     b->df = df;
-    if (!b->shape_set)
-        default_shape(b, &b->depth, &b->tile_rows);
+    int depth, rows;
+    default_shape(b, &depth, &rows);
+    if (!b->depth_set)
+        b->depth = depth;
+    if (!b->rows_set)
+        b->tile_rows = rows;
     if (df)
         b->tile_rows = 256;  // the double-float kernel has the 256-row tile only
     b->R = R;
@@ -531,7 +535,7 @@ ge_status ge_batch_set_depth(ge_batch *b, int32_t depth)
         b->depth = depth;
     else
         default_shape(b, &b->depth, &rows);
-    b->shape_set = true;
+    b->depth_set = depth != 0;
     return GE_OK;
 }
 
@@ -576,7 +580,7 @@ ge_status ge_batch_set_geometry(ge_batch *b, int32_t tile_rows, int32_t ctas_per
         return bfail(GE_EINVAL, "ge_batch_set_geometry: ctas_per_sm beyond what fits on an SM");
     b->tile_rows = tile_rows;
     b->ctas_per_sm = ctas_per_sm;
-    b->shape_set = true;
+    b->rows_set = true;
     return GE_OK;
 }
 
@@ -710,7 +714,7 @@ ge_status ge_batch_tune(ge_batch *b, const void *u_dev, int64_t steps, int32_t *
     b->depth = best_d;
     b->tile_rows = best_tr;
     b->ctas_per_sm = best_c;
-    b->shape_set = true;
+    b->depth_set = b->rows_set = true;
     b->persistent = best_persist;
     if (best_depth)
         *best_depth = best_d;

@@ -58,3 +58,29 @@ def test_batch_shape_by_size(prec, sizes):
         tol = tol64(r[i]) if prec == B.GE_F64 else 1e-5
         assert np.max(np.abs(got[off[i]:off[i] + n[i]] - want)) <= tol * np.max(np.abs(want)), i
     B.ge_batch_destroy(plan)
+
+
+@pytest.mark.parametrize("problems", [4, 600])
+def test_a_plans_own_choice_follows_its_kernel(problems):
+    """Depth 0 is the plan's own choice, for the kernel it runs at the time; a
+    chosen depth or geometry stays."""
+    n = np.full(problems, 4096, np.int64)
+    off = np.arange(problems, dtype=np.int64) * 4096
+    r, zero = np.full(problems, 1.0), np.zeros(problems)
+
+    def shape(*calls):
+        plan = B.ge_batch_create(n, r, zero, zero, off, problems * 4096, B.GE_F64)
+        for f, *args in calls:
+            f(plan, *args)
+        got = B.ge_batch_get_depth(plan), B.ge_batch_get_geometry(plan)[0]
+        B.ge_batch_destroy(plan)
+        return got
+
+    df, auto = (B.ge_batch_set_kernel, B.GE_KERNEL_TEMPORAL_DF), (B.ge_batch_set_kernel, B.GE_KERNEL_AUTO)
+    own, own_df = shape(), shape(df)
+    assert own_df == (48, 256) and own != own_df
+    assert shape((B.ge_batch_set_depth, 0)) == own and shape((B.ge_batch_set_depth, 0), df) == own_df
+    assert shape((B.ge_batch_set_depth, 96), (B.ge_batch_set_depth, 0), df) == own_df
+    assert shape((B.ge_batch_set_depth, 0), df, auto) == own
+    assert shape((B.ge_batch_set_depth, 96), df) == (96, 256)
+    assert shape((B.ge_batch_set_geometry, 256, 0), df, auto) == (own[0], 256)
