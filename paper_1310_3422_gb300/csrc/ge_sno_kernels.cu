@@ -919,42 +919,43 @@ __global__ void round_bf16_kernel(const float *__restrict__ x, float *__restrict
     }
 }
 
-// Lift without a GEMM (K = 4): one thread per point and 8 channels.
-// (see SnoPrepare)
+// (see SnoPrepare; I: an unsigned type that holds twice the parameters)
+template <typename I>
 __global__ void prepare_kernel(const SnoPrepare a)
 {
-    const unsigned c = a.c, cc = c * c, spec = a.modes * cc, lay0 = (unsigned)a.lay0, lay = (unsigned)a.lay_size;
-    const unsigned q1 = (unsigned)a.q1, d = 2 * c;
+    const I c = a.c, cc = c * c, spec = a.modes * cc, lay0 = (I)a.lay0, lay = (I)a.lay_size;
+    const I q1 = (I)a.q1, d = 2 * c;
     __nv_bfloat16 *pw16 = static_cast<__nv_bfloat16 *>(a.pw16), *wt = static_cast<__nv_bfloat16 *>(a.wt);
     __nv_bfloat16 *ws = static_cast<__nv_bfloat16 *>(a.ws), *wst = static_cast<__nv_bfloat16 *>(a.wst);
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (unsigned)a.count; i += gridDim.x * blockDim.x) {
+    for (I i = (I)blockIdx.x * blockDim.x + threadIdx.x; i < (I)a.count; i += (I)gridDim.x * blockDim.x) {
         const __nv_bfloat16 v = __float2bfloat16_rn(a.params[i]);
         a.pw[i] = __bfloat162float(v);
         pw16[i] = v;
         if (i >= lay0 && i - lay0 < lay * a.layers) {
-            const unsigned rel = i - lay0, l = rel / lay, o = rel - l * lay;
+            const I rel = i - lay0, l = rel / lay, o = rel - l * lay;
             if (o < 2 * spec) {
                 const bool im = o >= spec;
-                const unsigned q = im ? o - spec : o, m = q / cc, r = q - m * cc, out = r / c, in = r - out * c;
+                const I q = im ? o - spec : o, m = q / cc, r = q - m * cc, out = r / c, in = r - out * c;
                 const size_t base = (size_t)(l * a.modes + m) * 4 * cc;
                 // [[Rr^T, Ri^T], [-Ri^T, Rr^T]]
-                const unsigned r0 = in, c0 = im ? c + out : out, r1 = c + in, c1 = im ? out : c + out;
+                const I r0 = in, c0 = im ? c + out : out, r1 = c + in, c1 = im ? out : c + out;
                 const __nv_bfloat16 v1 = im ? __hneg(v) : v;
                 ws[base + r0 * d + c0] = v;
                 ws[base + r1 * d + c1] = v1;
                 wst[base + c0 * d + r0] = v;
                 wst[base + c1 * d + r1] = v1;
             } else if (o < 2 * spec + cc) {
-                const unsigned r = o - 2 * spec;
+                const I r = o - 2 * spec;
                 wt[(size_t)l * cc + (r % c) * c + r / c] = v;
             }
         } else if (i >= q1 && i - q1 < c * a.h) {
-            const unsigned r = i - q1;
+            const I r = i - q1;
             static_cast<__nv_bfloat16 *>(a.q1t)[(r % a.h) * c + r / a.h] = v;
         }
     }
 }
 
+// Lift without a GEMM (K = 4): one thread per point and 8 channels.
 constexpr int kLiftMaxC = 256;
 
 template <typename T, typename I>
@@ -1307,9 +1308,11 @@ cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int mod
 
 cudaError_t sno_prepare(const SnoPrepare &a, cudaStream_t s)
 {
-    if (a.count >= 1LL << 31)  // the kernel's 32-bit indices
-        return cudaErrorInvalidValue;
-    prepare_kernel<<<grid_for(a.count), 256, 0, s>>>(a);
+    // (64-bit divisions take three times as long)
+    if (a.count < 1LL << 31)
+        prepare_kernel<unsigned><<<grid_for(a.count), 256, 0, s>>>(a);
+    else
+        prepare_kernel<unsigned long long><<<grid_for(a.count), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

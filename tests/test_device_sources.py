@@ -87,3 +87,10 @@ def test_kernel_attributes_are_set_for_every_model():
     prepared = re.search(r"cudaError_t sno_tc_prepare.*?\n\}", text, re.S).group(0)
     assert kernels and kernels == set(re.findall(r"prepare_kernel\((\w+)", prepared))
     assert "sno_tc_prepare(&s->grid" in code("ge_sno.cpp")
+
+
+def test_weights_of_any_number_are_prepared():
+    """Models of 2^31 parameters and more (100 GB: no test makes one) take
+    64-bit indices instead of an error."""
+    body = re.search(r"cudaError_t sno_prepare\(.*?\n\}", code("ge_sno_kernels.cu"), re.S).group(0)
+    assert "cudaErrorInvalidValue" not in body and "prepare_kernel<unsigned long long>" in body
