@@ -41,8 +41,8 @@ void tb_fill_base(double r, double beta_l, double beta_r, int prec, TbParams *ou
         // and stays below 2^headroom (data magnitudes up to 2^(max_exp -
         // headroom - 1) are safe)
         const double headroom = (prec == 0) ? kF64Headroom : GE_F32_HEADROOM;
-        const int every = (int)std::floor(headroom / std::log2(1.0 + 2.0 * r));
-        p.rescale_every = every < 1 ? 1 : every;
+        const double every = std::floor(headroom / std::log2(1.0 + 2.0 * r));
+        p.rescale_every = every < 1.0 ? 1 : every > 1e9 ? 1000000000 : (int)every;
     }
     *out = p;
 }
@@ -50,7 +50,7 @@ void tb_fill_base(double r, double beta_l, double beta_r, int prec, TbParams *ou
 int tb_clamp_depth(const TbParams &base, int depth)
 {
     const int every = base.rescale_every;
-    if (every > 0 && depth > (kMaxRescale - 1) * every)
+    if (every > 0 && depth / (kMaxRescale - 1) >= every)
         depth = (kMaxRescale - 1) * every;
     if (depth > kMaxTableSteps)
         depth = kMaxTableSteps;
