@@ -173,9 +173,15 @@ void prop_carve(PropState *st, void *mem, long long n, int f64)
 //     costs what 200 steps of the FP32 pipes do; compensated 64 steps 95 /
 //     102 (2^20), 285 / 253 (2^24), 128 steps 308 / 441.
 // Later calls take half of that or less at these step counts.
+//   The compensated kernel rounds the state to FP32 where a launch ends, an
+// operator where it ends: grids too short for operators of as many steps (n -
+// 2 at most) keep the kernel (n = 19, r = 1e-4, 958 steps: 6.6e-8, composed
+// 3.4e-7).
 bool prop_takes(long long n, double r, long long steps, int prec)
 {
     if (n < kMinPoints || r < kMinR || r > kMaxR)
+        return false;
+    if (prec == 2 && n < kDefaultDepthF32 + 2)
         return false;
     const bool tiles = n >= kPropTileMin;
     long long least;

@@ -103,3 +103,24 @@ def test_quiet_stretches_keep_their_precision(prec, r, steps, level):
         inner[a + margin:a + 3000 - margin] = True
     auto, tiled = rms_errors(u0, r, 0.3, -0.8, steps, prec, inner)
     assert auto <= SLACK * tiled, (auto, tiled)
+
+
+# shorter than a launch of the compensated kernel, as long, and longer
+@pytest.mark.parametrize("n", [19, 41, 129, 130, 400])
+def test_short_compensated_grids(n):
+    """A state rounded to FP32 at the end of every operator errs no more than
+    one rounded at the end of every launch of the tiled kernel."""
+    auto, tiled = rms_errors(rough(16, n, np.float32), 1e-4, 0.25, -0.75, 958, B.GE_F32_COMP)
+    assert auto <= SLACK * tiled, (auto, tiled)
+
+
+@pytest.mark.parametrize("prec", [B.GE_F64, B.GE_F32])
+@pytest.mark.parametrize("r", [1.4e-6, 1e-7, 1e-12, 1e-300])
+def test_steps_that_hardly_move(prec, r):
+    """The tiled kernel at mesh ratios where its scale never needs taking down,
+    and the default path, whichever it takes."""
+    u0 = rough(1, 3000, np.float64 if prec == B.GE_F64 else np.float32)
+    want = exact(u0, r, 0.3, -0.8, 60)[0]
+    for kernel in (B.GE_KERNEL_TEMPORAL, B.GE_KERNEL_AUTO):
+        got = run(u0[0], r, 0.3, -0.8, 60, kernel, prec)
+        assert np.max(np.abs(got - want)) <= (1e-12 if prec == B.GE_F64 else 1e-5) * np.max(np.abs(want))
