@@ -320,6 +320,24 @@ __global__ void __launch_bounds__(128) prop_level_kernel(const PropLevel P)
     }
 }
 
+// round(x 2^E), at most 2^62 in magnitude.
+__device__ __forceinline__ long long fixed_of(double x, int E)
+{
+    const long long u = __double_as_longlong(x);
+    const int e = (int)(u >> 52) & 0x7ff;
+    unsigned long long m = (unsigned long long)u & 0x000fffffffffffffull;
+    if (e)
+        m |= 0x0010000000000000ull;
+    const int sh = (e ? e : 1) - 1075 + E;
+    if (sh >= 0) {
+        m <<= sh;
+    } else {
+        const int n = -sh < 60 ? -sh : 60;
+        m = (m + (1ull << (n - 1))) >> n;
+    }
+    return u < 0 ? -(long long)m : (long long)m;
+}
+
 // ---- the finished operator
 
 // The finished operator from the last level's arrays (small blocks, to spread
@@ -337,27 +355,27 @@ constexpr int kFinishThreads = 64;
 
 __global__ void __launch_bounds__(kFinishThreads) prop_finish_kernel(const PropLevel P, const PropFinish Q)
 {
-    __shared__ double part[kFinishThreads / 32];
+    __shared__ long long part[kFinishThreads / 32];
     __shared__ double s_miss;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, R = P.R1;
     {
-        double s = 0.0;
+        // (as integers: rounded sums would leave every row a common error of
+        // 2^-53, which adds up over the operators of a call)
+        long long s = 0;
         for (int i = -R + t; i <= R; i += kFinishThreads)
-            s += P.e0[i];
-        s = warp_sum(s);
+            s += fixed_of(P.e0[i], 62) + fixed_of(P.el0[i], 62);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0)
             part[warp] = s;
     }
     __syncthreads();
-    if (warp == 0) {
-        Dd m{-1.0, 0.0};
-        for (int i = 0; i < kFinishThreads / 32; ++i) {
-            const Dd x = two_sum(m.hi, part[i]);
-            m.hi = x.hi;
-            m.lo += x.lo;
-        }
-        if (t == 0)
-            s_miss = -(m.hi + m.lo);
+    if (t == 0) {
+        long long s = 1ll << 62;
+        for (int i = 0; i < kFinishThreads / 32; ++i)
+            s -= part[i];
+        s_miss = (double)s * 0x1p-62;
     }
     __syncthreads();
     const double miss = s_miss;
@@ -419,24 +437,6 @@ __global__ void __launch_bounds__(kFinishThreads) prop_finish_kernel(const PropL
 // d = 56 + W_i - rho + t, t = 0..7, and the operand's piece (n, k = 8c) is
 // row n - 8c + 56 + 2 W_i.
 constexpr int kPropQ = 2 * kPropRMax + 13;
-
-// round(x 2^E), below 2^62 in magnitude.
-__device__ __forceinline__ long long fixed_of(double x, int E)
-{
-    const long long u = __double_as_longlong(x);
-    const int e = (int)(u >> 52) & 0x7ff;
-    unsigned long long m = (unsigned long long)u & 0x000fffffffffffffull;
-    if (e)
-        m |= 0x0010000000000000ull;
-    const int sh = (e ? e : 1) - 1075 + E;
-    if (sh >= 0) {
-        m <<= sh;
-    } else {
-        const int n = -sh < 60 ? -sh : 60;
-        m = (m + (1ull << (n - 1))) >> n;
-    }
-    return u < 0 ? -(long long)m : (long long)m;
-}
 
 __global__ void __launch_bounds__(1024) prop_digits_kernel(const double *x, const unsigned long long *x_max, int R,
                                                            int nd, int comp, int hb_max, int tab_cap, unsigned char *tab,

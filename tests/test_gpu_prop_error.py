@@ -124,3 +124,13 @@ def test_steps_that_hardly_move(prec, r):
     for kernel in (B.GE_KERNEL_TEMPORAL, B.GE_KERNEL_AUTO):
         got = run(u0[0], r, 0.3, -0.8, 60, kernel, prec)
         assert np.max(np.abs(got - want)) <= (1e-12 if prec == B.GE_F64 else 1e-5) * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("n,r,steps", [(24, 0.003, 2000), (100, 1.0, 4000), (300, 1.0, 6000), (1000, 4.0, 5000)])
+def test_many_operators_one_after_the_other(n, r, steps):
+    """Twenty and more operators: what each has wrong in common with the last
+    adds up, and stays below what the steps one by one add up."""
+    x = np.arange(1, n + 1) / (n + 1)
+    for u0 in (rough(2, n), np.stack([np.sin(3 * np.pi * x) + 0.2 * np.sin(40 * np.pi * x)])):
+        auto, tiled = rms_errors(u0, r, 0.3, -0.8, steps, B.GE_F64)
+        assert auto <= SLACK * tiled, (auto, tiled)
