@@ -141,7 +141,9 @@ ge_status ge_create(ge_ctx **out, int64_t n, double r, double beta_l, double bet
 
 /* Select the kernel used by later ge_step_n calls.  depth: steps per launch
  * for GE_KERNEL_TEMPORAL and GE_KERNEL_TEMPORAL_DF, 1..1023 (0 = built-in
- * default); ignored otherwise.
+ * default).  GE_KERNEL_AUTO takes it for the calls that it leaves to
+ * GE_KERNEL_TEMPORAL and for sub-domains of width k > 1; composed steps have
+ * no depth.  Ignored otherwise.
  * Errors: GE_EINVAL (NULL ctx, unknown kernel, depth out of range,
  * GE_KERNEL_CANONICAL with GE_F32_COMP, GE_KERNEL_TEMPORAL_DF with a
  * precision other than GE_F64 or with r > 2^20). */
@@ -155,7 +157,10 @@ ge_status ge_get_kernel(const ge_ctx *ctx, ge_kernel *kernel, int32_t *depth);
  * current state at each candidate depth (FP64: 24, 32, 48, 64, 96; FP32:
  * 64 ... 256; double-float: 32 ... 128), keeps the fastest (returned in *best_depth, may be NULL) and
  * leaves the state and the step counter as they were.  A context on the
- * canonical, one-step or width-k path keeps its setting.  Synchronous;
+ * canonical, one-step or width-k path keeps its setting.  With GE_KERNEL_AUTO
+ * the depth is for the calls left to GE_KERNEL_TEMPORAL, as it is from the
+ * tuning table: composed steps, which most calls of 130 steps and more take,
+ * are faster than any depth and not timed here.  Synchronous;
  * allocates one scratch copy of the state.  Errors: GE_EINVAL, GE_ENOMEM,
  * GE_ECUDA. */
 ge_status ge_tune(ge_ctx *ctx, int64_t steps, int32_t *best_depth);
