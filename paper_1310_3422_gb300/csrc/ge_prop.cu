@@ -313,10 +313,8 @@ __global__ void __launch_bounds__(128) prop_level_kernel(const PropLevel P)
         return;
     if (wall) {
         P.h1[pb * P.hs + j] = v;
-        P.hl1[pb * P.hs + j] = 0.0;
     } else {
         P.e1[j] = v;
-        P.el1[j] = 0.0;
     }
 }
 
@@ -355,6 +353,7 @@ constexpr int kFinishThreads = 64;
 
 __global__ void __launch_bounds__(kFinishThreads) prop_finish_kernel(const PropLevel P, const PropFinish Q)
 {
+    auto e_low = [&](int d) { return P.el0 ? P.el0[d] : 0.0; };
     __shared__ long long part[kFinishThreads / 32];
     __shared__ double s_miss;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, R = P.R1;
@@ -363,7 +362,7 @@ __global__ void __launch_bounds__(kFinishThreads) prop_finish_kernel(const PropL
         // 2^-53, which adds up over the operators of a call)
         long long s = 0;
         for (int i = -R + t; i <= R; i += kFinishThreads)
-            s += fixed_of(P.e0[i], 62) + fixed_of(P.el0[i], 62);
+            s += fixed_of(P.e0[i], 62) + fixed_of(e_low(i), 62);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
             s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -381,19 +380,20 @@ __global__ void __launch_bounds__(kFinishThreads) prop_finish_kernel(const PropL
     const double miss = s_miss;
     const int gid = blockIdx.x * kFinishThreads + t, n_int = 2 * R + 1, n_h = 4 * (R + 1), RX = R + 4, n_x = 2 * (2 * RX + 1);
     if (gid < n_int) {
-        P.e1[gid - R] = P.e0[gid - R] + fma(miss, P.e0[gid - R], P.el0[gid - R]);
+        P.e1[gid - R] = P.e0[gid - R] + fma(miss, P.e0[gid - R], e_low(gid - R));
     } else if (gid < n_int + n_h) {
         const int w = gid - n_int, i = w / (R + 1) * P.hs + w % (R + 1);
-        P.h1[i] = P.h0[i] + fma(miss, P.h0[i], P.hl0[i]);
+        P.h1[i] = P.h0[i] + fma(miss, P.h0[i], P.hl0 ? P.hl0[i] : 0.0);
     } else if (Q.x && gid < n_int + n_h + n_x) {
         const int i = gid - n_int - n_h, phase = i & 1, d = (i >> 1) - RX;
         const int s = ((phase ^ Q.p0 ^ Q.k) & 1) ? -1 : 1, a = Q.p0 ^ phase;
         // the row with the exit, at column phase + d
         auto row = [&](int d) {
-            Dd v{tap(P.e0, R, a, d), tap(P.el0, R, a, d)};
+            auto low = [&](int q_phase, int x) { return P.el0 ? tap(P.el0, R, q_phase, x) : 0.0; };
+            Dd v{tap(P.e0, R, a, d), low(a, d)};
             if (Q.exit)
                 v = dd_add(dd_mul(Dd{Q.x1, 0.0}, v),
-                           dd_mul(Dd{Q.x2, 0.0}, Dd{tap(P.e0, R, a ^ 1, d - s), tap(P.el0, R, a ^ 1, d - s)}));
+                           dd_mul(Dd{Q.x2, 0.0}, Dd{tap(P.e0, R, a ^ 1, d - s), low(a ^ 1, d - s)}));
             return v;
         };
         Dd v = row(d);

@@ -151,8 +151,8 @@ struct PropCoef {
 
 // One doubling of the chain (k1 -> 2 k1 + delta), or its end.
 struct PropLevel {
-    const double *e0, *el0, *h0, *hl0;
-    double *e1, *el1, *h1, *hl1;
+    const double *e0, *el0, *h0, *hl0;  // el0, hl0: the low parts, or NULL
+    double *e1, *h1;
     int k1, R1, R2, delta, hs;
     int par;  // start parities whose wall arrays are needed (bit p)
     PropCoef c;

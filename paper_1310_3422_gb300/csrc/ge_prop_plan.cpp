@@ -281,18 +281,16 @@ cudaError_t build_set(PropState *st, const PropTarget &t, PropSet &s, int pr, in
     }
     auto set_in = [&] {
         a.e0 = in[0];
-        a.el0 = in[1];
+        a.el0 = k1 == s.k >> levels ? in[1] : nullptr;  // a doubling leaves FP64 taps
         a.h0 = in[2];
-        a.hl0 = in[3];
+        a.hl0 = a.el0 ? in[3] : nullptr;
         a.k1 = k1;
         a.R1 = std::min(k1 + 1, Rlim);
     };
     for (int bit = levels - 1; bit >= 0 && e == cudaSuccess; --bit) {
         set_in();
         a.e1 = out[0];
-        a.el1 = out[1];
         a.h1 = out[2];
-        a.hl1 = out[3];
         a.delta = (s.k >> bit) & 1;
         k1 = 2 * k1 + a.delta;
         a.R2 = std::min(k1 + 1, Rlim);

@@ -265,7 +265,7 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
         if (rc != GE_OK)
             return rc;
     } else {
-        SNO_TRY(ge::sno_round_bf16(s->params, s->pw, nullptr, s->n_params, st));
+        SNO_TRY(ge::sno_round_bf16(s->params, s->pw, s->n_params, st));
     }
     // lift (K = 4: no GEMM); the features themselves only for the backward pass
     if (keep)
@@ -276,7 +276,7 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
         const LayerOff &o = s->lay[l];
         void *ws = at(s->wspec, (long long)l * M * 4 * C * C, bf);
         if (!bf)
-            SNO_TRY(ge::sno_spec_assemble(P + o.rr, P + o.ri, ws, M, C, 0, st));
+            SNO_TRY(ge::sno_spec_assemble(P + o.rr, P + o.ri, static_cast<float *>(ws), M, C, st));
         // truncated DFT along the grid: vh[b] = F [2M x n] * v[b] [n x C]
         g = gemm(F, n, 1, s->v[l], C, 1, s->vh[l], C, 2 * M, C, n);
         g.sA = 0;
@@ -332,8 +332,9 @@ ge_status forward(ge_sno *s, int B, const float *u0, const float *r, const float
     g.bias = P + s->off_qb1;
     g.act = s->h;
     SNO_TRY(ge::sno_gemm(act_fmt(g, bf), 1, s->split, st));
-    // (a warp per row takes 16 us instead of 23, but sums in another order: where
-    // pred is close to its target, 1e-8 of pred is 2e-6 of the gradients)
+    // (23 us for 64 problems, a GEMM tile of which one column is used; but the
+    // loss sees the order of this sum: where pred is close to its target, 1e-8
+    // of pred is 2e-6 of the gradients)
     g = gemm(s->h, H, 1, weight(s, s->off_q2), 1, 1, out, 1, (int)R, 1, H);
     g.bias = P + s->off_qb2;
     g.C0 = u0;

@@ -145,7 +145,7 @@ cudaError_t sno_tc_grad_spec(const void *map_vh, const void *map_dy, const SnoTc
                              cudaStream_t s);
 cudaError_t sno_features(const float *u0, const float *r, const float *bl, const float *br, void *f, int batch,
                          int n, int bf16, cudaStream_t s);
-cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int modes, int c, int bf16, cudaStream_t s);
+cudaError_t sno_spec_assemble(const float *rr, const float *ri, float *w, int modes, int c, cudaStream_t s);
 cudaError_t sno_spec_reduce(const float *dw, float *drr, float *dri, int modes, int c, cudaStream_t s);
 // Column sums of x [rows][cols], plain and weighted by w [rows][ldw]'s first
 // nw (0, 1 or 4) columns; sum, wsum [nw][cols] and wtot (of w's first column)
@@ -160,7 +160,7 @@ struct SnoSums {
     float *part;
     int *ticket;
     float *sum, *wsum, *wtot;
-    // nw = 1: also out[i, j] = w[i] q[j] GELU'(pre[i, j]), unless out is NULL
+    // nw = 1: also out[i, j] = w[i] q[j] GELU'(pre[i, j])
     const void *q, *pre;
     void *out;
 };
@@ -185,7 +185,7 @@ struct SnoPrepare {
     long long q1;              // first parameter of Q1
 };
 cudaError_t sno_prepare(const SnoPrepare &a, cudaStream_t s);
-cudaError_t sno_round_bf16(const float *x, float *y, void *y16, long long n, cudaStream_t s);
+cudaError_t sno_round_bf16(const float *x, float *y, long long n, cudaStream_t s);
 // v0[b n + j][c] = b0[c] + sum_k feature_k(b, j) W0[k][c] (features as in
 // sno_features, rounded to BF16 when bf16); W0 BF16 or FP32 as v0.
 cudaError_t sno_lift(const float *u0, const float *r, const float *bl, const float *br, const void *w0,

@@ -620,7 +620,7 @@ __global__ void features_kernel(const float *__restrict__ u0, const float *__res
 // vector (re, im): [[Rr^T, Ri^T], [-Ri^T, Rr^T]] with R = Rr + i Ri (C x C,
 // out x in).  Layout of rr/ri: [m][out][in]; of w: [m][2C][2C].
 __global__ void spec_assemble_kernel(const float *__restrict__ rr, const float *__restrict__ ri,
-                                     void *__restrict__ w, int modes, int c, int bf16)
+                                     float *__restrict__ w, int modes, int c)
 {
     const long long total = (long long)modes * 2 * c * 2 * c;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
@@ -639,10 +639,7 @@ __global__ void spec_assemble_kernel(const float *__restrict__ rr, const float *
             v = -ri[ro];
         else
             v = rr[ro];
-        if (bf16)
-            static_cast<__nv_bfloat16 *>(w)[e] = __float2bfloat16_rn(v);
-        else
-            static_cast<float *>(w)[e] = v;
+        w[e] = v;
     }
 }
 
@@ -699,7 +696,7 @@ __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float
 // With NW = 4 and w the features it is the lift's weight gradient, with NW =
 // 1 and w the output's gradient that of the last projection: products with 4
 // or 1 rows, which a 64-row GEMM tile took 81 and 42 us for (65,536 rows).
-// HEAD (with NW = 1) also writes the gradient of the hidden layer's
+// NW = 1 also writes the gradient of the hidden layer's
 // pre-activation in the same pass, out[i, j] = w[i] q[j] GELU'(pre[i, j]); as
 // a GEMM with K = 1 it took 52 us for 65,536 x 128 BF16.
 // Bound by reading x once: blocks of 256 threads take rows in turn, 16 bytes
@@ -712,11 +709,11 @@ __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float
 // (21.6 + 12.4 and 32.7 us before the last block's sums were shared).
 constexpr int kSumBlocks = 192;
 
-template <typename T, int NW, bool V, bool HEAD>
+template <typename T, int NW, bool V>
 __global__ void __launch_bounds__(256) colsum_kernel(const SnoSums a)
 {
     constexpr int E = V ? Chunk<T>::E : 1, TPR = V ? 64 / E : 32, CW = E * TPR, G = 256 / TPR, S = 1 + NW;
-    static_assert(!HEAD || NW == 1, "the weight is the output's gradient");
+    constexpr bool HEAD = NW == 1;
     __shared__ float red[256 / CW > G ? 256 / CW : G][CW];
     __shared__ float tot[G];
     __shared__ int last;
@@ -908,14 +905,10 @@ __global__ void adam_kernel(float *__restrict__ p, const float *__restrict__ g, 
 
 // Round to the nearest BF16 value: the network's weights as the BF16 model
 // sees them, kept in FP32 storage (y) and, when y16 is set, as BF16.
-__global__ void round_bf16_kernel(const float *__restrict__ x, float *__restrict__ y, __nv_bfloat16 *__restrict__ y16,
-                                  long long n)
+__global__ void round_bf16_kernel(const float *__restrict__ x, float *__restrict__ y, long long n)
 {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(x[i]);
-        y[i] = __bfloat162float(h);
-        if (y16)
-            y16[i] = h;
+        y[i] = __bfloat162float(__float2bfloat16_rn(x[i]));
     }
 }
 
@@ -1300,9 +1293,9 @@ cudaError_t sno_features(const float *u0, const float *r, const float *bl, const
     return cudaGetLastError();
 }
 
-cudaError_t sno_spec_assemble(const float *rr, const float *ri, void *w, int modes, int c, int bf16, cudaStream_t s)
+cudaError_t sno_spec_assemble(const float *rr, const float *ri, float *w, int modes, int c, cudaStream_t s)
 {
-    spec_assemble_kernel<<<grid_for(4LL * modes * c * c), 256, 0, s>>>(rr, ri, w, modes, c, bf16);
+    spec_assemble_kernel<<<grid_for(4LL * modes * c * c), 256, 0, s>>>(rr, ri, w, modes, c);
     return cudaGetLastError();
 }
 
@@ -1324,32 +1317,30 @@ cudaError_t sno_spec_reduce(const float *dw, float *drr, float *dri, int modes, 
 
 namespace {
 
-template <typename T, int NW, bool HEAD>
+template <typename T, int NW>
 void launch_colsum(const SnoSums &a, cudaStream_t s)
 {
     const uintptr_t at = reinterpret_cast<uintptr_t>(a.x) |
-                         (HEAD ? reinterpret_cast<uintptr_t>(a.pre) | reinterpret_cast<uintptr_t>(a.out) : 0) |
+                         (NW == 1 ? reinterpret_cast<uintptr_t>(a.pre) | reinterpret_cast<uintptr_t>(a.out) : 0) |
                          (NW == 4 ? reinterpret_cast<uintptr_t>(a.w) : 0);
     const bool v = a.cols % Chunk<T>::E == 0 && (at & 15) == 0 && (NW != 4 || a.ldw == Chunk<T>::E);
     const int cw = v ? 64 : 32;
     const dim3 grid(kSumBlocks, (a.cols + cw - 1) / cw);
     if (v)
-        colsum_kernel<T, NW, true, HEAD><<<grid, 256, 0, s>>>(a);
+        colsum_kernel<T, NW, true><<<grid, 256, 0, s>>>(a);
     else
-        colsum_kernel<T, NW, false, HEAD><<<grid, 256, 0, s>>>(a);
+        colsum_kernel<T, NW, false><<<grid, 256, 0, s>>>(a);
 }
 
 template <typename T>
 cudaError_t pick_colsum(const SnoSums &a, cudaStream_t s)
 {
     if (a.nw == 0)
-        launch_colsum<T, 0, false>(a, s);
-    else if (a.nw == 1 && a.out)
-        launch_colsum<T, 1, true>(a, s);
+        launch_colsum<T, 0>(a, s);
     else if (a.nw == 1)
-        launch_colsum<T, 1, false>(a, s);
+        launch_colsum<T, 1>(a, s);
     else if (a.nw == 4)
-        launch_colsum<T, 4, false>(a, s);
+        launch_colsum<T, 4>(a, s);
     else
         return cudaErrorInvalidValue;
     return cudaGetLastError();
@@ -1450,9 +1441,9 @@ cudaError_t sno_dot_finish(const float *u0, const float *q2, const float *part, 
     return cudaGetLastError();
 }
 
-cudaError_t sno_round_bf16(const float *x, float *y, void *y16, long long n, cudaStream_t s)
+cudaError_t sno_round_bf16(const float *x, float *y, long long n, cudaStream_t s)
 {
-    round_bf16_kernel<<<grid_for(n), 256, 0, s>>>(x, y, static_cast<__nv_bfloat16 *>(y16), n);
+    round_bf16_kernel<<<grid_for(n), 256, 0, s>>>(x, y, n);
     return cudaGetLastError();
 }
 
