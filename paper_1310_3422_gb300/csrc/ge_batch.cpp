@@ -124,9 +124,10 @@ void release_batch(ge_batch *b)
 // steps: 4971 -> 4803 us at 64), and with few tiles, where a run is a chain
 // of launches each as long as one tile, deeper (64 problems of up to 4096
 // points, 300 steps: 532 -> 417 us at 192).  FP32 launches keep their 64
-// steps: where a launch ends decides where the scaled form rounds, and FP32
-// results, the surrogate's training targets among them, stay what they were
-// bit for bit (128 steps would take 5916 us; ge_batch_tune finds it).  The
+// steps, although 128 take 5916 us (ge_batch_tune finds them): where a launch
+// ends decides where the scaled form rounds, and targets 1e-7 off move the
+// gradient of the surrogate's relative loss by up to 1.5e-3 of a block's
+// largest where a prediction is close to its target.  The
 // compensated and the double-float plans keep the shape they were tuned at.
 void default_shape(const ge_batch *b, int *depth, int *tile_rows)
 {

@@ -991,7 +991,7 @@ static_assert((kDotWin + kEdgeScratch + dot_taps(kPropR64Max)) * 8 <= kTileSmem<
 // The conversion is not shared: a digit product's window is its own, and
 // their union is nearly the whole one.  The launcher weighs the tile's time
 // against that of the wall rows, which need the CTAs without a tile: n =
-// 100,003, k = 1999, FP64 takes 4 CTAs a tile, 68 -> 49 us a call (8: 57, 2:
+// 100,003, k = 1999, FP64 takes 4 CTAs a tile, 68 -> 42 us a call (8: 57, 2:
 // 59); n = 500,000 takes 2, 82 -> 67 us; n = 300,001, FP32, two operators:
 // 100 -> 82 us.
 template <typename T>

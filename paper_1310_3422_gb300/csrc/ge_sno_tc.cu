@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(kMixThreads) sno_tc_mix_kernel(const __grid_co
 //       few more CTAs add the bias parts meanwhile.
 // Bound by the latency of the loads and of the adds (16 MB in KIND 0: 2.4 us
 // at the copy rate).  65,536 rows, cold caches: KIND 0 takes 11.1 us, KIND 1
-// 12.9 us; as mma.sync tiles with split K, a column-sum pass and a memset
+// 12.5 us; as mma.sync tiles with split K, a column-sum pass and a memset
 // they took 38 and 40 us.  KIND 2, 64 problems: 7.5 us, before 19.4 us with
 // the folding as a pass of its own.
 template <int KIND>
