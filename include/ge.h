@@ -71,10 +71,9 @@ typedef enum {
                                 and 2^-39; one rounding a pass) and as dot
                                 products near the walls and in the blocks of
                                 64 points that would keep fewer digits so than
-                                step by step: those whose values lie below
-                                2^-8 (FP32: 2^-5; less where the taps smooth
-                                more) of the values that reach them, or whose
-                                results need more bits than the sums have; the
+                                step by step: those whose results need more
+                                bits than the sums have, or whose values lie
+                                below 2^-10 of the values that reach them; the
                                 dot products keep them down to 2^-100 of what
                                 reaches them.  Each tap of more than 31 steps
                                 carries a few FP64 roundings (2^-53 of itself).

@@ -708,11 +708,13 @@ template <typename T>
 constexpr int kCodeInf = sizeof(T) == 8 ? 2047 : 255;
 
 // Whether a tile leaves a block to dot products for its values: the code of
-// its largest, of the window's and of the cone's.
+// its largest, of the window's and of the cone's.  (Where the results will be
+// looked at, they decide, and the values only spare the tile a lost cause:
+// where a smooth field crosses zero they may be small.)
 template <typename T>
-__device__ __forceinline__ bool values_too_small(const PropRun &P, int q, int ref, int cone)
+__device__ __forceinline__ bool values_too_small(const PropRun &P, int keep, int q, int ref, int cone)
 {
-    return cone == kCodeInf<T> || q == 0 || q < ref - P.range || q < cone - TileShape<T>::kFar;
+    return cone == kCodeInf<T> || q == 0 || q < ref - P.range - (keep > 0 ? 4 : 0) || q < cone - TileShape<T>::kFar;
 }
 
 // Whether it does for its results: bits[0] those of block `row`'s largest sum.
@@ -1237,7 +1239,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_tile_kernel(const __grid
         bool listed = false;  // block t
         if (t < nb) {
             s_bits[t] = 0;
-            listed = cone > 0 && (!ok_tab || values_too_small<T>(P, s_code[hb + t], ref, cone));
+            listed = cone > 0 && (!ok_tab || values_too_small<T>(P, s_hdr.keep, s_code[hb + t], ref, cone));
             if (listed && rank == 0)
                 P.list[atomicAdd(P.count, 1)] = (int)(b0 + t);
             else if (!listed && cone > 0)
@@ -1684,7 +1686,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) prop_duo_kernel(const __grid_
             bool listed = false;  // block tt
             if (tt < nb) {
                 s_bits[m][tt] = 0;
-                listed = cone > 0 && (!ok_tab || values_too_small<T>(P, s_code[m][hb + tt], ref, cone));
+                listed = cone > 0 && (!ok_tab || values_too_small<T>(P, s_hdr.keep, s_code[m][hb + tt], ref, cone));
                 if (listed)
                     P.list[atomicAdd(P.count, 1)] = (int)(b0 + tt);
                 else if (cone > 0)

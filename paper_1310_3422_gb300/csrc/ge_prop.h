@@ -130,9 +130,10 @@ struct PropRun {
     // tiles: blocks [blk0, blk1) in tiles of `per`, hb halo blocks per side
     long long blk0, blk1, tiles;
     int per, hb;
-    // a block is left to dot products when its values lie below 2^-range of
-    // the largest of the tile's window, or when its results (and those of
-    // `near` blocks a side) are too far below that (PropHeader::keep)
+    // a block is left to dot products when its values lie below 2^-range
+    // (2^-(range + 4) with a PropHeader::keep) of the largest of the tile's
+    // window, or its results and those of `near` blocks a side have fewer bits
+    // than PropHeader::keep
     int range, near;
     // dot products: rows [0, rows_l) and [row_r, n), and the listed blocks
     long long rows_l, row_r;

@@ -77,7 +77,8 @@ int halo_blocks(double r, int k, int f64)
 // window's largest, and the rounding of that is smoothed as the values are:
 // for taps of standard deviation d its root mean square shrinks by S =
 // (2 sqrt(pi) d)^-1/2.  `range` keeps it below 2^-54 (2^-25) of a block's
-// largest value, which storing the result may cost as well.
+// largest value, which storing the result may cost as well; where the results
+// are looked at (PropHeader::keep), blocks of 2^-4 of that go on to there.
 //   Past d = 48 points the steps one by one give a block the errors of the
 // blocks beside it (where a smooth field crosses zero, say), and its results
 // are looked at together with theirs.
