@@ -474,11 +474,12 @@ cudaError_t prop_run(PropState *st, const PropTarget &t, int *cur, long long ste
             a.row_r = a.blk1 * kPropBlk;
             // listed blocks past which the whole grid step by step is sooner
             // done than their dot products: a block's 64 rows of 2 R taps at
-            // 2e11 multiply-adds a second, against the tiled kernel's rate
-            // and its wall tiles' time a step
+            // 2e11 multiply-adds a second and 85 ns for its eight items' set-up
+            // (3 us each on 304 CTAs), against the tiled kernel's rate and its
+            // wall tiles' time a step
             const double rate = t.prec == 0 ? 8e11 : t.prec == 1 ? 1.8e13 : 5.8e12, wall = t.prec == 0 ? 4.4e-6 : 0.85e-6;
             const double tiled_s = std::max((double)t.n * s.k / rate, wall * s.k) + 20e-6;
-            a.gate_min = (int)std::min(tiled_s / (128.0 * a.R / 2e11), 2e9);
+            a.gate_min = (int)std::min(tiled_s / (128.0 * a.R / 2e11 + 85e-9), 2e9);
             const bool gated = a.gate_min < a.blk1 - a.blk0 &&
                                tb_plan_rounds(t.tiled, *t.base, t.growth_lo, t.prec, *cur, p0, s.k, s.entry, s.exit,
                                               t.depth, &st->rounds);

@@ -248,3 +248,29 @@ def test_two_teams_with_the_largest_tables(r, steps):
     n = 304 * 8192 + 64 * 22 * 2 + 1
     u0 = inputs.random_state(n, seed=7).astype(np.float32).astype(np.float64)
     assert rel_max(auto_run(u0, r, 0.3, -0.8, steps, B.GE_F32), tiled_run(u0, r, 0.3, -0.8, steps, B.GE_F32)) <= 2e-5
+
+
+@pytest.mark.parametrize("prec,n,r,steps", [(B.GE_F64, 327663, 7.0, 36), (B.GE_F32, 1942719, 3e-5, 803)])
+def test_spikes_cost_no_multiple_of_the_tiled_kernel(prec, n, r, steps):
+    """Taps of a few points, nearly every block left to dot products: their
+    set-up counts, and the steps themselves are sooner done.  (The pass of the
+    tiles that finds out costs up to a third of a call here: twice is allowed.)"""
+    x = torch.zeros(n, dtype=B.dtype_of(prec), device=DEV)
+    x[::4999] = 1.0
+    ms = {}
+    for kernel in (B.GE_KERNEL_AUTO, B.GE_KERNEL_TEMPORAL):
+        ctx = B.ge_create(n, r, 0.5, 0.0, prec, x)
+        B.ge_set_kernel(ctx, kernel, 0)
+        times = []
+        for _ in range(6):
+            start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            B.ge_write_state(ctx, x, 0)
+            start.record()
+            B.ge_step_n(ctx, steps)
+            end.record()
+            B.ge_sync(ctx)
+            torch.cuda.synchronize()
+            times.append(start.elapsed_time(end))
+        ms[kernel] = min(times)
+        B.ge_destroy(ctx)
+    assert ms[B.GE_KERNEL_AUTO] <= 2.0 * ms[B.GE_KERNEL_TEMPORAL], ms
