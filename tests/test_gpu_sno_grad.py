@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from paper_1310_3422_gb300 import binding as B
-from test_gpu_sno import FULL, make_model
+from test_gpu_sno import FULL, make_model, test_tensor_core_path_matches_the_mma_path as inference_matches
 from test_gpu_sno_train import loss_grad
 
 pytestmark = pytest.mark.gpu
@@ -44,3 +44,10 @@ def test_all_but_the_matrices_are_the_same_from_run_to_run(batch):
             if k[0] != "W" and k != "Q1":
                 assert np.array_equal(got[k], want[k]), k
     B.ge_sno_destroy(m)
+
+
+@pytest.mark.parametrize("batch", [152, 153])
+def test_inference_on_either_side_of_the_transform_kernels_line(batch):
+    """One problem per SM has all eight chunks of its transform in flight, more
+    problems two: the last batch of the one kernel on 152 SMs, the first of the other."""
+    inference_matches(batch)
